@@ -324,7 +324,7 @@ int adg_step_noalloc(adg_ctx* ctx, void* d_Q, int n_steps, void* stream);
  * into launches is chosen per kernel kind by timing the candidates on this
  * context's own clusters with CUDA events (whole macro steps, per-phase
  * events as in adg_profile, after one untimed macro step):
- *   choice[0] / [1]: threads per element block of the CUDA-core local /
+ *   choice[0] / [1]: threads per block of the CUDA-core local /
  *                    neighbour kernels, of {64, 128, 256};
  *   choice[2] / [3]: consecutive 12-element tiles one CTA slot of the
  *                    tensor-core local / neighbour kernel takes per sweep

@@ -167,6 +167,51 @@ M9 boundary_matrix(const M9& TA, const M9& Ti, double Zp, double Zs, int tag) {
 }
 
 // ---------------- Gauss-Legendre on [0,1] (Newton on P_n) ----------------
+// Coefficients of one face for the row kernels (kernels.cuh, CREC) from the
+// middle state of Sec. 4.2 (Eq. boundary-state), a linear boundary's ghost
+// folded into the own side (free surface: traction mirrored; rigid wall: normal
+// velocity and shear traction mirrored; absorbing: zero).  A gravitational
+// face keeps the own tangential velocity and takes its normal state from the
+// (eta, H) ODE; a fault face's flux is the friction solve's.
+void face_coefficients(const double n[3], int tag, double Zp, double Zs, double Zpp, double Zsp, double rho, double lam,
+                       double mu, double sf, double* c) {
+  for (int d = 0; d < 3; ++d) c[d] = n[d];
+  if (tag == ADG_TAG_FAULT) return;
+  // normal pair: (t^b, v^b) from own (t, v) and the neighbour's; tangential the same
+  const double z = Zp * Zpp / (Zp + Zpp);
+  double an[4] = {1 - z / Zpp, -z, -z / (Zpp * Zp), 1 - z / Zp}, bn[4] = {z / Zpp, z, z / (Zpp * Zp), z / Zp};
+  double at[4] = {0, 0, Zs > 0 ? -1 / Zs : 0.0, 1}, bt[4] = {0, 0, 0, 0};
+  if (Zs > 0 && Zsp > 0) {
+    const double zs = Zs * Zsp / (Zs + Zsp);
+    at[0] = 1 - zs / Zsp; at[1] = -zs; at[2] = -zs / (Zsp * Zs); at[3] = 1 - zs / Zs;
+    bt[0] = zs / Zsp; bt[1] = zs; bt[2] = zs / (Zsp * Zs); bt[3] = zs / Zs;
+  }
+  if (tag == ADG_TAG_GRAVITY) {
+    an[0] = an[1] = an[2] = an[3] = at[0] = at[1] = 0;
+    at[2] = Zs > 0 ? -1 / Zs : 0.0;
+    at[3] = 1;
+  } else if (tag != ADG_TAG_INTERIOR && tag != ADG_TAG_PERIODIC) {
+    const double gtn = tag == ADG_TAG_FREE ? -1 : tag == ADG_TAG_RIGID ? 1 : 0;
+    const double gvn = tag == ADG_TAG_FREE ? 1 : tag == ADG_TAG_RIGID ? -1 : 0;
+    const double gts = tag == ADG_TAG_ABSORB ? 0 : -1, gvs = tag == ADG_TAG_ABSORB ? 0 : 1;
+    for (int k = 0; k < 4; ++k) {
+      an[k] += bn[k] * (k % 2 ? gvn : gtn);
+      at[k] += bt[k] * (k % 2 ? gvs : gts);
+    }
+  }
+  const bool nb = tag == ADG_TAG_INTERIOR || tag == ADG_TAG_PERIODIC;
+  for (int k = 0; k < 4; ++k) {
+    const double s = nb ? (k % 2 ? 1.0 : -1.0) : 0.0;  // the neighbour's traction has the opposite normal
+    c[3 + k] = at[k];
+    c[7 + k] = s * bt[k];
+    c[11 + k] = an[k] - at[k];
+    c[15 + k] = s * (bn[k] - bt[k]);
+  }
+  c[19] = -sf * lam;
+  c[20] = -sf * mu;
+  c[21] = -sf / rho;
+}
+
 void gauss01(int n, std::vector<double>& x, std::vector<double>& w) {
   x.resize(n);
   w.resize(n);
@@ -463,21 +508,23 @@ void Ctx::setup() {
   // instantiation), 2 the CUDA-core kernels: a fault face or more than one
   // gravitational face)
   std::vector<char> special(E, 0), lts_face(E, 0);
-  if (tc)
-    for (int64_t e = 0; e < E; ++e) {
-      int ng_e = 0;
-      bool cc = false, coarser = false, finer = false;
-      for (int f = 0; f < 4; ++f) {
-        const int tg = tag[4 * e + f];
-        const int64_t e2 = nbr_u[4 * e + f];
-        ng_e += tg == ADG_TAG_GRAVITY;
-        cc = cc || tg == ADG_TAG_FAULT;
-        coarser = coarser || (e2 >= 0 && cl[e2] > cl[e]);
-        finer = finer || (e2 >= 0 && cl[e2] < cl[e]);
-      }
-      special[e] = (cc || ng_e > 1) ? 2 : ((ng_e == 1 || finer) ? 3 : (coarser ? 1 : 0));
-      lts_face[e] = coarser || finer;
+  for (int64_t e = 0; e < E; ++e) {
+    int ng_e = 0;
+    bool cc = false, coarser = false, finer = false;
+    for (int f = 0; f < 4; ++f) {
+      const int tg = tag[4 * e + f];
+      const int64_t e2 = nbr_u[4 * e + f];
+      ng_e += tg == ADG_TAG_GRAVITY;
+      cc = cc || tg == ADG_TAG_FAULT;
+      coarser = coarser || (e2 >= 0 && cl[e2] > cl[e]);
+      finer = finer || (e2 >= 0 && cl[e2] < cl[e]);
     }
+    lts_face[e] = coarser || finer;
+    if (tc)
+      special[e] = (cc || ng_e > 1) ? 2 : ((ng_e == 1 || finer) ? 3 : (coarser ? 1 : 0));
+    else  // the row kernels: their special instantiation takes all of these
+      special[e] = cc || ng_e || lts_face[e] ? 2 : 0;
+  }
   // order key within a cluster: 0 plain elastic, 1 plain fluid on the
   // acoustic local kernel, 2 with a coarser neighbour, 3 with a gravitational
   // face or a finer neighbour (all four on the tensor-core kernels), 4 the
@@ -495,6 +542,7 @@ void Ctx::setup() {
   for (int64_t i = 0; i < E; ++i) inv[order[i]] = i;
   cl_begin.assign(ncl + 1, 0);
   cl_plain.assign(ncl, 0);
+  cl_row.assign(ncl, 0);
   cl_elastic.assign(ncl, 0);
   cl_fluid.assign(ncl, 0);
   cl_grav.assign(ncl, 0);
@@ -503,6 +551,7 @@ void Ctx::setup() {
     const int k = key[order[i]], c = cl[order[i]];
     cl_begin[c + 1]++;
     if (tc && k < 4) cl_plain[c]++;
+    if (!tc && k == 0) cl_row[c]++;
     if (tc && k == 0) cl_elastic[c]++;
     if (tc && k == 1) cl_fluid[c]++;
     if (tc && k == 3) cl_grav[c]++;
@@ -513,7 +562,15 @@ void Ctx::setup() {
   for (int64_t i = 0; i < E; ++i) cluster[i] = cl[order[i]];
 
   // ---- per-element / per-face device data (internal order)
-  std::vector<double> par((size_t)E * PAR), Fm((size_t)E * 324, 0.0), Fp((size_t)E * 324, 0.0);
+  // the nodal kernels (a tensor-core context's remaining elements) read flux
+  // matrices, the row kernels (without tensor cores, and adg_step_noalloc in
+  // the contexts that it accepts) coefficient records
+  bool nodal = false, faults = false;
+  for (int c = 0; c < ncl; ++c) nodal = nodal || (tc && cl_plain[c] < cl_begin[c + 1] - cl_begin[c]);
+  for (int64_t k = 0; k < 4 * E; ++k) faults = faults || tag[k] == ADG_TAG_FAULT || tag[k] == ADG_TAG_GRAVITY;
+  const bool rows = !tc || (ncl == 1 && S == 1 && !faults);
+  std::vector<double> par((size_t)E * PAR), Fm(nodal ? (size_t)E * 324 : 0, 0.0), Fp(nodal ? (size_t)E * 324 : 0, 0.0),
+      crec(rows ? (size_t)E * 4 * CREC : 0, 0.0);
   std::vector<float> frec(tc ? (size_t)E * 4 * FREC : 0, 0.f);
   std::vector<int> nbr((size_t)E * 4, -1), ninfo((size_t)E * 4, 0), gslot((size_t)E * 4, -1),
       bslot(E, -1), dslot((size_t)E * 4, -1);
@@ -605,9 +662,20 @@ void Ctx::setup() {
       } else {
         FmM = boundary_matrix(TA, Ti, Zpm, Zsm, tg);  // free, rigid, absorbing
       }
-      for (int k = 0; k < 81; ++k) {
-        Fm[(i * 4 + f) * 81 + k] = FmM[k];
-        Fp[(i * 4 + f) * 81 + k] = FpM[k];
+      if (nodal)
+        for (int k = 0; k < 81; ++k) {
+          Fm[(i * 4 + f) * 81 + k] = FmM[k];
+          Fp[(i * 4 + f) * 81 + k] = FpM[k];
+        }
+      if (rows) {
+        double Zpp = Zpm, Zsp = Zsm;
+        if (kind != NK_NONE) {
+          const int64_t e2u = nbr_u[4 * eu + f];
+          Zpp = std::sqrt(rho[e2u] * (lam[e2u] + 2 * mu[e2u]));
+          Zsp = std::sqrt(rho[e2u] * mu[e2u]);
+        }
+        face_coefficients(n, tg, Zpm, Zsm, Zpp, Zsp, rho[eu], lam[eu], mu[eu], par[i * PAR + 12 + f],
+                          &crec[((size_t)i * 4 + f) * CREC]);
       }
     }
     if (has_coarse) bslot[i] = 1;
@@ -684,6 +752,9 @@ void Ctx::setup() {
         liftT[((size_t)f * Bf + n) * B + l] = ops.lift[((size_t)f * B + l) * Bf + n];
       }
 
+  const RowTables rt = make_row_tables(ops);
+  if (rt.max_err > 1e-10) throw Err(ADG_E_STATE, "internal: the sparse operators do not match the basis");
+
   // ---- device allocations
   if (cfg.cuda_stream) {
     stream = (cudaStream_t)cfg.cuda_stream;
@@ -704,6 +775,10 @@ void Ctx::setup() {
     dPar = upload_vec<double>(par, owned, dev_bytes);
     dFm = upload_vec<double>(Fm, owned, dev_bytes);
     dFp = upload_vec<double>(Fp, owned, dev_bytes);
+    dCrec = upload_vec<double>(crec, owned, dev_bytes);
+    dRfc = upload_vec<double>(rt.rfcT, owned, dev_bytes);
+    dModal = upload_vec<double>(rt.modalT, owned, dev_bytes);
+    dReorient = upload_vec<double>(rt.reorient, owned, dev_bytes);
     dKt = upload_vec<double>(ktT, owned, dev_bytes);
     dKvol = upload_vec<double>(kvolT, owned, dev_bytes);
     dEfc = upload_vec<double>(efcT, owned, dev_bytes);
@@ -712,6 +787,10 @@ void Ctx::setup() {
     dPar = upload_vec<float>(par, owned, dev_bytes);
     dFm = upload_vec<float>(Fm, owned, dev_bytes);
     dFp = upload_vec<float>(Fp, owned, dev_bytes);
+    dCrec = upload_vec<float>(crec, owned, dev_bytes);
+    dRfc = upload_vec<float>(rt.rfcT, owned, dev_bytes);
+    dModal = upload_vec<float>(rt.modalT, owned, dev_bytes);
+    dReorient = upload_vec<float>(rt.reorient, owned, dev_bytes);
     dKt = upload_vec<float>(ktT, owned, dev_bytes);
     dKvol = upload_vec<float>(kvolT, owned, dev_bytes);
     dEfc = upload_vec<float>(efcT, owned, dev_bytes);
@@ -760,7 +839,9 @@ void Ctx::setup() {
   // configure kernels once (outside any stream capture)
   StepArgs a0 = base_args();
   const Segs none = make_segs(nullptr, 0, 1);
-  int rc = launch_local(fp64, N, a0, none, stream);
+  int rc = launch_local_row(fp64, N, a0, none, stream, 128, false);
+  if (!rc) rc = launch_neighbour_row(fp64, N, a0, none, stream, 128, false);
+  if (!rc && tc) rc = launch_local(N, a0, none, stream);
   if (!rc && tc) rc = launch_local_tc(N, a0, none, n_sms, stream, false);
   if (!rc && tc) rc = launch_neighbour_tc(N, a0, none, n_sms, stream, false);
   if (rc) throw Err(ADG_E_CUDA, std::string("kernel configuration: ") + cudaGetErrorString((cudaError_t)rc));
@@ -778,6 +859,7 @@ StepArgs Ctx::base_args() const {
   a.S = S; a.err = dErr;
   a.fslot = dFslot; a.drout = dDrout; a.gflux = dGflux; a.tc_local = dTcLocal; a.tc_lift = dTcLift;
   a.frec = dFrec; a.gscr = dGscr;
+  a.crec = dCrec; a.rfcT = dRfc; a.modalT = dModal; a.reorient = dReorient;
   return a;
 }
 
@@ -805,7 +887,8 @@ void Ctx::launch_tick(int s, double dtm) {
     // acoustic and gravitational-face (local phase only), CUDA-core
     // (tcb: the local phase's elements with a coarser neighbour outside the
     // special range, on the instantiation with the LTS-buffer code)
-    std::vector<Seg> tcs, tcb, fls, grs, ccs;
+    // (rws, rss: the row kernels' plain and special elements)
+    std::vector<Seg> tcs, tcb, fls, grs, ccs, rws, rss;
     bool ltsf = false;
     for (int c = 0; c < ncl; ++c) {
       const bool active = phase == 0 ? s % (1 << c) == 0 : (s + 1) % (1 << c) == 0;
@@ -844,9 +927,15 @@ void Ctx::launch_tick(int s, double dtm) {
           tcs.push_back(seg(cl_begin[c], np));
         }
       }
-      if (n > np) ccs.push_back(seg(cl_begin[c] + np, n - np));
+      if (tc) {
+        if (n > np) ccs.push_back(seg(cl_begin[c] + np, n - np));
+      } else {
+        if (cl_row[c] > 0) rws.push_back(seg(cl_begin[c], cl_row[c]));
+        if (n > cl_row[c]) rss.push_back(seg(cl_begin[c] + cl_row[c], n - cl_row[c]));
+      }
     }
-    if (tcs.empty() && tcb.empty() && fls.empty() && grs.empty() && ccs.empty()) continue;
+    if (tcs.empty() && tcb.empty() && fls.empty() && grs.empty() && ccs.empty() && rws.empty() && rss.empty())
+      continue;
     ProfEv ev{phase, nullptr, nullptr, 0};
     if (prof) {
       CK(cudaEventCreate(&ev.a));
@@ -858,7 +947,7 @@ void Ctx::launch_tick(int s, double dtm) {
     auto launch = [&](const std::vector<Seg>& v, int unit, auto&& fn) {
       for (size_t i = 0; i < v.size() && !rc; i += kMaxSeg) {
         const int k = (int)std::min<size_t>(kMaxSeg, v.size() - i);
-        rc = fn(make_segs(v.data() + i, k, unit, unit == 1 ? 1 : tc_chunk[phase]));
+        rc = fn(make_segs(v.data() + i, k, unit, unit == 1 || unit == kRowElems ? 1 : tc_chunk[phase]));
         ev.launches++;
       }
     };
@@ -875,9 +964,14 @@ void Ctx::launch_tick(int s, double dtm) {
       CK(cudaEventRecord(ev.m, stream));
     }
     launch(ccs, 1, [&](const Segs& g) {
-      return phase == 0 ? launch_local(fp64, N, a, g, stream, cc_threads[0])
-                        : launch_neighbour(fp64, N, a, g, stream, cc_threads[1]);
+      return phase == 0 ? launch_local(N, a, g, stream, cc_threads[0])
+                        : launch_neighbour(N, a, g, stream, cc_threads[1]);
     });
+    for (const bool spec : {true, false})
+      launch(spec ? rss : rws, kRowElems, [&](const Segs& g) {
+        return phase == 0 ? launch_local_row(fp64, N, a, g, stream, cc_threads[0], spec)
+                          : launch_neighbour_row(fp64, N, a, g, stream, cc_threads[1], spec);
+      });
     if (prof) { CK(cudaEventRecord(ev.b, stream)); prof->push_back(ev); }
     if (rc)
       throw Err(ADG_E_CUDA, std::string(phase == 0 ? "local kernel: " : "neighbour kernel: ") +
@@ -921,7 +1015,7 @@ int64_t Ctx::launches_per_macro() const {
   const int ticks = 1 << (ncl - 1);
   for (int s = 0; s < ticks; ++s)
     for (int phase = 0; phase < 2; ++phase) {
-      bool tcl = false, tbl = false, fll = false, grl = false, ccl = false;
+      bool tcl = false, tbl = false, fll = false, grl = false, ccl = false, rwl = false;
       for (int c = 0; c < ncl; ++c) {
         const int64_t n = cl_begin[c + 1] - cl_begin[c];
         if (!n || (phase == 0 ? s % (1 << c) : (s + 1) % (1 << c))) continue;
@@ -936,9 +1030,10 @@ int64_t Ctx::launches_per_macro() const {
         } else {
           tcl = tcl || np > 0;
         }
-        ccl = ccl || n > np;
+        ccl = ccl || (tc ? n > np : n > cl_row[c]);
+        rwl = rwl || (!tc && cl_row[c] > 0);
       }
-      L += tcl + tbl + fll + grl + ccl;
+      L += tcl + tbl + fll + grl + ccl + rwl;
     }
   return L;
 }

@@ -40,6 +40,14 @@ int launch_isotropic_fluid(int fp64, void* Q, const int64_t* elems, int64_t n, i
 int launch_receivers(int fp64, int B, const void* Q, int S, int64_t n, const int64_t* elem,
                      const double* phi, double* out, void* stream);
 
+// Tables of the row kernels (StepArgs rfcT, modalT, reorient); max_err: the
+// largest difference between the operators' compiled-in entries and `o`'s
+struct RowTables {
+  std::vector<double> rfcT, modalT, reorient;
+  double max_err = 0;
+};
+RowTables make_row_tables(const RefOps& o);
+
 // Host-side plan of a mesh (caller's element order): geometry, face
 // connectivity, CFL time steps and rate-2 clusters (Sec. 4.4)
 struct MeshPlan {
@@ -77,6 +85,10 @@ struct Ctx {
   // elements [cl_begin[c], cl_begin[c] + cl_plain[c]) of cluster c have no
   // gravitational face, fault face or LTS buffer (tensor-core local kernel)
   std::vector<int64_t> cl_plain;
+  // without the tensor-core kernels: the first cl_row[c] elements of cluster c
+  // have no gravitational or fault face and no neighbour in another cluster
+  // (the row kernels' plain instantiation)
+  std::vector<int64_t> cl_row;
   // cluster c's tensor-core range includes elements with a coarser or finer
   // neighbour (the neighbour kernel's LTS-face code)
   std::vector<char> cl_tc_lts;
@@ -108,6 +120,7 @@ struct Ctx {
   double *dBtrace = nullptr, *dEta = nullptr, *dGpar = nullptr;
   void *dPar = nullptr, *dFm = nullptr, *dFp = nullptr;
   float* dFrec = nullptr;  // face records of the tensor-core neighbour kernel
+  void *dCrec = nullptr, *dRfc = nullptr, *dModal = nullptr, *dReorient = nullptr;  // row kernels
   void *dKt = nullptr, *dKvol = nullptr, *dEfc = nullptr, *dLift = nullptr;
   int *dNbr = nullptr, *dNinfo = nullptr, *dGslot = nullptr, *dBslot = nullptr, *dDslot = nullptr,
       *dPerm = nullptr;

@@ -1,6 +1,6 @@
 // Autotuner of the launch shapes (adg_autotune).  The work of a step is fixed
 // by the scheme; how it is cut into launches is a choice per kernel kind:
-//   knob 0 / 1: threads per element block of the CUDA-core local / neighbour
+//   knob 0 / 1: threads per block of the CUDA-core local / neighbour
 //               kernels (64, 128, 256);
 //   knob 2 / 3: consecutive 12-element tiles a CTA slot of the tensor-core
 //               local / neighbour kernel takes per sweep (1, 2, 4), i.e. the

@@ -1,5 +1,4 @@
-// ADER-DG element-update kernels (CUDA cores), templated on the working
-// precision T (double or float) and the polynomial degree N.
+// ADER-DG element-update kernels: what they compute, their arguments and launchers.
 //
 // Per element v (virtual index; ensembles stack S scenarios per element) over
 // one own step:
@@ -15,8 +14,9 @@
 //                     numerical-flux): F^- on the own traces, F^+ on the
 //                     neighbours' (re-oriented by a node permutation), the
 //                     stored fluxes of gravitational and fault faces; one lift.
-// Dofs layout: Q[v][9][B] (basis fastest); traces [v][4][face_stride(N)], each face
-// block [9][Bf] (node fastest) followed by padding.
+// Dofs layout: Q[v][9][B] (basis fastest).  Traces: the tensor-core kernels and
+// the nodal kernels beside them [v][4][face_stride(N)], each face block [9][Bf]
+// (node fastest) followed by padding; the row kernels as in row_common.cuh.
 #pragma once
 #include <cstdint>
 
@@ -66,7 +66,20 @@ struct StepArgs {
   const float* tc_lift;  // tensor-core lift operand of the neighbour kernel (hi/lo, canonical layout), degree 5 or 4
   const float* frec;     // [E][4][FREC] face records of the tensor-core neighbour kernel (FP32 dofs)
   float* gscr;           // [ngslot*S][gscr_floats(N)] scratch of the tensor-core local kernel's gravity faces
+  // row kernels
+  const void* crec;      // T [E][4][CREC] face coefficients
+  const void* rfcT;      // T [4][B(l)][Bf(r)]  face modes of phi_l, l-major
+  const void* modalT;    // T [Bf(n)][Bf(r)]    face nodes to face modes, n-major
+  const void* reorient;  // T [6][sum (n+1)^2]  a neighbour's face modes in this side's, blocks by degree
 };
+// Virtual elements per warp of the row kernels
+constexpr int kRowElems = 3;
+// Face coefficients of the row kernels: outward normal n[3]; the middle
+// state's tangential coefficients of the own and of the neighbour's side (t^b
+// from t and v, v^b from t and v) and what the normal components add to them
+// (the same four), the neighbour's traction taken with its own normal; then
+// -s_f lambda, -s_f mu, -s_f / rho of the element (s_f = 2|S_f|/|J|); padding.
+constexpr int CREC = 24;
 // Per gravity slot and scenario, the tensor-core local kernel's scratch: the
 // normal-projected derivative rows g_m[l] = sum_p w_p D^m[p][l] (m = 0..N,
 // l < B(N - m); w: v_n - sigma_nn / Z), then the own-trace flux part
@@ -192,10 +205,16 @@ int launch_rupture(int fp64, int N, const DRArgs& a, void* stream);
 
 enum { ERR_NAN = 1u, ERR_TIMEOUT = 2u, ERR_NEWTON = 4u };
 
-// host-side launchers (kernels_f64.cu / kernels_f32.cu); return cudaError_t as int
-// (threads: per element block, a multiple of 32 up to 256)
-int launch_local(int fp64, int N, const StepArgs& a, const Segs& g, void* stream, int threads = 128);
-int launch_neighbour(int fp64, int N, const StepArgs& a, const Segs& g, void* stream, int threads = 128);
-int local_smem_bytes(int fp64, int N);
+// host-side launchers; return cudaError_t as int
+// (threads: per block, a multiple of 32 up to 256)
+// row kernels (row_local.cuh, row_neighbour.cuh): both precisions, every degree;
+// spec: the launch's elements may have gravitational or fault faces or
+// neighbours in another cluster
+int launch_local_row(int fp64, int N, const StepArgs& a, const Segs& g, void* stream, int threads, bool spec);
+int launch_neighbour_row(int fp64, int N, const StepArgs& a, const Segs& g, void* stream, int threads, bool spec);
+// nodal kernels (kernels_impl.cuh): the elements of a tensor-core context
+// (FP32 dofs, degree 5 or 4) that the tensor-core kernels do not take
+int launch_local(int N, const StepArgs& a, const Segs& g, void* stream, int threads = 128);
+int launch_neighbour(int N, const StepArgs& a, const Segs& g, void* stream, int threads = 128);
 
 }  // namespace adg

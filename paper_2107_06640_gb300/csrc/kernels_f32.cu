@@ -1,26 +1,27 @@
-// FP32 instantiations of the element-update kernels.
+// FP32 instantiations of the nodal kernels, and the launchers shared by the kernel kinds.
 #include "kernels_impl.cuh"
 
 namespace adg {
-int launch_local_f32(int N, const StepArgs& a, const Segs& nb, int th, void* st) {
-  return dispatch_local<float>(N, a, nb, th, (cudaStream_t)st);
+int launch_local(int N, const StepArgs& a, const Segs& g, void* stream, int threads) {
+  return dispatch_local(N, a, g, threads, (cudaStream_t)stream);
 }
-int launch_neighbour_f32(int N, const StepArgs& a, const Segs& nb, int th, void* st) {
-  return dispatch_neighbour<float>(N, a, nb, th, (cudaStream_t)st);
+int launch_neighbour(int N, const StepArgs& a, const Segs& g, void* stream, int threads) {
+  return dispatch_neighbour(N, a, g, threads, (cudaStream_t)stream);
 }
-int smem_f32(int N) { return smem_of<float>(N); }
 
-int launch_local_f64(int N, const StepArgs& a, const Segs& nb, int th, void* st);
-int launch_neighbour_f64(int N, const StepArgs& a, const Segs& nb, int th, void* st);
-int smem_f64(int N);
+int launch_local_row_f32(int N, const StepArgs& a, const Segs& g, int threads, bool spec, void* stream);
+int launch_local_row_f64(int N, const StepArgs& a, const Segs& g, int threads, bool spec, void* stream);
+int launch_neighbour_row_f32(int N, const StepArgs& a, const Segs& g, int threads, bool spec, void* stream);
+int launch_neighbour_row_f64(int N, const StepArgs& a, const Segs& g, int threads, bool spec, void* stream);
 
-int launch_local(int fp64, int N, const StepArgs& a, const Segs& g, void* stream, int threads) {
-  return fp64 ? launch_local_f64(N, a, g, threads, stream) : launch_local_f32(N, a, g, threads, stream);
+int launch_local_row(int fp64, int N, const StepArgs& a, const Segs& g, void* stream, int threads, bool spec) {
+  return fp64 ? launch_local_row_f64(N, a, g, threads, spec, stream)
+              : launch_local_row_f32(N, a, g, threads, spec, stream);
 }
-int launch_neighbour(int fp64, int N, const StepArgs& a, const Segs& g, void* stream, int threads) {
-  return fp64 ? launch_neighbour_f64(N, a, g, threads, stream) : launch_neighbour_f32(N, a, g, threads, stream);
+int launch_neighbour_row(int fp64, int N, const StepArgs& a, const Segs& g, void* stream, int threads, bool spec) {
+  return fp64 ? launch_neighbour_row_f64(N, a, g, threads, spec, stream)
+              : launch_neighbour_row_f32(N, a, g, threads, spec, stream);
 }
-int local_smem_bytes(int fp64, int N) { return fp64 ? smem_f64(N) : smem_f32(N); }
 
 Segs make_segs(const Seg* s, int n, int unit, int chunk) {
   Segs g{};

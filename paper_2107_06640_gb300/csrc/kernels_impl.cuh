@@ -1,4 +1,5 @@
-// Template bodies of the element-update kernels (see kernels.cuh).
+// Nodal CUDA-core element kernels (see kernels.cuh): the elements of a
+// tensor-core context that have a fault face or several gravitational faces.
 //
 // Shared-memory working arrays keep the 9 quantities of one basis function
 // (or face node) contiguous, padded to P values so that a row is read with
@@ -524,38 +525,13 @@ int launch_neighbour_t(const StepArgs& a, const Segs& g, int threads, cudaStream
   return (int)cudaGetLastError();
 }
 
-template <typename T>
-int dispatch_local(int N, const StepArgs& a, const Segs& nb, int th, cudaStream_t st) {
-  switch (N) {
-    case 1: return launch_local_t<T, 1>(a, nb, th, st);
-    case 2: return launch_local_t<T, 2>(a, nb, th, st);
-    case 3: return launch_local_t<T, 3>(a, nb, th, st);
-    case 4: return launch_local_t<T, 4>(a, nb, th, st);
-    case 5: return launch_local_t<T, 5>(a, nb, th, st);
-  }
-  return (int)cudaErrorInvalidValue;
+inline int dispatch_local(int N, const StepArgs& a, const Segs& nb, int th, cudaStream_t st) {
+  return N == 4 ? launch_local_t<float, 4>(a, nb, th, st)
+                : N == 5 ? launch_local_t<float, 5>(a, nb, th, st) : (int)cudaErrorInvalidValue;
 }
-template <typename T>
-int dispatch_neighbour(int N, const StepArgs& a, const Segs& nb, int th, cudaStream_t st) {
-  switch (N) {
-    case 1: return launch_neighbour_t<T, 1>(a, nb, th, st);
-    case 2: return launch_neighbour_t<T, 2>(a, nb, th, st);
-    case 3: return launch_neighbour_t<T, 3>(a, nb, th, st);
-    case 4: return launch_neighbour_t<T, 4>(a, nb, th, st);
-    case 5: return launch_neighbour_t<T, 5>(a, nb, th, st);
-  }
-  return (int)cudaErrorInvalidValue;
-}
-template <typename T>
-int smem_of(int N) {
-  switch (N) {
-    case 1: return Smem<T, 1>::bytes;
-    case 2: return Smem<T, 2>::bytes;
-    case 3: return Smem<T, 3>::bytes;
-    case 4: return Smem<T, 4>::bytes;
-    case 5: return Smem<T, 5>::bytes;
-  }
-  return 0;
+inline int dispatch_neighbour(int N, const StepArgs& a, const Segs& nb, int th, cudaStream_t st) {
+  return N == 4 ? launch_neighbour_t<float, 4>(a, nb, th, st)
+                : N == 5 ? launch_neighbour_t<float, 5>(a, nb, th, st) : (int)cudaErrorInvalidValue;
 }
 
 }  // namespace adg

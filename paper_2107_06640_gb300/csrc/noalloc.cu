@@ -90,10 +90,10 @@ extern "C" int adg_step_noalloc(adg_ctx* ctx, void* d_Q, int n_steps, void* stre
     sg.tcoef[k] = (fb - fa) / fac;
     fb *= c.dtmin;
   }
-  const adg::Segs g = adg::make_segs(&sg, 1, 1);
+  const adg::Segs g = adg::make_segs(&sg, 1, adg::kRowElems);
   for (int i = 0; i < n_steps; ++i) {
-    int rc = adg::launch_local(c.fp64, c.N, a, g, st);
-    if (!rc) rc = adg::launch_neighbour(c.fp64, c.N, a, g, st);
+    int rc = adg::launch_local_row(c.fp64, c.N, a, g, st, 128, false);
+    if (!rc) rc = adg::launch_neighbour_row(c.fp64, c.N, a, g, st, 128, false);
     if (rc) {
       c.last_error = std::string("adg_step_noalloc: launch failed: ") + cudaGetErrorString((cudaError_t)rc);
       return ADG_E_CUDA;

@@ -1,0 +1,119 @@
+// What the two row kernels (row_local.cuh, row_neighbour.cuh) share.
+//
+// They are the CUDA-core form of the element update, in both precisions and at
+// every degree: one warp works on three (virtual) elements, lane 9 j + p holds
+// the row of quantity p of element j in registers (lanes 27..31 idle), the
+// operators are straight-line sparse code (sparse_ops.cuh), the quantities of
+// an element meet in warp shuffles, and no block barrier is needed.
+//
+// Face data are modal: a face block holds traction sigma n (n the owner's
+// outward normal) and velocity, the six quantities that the Godunov flux
+// reads, in the face's orthonormal Dubiner modes, [6][Bf].  An element's four
+// blocks follow one another ([v][4][6][Bf] in the trace array).  LTS buffers
+// ([slot*S][4][6][Bf], FP64) and the derivative traces of faces with a finer
+// neighbour ([slot*S][N+1][6][Bf]) are modal as well; those of fault faces stay
+// nodal in all nine quantities ([N+1][9][Bf]), as the friction solve reads them.
+//
+// What bounds them: FP64, the 2 FMA per clock and SM (the sparse form has 3.4
+// to 4 times fewer of them than dense nodal products, and no lane waits on an
+// operand); FP32, instruction issue.  Against one block per element with dense
+// operands in global memory and block barriers between the levels: degree 3
+// FP64, 3,072 tets, 366 -> 130 us per step; degree 5 FP64, 33,696 tets, 17.2 ->
+// 5.9 ms; degree 3 FP32, 13,182 tets, 130 -> 35 us; 102,258 tets, 1.13 -> 0.33
+// ms (steps as a caller sees them, transfers included).
+#pragma once
+#include <cuda_runtime.h>
+
+#include "func_attr.hpp"
+#include "kernels.cuh"
+#include "sparse_ops.cuh"
+
+namespace adg {
+namespace row {
+
+constexpr int EW = kRowElems;  // elements per warp
+constexpr int kMaxThreads = 256;
+
+// Shapes of degree N in type T: vector width VW of the copies between global
+// and shared memory (16 bytes where a row allows it), and the row stride SB
+// in shared memory, padded so that the vector accesses of a quarter warp's
+// eight rows fall on distinct banks.
+template <class T, int N>
+struct Shape {
+  static constexpr int B = nb3(N), Bf = nb2(N), B1 = nb3(N - 1);
+  static constexpr int V16 = 16 / (int)sizeof(T);
+  static constexpr int VW = B % V16 == 0 ? V16 : 1;
+  static constexpr int words(int s) { return s * (int)sizeof(T) / 4; }
+  // 16-byte accesses: the stride in 16-byte units must be odd
+  static constexpr int SB = VW == 1 ? (sizeof(T) == 4 ? (B | 1) : B) : (B / VW % 2 ? B : B + VW);
+  static constexpr int FS = 6 * Bf;            // values of a face block
+  static constexpr int ND = nb3(N) + nb3(N - 1) + nb3(N - 2) + nb3(N - 3) + nb3(N - 4) + nb3(N - 5);
+};
+// row offset of D^k in a row's derivative stack
+__host__ __device__ constexpr int stack_off(int k, int N) {
+  int s = 0;
+  for (int j = 0; j < k; ++j) s += nb3(N - j);
+  return s;
+}
+
+template <class T, int VW>
+struct alignas(VW * sizeof(T)) Vec {
+  T x[VW];
+};
+
+// f(row, column, offset) for every VW values of nE elements' rows, offset the place in global memory
+template <class T, int N, int VW, class F>
+__device__ __forceinline__ void each_chunk(int nE, int lane, F&& f) {
+  constexpr int C = Shape<T, N>::B / VW;
+  for (int i = lane; i < nE * 9 * C; i += 32) f(i / C, (i % C) * VW, i);
+}
+// adg_step_noalloc's caller may pass dofs on any multiple of sizeof(T)
+template <class T, int N>
+__device__ __forceinline__ bool vector_rows(const T* Q) {
+  return Shape<T, N>::VW > 1 && (reinterpret_cast<uintptr_t>(Q) & 15) == 0;
+}
+template <class T, int N, int VW>
+__device__ __forceinline__ void rows_in_v(T* sQ, const T* Q, int nE, int lane) {
+  using V = Vec<T, VW>;
+  each_chunk<T, N, VW>(nE, lane, [&](int r, int c, int i) {
+    *reinterpret_cast<V*>(sQ + r * Shape<T, N>::SB + c) = reinterpret_cast<const V*>(Q)[i];
+  });
+}
+template <class T, int N, int VW>
+__device__ __forceinline__ void rows_out_v(const T* sQ, T* Q, int nE, int lane) {
+  using V = Vec<T, VW>;
+  each_chunk<T, N, VW>(nE, lane, [&](int r, int c, int i) {
+    reinterpret_cast<V*>(Q)[i] = *reinterpret_cast<const V*>(sQ + r * Shape<T, N>::SB + c);
+  });
+}
+// the warp's nE elements' dofs rows, global <-> shared (row stride SB)
+template <class T, int N>
+__device__ __forceinline__ void rows_in(T* sQ, const T* Q, int nE, int lane) {
+  if (vector_rows<T, N>(Q))
+    rows_in_v<T, N, Shape<T, N>::VW>(sQ, Q, nE, lane);
+  else
+    rows_in_v<T, N, 1>(sQ, Q, nE, lane);
+}
+template <class T, int N>
+__device__ __forceinline__ void rows_out(const T* sQ, T* Q, int nE, int lane) {
+  if (vector_rows<T, N>(Q))
+    rows_out_v<T, N, Shape<T, N>::VW>(sQ, Q, nE, lane);
+  else
+    rows_out_v<T, N, 1>(sQ, Q, nE, lane);
+}
+
+// this warp's work unit: its segment, first virtual element and element count (0: none)
+struct Unit {
+  int seg, nE;
+  int64_t v0;
+};
+__device__ __forceinline__ Unit unit_of(const Segs& g) {
+  const int64_t u = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (u >= g.first[g.n]) return {0, 0, 0};
+  const int i = seg_find(g, u);
+  const int64_t o = (u - g.first[i]) * EW, left = g.s[i].n - o;
+  return {i, (int)(left < EW ? left : EW), g.s[i].v_begin + o};
+}
+
+}  // namespace row
+}  // namespace adg

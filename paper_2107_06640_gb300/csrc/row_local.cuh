@@ -1,0 +1,394 @@
+// Row form of the local kernel (Sec. 4.1; see row_common.cuh for the layout):
+// Cauchy-Kovalewski predictor, time integral, modal face traces and volume
+// term of three elements per warp.  kSpec: the launch's elements may have
+// gravitational faces (Sec. 4.3), fault faces or neighbours in another LTS
+// cluster (Sec. 4.4); their derivative stack is kept in shared memory for it.
+#pragma once
+#include "row_common.cuh"
+
+namespace adg {
+namespace row {
+
+// Star product of this lane's quantity: D[p] = sum_d c_d X_d[src_d] with
+// X_d = sum_b G_b,d Y_b over the three parity-respecting directions b of
+// sparse_ops.inc (Jacobian form of -sum_a A*_a Y_a).
+// FP32: X_d here, one shuffle per direction.  FP64: the arithmetic is what
+// counts (2 FMA per clock and SM), so the Y_b travel and the products
+// c_d G_b,d are formed once: 9 FMAs instead of 12 operations.
+template <class T>
+struct RowStar {
+  T w[9];      // FP32: G_b,d at 3 b + d; FP64: c_d G_b,d
+  T c[3];
+  int src[3];
+  __device__ __forceinline__ void setup(int lane, bool valid, const T* par) {
+    const int j = lane / 9, p = lane - 9 * j, base = 9 * j;
+    T lam = 0, mu = 0, irho = 0;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) w[k] = T(0);
+    if (valid) {
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        const T gx = par[d], gy = par[3 + d], gz = par[6 + d];
+        w[d] = gx + T(0.5) * (gy + gz);
+        w[3 + d] = gy + gz;
+        w[6 + d] = gz;
+      }
+      irho = T(1) / par[9];
+      lam = par[10];
+      mu = par[11];
+    }
+    const T l2m = lam + T(2) * mu;
+    int q0 = p, q1 = p, q2 = p;
+    T c0 = 0, c1 = 0, c2 = 0;
+    switch (p) {
+      case 0: q0 = 6; c0 = l2m; q1 = 7; c1 = lam; q2 = 8; c2 = lam; break;
+      case 1: q0 = 6; c0 = lam; q1 = 7; c1 = l2m; q2 = 8; c2 = lam; break;
+      case 2: q0 = 6; c0 = lam; q1 = 7; c1 = lam; q2 = 8; c2 = l2m; break;
+      case 3: q0 = 7; c0 = mu; q1 = 6; c1 = mu; break;
+      case 4: q1 = 8; c1 = mu; q2 = 7; c2 = mu; break;
+      case 5: q0 = 8; c0 = mu; q2 = 6; c2 = mu; break;
+      case 6: q0 = 0; c0 = irho; q1 = 3; c1 = irho; q2 = 5; c2 = irho; break;
+      case 7: q0 = 3; c0 = irho; q1 = 1; c1 = irho; q2 = 4; c2 = irho; break;
+      default: q0 = 5; c0 = irho; q1 = 4; c1 = irho; q2 = 2; c2 = irho; break;
+    }
+    const bool on = lane < 27;
+    src[0] = on ? base + q0 : lane;
+    src[1] = on ? base + q1 : lane;
+    src[2] = on ? base + q2 : lane;
+    c[0] = c0; c[1] = c1; c[2] = c2;
+    if constexpr (sizeof(T) == 8) {
+#pragma unroll
+      for (int k = 0; k < 9; ++k) w[k] *= c[k % 3];
+    }
+  }
+  __device__ __forceinline__ T apply(T y0, T y1, T y2) const {
+    if constexpr (sizeof(T) == 8) {
+      T s = T(0);
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        s = fma(w[d], __shfl_sync(0xffffffffu, y0, src[d]), s);
+        s = fma(w[3 + d], __shfl_sync(0xffffffffu, y1, src[d]), s);
+        s = fma(w[6 + d], __shfl_sync(0xffffffffu, y2, src[d]), s);
+      }
+      return s;
+    } else {
+      T s = T(0);
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        const T X = fma(w[6 + d], y2, fma(w[3 + d], y1, w[d] * y0));
+        s = fma(c[d], __shfl_sync(0xffffffffu, X, src[d]), s);
+      }
+      return s;
+    }
+  }
+};
+
+// shared memory of one warp (values of T): dofs rows, the nine-quantity modes
+// of two faces, and with kSpec the rows' derivative stacks
+template <class T, int N, bool kSpec>
+struct LocalSmem {
+  using S = Shape<T, N>;
+  static constexpr int nQ = (9 * EW * S::SB + 3) / 4 * 4, nT = (2 * 9 * EW * S::Bf + 3) / 4 * 4;
+  static constexpr int nD = kSpec ? 9 * EW * S::ND + (S::ND + 3) / 4 * 4 + 2 * S::Bf + 2 : 0;
+  static constexpr int warp = (nQ + nT + nD + 3) / 4 * 4;
+  static constexpr int bytes(int threads) { return warp * (int)sizeof(T) * (threads / 32); }
+};
+
+static __constant__ double kRowRcp[48] = {
+    0.0, 1.0 / 1, 1.0 / 2, 1.0 / 3, 1.0 / 4, 1.0 / 5, 1.0 / 6, 1.0 / 7, 1.0 / 8, 1.0 / 9, 1.0 / 10, 1.0 / 11,
+    1.0 / 12, 1.0 / 13, 1.0 / 14, 1.0 / 15, 1.0 / 16, 1.0 / 17, 1.0 / 18, 1.0 / 19, 1.0 / 20, 1.0 / 21, 1.0 / 22,
+    1.0 / 23, 1.0 / 24, 1.0 / 25, 1.0 / 26, 1.0 / 27, 1.0 / 28, 1.0 / 29, 1.0 / 30, 1.0 / 31, 1.0 / 32, 1.0 / 33,
+    1.0 / 34, 1.0 / 35, 1.0 / 36, 1.0 / 37, 1.0 / 38, 1.0 / 39, 1.0 / 40, 1.0 / 41, 1.0 / 42, 1.0 / 43, 1.0 / 44,
+    1.0 / 45, 1.0 / 46, 1.0 / 47};
+static __constant__ double kRowRcpFact[6] = {1.0, 1.0, 1.0 / 2, 1.0 / 6, 1.0 / 24, 1.0 / 120};
+
+// D^{K+1} rows from D^K, then the next levels; I accumulates the time integral
+template <class T, int N, int K, bool kSpec>
+__device__ __forceinline__ void predict(const T* D, T* I, const RowStar<T>& st, const double* tc, T* stack) {
+  constexpr int L = nb3(N - K), M = nb3(N - K - 1);
+  T Dn[M];
+  sp::each<M>([&](auto mc) {
+    constexpr int m = decltype(mc)::value;
+    Dn[m] = st.apply(sp::dot<sp::KX, m, L>(T(0), D), sp::dot<sp::KY, m, L>(T(0), D), sp::dot<sp::KZ, m, L>(T(0), D));
+  });
+  if constexpr (K == 0) {  // D^0 is not needed any more: its registers become I
+    const T c0 = (T)tc[0];
+#pragma unroll
+    for (int l = 0; l < L; ++l) I[l] = c0 * D[l];
+  }
+  const T ck = (T)tc[K + 1];
+#pragma unroll
+  for (int m = 0; m < M; ++m) I[m] = fma(ck, Dn[m], I[m]);
+  if constexpr (kSpec) {
+    if (stack) {
+#pragma unroll
+      for (int m = 0; m < M; ++m) stack[stack_off(K + 1, N) + m] = Dn[m];
+    }
+  }
+  if constexpr (K + 1 < N) predict<T, N, K + 1, kSpec>(Dn, I, st, tc, stack);
+}
+
+// the faces F0, F0 + 1 of the warp's elements: staged modes -> traction and
+// velocity blocks of the trace array (and the LTS buffers, in FP64)
+template <class T, int N, bool kSpec>
+__device__ __forceinline__ void faces_out(const StepArgs& a, const Seg& sg, int64_t v0, int nE, int f0, const T* sT,
+                                          int lane) {
+  using S = Shape<T, N>;
+  constexpr int Bf = S::Bf;
+  T* const trace = reinterpret_cast<T*>(a.trace);
+  const T* const crec = reinterpret_cast<const T*>(a.crec);
+  for (int i = lane; i < nE * 2 * Bf; i += 32) {
+    const int jf = i / Bf, n = i - jf * Bf, j = jf >> 1, f = f0 + (jf & 1);
+    const int64_t v = v0 + j, e = v / a.S;
+    const T* const s = sT + ((jf & 1) * 9 * EW + 9 * j) * Bf + n;
+    T q[9];
+#pragma unroll
+    for (int p = 0; p < 9; ++p) q[p] = s[p * Bf];
+    const T* const c = crec + (e * 4 + f) * CREC;
+    const T nx = c[0], ny = c[1], nz = c[2];
+    const T o[6] = {fma(q[5], nz, fma(q[3], ny, q[0] * nx)), fma(q[4], nz, fma(q[1], ny, q[3] * nx)),
+                    fma(q[2], nz, fma(q[4], ny, q[5] * nx)), q[6], q[7], q[8]};
+    T* const out = trace + (v * 4 + f) * S::FS + n;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) out[k * Bf] = o[k];
+    if constexpr (kSpec) {
+      if (sg.btrace_mode && a.bslot) {
+        const int bs = a.bslot[e];
+        if (bs >= 0) {
+          double* const b = a.btrace + (((int64_t)bs * a.S + (v - e * a.S)) * 4 + f) * S::FS + n;
+#pragma unroll
+          for (int k = 0; k < 6; ++k) b[k * Bf] = (sg.btrace_mode == 1 ? 0.0 : b[k * Bf]) + (double)o[k];
+        }
+      }
+    }
+  }
+}
+
+// faces of one element that need more than its trace (kSpec): derivative
+// traces for fault faces and finer neighbours, and the gravitational surface's
+// ODE.  sD: the element's nine stacks (stride ND), sW: scratch of ND + 2 Bf values.
+template <class T, int N>
+__device__ void special_faces(const StepArgs& a, const Seg& sg, int64_t v, const T* sD, T* sW, int lane) {
+  using S = Shape<T, N>;
+  constexpr int B = S::B, Bf = S::Bf, ND = S::ND;
+  const int64_t e = v / a.S;
+  const int s = (int)(v - e * a.S);
+#pragma unroll 1
+  for (int f = 0; f < 4; ++f) {
+    const T* const c = reinterpret_cast<const T*>(a.crec) + (e * 4 + f) * CREC;
+    const int ds = a.dslot ? a.dslot[e * 4 + f] : -1;
+    if (ds >= 0) {
+      const bool fault = ((a.ninfo[e * 4 + f] >> 5) & 7) == NK_FAULT;
+      const T* const tab = reinterpret_cast<const T*>(fault ? a.efcT : a.rfcT) + (size_t)f * B * Bf;
+      T* const out = reinterpret_cast<T*>(a.dtrace) + ((int64_t)ds * a.S + s) * (N + 1) * 9 * Bf;
+      for (int i = lane; i < (N + 1) * Bf; i += 32) {
+        const int k = i / Bf, n = i - k * Bf, Bk = nb3(N - k), o = stack_off(k, N);
+        T q[9];
+#pragma unroll
+        for (int p = 0; p < 9; ++p) q[p] = T(0);
+        for (int l = 0; l < Bk; ++l) {
+          const T w = tab[(size_t)l * Bf + n];
+#pragma unroll
+          for (int p = 0; p < 9; ++p) q[p] = fma(w, sD[p * ND + o + l], q[p]);
+        }
+        if (fault) {
+#pragma unroll
+          for (int p = 0; p < 9; ++p) out[(k * 9 + p) * Bf + n] = q[p];
+        } else {
+          T* const d = out + k * S::FS + n;
+          d[0] = q[0] * c[0] + q[3] * c[1] + q[5] * c[2];
+          d[Bf] = q[3] * c[0] + q[1] * c[1] + q[4] * c[2];
+          d[2 * Bf] = q[5] * c[0] + q[4] * c[1] + q[2] * c[2];
+          d[3 * Bf] = q[6];
+          d[4 * Bf] = q[7];
+          d[5 * Bf] = q[8];
+        }
+      }
+    }
+    const int gs = a.gslot ? a.gslot[e * 4 + f] : -1;
+    if (gs >= 0) {
+      // g_m[l]: v_n - sigma_nn / Z of the derivative rows, then per face node
+      // f_m = E g_m / m!, the (eta, H) series in FP64, and the modes of
+      // -rho g H and eta^{n+1} - eta^n
+      const double* const gp = a.gpar + (size_t)gs * GPAR;
+      const T nx = (T)gp[0], ny = (T)gp[1], nz = (T)gp[2], iz = (T)(1.0 / gp[3]);
+      T* const sS = sW + (ND + 3) / 4 * 4;
+      for (int l = lane; l < ND; l += 32) {
+        const T snn = nx * nx * sD[l] + ny * ny * sD[ND + l] + nz * nz * sD[2 * ND + l] +
+                      T(2) * (nx * ny * sD[3 * ND + l] + ny * nz * sD[4 * ND + l] + nx * nz * sD[5 * ND + l]);
+        const T vn = nx * sD[6 * ND + l] + ny * sD[7 * ND + l] + nz * sD[8 * ND + l];
+        sW[l] = vn - snn * iz;
+      }
+      __syncwarp();
+      if (lane < Bf) {
+        const T* const tab = reinterpret_cast<const T*>(a.efcT) + (size_t)f * B * Bf + lane;
+        double fm[N + 1];
+#pragma unroll
+        for (int m = 0; m <= N; ++m) {
+          T acc = T(0);
+          for (int l = 0; l < nb3(N - m); ++l) acc = fma(tab[(size_t)l * Bf], sW[stack_off(m, N) + l], acc);
+          fm[m] = (double)acc * kRowRcpFact[m];
+        }
+        double* const eta = a.eta + ((int64_t)gs * a.S + s) * Bf + lane;
+        const double kappa = gp[4], rg = gp[5], dt = sg.dt, eta0 = *eta;
+        double cm = eta0, e1 = eta0, H = eta0 * dt, pw = 1.0;
+#pragma unroll 1
+        for (int m = 0; m < N + 40; ++m) {
+          double fv = 0.0;
+#pragma unroll
+          for (int k = 0; k <= N; ++k)
+            if (k == m) fv = fm[k];
+          cm = (fv - kappa * cm) * kRowRcp[m + 1];
+          pw *= dt;
+          const double t = cm * pw;
+          e1 += t;
+          H += t * dt * kRowRcp[m + 2];
+          if (m > N && fabs(t) <= 1e-17 * fabs(e1)) break;
+        }
+        *eta = e1;
+        sS[lane] = (T)(-rg * H);
+        sS[Bf + lane] = (T)(e1 - eta0);
+      }
+      __syncwarp();
+      if (lane < Bf) {
+        const T* const mn = reinterpret_cast<const T*>(a.modalT) + lane;
+        T h = T(0), d = T(0);
+        for (int n = 0; n < Bf; ++n) {
+          const T w = mn[n * Bf];
+          h = fma(w, sS[n], h);
+          d = fma(w, sS[Bf + n], d);
+        }
+        T* const out = reinterpret_cast<T*>(a.gflux) + ((int64_t)gs * a.S + s) * 9 * Bf + lane;
+        out[0] = h;
+        out[Bf] = d;
+      }
+      __syncwarp();
+    }
+  }
+}
+
+template <class T, int N, bool kSpec>
+__global__ void __launch_bounds__(kMaxThreads, sizeof(T) == 4 ? 2 : 1) local_row_kernel(StepArgs a, const __grid_constant__ Segs g) {
+  using S = Shape<T, N>;
+  using M = LocalSmem<T, N, kSpec>;
+  constexpr int B = S::B, Bf = S::Bf, VW = S::VW;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int lane = threadIdx.x & 31;
+  T* const sQ = reinterpret_cast<T*>(smem_raw) + (threadIdx.x >> 5) * M::warp;
+  T* const sT = sQ + M::nQ;
+  const Unit u = unit_of(g);
+  if (u.nE == 0) return;
+  const Seg& sg = g.s[u.seg];
+  T* const Q = reinterpret_cast<T*>(a.Q) + u.v0 * 9 * B;
+  rows_in<T, N>(sQ, Q, u.nE, lane);
+  const int j = lane / 9;
+  const bool valid = lane < 9 * u.nE;
+  RowStar<T> st;
+  st.setup(lane, valid, reinterpret_cast<const T*>(a.par) + (u.v0 + (valid ? j : 0)) / a.S * PAR);
+  T* const row = sQ + (valid ? lane : 0) * S::SB;
+  T* const stack = kSpec && valid ? sT + M::nT + lane * S::ND : nullptr;
+  __syncwarp();
+
+  // ---- D^0, the predictor levels and the time integral
+  T I[B];
+#pragma unroll
+  for (int c = 0; c < B / VW; ++c) {
+    const Vec<T, VW> x = *reinterpret_cast<const Vec<T, VW>*>(row + c * VW);
+#pragma unroll
+    for (int k = 0; k < VW; ++k) I[c * VW + k] = valid ? x.x[k] : T(0);
+  }
+  if constexpr (kSpec) {
+    if (valid) {
+#pragma unroll
+      for (int l = 0; l < B; ++l) stack[l] = I[l];
+    }
+  }
+  predict<T, N, 0, kSpec>(I, I, st, sg.tcoef, stack);
+
+  // ---- modal face traces, two faces at a time through shared memory
+  {
+    T* const s0 = sT + lane * Bf;
+    if (valid) {
+      sp::each<Bf>([&](auto rc) {
+        constexpr int r = decltype(rc)::value;
+        const T ev = sp::dot<sp::R0, r, B, 0>(T(0), I), od = sp::dot<sp::R0, r, B, 1>(T(0), I);
+        s0[r] = ev + od;
+        s0[9 * EW * Bf + r] = ev - od;
+      });
+    }
+    __syncwarp();
+    faces_out<T, N, kSpec>(a, sg, u.v0, u.nE, 0, sT, lane);
+    __syncwarp();
+    if (valid) {
+      sp::each<Bf>([&](auto rc) {
+        constexpr int r = decltype(rc)::value;
+        s0[r] = sp::dot<sp::R2, r, B>(T(0), I);
+        s0[9 * EW * Bf + r] = sp::dot<sp::R3, r, B>(T(0), I);
+      });
+    }
+    __syncwarp();
+    faces_out<T, N, kSpec>(a, sg, u.v0, u.nE, 2, sT, lane);
+  }
+
+  // ---- volume: Q += sum_a A*_a K_a I (face terms follow in the neighbour kernel)
+  sp::each<B / VW>([&](auto cc) {
+    constexpr int m0 = decltype(cc)::value * VW;
+    T x[VW];
+    sp::each<VW>([&](auto kc) {
+      constexpr int m = m0 + decltype(kc)::value;
+      x[decltype(kc)::value] = st.apply(sp::dot<sp::KXt, m, S::B1>(T(0), I), sp::dot<sp::KYt, m, S::B1>(T(0), I),
+                                        sp::dot<sp::KZt, m, S::B1>(T(0), I));
+    });
+    if (valid) {
+      Vec<T, VW> q = *reinterpret_cast<const Vec<T, VW>*>(row + m0);
+#pragma unroll
+      for (int k = 0; k < VW; ++k) q.x[k] -= x[k];
+      *reinterpret_cast<Vec<T, VW>*>(row + m0) = q;
+    }
+  });
+  __syncwarp();
+  rows_out<T, N>(sQ, Q, u.nE, lane);
+  if constexpr (kSpec) {
+    for (int k = 0; k < u.nE; ++k)
+      special_faces<T, N>(a, sg, u.v0 + k, sT + M::nT + 9 * k * S::ND, sT + M::nT + 9 * EW * S::ND, lane);
+  }
+}
+
+template <class T, int N>
+int launch_local_row_t(const StepArgs& a, const Segs& g, int threads, bool spec, cudaStream_t st) {
+  const int rc = configure_on_device((const void*)local_row_kernel<T, N, false>, [] {
+    cudaError_t ce = cudaFuncSetAttribute(local_row_kernel<T, N, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          LocalSmem<T, N, false>::bytes(kMaxThreads));
+    if (ce == cudaSuccess)
+      ce = cudaFuncSetAttribute(local_row_kernel<T, N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                LocalSmem<T, N, true>::bytes(64));
+    return ce;
+  });
+  if (rc) return rc;
+  const int64_t units = g.n ? g.first[g.n] : 0;
+  if (units <= 0) return 0;
+  if (threads < 32 || threads > kMaxThreads || threads % 32) return (int)cudaErrorInvalidValue;
+  if (spec && threads > 64) threads = 64;  // (the derivative stacks in shared memory)
+  const int w = threads / 32;
+  const unsigned blocks = (unsigned)((units + w - 1) / w);
+  if (spec)
+    local_row_kernel<T, N, true><<<blocks, threads, LocalSmem<T, N, true>::bytes(threads), st>>>(a, g);
+  else
+    local_row_kernel<T, N, false><<<blocks, threads, LocalSmem<T, N, false>::bytes(threads), st>>>(a, g);
+  return (int)cudaGetLastError();
+}
+
+template <class T>
+int launch_local_row_n(int N, const StepArgs& a, const Segs& g, int th, bool spec, cudaStream_t st) {
+  switch (N) {
+    case 1: return launch_local_row_t<T, 1>(a, g, th, spec, st);
+    case 2: return launch_local_row_t<T, 2>(a, g, th, spec, st);
+    case 3: return launch_local_row_t<T, 3>(a, g, th, spec, st);
+    case 4: return launch_local_row_t<T, 4>(a, g, th, spec, st);
+    case 5: return launch_local_row_t<T, 5>(a, g, th, spec, st);
+  }
+  return (int)cudaErrorInvalidValue;
+}
+
+}  // namespace row
+}  // namespace adg

@@ -1,0 +1,8 @@
+// Row form of the local kernel, float.
+#include "row_local.cuh"
+
+namespace adg {
+int launch_local_row_f32(int N, const StepArgs& a, const Segs& g, int threads, bool spec, void* stream) {
+  return row::launch_local_row_n<float>(N, a, g, threads, spec, (cudaStream_t)stream);
+}
+}  // namespace adg

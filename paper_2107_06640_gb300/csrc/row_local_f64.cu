@@ -1,0 +1,8 @@
+// Row form of the local kernel, double.
+#include "row_local.cuh"
+
+namespace adg {
+int launch_local_row_f64(int N, const StepArgs& a, const Segs& g, int threads, bool spec, void* stream) {
+  return row::launch_local_row_n<double>(N, a, g, threads, spec, (cudaStream_t)stream);
+}
+}  // namespace adg

@@ -1,0 +1,55 @@
+"""The row kernels (CUDA cores, three elements per warp) against the oracle at
+every degree: boxes with all face kinds and LTS neighbours whose plain and
+special element ranges are not multiples of three, ensembles whose warps mix
+scenarios and elements, and a caller's dofs that are not 16-byte aligned."""
+
+import numpy as np
+import pytest
+
+from _cases import make_pair, rel_l2, to_gpu_layout, to_oracle_layout
+
+pytestmark = pytest.mark.gpu
+
+TOL = {0: 1e-10, 1: 2e-5}  # the repository's parity tolerances of ADG_FP64 and ADG_FP32
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("N,S", [(1, 1), (2, 5), (3, 2), (4, 1), (5, 2)])
+def test_lts_box_every_degree(N, S, precision):
+    from synthetic.workloads import coupled_box, random_dofs
+    m, mat = coupled_box(nxy=5, n_water=1, n_crust=2, L=20e3, depth=6e3, water=1e3, grading=6.0, rigid_bottom=True)
+    m.face_tag[(m.face_tag == 3) & (np.arange(m.nt)[:, None] % 2 == 0)] = 1  # some free surfaces among the absorbing
+    o, s = make_pair(m, mat, N, precision=precision, max_clusters=3, ensemble=S)
+    info = s.info
+    assert info.n_clusters > 1
+    Q0 = random_dofs((S, m.nt, s.B, 9), 5, N=N)
+    s.set_dofs(np.ascontiguousarray(np.stack([to_gpu_layout(q) for q in Q0], axis=1)))
+    s.set_eta(np.zeros((int(info.n_gravity_faces), S, s.Bf)))
+    s.advance(2)
+    got = s.get_dofs().reshape(m.nt, S, 9, s.B)
+    for k in range(S):
+        o.Q, o._D, o.t = Q0[k].copy(), None, 0.0
+        o.eta[:] = 0
+        for _ in range(2):
+            o.advance_macro()
+        assert rel_l2(to_oracle_layout(got[:, k]), o.Q) <= TOL[precision]
+
+
+@pytest.mark.parametrize("precision,N", [(0, 3), (1, 3), (1, 5), (0, 2)])
+def test_noalloc_dofs_at_any_element_alignment(precision, N):
+    import torch
+    from paper_2107_06640_gb300 import _lib
+    from synthetic.workloads import plane_wave_case, random_dofs
+    m, mat = plane_wave_case(2)
+    _, s = make_pair(m, mat, N, precision=precision)
+    Q0 = torch.from_numpy(random_dofs((m.nt, 9, s.B), 3, N=N)).to(torch.float64 if precision == 0 else torch.float32)
+    out = []
+    for off in (0, 1):
+        buf = torch.zeros(Q0.numel() + 4, dtype=Q0.dtype, device="cuda")
+        d = buf[off:off + Q0.numel()]
+        d.copy_(Q0.reshape(-1))
+        _lib.adg_step_noalloc(s.ctx, d.data_ptr(), 2, torch.cuda.current_stream().cuda_stream)
+        out.append(d.cpu().numpy())
+        assert float(buf[:off].abs().sum()) == 0 and float(buf[off + Q0.numel():].abs().sum()) == 0
+    s.sync()
+    assert np.array_equal(out[0], out[1])

@@ -52,6 +52,9 @@ def build(force=False, verbose=False):
     os.makedirs(obj, exist_ok=True)
     os.makedirs(LIBDIR, exist_ok=True)
     cu, cpp = _sources()
+    for f in os.listdir(obj):  # objects of sources that are gone
+        if f.endswith(".o") and f[:-2] not in cu + cpp:
+            os.remove(os.path.join(obj, f))
     common = ["-O3", "-std=c++17", "-Xcompiler", "-fPIC", "-I" + os.path.join(ROOT, "include")]
     jobs = []
     for f in cu:

@@ -7,6 +7,7 @@
 #include <array>
 #include <cmath>
 #include <cstring>
+#include <functional>
 #include <map>
 #include <stdexcept>
 #include <string>
@@ -507,7 +508,7 @@ void Ctx::setup() {
   // neighbour (both on the tensor-core kernels, 3 on their special local
   // instantiation), 2 the CUDA-core kernels: a fault face or more than one
   // gravitational face)
-  std::vector<char> special(E, 0), lts_face(E, 0);
+  std::vector<char> special(E, 0);
   for (int64_t e = 0; e < E; ++e) {
     int ng_e = 0;
     bool cc = false, coarser = false, finer = false;
@@ -519,11 +520,10 @@ void Ctx::setup() {
       coarser = coarser || (e2 >= 0 && cl[e2] > cl[e]);
       finer = finer || (e2 >= 0 && cl[e2] < cl[e]);
     }
-    lts_face[e] = coarser || finer;
     if (tc)
       special[e] = (cc || ng_e > 1) ? 2 : ((ng_e == 1 || finer) ? 3 : (coarser ? 1 : 0));
     else  // the row kernels: their special instantiation takes all of these
-      special[e] = cc || ng_e || lts_face[e] ? 2 : 0;
+      special[e] = cc || ng_e || coarser || finer ? 2 : 0;
   }
   // order key within a cluster: 0 plain elastic, 1 plain fluid on the
   // acoustic local kernel, 2 with a coarser neighbour, 3 with a gravitational
@@ -555,23 +555,14 @@ void Ctx::setup() {
     if (tc && k == 0) cl_elastic[c]++;
     if (tc && k == 1) cl_fluid[c]++;
     if (tc && k == 3) cl_grav[c]++;
-    if (tc && (k == 2 || k == 3) && lts_face[order[i]]) cl_tc_lts[c] = 1;  // (the neighbour kernel's LTS-face code)
+    if (tc && (k == 2 || k == 3)) cl_tc_lts[c] = 1;
   }
   for (int c = 0; c < ncl; ++c) cl_begin[c + 1] += cl_begin[c];
   cluster.resize(E);
   for (int64_t i = 0; i < E; ++i) cluster[i] = cl[order[i]];
 
   // ---- per-element / per-face device data (internal order)
-  // the nodal kernels (a tensor-core context's remaining elements) read flux
-  // matrices, the row kernels (without tensor cores, and adg_step_noalloc in
-  // the contexts that it accepts) coefficient records
-  bool nodal = false, faults = false;
-  for (int c = 0; c < ncl; ++c) nodal = nodal || (tc && cl_plain[c] < cl_begin[c + 1] - cl_begin[c]);
-  for (int64_t k = 0; k < 4 * E; ++k) faults = faults || tag[k] == ADG_TAG_FAULT || tag[k] == ADG_TAG_GRAVITY;
-  const bool rows = !tc || (ncl == 1 && S == 1 && !faults);
-  std::vector<double> par((size_t)E * PAR), Fm(nodal ? (size_t)E * 324 : 0, 0.0), Fp(nodal ? (size_t)E * 324 : 0, 0.0),
-      crec(rows ? (size_t)E * 4 * CREC : 0, 0.0);
-  std::vector<float> frec(tc ? (size_t)E * 4 * FREC : 0, 0.f);
+  std::vector<double> par((size_t)E * PAR), crec((size_t)E * 4 * CREC, 0.0);
   std::vector<int> nbr((size_t)E * 4, -1), ninfo((size_t)E * 4, 0), gslot((size_t)E * 4, -1),
       bslot(E, -1), dslot((size_t)E * 4, -1);
   std::vector<double> gpar;
@@ -598,85 +589,32 @@ void Ctx::setup() {
     par[i * PAR + 11] = mu[eu];
     for (int f = 0; f < 4; ++f) par[i * PAR + 12 + f] = 2.0 * area[4 * eu + f] / detJ[eu];
     const double Zpm = std::sqrt(rho[eu] * (lam[eu] + 2 * mu[eu])), Zsm = std::sqrt(rho[eu] * mu[eu]);
-    const M9 Am = jac_x(rho[eu], lam[eu], mu[eu]);
     bool has_coarse = false;
     for (int f = 0; f < 4; ++f) {
       const double* n = &nrm[12 * eu + 3 * f];
-      M9 T, Ti;
-      rot_mats(n, T, Ti);
-      const M9 TA = mm(T, Am);
       const int tg = tag[4 * eu + f];
-      M9 Mm, Mp, FmM{}, FpM{};
-      int kind = NK_NONE;
-      float* rec = tc ? &frec[((size_t)i * 4 + f) * FREC] : nullptr;
-      if (rec) {
-        for (int d = 0; d < 3; ++d) rec[d] = (float)n[d];
-        rec[5] = (float)(tg == ADG_TAG_FREE ? FACE_FREE
-                         : tg == ADG_TAG_RIGID ? FACE_RIGID
-                         : tg == ADG_TAG_ABSORB ? FACE_ABSORB : FACE_NEIGHBOUR);
-      }
-      if (tg == ADG_TAG_INTERIOR || tg == ADG_TAG_PERIODIC) {
-        const int64_t e2u = nbr_u[4 * eu + f];
-        const double Zpp = std::sqrt(rho[e2u] * (lam[e2u] + 2 * mu[e2u])), Zsp = std::sqrt(rho[e2u] * mu[e2u]);
-        if (rec) {
-          rec[3] = (float)Zpp;
-          rec[4] = (float)Zsp;
-        }
-        godunov_pair(TA, Ti, Zpm, Zpp, Zsm, Zsp, FmM, FpM);
+      const int64_t e2u = nbr_u[4 * eu + f];
+      double Zpp = Zpm, Zsp = Zsm;
+      if (tg == ADG_TAG_INTERIOR || tg == ADG_TAG_PERIODIC || tg == ADG_TAG_FAULT) {
+        Zpp = std::sqrt(rho[e2u] * (lam[e2u] + 2 * mu[e2u]));
+        Zsp = std::sqrt(rho[e2u] * mu[e2u]);
         const int64_t e2 = inv[e2u];
-        nbr[i * 4 + f] = (int)e2;
         const int c1 = cluster[i], c2 = cluster[e2];
-        kind = c1 == c2 ? NK_SAME : (c2 > c1 ? NK_COARSE : NK_FINE);
+        // (a fault face's flux is supplied by the rupture solver from both sides' derivative traces)
+        const int kind = tg == ADG_TAG_FAULT ? NK_FAULT : c1 == c2 ? NK_SAME : (c2 > c1 ? NK_COARSE : NK_FINE);
         if (kind == NK_COARSE) has_coarse = true;
-        if (kind == NK_FINE) dslot[i * 4 + f] = 1;
+        if (kind == NK_FINE || kind == NK_FAULT) dslot[i * 4 + f] = 1;
+        nbr[i * 4 + f] = (int)e2;
         ninfo[i * 4 + f] = nface_u[4 * eu + f] | (nperm_u[4 * eu + f] << 2) | (kind << 5);
       } else if (tg == ADG_TAG_GRAVITY) {
-        if (rec) {
-          const int g = gslot[i * 4 + f];
-          rec[5] = (float)FACE_GRAVITY;
-          std::memcpy(&rec[6], &g, sizeof(int));
-        }
-        middle_state(Zpm, Zpm, Zsm, Zsm, Mm, Mp);
-        // time-integrated middle state: w1 = -rho g H, w7 = eta^{n+1}-eta^n, w4 = w6 = 0,
-        // w8/w9 = w8/w9 - w4/w6 / Z_s (solid) ; Fg applies the shear part to int q^-
-        M9 Sm{};
-        const int pairs[2][2] = {{3, 7}, {5, 8}};
-        for (auto& pr : pairs) {
-          Sm[pr[1] * 9 + pr[1]] = 1;
-          if (Zsm > 0) Sm[pr[1] * 9 + pr[0]] = -1.0 / Zsm;
-        }
-        const M9 Fg = mm(mm(TA, Sm), Ti);
-        const int g = gslot[i * 4 + f];
-        double* gp = &gpar[(size_t)g * GPAR];
+        double* gp = &gpar[(size_t)gslot[i * 4 + f] * GPAR];
         gp[0] = n[0]; gp[1] = n[1]; gp[2] = n[2];
         gp[3] = Zpm;
         gp[4] = rho[eu] * cfg.gravity / Zpm;
         gp[5] = rho[eu] * cfg.gravity;
-        for (int k = 0; k < 81; ++k) gp[6 + k] = Fg[k];
-        for (int q = 0; q < 9; ++q) { gp[87 + q] = TA[q * 9 + 0]; gp[96 + q] = TA[q * 9 + 6]; }
-      } else if (tg == ADG_TAG_FAULT) {
-        kind = NK_FAULT;  // flux supplied by the rupture solver from both sides' derivative traces
-        dslot[i * 4 + f] = 1;
-        nbr[i * 4 + f] = (int)inv[nbr_u[4 * eu + f]];
-        ninfo[i * 4 + f] = nface_u[4 * eu + f] | (nperm_u[4 * eu + f] << 2) | (kind << 5);
-      } else {
-        FmM = boundary_matrix(TA, Ti, Zpm, Zsm, tg);  // free, rigid, absorbing
       }
-      if (nodal)
-        for (int k = 0; k < 81; ++k) {
-          Fm[(i * 4 + f) * 81 + k] = FmM[k];
-          Fp[(i * 4 + f) * 81 + k] = FpM[k];
-        }
-      if (rows) {
-        double Zpp = Zpm, Zsp = Zsm;
-        if (kind != NK_NONE) {
-          const int64_t e2u = nbr_u[4 * eu + f];
-          Zpp = std::sqrt(rho[e2u] * (lam[e2u] + 2 * mu[e2u]));
-          Zsp = std::sqrt(rho[e2u] * mu[e2u]);
-        }
-        face_coefficients(n, tg, Zpm, Zsm, Zpp, Zsp, rho[eu], lam[eu], mu[eu], par[i * PAR + 12 + f],
-                          &crec[((size_t)i * 4 + f) * CREC]);
-      }
+      face_coefficients(n, tg, Zpm, Zsm, Zpp, Zsp, rho[eu], lam[eu], mu[eu], par[i * PAR + 12 + f],
+                        &crec[((size_t)i * 4 + f) * CREC]);
     }
     if (has_coarse) bslot[i] = 1;
   }
@@ -738,19 +676,10 @@ void Ctx::setup() {
   fault_set = false;
 
   // ---- reference operators in device layouts (l-major / n-major)
-  std::vector<double> ktT((size_t)3 * B * B), kvolT((size_t)3 * B1 * B), efcT((size_t)4 * B * Bf),
-      liftT((size_t)4 * Bf * B);
-  for (int a = 0; a < 3; ++a)
-    for (int m = 0; m < B; ++m) {
-      for (int l = 0; l < B; ++l) ktT[((size_t)a * B + l) * B + m] = ops.kt[((size_t)a * B + m) * B + l];
-      for (int l = 0; l < B1; ++l) kvolT[((size_t)a * B1 + l) * B + m] = ops.kvol[((size_t)a * B + m) * B1 + l];
-    }
+  std::vector<double> efcT((size_t)4 * B * Bf);
   for (int f = 0; f < 4; ++f)
     for (int n = 0; n < Bf; ++n)
-      for (int l = 0; l < B; ++l) {
-        efcT[((size_t)f * B + l) * Bf + n] = ops.efc[((size_t)f * Bf + n) * B + l];
-        liftT[((size_t)f * Bf + n) * B + l] = ops.lift[((size_t)f * B + l) * Bf + n];
-      }
+      for (int l = 0; l < B; ++l) efcT[((size_t)f * B + l) * Bf + n] = ops.efc[((size_t)f * Bf + n) * B + l];
 
   const RowTables rt = make_row_tables(ops);
   if (rt.max_err > 1e-10) throw Err(ADG_E_STATE, "internal: the sparse operators do not match the basis");
@@ -773,28 +702,18 @@ void Ctx::setup() {
   dGflux = dalloc((size_t)ng * S * 9 * Bf * ts, owned, dev_bytes);
   if (fp64) {
     dPar = upload_vec<double>(par, owned, dev_bytes);
-    dFm = upload_vec<double>(Fm, owned, dev_bytes);
-    dFp = upload_vec<double>(Fp, owned, dev_bytes);
     dCrec = upload_vec<double>(crec, owned, dev_bytes);
     dRfc = upload_vec<double>(rt.rfcT, owned, dev_bytes);
     dModal = upload_vec<double>(rt.modalT, owned, dev_bytes);
     dReorient = upload_vec<double>(rt.reorient, owned, dev_bytes);
-    dKt = upload_vec<double>(ktT, owned, dev_bytes);
-    dKvol = upload_vec<double>(kvolT, owned, dev_bytes);
     dEfc = upload_vec<double>(efcT, owned, dev_bytes);
-    dLift = upload_vec<double>(liftT, owned, dev_bytes);
   } else {
     dPar = upload_vec<float>(par, owned, dev_bytes);
-    dFm = upload_vec<float>(Fm, owned, dev_bytes);
-    dFp = upload_vec<float>(Fp, owned, dev_bytes);
     dCrec = upload_vec<float>(crec, owned, dev_bytes);
     dRfc = upload_vec<float>(rt.rfcT, owned, dev_bytes);
     dModal = upload_vec<float>(rt.modalT, owned, dev_bytes);
     dReorient = upload_vec<float>(rt.reorient, owned, dev_bytes);
-    dKt = upload_vec<float>(ktT, owned, dev_bytes);
-    dKvol = upload_vec<float>(kvolT, owned, dev_bytes);
     dEfc = upload_vec<float>(efcT, owned, dev_bytes);
-    dLift = upload_vec<float>(liftT, owned, dev_bytes);
   }
   dNbr = upload_raw<int>(nbr, owned, dev_bytes);
   dNinfo = upload_raw<int>(ninfo, owned, dev_bytes);
@@ -806,12 +725,11 @@ void Ctx::setup() {
   CK(cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, cfg.device));
   if (tc) {
     std::vector<float> tl(local_tc_floats(N));
-    pack_local_tc(N, ops.kt.data(), ops.kvol.data(), ops.efc.data(), tl.data());
+    pack_local_tc(N, ops.kt.data(), ops.kvol.data(), rt.rfcT.data(), tl.data());
     dTcLocal = upload_raw<float>(tl, owned, dev_bytes);
     std::vector<float> tf(lift_tc_floats(N));
-    pack_lift_tc(N, ops.lift.data(), tf.data());
+    pack_lift_tc(N, rt.rfcT.data(), tf.data());
     dTcLift = upload_raw<float>(tf, owned, dev_bytes);
-    dFrec = upload_raw<float>(frec, owned, dev_bytes);
     int64_t ngrav = 0;
     for (int c = 0; c < ncl; ++c) ngrav += cl_grav[c];
     if (ngrav > 0 && n_gslots > 0)
@@ -836,12 +754,16 @@ void Ctx::setup() {
     dMlp = (float*)dalloc(MLP_NPARAM * sizeof(float), owned, dev_bytes);
     dCapCount = (unsigned long long*)dalloc(sizeof(unsigned long long), owned, dev_bytes);
   }
+  for (int i = 0; i < kSide; ++i) {
+    CK(cudaStreamCreateWithFlags(&side[i], cudaStreamNonBlocking));
+    CK(cudaEventCreateWithFlags(&side_done[i], cudaEventDisableTiming));
+  }
+  CK(cudaEventCreateWithFlags(&side_fork, cudaEventDisableTiming));
   // configure kernels once (outside any stream capture)
   StepArgs a0 = base_args();
   const Segs none = make_segs(nullptr, 0, 1);
   int rc = launch_local_row(fp64, N, a0, none, stream, 128, false);
   if (!rc) rc = launch_neighbour_row(fp64, N, a0, none, stream, 128, false);
-  if (!rc && tc) rc = launch_local(N, a0, none, stream);
   if (!rc && tc) rc = launch_local_tc(N, a0, none, n_sms, stream, false);
   if (!rc && tc) rc = launch_neighbour_tc(N, a0, none, n_sms, stream, false);
   if (rc) throw Err(ADG_E_CUDA, std::string("kernel configuration: ") + cudaGetErrorString((cudaError_t)rc));
@@ -853,12 +775,12 @@ void Ctx::setup() {
 StepArgs Ctx::base_args() const {
   StepArgs a{};
   a.Q = dQ; a.trace = dTrace; a.btrace = dBtrace; a.dtrace = dDtrace; a.eta = dEta;
-  a.par = dPar; a.Fm = dFm; a.Fp = dFp; a.nbr = dNbr; a.ninfo = dNinfo;
+  a.par = dPar; a.nbr = dNbr; a.ninfo = dNinfo;
   a.gslot = dGslot; a.bslot = dBslot; a.dslot = dDslot;
-  a.ktT = dKt; a.kvolT = dKvol; a.efcT = dEfc; a.liftT = dLift; a.perm = dPerm; a.gpar = dGpar;
+  a.efcT = dEfc; a.perm = dPerm; a.gpar = dGpar;
   a.S = S; a.err = dErr;
   a.fslot = dFslot; a.drout = dDrout; a.gflux = dGflux; a.tc_local = dTcLocal; a.tc_lift = dTcLift;
-  a.frec = dFrec; a.gscr = dGscr;
+  a.gscr = dGscr;
   a.crec = dCrec; a.rfcT = dRfc; a.modalT = dModal; a.reorient = dReorient;
   return a;
 }
@@ -884,11 +806,11 @@ void Ctx::launch_tick(int s, double dtm) {
   StepArgs a = base_args();
   for (int phase = 0; phase < 2; ++phase) {
     // per kernel kind the clusters' segments: tensor-core elastic, tensor-core
-    // acoustic and gravitational-face (local phase only), CUDA-core
+    // acoustic and gravitational-face (local phase only), the row kernels' plain
+    // and special elements
     // (tcb: the local phase's elements with a coarser neighbour outside the
     // special range, on the instantiation with the LTS-buffer code)
-    // (rws, rss: the row kernels' plain and special elements)
-    std::vector<Seg> tcs, tcb, fls, grs, ccs, rws, rss;
+    std::vector<Seg> tcs, tcb, fls, grs, rws, rss;
     bool ltsf = false;
     for (int c = 0; c < ncl; ++c) {
       const bool active = phase == 0 ? s % (1 << c) == 0 : (s + 1) % (1 << c) == 0;
@@ -928,50 +850,89 @@ void Ctx::launch_tick(int s, double dtm) {
         }
       }
       if (tc) {
-        if (n > np) ccs.push_back(seg(cl_begin[c] + np, n - np));
+        if (n > np) rss.push_back(seg(cl_begin[c] + np, n - np));
       } else {
         if (cl_row[c] > 0) rws.push_back(seg(cl_begin[c], cl_row[c]));
         if (n > cl_row[c]) rss.push_back(seg(cl_begin[c] + cl_row[c], n - cl_row[c]));
       }
     }
-    if (tcs.empty() && tcb.empty() && fls.empty() && grs.empty() && ccs.empty() && rws.empty() && rss.empty())
-      continue;
+    if (tcs.empty() && tcb.empty() && fls.empty() && grs.empty() && rws.empty() && rss.empty()) continue;
     ProfEv ev{phase, nullptr, nullptr, 0};
     if (prof) {
       CK(cudaEventCreate(&ev.a));
       CK(cudaEventCreate(&ev.b));
       CK(cudaEventRecord(ev.a, stream));
     }
-    int rc = 0;
-    // one launch per kind and at most kMaxSeg segments
-    auto launch = [&](const std::vector<Seg>& v, int unit, auto&& fn) {
+    // The launches of a phase, the tensor-core kinds first.  They work on
+    // different elements and may run side by side.  A tensor-core kernel takes
+    // whole SMs for all of its tiles, so those are forked only where every CTA
+    // of all of them has an SM of its own from the start (small meshes and LTS
+    // ticks: 1,512 tets at degree 5, local phase, 107 us one after the other
+    // and 50 us side by side); with more tiles than that, kernels on shares of
+    // the SMs were no faster than one after the other on all (183,456 tets
+    // 1.29 against 1.31 ms per step, six-cluster box 6.86 against 6.57 ms).
+    // The row kernels' small blocks mix freely.  adg_profile measures the kinds
+    // one after the other.
+    struct Launch {
+      const std::vector<Seg>* v;
+      int unit, per_cta;  // elements of a work unit; of a tensor-core kernel: units in flight per CTA (0: row kernel)
+      std::function<int(const Segs&, void*)> fn;
+    };
+    const Launch all[] = {
+        {&grs, kTileElems, 2,
+         [&](const Segs& g, void* st) { return launch_local_tc(N, a, g, n_sms, st, true, false, true); }},
+        {&fls, kTileElemsFluid, 2,
+         [&](const Segs& g, void* st) { return launch_local_tc(N, a, g, n_sms, st, false, true); }},
+        {&tcb, kTileElems, 2,
+         [&](const Segs& g, void* st) { return launch_local_tc(N, a, g, n_sms, st, true); }},
+        {&tcs, kTileElems, phase == 0 ? 2 : 3,
+         [&](const Segs& g, void* st) {
+           return phase == 0 ? launch_local_tc(N, a, g, n_sms, st, false) : launch_neighbour_tc(N, a, g, n_sms, st, ltsf);
+         }},
+        {&rss, kRowElems, 0,
+         [&](const Segs& g, void* st) {
+           return phase == 0 ? launch_local_row(fp64, N, a, g, st, cc_threads[0], true)
+                             : launch_neighbour_row(fp64, N, a, g, st, cc_threads[1], true);
+         }},
+        {&rws, kRowElems, 0,
+         [&](const Segs& g, void* st) {
+           return phase == 0 ? launch_local_row(fp64, N, a, g, st, cc_threads[0], false)
+                             : launch_neighbour_row(fp64, N, a, g, st, cc_threads[1], false);
+         }}};
+    constexpr int kKinds = (int)(sizeof(all) / sizeof(all[0]));
+    int64_t units[kKinds] = {}, ctas = 0;
+    int kinds = 0, last = -1;
+    for (int k = 0; k < kKinds; ++k) {
+      for (const Seg& x : *all[k].v) units[k] += (x.n + all[k].unit - 1) / all[k].unit;
+      if (all[k].per_cta) ctas += (units[k] + all[k].per_cta - 1) / all[k].per_cta;
+      if (units[k]) ++kinds, last = k;
+    }
+    const bool fork = kinds > 1 && !prof && ctas <= n_sms;
+    int rc = 0, side_used = 0;
+    bool tc_open = prof != nullptr;
+    if (fork) CK(cudaEventRecord(side_fork, stream));
+    for (int k = 0; k < kKinds && !rc; ++k) {
+      if (tc_open && !all[k].per_cta && ctas) {  // (adg_profile: the tensor-core launches alone)
+        CK(cudaEventCreate(&ev.m));
+        CK(cudaEventRecord(ev.m, stream));
+        tc_open = false;
+      }
+      if (!units[k]) continue;
+      cudaStream_t st = stream;
+      if (fork && k != last) {
+        st = side[side_used];
+        CK(cudaStreamWaitEvent(st, side_fork, 0));
+      }
+      // one launch per kind and at most kMaxSeg segments
+      const std::vector<Seg>& v = *all[k].v;
       for (size_t i = 0; i < v.size() && !rc; i += kMaxSeg) {
-        const int k = (int)std::min<size_t>(kMaxSeg, v.size() - i);
-        rc = fn(make_segs(v.data() + i, k, unit, unit == 1 || unit == kRowElems ? 1 : tc_chunk[phase]));
+        const int n = (int)std::min<size_t>(kMaxSeg, v.size() - i);
+        rc = all[k].fn(make_segs(v.data() + i, n, all[k].unit, all[k].per_cta ? tc_chunk[phase] : 1), st);
         ev.launches++;
       }
-    };
-    launch(tcs, kTileElems, [&](const Segs& g) {
-      return phase == 0 ? launch_local_tc(N, a, g, n_sms, stream, false)
-                        : launch_neighbour_tc(N, a, g, n_sms, stream, ltsf);
-    });
-    launch(tcb, kTileElems, [&](const Segs& g) { return launch_local_tc(N, a, g, n_sms, stream, true); });
-    launch(fls, kTileElemsFluid, [&](const Segs& g) { return launch_local_tc(N, a, g, n_sms, stream, false, true); });
-    launch(grs, kTileElems,
-           [&](const Segs& g) { return launch_local_tc(N, a, g, n_sms, stream, true, false, true); });
-    if (prof && (!tcs.empty() || !tcb.empty() || !fls.empty() || !grs.empty())) {  // the tensor-core launches alone
-      CK(cudaEventCreate(&ev.m));
-      CK(cudaEventRecord(ev.m, stream));
+      if (st != stream) CK(cudaEventRecord(side_done[side_used++], st));
     }
-    launch(ccs, 1, [&](const Segs& g) {
-      return phase == 0 ? launch_local(N, a, g, stream, cc_threads[0])
-                        : launch_neighbour(N, a, g, stream, cc_threads[1]);
-    });
-    for (const bool spec : {true, false})
-      launch(spec ? rss : rws, kRowElems, [&](const Segs& g) {
-        return phase == 0 ? launch_local_row(fp64, N, a, g, stream, cc_threads[0], spec)
-                          : launch_neighbour_row(fp64, N, a, g, stream, cc_threads[1], spec);
-      });
+    for (int i = 0; i < side_used; ++i) CK(cudaStreamWaitEvent(stream, side_done[i], 0));
     if (prof) { CK(cudaEventRecord(ev.b, stream)); prof->push_back(ev); }
     if (rc)
       throw Err(ADG_E_CUDA, std::string(phase == 0 ? "local kernel: " : "neighbour kernel: ") +
@@ -1156,6 +1117,11 @@ Ctx::~Ctx() {
   aio_free();
   if (rec_stream) cudaStreamDestroy(rec_stream);
   if (graph_exec) cudaGraphExecDestroy(graph_exec);
+  for (int i = 0; i < kSide; ++i) {
+    if (side[i]) cudaStreamDestroy(side[i]);
+    if (side_done[i]) cudaEventDestroy(side_done[i]);
+  }
+  if (side_fork) cudaEventDestroy(side_fork);
   for (void* p : owned) cudaFree(p);
   if (hstage) cudaFreeHost(hstage);
   if (own_stream) cudaStreamDestroy(own_stream);

@@ -40,7 +40,7 @@ int launch_isotropic_fluid(int fp64, void* Q, const int64_t* elems, int64_t n, i
 int launch_receivers(int fp64, int B, const void* Q, int S, int64_t n, const int64_t* elem,
                      const double* phi, double* out, void* stream);
 
-// Tables of the row kernels (StepArgs rfcT, modalT, reorient); max_err: the
+// Modal face tables (StepArgs rfcT, modalT, reorient); max_err: the
 // largest difference between the operators' compiled-in entries and `o`'s
 struct RowTables {
   std::vector<double> rfcT, modalT, reorient;
@@ -90,7 +90,7 @@ struct Ctx {
   // (the row kernels' plain instantiation)
   std::vector<int64_t> cl_row;
   // cluster c's tensor-core range includes elements with a coarser or finer
-  // neighbour (the neighbour kernel's LTS-face code)
+  // neighbour or a gravitational face (the neighbour kernel's code for them)
   std::vector<char> cl_tc_lts;
   // acoustic ocean (adg_set_acoustic_ocean): the plain fluid elements of
   // cluster c, [cl_begin[c] + cl_elastic[c], + cl_fluid[c]), take the
@@ -118,13 +118,16 @@ struct Ctx {
   void *dQ = nullptr, *dTrace = nullptr, *dDtrace = nullptr, *dGflux = nullptr;
   int64_t* dOrder = nullptr;  // order on the device: the caller's element of library element i
   double *dBtrace = nullptr, *dEta = nullptr, *dGpar = nullptr;
-  void *dPar = nullptr, *dFm = nullptr, *dFp = nullptr;
-  float* dFrec = nullptr;  // face records of the tensor-core neighbour kernel
-  void *dCrec = nullptr, *dRfc = nullptr, *dModal = nullptr, *dReorient = nullptr;  // row kernels
-  void *dKt = nullptr, *dKvol = nullptr, *dEfc = nullptr, *dLift = nullptr;
+  void* dPar = nullptr;
+  void *dCrec = nullptr, *dRfc = nullptr, *dModal = nullptr, *dReorient = nullptr, *dEfc = nullptr;
   int *dNbr = nullptr, *dNinfo = nullptr, *dGslot = nullptr, *dBslot = nullptr, *dDslot = nullptr,
       *dPerm = nullptr;
   unsigned int* dErr = nullptr;
+  // the launches of one phase are independent of each other and run side by
+  // side: forked onto these streams from the library stream and joined with it
+  static constexpr int kSide = 4;
+  cudaStream_t side[kSide] = {nullptr, nullptr, nullptr, nullptr};
+  cudaEvent_t side_fork = nullptr, side_done[kSide] = {nullptr, nullptr, nullptr, nullptr};
   cudaGraphExec_t graph_exec = nullptr;
   bool use_graph = true;
   // launch shapes (adg_autotune; phase 0 local, 1 neighbour): threads per

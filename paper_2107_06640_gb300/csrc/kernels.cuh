@@ -14,9 +14,7 @@
 //                     numerical-flux): F^- on the own traces, F^+ on the
 //                     neighbours' (re-oriented by a node permutation), the
 //                     stored fluxes of gravitational and fault faces; one lift.
-// Dofs layout: Q[v][9][B] (basis fastest).  Traces: the tensor-core kernels and
-// the nodal kernels beside them [v][4][face_stride(N)], each face block [9][Bf]
-// (node fastest) followed by padding; the row kernels as in row_common.cuh.
+// Dofs layout: Q[v][9][B] (basis fastest).  Face data: modal, see row_common.cuh.
 #pragma once
 #include <cstdint>
 
@@ -24,8 +22,10 @@ namespace adg {
 
 __host__ __device__ constexpr int nb3(int n) { return n < 0 ? 0 : (n + 1) * (n + 2) * (n + 3) / 6; }
 __host__ __device__ constexpr int nb2(int n) { return (n + 1) * (n + 2) / 2; }
-// floats of one face's traces in the trace array: 9 x Bf values [quantity][node],
-// padded to a multiple of 4 so that every face block starts on 16 bytes
+// values of one face in the trace array: traction and velocity in the face's
+// modes, [6][Bf], padded to a multiple of 4 so that a block starts on 16 bytes
+__host__ __device__ constexpr int face_block(int n) { return (6 * nb2(n) + 3) / 4 * 4; }
+// values that the trace array (also the scratch of the FP32 dofs transfers) holds per face
 __host__ __device__ constexpr int face_stride(int n) { return (9 * nb2(n) + 3) / 4 * 4; }
 
 // neighbour-face kinds (ninfo bits 5..7)
@@ -34,39 +34,33 @@ enum { NK_NONE = 0, NK_SAME = 1, NK_COARSE = 2, NK_FINE = 3, NK_FAULT = 4 };
 // per-element parameters (stride PAR): Jinv[9] (d xi_a/d x_d, row a), rho, lam, mu, scale[4]
 constexpr int PAR = 16;
 // per-gravity-face parameters (double, stride GPAR):
-//   n[3], Z, kappa = rho g / Z, rho*g, Fg[81], a1[9], a7[9]
-constexpr int GPAR = 6 + 81 + 18;
+//   n[3], Z, kappa = rho g / Z, rho*g
+constexpr int GPAR = 6;
 
 struct StepArgs {
   void* Q;              // T [V][9][B]
-  void* trace;          // T [V][4][face_stride(N)]: [9][Bf] per face + padding
-  double* btrace;       // [nbslot*S][4][9][Bf]  (LTS buffer, FP64)
-  void* dtrace;         // T [ndslot*S][N+1][9][Bf] (LTS derivative traces)
+  void* trace;          // T [V][4][face_block(N)]
+  double* btrace;       // [nbslot*S][4][face_block(N)]  (LTS buffer, FP64)
+  void* dtrace;         // T [ndslot*S][N+1][9][Bf] (derivative traces; modal blocks, at fault faces nodal)
   double* eta;          // [ngslot*S][Bf]
   const void* par;      // T [E][PAR]
-  const void* Fm;       // T [E][4][81]  row-major F[q][p]
-  const void* Fp;       // T [E][4][81]
   const int* nbr;       // [E][4] internal neighbour element or -1
   const int* ninfo;     // [E][4] j | perm<<2 | kind<<5
   const int* gslot;     // [E][4] gravity slot or -1
   const int* bslot;     // [E]    LTS buffer slot or -1
   const int* dslot;     // [E][4] LTS derivative-trace slot or -1
-  const void* ktT;      // T [3][B(l)][B(m)]   KT_a[m][l] stored l-major
-  const void* kvolT;    // T [3][B1(l)][B(m)]  K_a[m][l]  stored l-major
   const void* efcT;     // T [4][B(l)][Bf(n)]  phi_l at node n stored l-major
-  const void* liftT;    // T [4][Bf(n)][B(m)]  lift[f][m][n] stored n-major
   const int* perm;      // [6][Bf]
   const double* gpar;   // [ngslot][GPAR]
   int S;                // ensemble size
   unsigned int* err;    // device error word
   const int* fslot;     // [E][4] 2*fault + side for fault faces, else -1
   const void* drout;    // T [nff*S][2][9][Bf] time-integrated fault flux per side
-  void* gflux;          // T [ngslot*S][9][Bf] time-integrated flux of gravitational faces
+  void* gflux;          // T [ngslot*S][9][Bf], the first two rows: the modes of the time-integrated normal
+                        // traction -rho g H and normal velocity of gravitational faces
   const float* tc_local; // tensor-core operands of the local kernel (hi/lo, canonical layout), degree 5 or 4
   const float* tc_lift;  // tensor-core lift operand of the neighbour kernel (hi/lo, canonical layout), degree 5 or 4
-  const float* frec;     // [E][4][FREC] face records of the tensor-core neighbour kernel (FP32 dofs)
   float* gscr;           // [ngslot*S][gscr_floats(N)] scratch of the tensor-core local kernel's gravity faces
-  // row kernels
   const void* crec;      // T [E][4][CREC] face coefficients
   const void* rfcT;      // T [4][B(l)][Bf(r)]  face modes of phi_l, l-major
   const void* modalT;    // T [Bf(n)][Bf(r)]    face nodes to face modes, n-major
@@ -74,7 +68,7 @@ struct StepArgs {
 };
 // Virtual elements per warp of the row kernels
 constexpr int kRowElems = 3;
-// Face coefficients of the row kernels: outward normal n[3]; the middle
+// Face coefficients: outward normal n[3]; the middle
 // state's tangential coefficients of the own and of the neighbour's side (t^b
 // from t and v, v^b from t and v) and what the normal components add to them
 // (the same four), the neighbour's traction taken with its own normal; then
@@ -82,20 +76,10 @@ constexpr int kRowElems = 3;
 constexpr int CREC = 24;
 // Per gravity slot and scenario, the tensor-core local kernel's scratch: the
 // normal-projected derivative rows g_m[l] = sum_p w_p D^m[p][l] (m = 0..N,
-// l < B(N - m); w: v_n - sigma_nn / Z), then the own-trace flux part
-// sum_p Fg[q][p] V[p][n] (q < 9, n < Bf).
+// l < B(N - m); w: v_n - sigma_nn / Z), then the face nodes' time-integrated
+// normal traction and velocity.
 __host__ __device__ constexpr int gscr_off(int n, int m) { return m <= 0 ? 0 : gscr_off(n, m - 1) + nb3(n - m + 1); }
-__host__ __device__ constexpr int gscr_floats(int n) { return gscr_off(n, n + 1) + 9 * nb2(n); }
-
-// Face record of the tensor-core neighbour kernel (floats): the outward unit
-// normal n[3], the plus side's impedances Zp+, Zs+ (interior and periodic
-// faces), the face code (FACE_* below), two zeros.  The kernel forms the
-// Godunov flux of Sec. 4.2 from it and the element's own material.
-constexpr int FREC = 8;
-// (FACE_GRAVITY: a gravitational free surface; the record's seventh float
-// holds the bits of its gravity slot, and the kernel lifts the flux the local
-// kernel stored for it)
-enum { FACE_NEIGHBOUR = 0, FACE_FREE = 1, FACE_RIGID = 2, FACE_ABSORB = 3, FACE_GRAVITY = 4 };
+__host__ __device__ constexpr int gscr_floats(int n) { return gscr_off(n, n + 1) + 2 * nb2(n); }
 
 // The clusters of one LTS phase (Sec. 4.4) in a single launch: segment i
 // covers the virtual elements [v_begin, v_begin + n) of one cluster with that
@@ -155,13 +139,13 @@ Segs make_segs(const Seg* s, int n, int unit, int chunk = 1);
 // the derivative traces of every level on faces with a finer neighbour)
 int launch_local_tc(int degree, const StepArgs& a, const Segs& g, int n_sms, void* stream, bool buffers,
                     bool acoustic = false, bool grav = false);
-void pack_local_tc(int degree, const double* kt, const double* kvol, const double* efc, float* out);
+void pack_local_tc(int degree, const double* kt, const double* kvol, const double* rfc, float* out);
 int local_tc_floats(int degree);
 // tensor-core (tcgen05, 3xTF32) neighbour kernel, degree 5 or 4, FP32 dofs
 // (neighbour_tc.cuh), for the same elements
-// coarse: the launch's elements include some with a coarser LTS neighbour
-int launch_neighbour_tc(int degree, const StepArgs& a, const Segs& g, int n_sms, void* stream, bool coarse);
-void pack_lift_tc(int degree, const double* lift, float* out);
+// lts: the launch's elements include some with a neighbour in another cluster or a gravitational face
+int launch_neighbour_tc(int degree, const StepArgs& a, const Segs& g, int n_sms, void* stream, bool lts);
+void pack_lift_tc(int degree, const double* rfc, float* out);
 int lift_tc_floats(int degree);
 
 // ---- dynamic rupture (rupture.cu) ----
@@ -212,9 +196,5 @@ enum { ERR_NAN = 1u, ERR_TIMEOUT = 2u, ERR_NEWTON = 4u };
 // neighbours in another cluster
 int launch_local_row(int fp64, int N, const StepArgs& a, const Segs& g, void* stream, int threads, bool spec);
 int launch_neighbour_row(int fp64, int N, const StepArgs& a, const Segs& g, void* stream, int threads, bool spec);
-// nodal kernels (kernels_impl.cuh): the elements of a tensor-core context
-// (FP32 dofs, degree 5 or 4) that the tensor-core kernels do not take
-int launch_local(int N, const StepArgs& a, const Segs& g, void* stream, int threads = 128);
-int launch_neighbour(int N, const StepArgs& a, const Segs& g, void* stream, int threads = 128);
 
 }  // namespace adg

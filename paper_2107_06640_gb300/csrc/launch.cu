@@ -1,13 +1,7 @@
-// FP32 instantiations of the nodal kernels, and the launchers shared by the kernel kinds.
-#include "kernels_impl.cuh"
+// Launchers shared by the kernel kinds.
+#include "kernels.cuh"
 
 namespace adg {
-int launch_local(int N, const StepArgs& a, const Segs& g, void* stream, int threads) {
-  return dispatch_local(N, a, g, threads, (cudaStream_t)stream);
-}
-int launch_neighbour(int N, const StepArgs& a, const Segs& g, void* stream, int threads) {
-  return dispatch_neighbour(N, a, g, threads, (cudaStream_t)stream);
-}
 
 int launch_local_row_f32(int N, const StepArgs& a, const Segs& g, int threads, bool spec, void* stream);
 int launch_local_row_f64(int N, const StepArgs& a, const Segs& g, int threads, bool spec, void* stream);

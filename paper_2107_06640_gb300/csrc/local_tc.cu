@@ -14,11 +14,11 @@ int launch_local_tc(int degree, const StepArgs& a, const Segs& g, int n_sms, voi
   return launch_local_tc_deg<5>(a, g, n_sms, stream, buffers, acoustic, grav);
 }
 
-void pack_local_tc(int degree, const double* kt, const double* kvol, const double* efc, float* out) {
+void pack_local_tc(int degree, const double* kt, const double* kvol, const double* rfc, float* out) {
   if (degree == 4)
-    pack_local_tc_deg<4>(kt, kvol, efc, out);
+    pack_local_tc_deg<4>(kt, kvol, rfc, out);
   else
-    pack_local_tc_deg<5>(kt, kvol, efc, out);
+    pack_local_tc_deg<5>(kt, kvol, rfc, out);
 }
 
 int local_tc_floats(int degree) { return degree == 4 ? LImg<4>::floats : LImg<5>::floats; }

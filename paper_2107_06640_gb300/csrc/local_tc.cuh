@@ -87,19 +87,18 @@ constexpr int r16(int x) { return (x + 15) / 16 * 16; }
 // (KU[l] rows used, K[l] padded to 8) by the three stacked KT_a, keeping the
 // M[l] rows of D^{l+1} per axis (padded to MP[l]; N = NN[l] = 3 MP[l] padded
 // to 16); the last tensor-core level leaves the 10 rows of D^{N-2}, and the
-// CUDA cores take D^{N-1} (4 rows) and D^N (1 row).  TS: floats per element in
-// the trace staging buffer (the face block, then zeros; 16-byte multiple).
+// CUDA cores take D^{N-1} (4 rows) and D^N (1 row).
 template <int N>
 struct LDeg;
 template <>
 struct LDeg<5> {
-  static constexpr int B = 56, B1 = 35, BF = 21, NL = 3, TS = 196;
+  static constexpr int B = 56, B1 = 35, BF = 21, NL = 3;
   static constexpr int K[3] = {56, 40, 24}, KU[3] = {56, 35, 20}, M[3] = {35, 20, 10}, MP[3] = {40, 24, 16},
                        NN[3] = {128, 80, 48};
 };
 template <>
 struct LDeg<4> {
-  static constexpr int B = 35, B1 = 20, BF = 15, NL = 2, TS = 140;
+  static constexpr int B = 35, B1 = 20, BF = 15, NL = 2;
   static constexpr int K[3] = {40, 24, 0}, KU[3] = {35, 20, 0}, M[3] = {20, 10, 0}, MP[3] = {24, 16, 0},
                        NN[3] = {80, 48, 0};
 };
@@ -112,7 +111,6 @@ struct LImg : LDeg<N> {
   static constexpr int B = D::B, B1 = D::B1, BF = D::BF, NL = D::NL;
   static constexpr int BP = r8(B);            // a row padded to whole 8-column chunks
   static constexpr int NCH = BP / 8;          // 8-column chunks of a row
-  static constexpr int FS = face_stride(N);   // floats per face block of the trace array
   static constexpr int NT = r16(4 * BF);      // traces: 4 faces x BF nodes, padded; K = BP
   static constexpr int NTCH = (4 * BF + 7) / 8;  // 8-column chunks holding traces
   static constexpr int KV = r8(B1);           // volume: K = the B1 rows of I that K_a reads
@@ -133,9 +131,11 @@ struct LImg : LDeg<N> {
   static_assert(BP <= 64 && D::NN[0] <= 128 && NT <= 128 && 2 * KV + NV <= 256, "TMEM columns of a slot");
 };
 
-// trace staging: per warp pair one face of its elements, two buffers
-// alternating over the faces (sized for degree 5, the larger)
-constexpr int kTB = 3 * LDeg<5>::TS;
+// trace staging: per warp pair one face of its 27 elastic rows, two buffers
+// alternating over the faces (sized for degree 5, the larger); the 32 acoustic
+// rows take both as one
+constexpr int kTB = 27 * LDeg<5>::BF + 1;
+static_assert(2 * kTB >= 32 * LDeg<5>::BF, "acoustic rows of a face");
 static_assert(LImg<5>::bytes + 2 * (2 * 128 + 4 * 2 * kTB) * 4 + 64 <= 232448 &&
                   LImg<4>::bytes + 2 * (2 * 128 + 4 * 2 * kTB) * 4 + 64 <= 232448,
               "operands exceed the shared memory of one CTA");
@@ -371,19 +371,31 @@ __device__ __forceinline__ void rows_store(const float* sQ, float* Q, int64_t v0
   }
 }
 
-// One tile, the share of half H (8-column chunks c with c % 2 == H); false
-// after a timed-out wait.
-// kBuf: some elements of the launch have an LTS buffer (a coarser neighbour)
-// tile: index within its segment; t2: this slot's tile after the next among
-// all tiles of the launch (kMulti: the launch has several segments)
+// One column of derivative traces on this row's face: the modes' traction and
+// velocity from the nine quantities of the element (the velocity lanes read the
+// stresses of sigma n, as in the star product), written by the velocity lanes.
+struct DFace {
+  float* d[4] = {nullptr, nullptr, nullptr, nullptr};  // the element's faces with a finer neighbour
+  float n[4][3];                                       // their normals
+  int p = 0;
+};
+template <int N>
+__device__ __forceinline__ void dtrace_out(const DFace& df, const Star& st, int f, int n, int m, float x) {
+  constexpr int BF = nb2(N), FS = face_block(N);
+  const float a0 = __shfl_sync(0xffffffffu, x, st.src[0]), a1 = __shfl_sync(0xffffffffu, x, st.src[1]),
+              a2 = __shfl_sync(0xffffffffu, x, st.src[2]);
+  if (df.d[f] && df.p >= 6) {
+    float* const o = df.d[f] + m * FS + (df.p - 6) * BF + n;
+    o[0] = a0 * df.n[f][0] + a1 * df.n[f][1] + a2 * df.n[f][2];
+    o[3 * BF] = x;
+  }
+}
 // Derivative traces of level m (Sec. 4.4: a finer neighbour integrates this
-// element's Taylor expansion over its sub-steps) on this row's faces with a
-// finer neighbour: one tensor-core round T = D^m E^T with D^m the A operand
-// in TMEM (K = KM), then this half's trace chunks to dtr[f] (null: no finer
-// neighbour on face f; [N+1][9][Bf] per face, this row's quantity already
-// offset).  False after a timed-out wait.
+// element's Taylor expansion over its sub-steps) on the rows' faces with a
+// finer neighbour: one tensor-core round T = D^m R^T with D^m the A operand
+// in TMEM (K = KM), then this half's columns.  False after a timed-out wait.
 template <int N, int H, int KM>
-__device__ __forceinline__ bool dtrace_round(Lane& L, const StepArgs& a, float* const (&dtr)[4], int m) {
+__device__ __forceinline__ bool dtrace_round(Lane& L, const StepArgs& a, const DFace& df, const Star& st, int m) {
   using I_ = LImg<N>;
   constexpr int BF = I_::BF, NTH = H == 0 ? (I_::NTCH + 1) / 2 : I_::NTCH / 2;
   if (!pair_round<H>(L, a.err, [&] {
@@ -405,15 +417,17 @@ __device__ __forceinline__ bool dtrace_round(Lane& L, const StepArgs& a, float* 
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const int col = 8 * (H + 2 * cj) + j;
-      if (col < 4 * BF) {
-        const int f = col / BF, n = col - f * BF;
-        if (dtr[f]) dtr[f][m * 9 * BF + n] = tv[8 * cj + j];
-      }
+      if (col < 4 * BF) dtrace_out<N>(df, st, col / BF, col % BF, m, tv[8 * cj + j]);
     }
   }
   return true;
 }
 
+// One tile, the share of half H (8-column chunks c with c % 2 == H); false
+// after a timed-out wait.
+// kBuf: some elements of the launch have an LTS buffer (a coarser neighbour)
+// tile: index within its segment; t2: this slot's tile after the next among
+// all tiles of the launch (kMulti: the launch has several segments)
 // kSpec: the launch's elements may have one gravitational face and faces with
 // a finer LTS neighbour (elastic instantiation)
 template <int N, class M, int H, bool kBuf, bool kMulti, bool kSpec>
@@ -421,7 +435,7 @@ __device__ __forceinline__ bool local_tile(Lane& L, const StepArgs& a, const Seg
                                            int64_t v_begin, int64_t n_virtual, int64_t tile) {
   using D = LDeg<N>;
   using I_ = LImg<N>;
-  constexpr int B = I_::B, BF = I_::BF, BP = I_::BP, NCH = I_::NCH, FS = I_::FS, TS = D::TS, NL = D::NL;
+  constexpr int B = I_::B, BF = I_::BF, BP = I_::BP, NCH = I_::NCH, FS = face_block(N), NL = D::NL;
   constexpr int TE = M::TE;
   float* const Q = reinterpret_cast<float*>(a.Q);
   const int64_t v0 = v_begin + tile * TE;
@@ -462,17 +476,20 @@ __device__ __forceinline__ bool local_tile(Lane& L, const StepArgs& a, const Seg
   }
   // faces with a finer neighbour: this row's derivative traces there; tile_fine:
   // some element of the tile has one (the same answer in every thread of the slot)
-  float* dtr[4] = {nullptr, nullptr, nullptr, nullptr};
+  DFace df;
   bool tile_fine = false;
   if constexpr (kSpec) {
+    df.p = p;
     if (a.dslot)
       for (int k = 0; k < 4 * nE; ++k) tile_fine |= a.dslot[((v0 + (k >> 2)) / a.S) * 4 + (k & 3)] >= 0;
     if (valid && a.dslot) {
 #pragma unroll
       for (int f = 0; f < 4; ++f) {
         const int ds = a.dslot[e * 4 + f];
-        if (ds >= 0)
-          dtr[f] = reinterpret_cast<float*>(a.dtrace) + ((int64_t)ds * a.S + (v - e * a.S)) * (N + 1) * 9 * BF + p * BF;
+        const float* const c = reinterpret_cast<const float*>(a.crec) + (e * 4 + f) * CREC;
+        if (ds >= 0) df.d[f] = reinterpret_cast<float*>(a.dtrace) + ((int64_t)ds * a.S + (v - e * a.S)) * (N + 1) * 9 * BF;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) df.n[f][d] = c[d];
       }
     }
   }
@@ -541,7 +558,7 @@ __device__ __forceinline__ bool local_tile(Lane& L, const StepArgs& a, const Seg
   // level's A operand, the last leaves the 10 rows of D^NL in registers
   if constexpr (NL == 3) {
     if constexpr (kSpec) {
-      if (tile_fine && !dtrace_round<N, H, D::K[0]>(L, a, dtr, 0)) return false;
+      if (tile_fine && !dtrace_round<N, H, D::K[0]>(L, a, df, st, 0)) return false;
     }
     if (!pair_round<H>(L, a.err, [&] {
           tc::mma3_ts<D::NN[0], D::K[0]>(tbase + cAcc, tbase + cAh, tbase + cAl, sbase + 4 * I_::oP0,
@@ -555,7 +572,7 @@ __device__ __forceinline__ bool local_tile(Lane& L, const StepArgs& a, const Seg
   constexpr int o1 = l1 == 0 ? I_::oP0 : I_::oP1, s1 = l1 == 0 ? I_::sP0 : I_::sP1;
   constexpr int o2 = l2 == 1 ? I_::oP1 : I_::oP2, s2 = l2 == 1 ? I_::sP1 : I_::sP2;
   if constexpr (kSpec) {
-    if (tile_fine && !dtrace_round<N, H, D::K[l1]>(L, a, dtr, l1)) return false;
+    if (tile_fine && !dtrace_round<N, H, D::K[l1]>(L, a, df, st, l1)) return false;
   }
   if (!pair_round<H>(L, a.err, [&] {
         tc::mma3_ts<D::NN[l1], D::K[l1]>(tbase + cAcc, tbase + cAh, tbase + cAl, sbase + 4 * o1,
@@ -565,7 +582,7 @@ __device__ __forceinline__ bool local_tile(Lane& L, const StepArgs& a, const Seg
   level_epilogue<H, D::M[l1], D::MP[l1], true, kSpec>(trow + cAcc, trow + cAh, trow + cAl, st, L.tcf[l1 + 1], I,
                                                      nullptr, gv, gscr_off(N, l1 + 1));
   if constexpr (kSpec) {
-    if (tile_fine && !dtrace_round<N, H, D::K[l2]>(L, a, dtr, l2)) return false;
+    if (tile_fine && !dtrace_round<N, H, D::K[l2]>(L, a, df, st, l2)) return false;
   }
   if (!pair_round<H>(L, a.err, [&] {
         tc::mma3_ts<D::NN[l2], D::K[l2]>(tbase + cAcc, tbase + cAh, tbase + cAl, sbase + 4 * o2,
@@ -617,11 +634,11 @@ __device__ __forceinline__ bool local_tile(Lane& L, const StepArgs& a, const Seg
       const float gsum = elem_sum9(gv.w * d5, gv.base);
       if (gv.dst) gv.dst[gscr_off(N, NL + 2)] = gsum;
       // derivative traces of the last three levels (10, 4 and 1 rows) on the
-      // faces with a finer neighbour, on the CUDA cores (E: hi + lo of the image)
+      // faces with a finer neighbour, on the CUDA cores (R: hi + lo of the image)
       const float* img = reinterpret_cast<const float*>(smem_raw);
 #pragma unroll 1
       for (int f = 0; f < 4; ++f) {
-        if (!dtr[f]) continue;
+        if (!__any_sync(0xffffffffu, df.d[f] != nullptr)) continue;
 #pragma unroll 1
         for (int n = 0; n < BF; ++n) {
           float t3 = 0.f, t4 = 0.f;
@@ -633,30 +650,41 @@ __device__ __forceinline__ bool local_tile(Lane& L, const StepArgs& a, const Seg
             if (l < 4) t4 += E * d4[l];
           }
           const int o0 = tc::canon(f * BF + n, 0, I_::NT);
-          dtr[f][NL * 9 * BF + n] = t3;
-          dtr[f][(NL + 1) * 9 * BF + n] = t4;
-          dtr[f][(NL + 2) * 9 * BF + n] = (img[I_::oT + o0] + img[I_::oT + I_::sT + o0]) * d5;
+          dtrace_out<N>(df, st, f, n, NL, t3);
+          dtrace_out<N>(df, st, f, n, NL + 1, t4);
+          dtrace_out<N>(df, st, f, n, NL + 2, (img[I_::oT + o0] + img[I_::oT + I_::sT + o0]) * d5);
         }
       }
     }
   }
 
-  // ---- face traces: T = I E^T (N = 4 x BF)
+  // ---- modal face traces: T = I R^T (N = 4 x BF)
 #pragma unroll
   for (int c = H; c < NCH; c += 2) tc::st_split8(trow + cAh + 8 * c, trow + cAl + 8 * c, I + 8 * c);
+  // (the normals of this thread's trace items, requested before the round: see below)
+  const int64_t vw = v0 + M::EW * L.w;
+  const int nmine = nE - M::EW * L.w < M::EW ? nE - M::EW * L.w : M::EW;  // elements of this warp (may be <= 0)
+  float nv[4][3];
+  if constexpr (!M::fluid) {
+    const int k = L.lane + 32 * H;
+    if (k < nmine * BF) {
+      const float* const c = reinterpret_cast<const float*>(a.crec) + (vw + k / BF) / a.S * (4 * CREC);
+#pragma unroll
+      for (int f = 0; f < 4; ++f)
+#pragma unroll
+        for (int d = 0; d < 3; ++d) nv[f][d] = c[f * CREC + d];
+    }
+  }
   if (!pair_round<H>(L, a.err, [&] {
         tc::mma3_ts<I_::NT, BP>(tbase + cAcc, tbase + cAh, tbase + cAl, sbase + 4 * I_::oT,
                                 sbase + 4 * (I_::oT + I_::sT), false);
       }))
     return false;
-  // traces leave face by face: the rows go to a shared buffer laid out like
-  // the element's face block in memory, then one thread of the warp pair
-  // copies each element's block with a bulk copy; two buffers alternate, the
-  // copier waits until the copy before the last has read its buffer
+  // traces leave face by face: the nine quantities' modes go to a shared buffer,
+  // then the warp pair forms traction and velocity, one (element, mode) per
+  // thread, and writes them
   {
     constexpr int NTH = H == 0 ? (I_::NTCH + 1) / 2 : I_::NTCH / 2;  // this half's trace chunks
-    const int nmine = nE - M::EW * L.w < M::EW ? nE - M::EW * L.w : M::EW;  // elements of this warp (may be <= 0)
-    const bool copier = H == 0 && L.lane == 0;
     // this half's chunks c = H, H + 2, ... of the trace columns, read once
     float tv[48];
     if constexpr (N == 5) {
@@ -667,118 +695,69 @@ __device__ __forceinline__ bool local_tile(Lane& L, const StepArgs& a, const Seg
       tc::ld3x8(trow + cAcc + 8 * H, trow + cAcc + 8 * (H + 2), trow + cAcc + 8 * (H + 4), tv);
       tc::ld8(trow + cAcc + 8 * (H + 6), tv + 24);
     }
-    // an element with a coarser neighbour also adds its four face traces to
-    // its LTS buffer, in FP64 (overwrite at the first of the two steps)
-    if (kBuf && !M::fluid && L.btrace_mode && a.bslot && valid) {
-      const int bs = a.bslot[e];
-      if (bs >= 0) {
-        double* bt = a.btrace + ((int64_t)bs * a.S + (v - e * a.S)) * 36 * BF;
 #pragma unroll
-        for (int cj = 0; cj < NTH; ++cj) {
+    for (int f = 0; f < 4; ++f) {
+      float* sTf = s_T[L.slot][L.w] + (M::fluid ? 0 : f & 1) * kTB;
+#pragma unroll
+      for (int cj = 0; cj < NTH; ++cj) {
+        const int c = H + 2 * cj;
+        if (8 * c + 7 < BF * f || 8 * c >= BF * (f + 1)) continue;  // chunk outside face f
+        if (valid) {
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
-            const int col = 8 * (H + 2 * cj) + j;
-            if (col < 4 * BF) {
-              const int f = col / BF, n = col - f * BF;
-              double* b = bt + (f * 9 + p) * BF + n;
-              *b = (L.btrace_mode == 1 ? 0.0 : *b) + (double)tv[8 * cj + j];
-            }
+            const int col = 8 * c + j;
+            if (col >= BF * f && col < BF * (f + 1)) sTf[(jj * M::Q + p) * BF + col - BF * f] = tv[8 * cj + j];
           }
         }
       }
-    }
-    if constexpr (M::fluid) {
-      // acoustic: this face's (p, v) rows of the warp's eight elements in a
-      // compact buffer [element][4][BF], then the warp pair writes each
-      // element's full face block (sigma_xx three times, zero shear, v,
-      // padding zeros) with 16-byte stores
-      float* sC = s_T[L.slot][L.w];
+      warp_pair_bar(L.slot, L.w);
 #pragma unroll
-      for (int f = 0; f < 4; ++f) {
-#pragma unroll
-        for (int cj = 0; cj < NTH; ++cj) {
-          const int c = H + 2 * cj;
-          if (8 * c + 7 < BF * f || 8 * c >= BF * (f + 1)) continue;  // chunk outside face f
-          if (valid) {
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              const int col = 8 * c + j;
-              if (col >= BF * f && col < BF * (f + 1)) sC[(jj * 4 + p) * BF + col - BF * f] = tv[8 * cj + j];
-            }
-          }
+      for (int it = 0; it < (M::EW * BF + 63) / 64; ++it) {
+        const int k = L.lane + 32 * H + 64 * it, ej = k / BF, n = k - ej * BF;
+        if (k >= nmine * BF) continue;
+        const int64_t ve = vw + ej, ee = ve / a.S;
+        float nx, ny, nz;
+        if constexpr (M::fluid) {
+          const float* const c = reinterpret_cast<const float*>(a.crec) + (ee * 4 + f) * CREC;
+          nx = c[0]; ny = c[1]; nz = c[2];
+        } else {
+          nx = nv[f][0]; ny = nv[f][1]; nz = nv[f][2];
         }
-        warp_pair_bar(L.slot, L.w);
-        for (int k = L.lane + 32 * H; k < nmine * (FS / 4); k += 64) {
-          const int ej = k / (FS / 4), c4 = k - ej * (FS / 4);
-          float x[4];
-#pragma unroll
-          for (int t = 0; t < 4; ++t) {
-            const int idx = 4 * c4 + t, r = idx / BF, n = idx - BF * (idx / BF);
-            x[t] = (idx >= 9 * BF || (r >= 3 && r < 6)) ? 0.f : sC[(ej * 4 + (r < 3 ? 0 : r - 5)) * BF + n];
-          }
-          reinterpret_cast<float4*>(reinterpret_cast<float*>(a.trace) +
-                                    ((v0 + M::EW * L.w + ej) * 4 + f) * FS)[c4] = make_float4(x[0], x[1], x[2], x[3]);
+        const float* const x = sTf + ej * M::Q * BF + n;
+        float o[6];
+        if constexpr (M::fluid) {
+          const float s = x[0];
+          o[0] = s * nx; o[1] = s * ny; o[2] = s * nz;
+          o[3] = x[BF]; o[4] = x[2 * BF]; o[5] = x[3 * BF];
+        } else {
+          const float sxy = x[3 * BF], syz = x[4 * BF], sxz = x[5 * BF];
+          o[0] = x[0] * nx + sxy * ny + sxz * nz;
+          o[1] = sxy * nx + x[BF] * ny + syz * nz;
+          o[2] = sxz * nx + syz * ny + x[2 * BF] * nz;
+          o[3] = x[6 * BF]; o[4] = x[7 * BF]; o[5] = x[8 * BF];
         }
-        warp_pair_bar(L.slot, L.w);  // the next face refills the buffer
-      }
-    } else {
+        float* const out = reinterpret_cast<float*>(a.trace) + (ve * 4 + f) * FS + n;
 #pragma unroll
-      for (int f = 0; f < 4; ++f) {
-        float* sTf = s_T[L.slot][L.w] + (f & 1) * kTB;
+        for (int d = 0; d < 6; ++d) out[d * BF] = o[d];
+        // an element with a coarser neighbour also adds its face traces to its
+        // LTS buffer, in FP64 (overwrite at the first of the two steps)
+        if (kBuf && !M::fluid && L.btrace_mode && a.bslot) {
+          const int bs = a.bslot[ee];
+          if (bs >= 0) {
+            double* const b = a.btrace + (((int64_t)bs * a.S + (ve - ee * a.S)) * 4 + f) * FS + n;
 #pragma unroll
-        for (int cj = 0; cj < NTH; ++cj) {
-          const int c = H + 2 * cj;
-          if (8 * c + 7 < BF * f || 8 * c >= BF * (f + 1)) continue;  // chunk outside face f
-          if (valid) {
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              const int col = 8 * c + j;
-              if (col >= BF * f && col < BF * (f + 1)) sTf[jj * TS + p * BF + col - BF * f] = tv[8 * cj + j];
-            }
-          }
-        }
-        tc::fence_async_smem();
-        if (copier) tc::bulk_wait_read();  // the other buffer is free for face f + 1
-        warp_pair_bar(L.slot, L.w);
-        if (copier) {
-          for (int ej = 0; ej < nmine; ++ej)
-            tc::bulk_store(reinterpret_cast<float*>(a.trace) + ((v0 + M::EW * L.w + ej) * 4 + f) * FS,
-                           sTf + ej * TS, FS * 4);
-          tc::bulk_commit();
-        }
-        if constexpr (kSpec) {
-          // the own-trace part of the gravitational face's flux, sum_p Fg[q][p] V[p][n],
-          // from this face's staged block, for the warp pair's elements whose gravitational face is f
-          int gfe[M::EW], gse[M::EW];
-#pragma unroll
-          for (int ej = 0; ej < M::EW; ++ej) {
-            gfe[ej] = __shfl_sync(0xffffffffu, gface, 9 * ej);
-            gse[ej] = __shfl_sync(0xffffffffu, gsl, 9 * ej);
-          }
-          for (int k = L.lane + 32 * H; k < nmine * 9 * BF; k += 64) {
-            const int ej = k / (9 * BF), r = k - ej * 9 * BF, q = r / BF, n = r - q * BF;
-            int gf = -1, gs = -1;
-#pragma unroll
-            for (int jx = 0; jx < M::EW; ++jx)
-              if (jx == ej) { gf = gfe[jx]; gs = gse[jx]; }
-            if (gf != f || gs < 0) continue;
-            const double* Fg = a.gpar + (int64_t)gs * GPAR + 6 + q * 9;
-            float acc = 0.f;
-#pragma unroll
-            for (int pp = 0; pp < 9; ++pp) acc += (float)Fg[pp] * sTf[ej * TS + pp * BF + n];
-            const int64_t ve = v0 + M::EW * L.w + ej;
-            a.gscr[((int64_t)gs * a.S + (ve - (ve / a.S) * a.S)) * gscr_floats(N) + gscr_off(N, N + 1) + q * BF + n] =
-                acc;
+            for (int d = 0; d < 6; ++d) b[d * BF] = (L.btrace_mode == 1 ? 0.0 : b[d * BF]) + (double)o[d];
           }
         }
       }
+      if constexpr (M::fluid) warp_pair_bar(L.slot, L.w);  // the next face refills the buffer
     }
   }
 
   // ---- gravitational faces: the face's normal-projected derivative traces
   // f_m = E g_m, the (eta, H) ODE of Sec. 4.3 in FP64 over the step (its
   // Taylor series, as in the CUDA-core kernel) and the face's time-integrated
-  // flux; one (element, node) per thread of the slot
+  // normal traction and velocity; one (element, node) per thread of the slot
   if constexpr (kSpec) {
     pair_bar(L.slot);  // the slot's scratch rows are written
     const int u = L.t + 128 * H;
@@ -793,17 +772,15 @@ __device__ __forceinline__ bool local_tile(Lane& L, const StepArgs& a, const Seg
         if (x >= 0) { gf = f; gs = x; }
       }
       if (gs >= 0) {
-        const float* gsrc = a.gscr + ((int64_t)gs * a.S + sc) * gscr_floats(N);
-        const float* img = reinterpret_cast<const float*>(smem_raw);
+        float* const gsrc = a.gscr + ((int64_t)gs * a.S + sc) * gscr_floats(N);
+        const float* const E = reinterpret_cast<const float*>(a.efcT) + (size_t)gf * B * BF + n;
         double fm[N + 1];
 #pragma unroll
         for (int m = 0; m <= N; ++m) {
           const int Bm = nb3(N - m);
           float acc = 0.f;
-          for (int l = 0; l < Bm; ++l) {
-            const int o = tc::canon(gf * BF + n, l, I_::NT);
-            acc += (img[I_::oT + o] + img[I_::oT + I_::sT + o]) * gsrc[gscr_off(N, m) + l];
-          }
+#pragma unroll 8
+          for (int l = 0; l < Bm; ++l) acc += E[(size_t)l * BF] * gsrc[gscr_off(N, m) + l];
           fm[m] = (double)acc * kRcpFact[m];
         }
         const double* gp = a.gpar + (int64_t)gs * GPAR;
@@ -825,11 +802,29 @@ __device__ __forceinline__ bool local_tile(Lane& L, const StepArgs& a, const Seg
           if (m > N && fabs(term) <= 1e-17 * fabs(e1)) break;
         }
         eta[n] = e1;
-        float* gfl = reinterpret_cast<float*>(a.gflux) + ((int64_t)gs * a.S + sc) * 9 * BF;
+        gsrc[gscr_off(N, N + 1) + n] = (float)(-rg * Hint);
+        gsrc[gscr_off(N, N + 1) + BF + n] = (float)(e1 - eta0);
+      }
+    }
+    pair_bar(L.slot);
+    // ... and the face modes of both
+    if (u < TE * BF && ei < nE && a.gslot) {
+      const int64_t ve = v0 + ei, ee = ve / a.S;
+      const int sc = (int)(ve - ee * a.S);
+      int gs = -1;
 #pragma unroll
-        for (int q = 0; q < 9; ++q)
-          gfl[q * BF + n] = (float)(gp[87 + q] * (-rg * Hint) + gp[96 + q] * (e1 - eta0) +
-                                    (double)gsrc[gscr_off(N, N + 1) + q * BF + n]);
+      for (int f = 0; f < 4; ++f) gs = max(gs, a.gslot[ee * 4 + f]);
+      if (gs >= 0) {
+        const float* const src = a.gscr + ((int64_t)gs * a.S + sc) * gscr_floats(N) + gscr_off(N, N + 1);
+        const float* const mn = reinterpret_cast<const float*>(a.modalT) + n;
+        float h = 0.f, d = 0.f;
+        for (int k = 0; k < BF; ++k) {
+          h += mn[k * BF] * src[k];
+          d += mn[k * BF] * src[BF + k];
+        }
+        float* const gfl = reinterpret_cast<float*>(a.gflux) + ((int64_t)gs * a.S + sc) * 9 * BF + n;
+        gfl[0] = h;
+        gfl[BF] = d;
       }
     }
   }
@@ -982,7 +977,6 @@ __global__ void __launch_bounds__(kThreadsL, 1) local_tc_kernel(StepArgs a, cons
   // after a timed-out wait, give this slot's MMAs in flight a bounded chance
   // to finish before the columns are freed
   if (half == 0 && L.t == 0 && s_abort[slot]) tc::mbar_wait(&mbar[slot], L.phase ^ 1u, kWaitIters);
-  if (half == 0 && L.lane == 0) tc::bulk_wait();  // trace copies complete before shared memory is released
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
@@ -1037,10 +1031,10 @@ int launch_local_tc_deg(const StepArgs& a, const Segs& g, int n_sms, void* strea
 }
 
 // Host-side image of the operands of degree N: kt[a][m][l], kvol[a][m][l]
-// (l < B1) and efc[f][n][l] of that degree's basis, split into tf32 hi / lo
+// (l < B1) and rfc[f][l][r] of that degree's basis, split into tf32 hi / lo
 // and laid out as the canonical K-major B operands of local_tc_kernel.
 template <int N>
-void pack_local_tc_deg(const double* kt, const double* kvol, const double* efc, float* out) {
+void pack_local_tc_deg(const double* kt, const double* kvol, const double* rfc, float* out) {
   using D = LDeg<N>;
   using I_ = LImg<N>;
   constexpr int B = I_::B, B1 = I_::B1, BF = I_::BF, BP = I_::BP;
@@ -1064,7 +1058,7 @@ void pack_local_tc_deg(const double* kt, const double* kvol, const double* efc, 
         put(I_::oV, I_::sV, I_::NV, ax * BP + m, l, kvol[((size_t)ax * B + m) * B1 + l]);
   for (int f = 0; f < 4; ++f)
     for (int n = 0; n < BF; ++n)
-      for (int l = 0; l < B; ++l) put(I_::oT, I_::sT, I_::NT, f * BF + n, l, efc[((size_t)f * BF + n) * B + l]);
+      for (int l = 0; l < B; ++l) put(I_::oT, I_::sT, I_::NT, f * BF + n, l, rfc[((size_t)f * B + l) * BF + n]);
   for (int ax = 0; ax < 3; ++ax)
     for (int m = 0; m < 4; ++m)
       for (int l = 0; l < 10; ++l) out[I_::oK3 + (ax * 4 + m) * 10 + l] = (float)kt[((size_t)ax * B + m) * B + l];

@@ -3,8 +3,8 @@
 
 namespace adg {
 
-int launch_neighbour_tc4(const StepArgs& a, const Segs& g, int n_sms, void* stream, bool coarse) {
-  return launch_neighbour_tc_deg<4>(a, g, n_sms, stream, coarse);
+int launch_neighbour_tc4(const StepArgs& a, const Segs& g, int n_sms, void* stream, bool lts) {
+  return launch_neighbour_tc_deg<4>(a, g, n_sms, stream, lts);
 }
 
 }  // namespace adg

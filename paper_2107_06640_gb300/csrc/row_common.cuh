@@ -1,17 +1,18 @@
 // What the two row kernels (row_local.cuh, row_neighbour.cuh) share.
 //
 // They are the CUDA-core form of the element update, in both precisions and at
-// every degree: one warp works on three (virtual) elements, lane 9 j + p holds
+// every degree (in a tensor-core context for its fault elements): one warp works on three (virtual) elements, lane 9 j + p holds
 // the row of quantity p of element j in registers (lanes 27..31 idle), the
 // operators are straight-line sparse code (sparse_ops.cuh), the quantities of
 // an element meet in warp shuffles, and no block barrier is needed.
 //
 // Face data are modal: a face block holds traction sigma n (n the owner's
 // outward normal) and velocity, the six quantities that the Godunov flux
-// reads, in the face's orthonormal Dubiner modes, [6][Bf].  An element's four
-// blocks follow one another ([v][4][6][Bf] in the trace array).  LTS buffers
-// ([slot*S][4][6][Bf], FP64) and the derivative traces of faces with a finer
-// neighbour ([slot*S][N+1][6][Bf]) are modal as well; those of fault faces stay
+// reads, in the face's orthonormal Dubiner modes: [6][Bf], padded to
+// face_block(N) values.  An element's four blocks follow one another in the
+// trace array.  LTS buffers ([slot*S][4] blocks, FP64) and the derivative
+// traces of faces with a finer neighbour ([slot*S][N+1] blocks in the space of
+// [N+1][9][Bf]) are modal as well; those of fault faces stay
 // nodal in all nine quantities ([N+1][9][Bf]), as the friction solve reads them.
 //
 // What bounds them: FP64, the 2 FMA per clock and SM (the sparse form has 3.4
@@ -46,7 +47,7 @@ struct Shape {
   static constexpr int words(int s) { return s * (int)sizeof(T) / 4; }
   // 16-byte accesses: the stride in 16-byte units must be odd
   static constexpr int SB = VW == 1 ? (sizeof(T) == 4 ? (B | 1) : B) : (B / VW % 2 ? B : B + VW);
-  static constexpr int FS = 6 * Bf;            // values of a face block
+  static constexpr int FS = face_block(N);     // values of a face block
   static constexpr int ND = nb3(N) + nb3(N - 1) + nb3(N - 2) + nb3(N - 3) + nb3(N - 4) + nb3(N - 5);
 };
 // row offset of D^k in a row's derivative stack

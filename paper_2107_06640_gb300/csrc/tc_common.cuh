@@ -203,6 +203,30 @@ __device__ __forceinline__ void ld8(uint32_t t, float o[8]) {
   for (int j = 0; j < 8; ++j) o[j] = __uint_as_float(r[j]);
 }
 
+// 8 C consecutive fp32 columns of this warp's lanes (one wait)
+template <int C>
+__device__ __forceinline__ void ld8s(uint32_t t, float* o) {
+  uint32_t r[8 * C];
+#pragma unroll
+  for (int c = 0; c < C; ++c)
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[8 * c]), "=r"(r[8 * c + 1]), "=r"(r[8 * c + 2]), "=r"(r[8 * c + 3]), "=r"(r[8 * c + 4]),
+                   "=r"(r[8 * c + 5]), "=r"(r[8 * c + 6]), "=r"(r[8 * c + 7])
+                 : "r"(t + 8 * c));
+  // (the wait ties every loaded register: none may be read before it)
+#pragma unroll
+  for (int c = 0; c < C; ++c) {
+    if (c == 0)
+      asm volatile("tcgen05.wait::ld.sync.aligned;"
+                   : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]));
+    else
+      asm volatile("" : "+r"(r[8 * c]), "+r"(r[8 * c + 1]), "+r"(r[8 * c + 2]), "+r"(r[8 * c + 3]),
+                   "+r"(r[8 * c + 4]), "+r"(r[8 * c + 5]), "+r"(r[8 * c + 6]), "+r"(r[8 * c + 7]));
+  }
+#pragma unroll
+  for (int k = 0; k < 8 * C; ++k) o[k] = __uint_as_float(r[k]);
+}
+
 // 8 values of this lane's row -> tf32 hi at column th, lo (the remainder) at column tl
 __device__ __forceinline__ void st_split8(uint32_t th, uint32_t tl, const float x[8]) {
   uint32_t h[8], l[8];

@@ -876,35 +876,35 @@ void Ctx::launch_tick(int s, double dtm) {
     struct Launch {
       const std::vector<Seg>* v;
       int unit, per_cta;  // elements of a work unit; of a tensor-core kernel: units in flight per CTA (0: row kernel)
-      std::function<int(const Segs&, void*)> fn;
+      std::function<int(const Segs&, int, void*)> fn;  // (segments, SMs to use, stream)
     };
     const Launch all[] = {
-        {&grs, kTileElems, 2,
-         [&](const Segs& g, void* st) { return launch_local_tc(N, a, g, n_sms, st, true, false, true); }},
+        {&grs, kTileElems, 1,
+         [&](const Segs& g, int sms, void* st) { return launch_local_tc(N, a, g, sms, st, true, false, true); }},
         {&fls, kTileElemsFluid, 2,
-         [&](const Segs& g, void* st) { return launch_local_tc(N, a, g, n_sms, st, false, true); }},
+         [&](const Segs& g, int sms, void* st) { return launch_local_tc(N, a, g, sms, st, false, true); }},
         {&tcb, kTileElems, 2,
-         [&](const Segs& g, void* st) { return launch_local_tc(N, a, g, n_sms, st, true); }},
+         [&](const Segs& g, int sms, void* st) { return launch_local_tc(N, a, g, sms, st, true); }},
         {&tcs, kTileElems, phase == 0 ? 2 : 3,
-         [&](const Segs& g, void* st) {
-           return phase == 0 ? launch_local_tc(N, a, g, n_sms, st, false) : launch_neighbour_tc(N, a, g, n_sms, st, ltsf);
+         [&](const Segs& g, int sms, void* st) {
+           return phase == 0 ? launch_local_tc(N, a, g, sms, st, false) : launch_neighbour_tc(N, a, g, sms, st, ltsf);
          }},
         {&rss, kRowElems, 0,
-         [&](const Segs& g, void* st) {
+         [&](const Segs& g, int sms, void* st) {
            return phase == 0 ? launch_local_row(fp64, N, a, g, st, cc_threads[0], true)
                              : launch_neighbour_row(fp64, N, a, g, st, cc_threads[1], true);
          }},
         {&rws, kRowElems, 0,
-         [&](const Segs& g, void* st) {
+         [&](const Segs& g, int sms, void* st) {
            return phase == 0 ? launch_local_row(fp64, N, a, g, st, cc_threads[0], false)
                              : launch_neighbour_row(fp64, N, a, g, st, cc_threads[1], false);
          }}};
     constexpr int kKinds = (int)(sizeof(all) / sizeof(all[0]));
-    int64_t units[kKinds] = {}, ctas = 0;
+    int64_t units[kKinds] = {}, ctas = 0, tiles = 0;
     int kinds = 0, last = -1;
     for (int k = 0; k < kKinds; ++k) {
       for (const Seg& x : *all[k].v) units[k] += (x.n + all[k].unit - 1) / all[k].unit;
-      if (all[k].per_cta) ctas += (units[k] + all[k].per_cta - 1) / all[k].per_cta;
+      if (all[k].per_cta) ctas += (units[k] + all[k].per_cta - 1) / all[k].per_cta, tiles += units[k];
       if (units[k]) ++kinds, last = k;
     }
     const bool fork = kinds > 1 && !prof && ctas <= n_sms;
@@ -924,10 +924,12 @@ void Ctx::launch_tick(int s, double dtm) {
         CK(cudaStreamWaitEvent(st, side_fork, 0));
       }
       // one launch per kind and at most kMaxSeg segments
+      // (side by side: a CTA per tile where that fits, else full CTAs)
+      const int sms = fork && all[k].per_cta && tiles > n_sms ? (int)((units[k] + all[k].per_cta - 1) / all[k].per_cta) : n_sms;
       const std::vector<Seg>& v = *all[k].v;
       for (size_t i = 0; i < v.size() && !rc; i += kMaxSeg) {
         const int n = (int)std::min<size_t>(kMaxSeg, v.size() - i);
-        rc = all[k].fn(make_segs(v.data() + i, n, all[k].unit, all[k].per_cta ? tc_chunk[phase] : 1), st);
+        rc = all[k].fn(make_segs(v.data() + i, n, all[k].unit, all[k].per_cta ? tc_chunk[phase] : 1), sms, st);
         ev.launches++;
       }
       if (st != stream) CK(cudaEventRecord(side_done[side_used++], st));

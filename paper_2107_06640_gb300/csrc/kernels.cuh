@@ -66,6 +66,13 @@ struct StepArgs {
   const void* modalT;    // T [Bf(n)][Bf(r)]    face nodes to face modes, n-major
   const void* reorient;  // T [6][sum (n+1)^2]  a neighbour's face modes in this side's, blocks by degree
 };
+// Element of a virtual element, S scenarios per element: the 64-bit division
+// (some 100 instructions) only where it is needed.
+__host__ __device__ inline int64_t elem_of(int64_t v, int S) {
+  if (S == 1) return v;
+  if ((v >> 32) == 0) return (int64_t)((uint32_t)v / (uint32_t)S);
+  return v / S;
+}
 // Virtual elements per warp of the row kernels
 constexpr int kRowElems = 3;
 // Face coefficients: outward normal n[3]; the middle
@@ -97,9 +104,18 @@ struct Seg {
   int64_t v_begin, n;
   double tcoef[8];   // dt^{k+1}/(k+1)!, k = 0..N (the cluster's own step)
   double ccoef[8];   // (tb^{k+1}-ta^{k+1})/(k+1)! on a coarser neighbour's expansion
+  float tcoef32[8], ccoef32[8];  // the same in FP32 (make_segs): a conversion in the kernel would run on the FP64 pipe
   double dt;         // the cluster's step (gravity ODE)
   int btrace_mode;   // 0 none, 1 overwrite, 2 accumulate (LTS buffers)
 };
+template <class T>
+__host__ __device__ inline T seg_tcoef(const Seg& s, int k) {
+  if constexpr (sizeof(T) == 4) return s.tcoef32[k]; else return s.tcoef[k];
+}
+template <class T>
+__host__ __device__ inline T seg_ccoef(const Seg& s, int k) {
+  if constexpr (sizeof(T) == 4) return s.ccoef32[k]; else return s.ccoef[k];
+}
 struct Segs {
   int n;                        // segments
   int chunk;                    // tensor-core kernels: consecutive tiles a CTA slot takes per sweep
@@ -118,11 +134,6 @@ __host__ __device__ inline int seg_find(const Segs& g, int64_t u) {
   int i = 0;
   while (i + 1 < g.n && u >= g.first[i + 1]) ++i;
   return i;
-}
-// segment of work unit u in a launch that may have several (kMulti) or has one
-template <bool kMulti>
-__host__ __device__ inline int seg_of(const Segs& g, int64_t u) {
-  return kMulti ? seg_find(g, u) : 0;
 }
 // Segs of the given segments with `unit` virtual elements per work unit
 Segs make_segs(const Seg* s, int n, int unit, int chunk = 1);

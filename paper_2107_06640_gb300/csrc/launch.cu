@@ -24,6 +24,10 @@ Segs make_segs(const Seg* s, int n, int unit, int chunk) {
   for (int i = 0; i < n && g.n < kMaxSeg; ++i) {
     if (s[i].n <= 0) continue;
     g.s[g.n] = s[i];
+    for (int k = 0; k < 8; ++k) {
+      g.s[g.n].tcoef32[k] = (float)s[i].tcoef[k];
+      g.s[g.n].ccoef32[k] = (float)s[i].ccoef[k];
+    }
     g.first[g.n] = u;
     u += (s[i].n + unit - 1) / unit;
     g.n++;

@@ -36,38 +36,15 @@ namespace {
 
 constexpr int TE = kTileElems;
 constexpr int kSlotsN = 3, kThreadsN = 128 * kSlotsN;
-constexpr int kWaitIters = 1 << 22;
+using tc::kWaitIters;
 
-__host__ __device__ constexpr int up8(int x) { return (x + 7) / 8 * 8; }
-__host__ __device__ constexpr int up16(int x) { return (x + 15) / 16 * 16; }
-
-// modes of parity p among the first n of the element's basis / a face's basis
-__host__ __device__ constexpr int count_par(int n, int p) {
-  int c = 0;
-  for (int l = 0; l < n; ++l) c += sp::parity(l) == p;
-  return c;
-}
-__host__ __device__ constexpr int fparity(int r) {  // of i in psi_ij (order: degree, then i)
-  int n = 0;
-  while ((n + 1) * (n + 2) / 2 <= r) ++n;
-  return (r - n * (n + 1) / 2) & 1;
-}
-__host__ __device__ constexpr int count_fpar(int n, int p) {
-  int c = 0;
-  for (int r = 0; r < n; ++r) c += fparity(r) == p;
-  return c;
-}
-// place of mode l among those of its parity
-__host__ __device__ constexpr int par_index(int l) {
-  int c = 0;
-  for (int k = 0; k < l; ++k) c += sp::parity(k) == sp::parity(l);
-  return c;
-}
-__host__ __device__ constexpr int fpar_index(int r) {
-  int c = 0;
-  for (int k = 0; k < r; ++k) c += fparity(k) == fparity(r);
-  return c;
-}
+using sp::count_fpar;
+using sp::count_par;
+using sp::fpar_index;
+using sp::fparity;
+using sp::par_index;
+using tc::up16;
+using tc::up8;
 
 template <int N>
 struct NImg {
@@ -90,7 +67,6 @@ struct NImg {
   static_assert(bytes + 256 <= 232448, "neighbour tensor-core kernel exceeds the shared memory of one CTA");
 };
 
-__device__ __forceinline__ void slot_bar(int slot) { asm volatile("bar.sync %0, 128;" ::"r"(slot + 1)); }
 // kOne: one scenario (S = 1), where a virtual element is its element and the
 // 64-bit divisions by S drop out; kLts: the launch's elements may have a
 // neighbour in another cluster or a gravitational face (without, that code
@@ -142,9 +118,8 @@ __global__ void __launch_bounds__(kThreadsN, 1) neighbour_tc_kernel(StepArgs a, 
   float* const sStage = sm + NI::oW + (slot * 4 + w) * NI::sW;
   float* const sG = sStage + 2 * F::stage;
   float* const sRows = sStage + F::stage;  // the lifted rows at a tile's end
-  const int S = kOne ? 1 : a.S;
   const float* const trace = reinterpret_cast<const float*>(a.trace);
-  auto elem = [&](int64_t vv) -> int64_t { return kOne ? vv : vv / S; };
+  auto elem = [&](int64_t vv) -> int64_t { return kOne ? vv : elem_of(vv, a.S); };
   const int64_t ntiles = g.first[g.n];
   const int slots = (int)gridDim.x * kSlotsN, me = (int)blockIdx.x * kSlotsN + slot;
 
@@ -172,39 +147,15 @@ __global__ void __launch_bounds__(kThreadsN, 1) neighbour_tc_kernel(StepArgs a, 
     face_stage<float, N, kOne>(a, sStage + buf * F::stage, p.v0, p.nE, info, nbr, f, lane);
   };
 
-  uint32_t phase = 0;
   float bad = 0.f;  // stays 0 while every updated dof is finite (x * 0 is NaN for x = inf, NaN)
-  // a lift product: the A columns written, all warps of the slot there, issued by one thread
-  auto issue = [&](auto&& mma) {
-    asm volatile("tcgen05.wait::st.sync.aligned;");
-    tc::fence_before();
-    slot_bar(slot);
-    tc::fence_after();
-    if (t == 0) {
-      mma();
-      tc::commit(&mbar[slot]);
-    }
-  };
-  // ... complete (bounded: a thread whose wait runs out reports it and goes on
-  // to the end of the tile, where the slot leaves together)
-  auto done = [&] {
-    if (!tc::mbar_wait(&mbar[slot], phase, *(volatile int*)&s_abort[slot] ? 1 : kWaitIters)) {
-      atomicOr(a.err, ERR_TIMEOUT);
-      s_abort[slot] = 1;
-    }
-    phase ^= 1u;
-    tc::fence_after();
-  };
-  // 8-column chunks of an operand row, zero past `cnt`
+  tc::SlotMma mma{&mbar[slot], &s_abort[slot], a.err, slot, t, lane, 0};
+  // an operand row (zero past `cnt`) into the A columns
   auto put = [&](const auto& x, auto cc) {
     constexpr int cnt = decltype(cc)::value;
-#pragma unroll
-    for (int c = 0; c < up8(cnt) / 8; ++c) {
-      float y[8];
-#pragma unroll
-      for (int k = 0; k < 8; ++k) y[k] = 8 * c + k < cnt ? x[8 * c + k < cnt ? 8 * c + k : 0] : 0.f;
-      tc::st_split8(trow + 8 * c, trow + NI::cAl + 8 * c, y);
-    }
+    tc::put_row<up8(cnt) / 8>(trow, trow + NI::cAl, [&](auto kc) {
+      constexpr int k = decltype(kc)::value;
+      if constexpr (k < cnt) return x[k]; else return 0.f;
+    });
   };
 
   int it = 0;
@@ -247,7 +198,7 @@ __global__ void __launch_bounds__(kThreadsN, 1) neighbour_tc_kernel(StepArgs a, 
     for (int r = 0; r < BF; ++r) g0[r] = g1[r] = 0.f;
 #pragma unroll 1
     for (int f = 0; f < 4; ++f) {
-      cp_wait_all();
+      tc::cp_async_wait<0>();
       __syncwarp();
       if (f < 3)
         stage(p, info, nbr, f + 1, (f + 1) & 1);
@@ -273,14 +224,14 @@ __global__ void __launch_bounds__(kThreadsN, 1) neighbour_tc_kernel(StepArgs a, 
           g0[r] += x[r];
         }
         put(g0, std::integral_constant<int, BF>{});
-        issue([&] {
+        mma.issue([&] {
           tc::mma3_ts<NI::NE, NI::KS>(tbase + NI::cE, tbase, tbase + NI::cAl, sL + 4 * NI::oA,
                                       sL + 4 * (NI::oA + NI::sA), false);
         });
       } else if (f == 2) {
-        done();
+        mma.done();
         put(g1, std::integral_constant<int, BF>{});
-        issue([&] {
+        mma.issue([&] {
           tc::mma3_ts<NI::NO, NI::KS>(tbase + NI::cO, tbase, tbase + NI::cAl, sL + 4 * NI::oB,
                                       sL + 4 * (NI::oB + NI::sB), false);
         });
@@ -291,7 +242,7 @@ __global__ void __launch_bounds__(kThreadsN, 1) neighbour_tc_kernel(StepArgs a, 
         for (int r = 0; r < BF; ++r) g1[r] = x[r];
       }
     }
-    done();
+    mma.done();
     {
       float x[2 * NI::FE];
       sp::each<BF>([&](auto rc) {
@@ -303,7 +254,7 @@ __global__ void __launch_bounds__(kThreadsN, 1) neighbour_tc_kernel(StepArgs a, 
       });
       put(x, std::integral_constant<int, 2 * NI::FE>{});
     }
-    issue([&] {
+    mma.issue([&] {
       tc::mma3_ts<NI::NE, NI::KE>(tbase + NI::cE, tbase, tbase + NI::cAl, sL + 4 * NI::oC, sL + 4 * (NI::oC + NI::sC),
                                   true);
     });
@@ -312,7 +263,7 @@ __global__ void __launch_bounds__(kThreadsN, 1) neighbour_tc_kernel(StepArgs a, 
 #pragma unroll
     for (int k = 0; k < (nV + 31) / 32; ++k)
       if (lane + 32 * k < cnt) q[k] = reinterpret_cast<const V*>(Q)[lane + 32 * k];
-    done();
+    mma.done();
     {
       float x[2 * NI::FO];
       sp::each<BF>([&](auto rc) {
@@ -324,11 +275,11 @@ __global__ void __launch_bounds__(kThreadsN, 1) neighbour_tc_kernel(StepArgs a, 
       });
       put(x, std::integral_constant<int, 2 * NI::FO>{});
     }
-    issue([&] {
+    mma.issue([&] {
       tc::mma3_ts<NI::NO, NI::KO>(tbase + NI::cO, tbase, tbase + NI::cAl, sL + 4 * NI::oD, sL + 4 * (NI::oD + NI::sD),
                                   true);
     });
-    done();
+    mma.done();
     // ---- Q -= lift: the rows through shared memory, laid out as in memory
     {
       constexpr int CE = (count_par(B, 0) + 7) / 8, CO = (count_par(B, 1) + 7) / 8;
@@ -363,7 +314,7 @@ __global__ void __launch_bounds__(kThreadsN, 1) neighbour_tc_kernel(StepArgs a, 
       }
       __syncwarp();  // the rows are read before the next tile's fluxes overwrite them
     }
-    slot_bar(slot);
+    tc::slot_bar(slot);
     if (*(volatile int*)&s_abort[slot]) break;
     ++it;
     tile = next;
@@ -374,7 +325,7 @@ __global__ void __launch_bounds__(kThreadsN, 1) neighbour_tc_kernel(StepArgs a, 
   if (__any_sync(0xffffffffu, bad != 0.f) && lane == 0) atomicOr(a.err, ERR_NAN);
   tc::cp_async_wait<0>();  // no copy into shared memory outlives the loop
   // after a timed-out wait, give this slot's products in flight a bounded chance to finish
-  if (t == 0 && s_abort[slot]) tc::mbar_wait(&mbar[slot], phase ^ 1u, kWaitIters);
+  if (t == 0 && s_abort[slot]) tc::mbar_wait(&mbar[slot], mma.phase ^ 1u, kWaitIters);
   tc::fence_before();
   __syncthreads();
   tc::fence_after();

@@ -20,6 +20,7 @@
 
 #include "kernels.cuh"
 #include "sparse_ops.cuh"
+#include "tc_common.cuh"
 
 namespace adg {
 
@@ -46,13 +47,6 @@ __device__ __forceinline__ void reorient_table(T* sP, const T* blocks, int t, in
   }
 }
 
-__device__ __forceinline__ void cp16(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
-               : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
-
 // info, nbr: of face f of element j in lane 4 j + f; kOne: one scenario
 template <class T, int N, bool kOne>
 __device__ __forceinline__ void face_stage(const StepArgs& a, T* st, int64_t v0, int nE, int info, int nbr, int f,
@@ -67,20 +61,20 @@ __device__ __forceinline__ void face_stage(const StepArgs& a, T* st, int64_t v0,
     const int in = __shfl_sync(0xffffffffu, info, 4 * j + f), nb = __shfl_sync(0xffffffffu, nbr, 4 * j + f);
     if (i >= nE * C) continue;
     const int64_t v = v0 + j;
-    cp16(st + i * F::V, trace + (v * 4 + f) * F::FS + c * F::V);
+    tc::cp_async16(st + i * F::V, trace + (v * 4 + f) * F::FS + c * F::V);
     if (((in >> 5) & 7) == NK_SAME) {
-      const int64_t vn = kOne ? (int64_t)nb : (int64_t)nb * a.S + v % a.S;
-      cp16(st + 3 * F::FS + i * F::V, trace + (vn * 4 + (in & 3)) * F::FS + c * F::V);
+      const int64_t vn = kOne ? (int64_t)nb : (int64_t)nb * a.S + (v - elem_of(v, a.S) * a.S);
+      tc::cp_async16(st + 3 * F::FS + i * F::V, trace + (vn * 4 + (in & 3)) * F::FS + c * F::V);
     }
   }
 #pragma unroll
   for (int k = 0; k < (3 * CC + 31) / 32; ++k) {
     const int i = lane + 32 * k, j = i / CC, c = i - j * CC;
     if (i >= nE * CC) continue;
-    const int64_t v = v0 + j, e = kOne ? v : v / a.S;
-    cp16(st + 6 * F::FS + i * F::V, crec + (e * 4 + f) * CREC + c * F::V);
+    const int64_t v = v0 + j, e = kOne ? v : elem_of(v, a.S);
+    tc::cp_async16(st + 6 * F::FS + i * F::V, crec + (e * 4 + f) * CREC + c * F::V);
   }
-  cp_commit();
+  tc::cp_async_commit();
 }
 
 // the neighbours' blocks of face f that are not in the trace array: a finer
@@ -93,7 +87,7 @@ __device__ void face_lts(const StepArgs& a, const Seg& sg, T* st, int64_t v0, in
   for (int j = 0; j < nE; ++j) {
     const int in = __shfl_sync(0xffffffffu, info, 4 * j + f), nb = __shfl_sync(0xffffffffu, nbr, 4 * j + f);
     const int kind = (in >> 5) & 7;
-    const int s = (int)((v0 + j) % a.S);
+    const int s = (int)(v0 + j - elem_of(v0 + j, a.S) * a.S);
     T* const out = st + (3 + j) * F::FS;
     if (kind == NK_FINE) {
       const double* const src = a.btrace + (((int64_t)a.bslot[nb] * a.S + s) * 4 + (in & 3)) * F::FS;
@@ -104,7 +98,7 @@ __device__ void face_lts(const StepArgs& a, const Seg& sg, T* st, int64_t v0, in
       for (int i = lane; i < 6 * F::BF; i += 32) {
         T x = T(0);
 #pragma unroll
-        for (int d = 0; d <= N; ++d) x = fma((T)sg.ccoef[d], src[d * F::FS + i], x);
+        for (int d = 0; d <= N; ++d) x = fma(seg_ccoef<T>(sg, d), src[d * F::FS + i], x);
         out[i] = x;
       }
     }
@@ -144,7 +138,7 @@ __device__ __forceinline__ void face_items(const StepArgs& a, const T* st, const
       }
     } else if (kLts && a.gslot) {
       // a gravitational surface's normal traction and velocity
-      const int64_t v = v0 + je, e = v / a.S;
+      const int64_t v = v0 + je, e = elem_of(v, a.S);
       const int gs = a.gslot[e * 4 + f];
       if (gs >= 0) {
         const T* const src = reinterpret_cast<const T*>(a.gflux) + ((int64_t)gs * a.S + (v - e * a.S)) * 9 * BF + n;

@@ -5,34 +5,78 @@
 // cluster (Sec. 4.4); their derivative stack is kept in shared memory for it.
 #pragma once
 #include "row_common.cuh"
+#include "tc_common.cuh"
+
+#include <type_traits>
 
 namespace adg {
 namespace row {
 
+// two FP32 values in a register pair, and their packed multiply and fused multiply-add
+struct F2 {
+  uint64_t v;
+};
+__device__ __forceinline__ F2 f2(float a, float b) {
+  F2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void f2_get(F2 x, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x.v));
+}
+__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
+  F2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F2 f2_fma(F2 a, F2 b, F2 c) {
+  F2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+  return r;
+}
+
 // Star product of this lane's quantity: D[p] = sum_d c_d X_d[src_d] with
 // X_d = sum_b G_b,d Y_b over the three parity-respecting directions b of
-// sparse_ops.inc (Jacobian form of -sum_a A*_a Y_a).
-// FP32: X_d here, one shuffle per direction.  FP64: the arithmetic is what
-// counts (2 FMA per clock and SM), so the Y_b travel and the products
-// c_d G_b,d are formed once: 9 FMAs instead of 12 operations.
+// sparse_ops.inc (Jacobian form of -sum_a A*_a Y_a), for two basis functions at
+// a time.
+// FP32: X_d here, one shuffle per direction and function, the arithmetic
+// packed in pairs (18 instructions for two functions, 30 without: the kernels
+// are bound by instruction issue).  FP64: the arithmetic is what counts (2 FMA
+// per clock and SM), so the Y_b travel and the products c_d G_b,d are formed
+// once: 9 FMAs per function instead of 12 operations.
 template <class T>
 struct RowStar {
-  T w[9];      // FP32: G_b,d at 3 b + d; FP64: c_d G_b,d
-  T c[3];
+  static constexpr bool f32 = sizeof(T) == 4;
+  using W = std::conditional_t<f32, F2, T>;
+  W w[9];      // FP32: G_b,d at 3 b + d, twice; FP64: c_d G_b,d
+  W c[3];
   int src[3];
+  __device__ __forceinline__ void set(const T (&G)[9], const T (&cc)[3]) {
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      if constexpr (f32) w[k] = f2(G[k], G[k]);
+      else w[k] = G[k] * cc[k % 3];
+    }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      if constexpr (f32) c[d] = f2(cc[d], cc[d]);
+      else c[d] = cc[d];
+    }
+  }
+  __device__ __forceinline__ void metric(bool valid, const T* par, T (&G)[9]) {
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const T gx = valid ? par[d] : T(0), gy = valid ? par[3 + d] : T(0), gz = valid ? par[6 + d] : T(0);
+      G[d] = gx + T(0.5) * (gy + gz);
+      G[3 + d] = gy + gz;
+      G[6 + d] = gz;
+    }
+  }
   __device__ __forceinline__ void setup(int lane, bool valid, const T* par) {
     const int j = lane / 9, p = lane - 9 * j, base = 9 * j;
-    T lam = 0, mu = 0, irho = 0;
-#pragma unroll
-    for (int k = 0; k < 9; ++k) w[k] = T(0);
+    T lam = 0, mu = 0, irho = 0, G[9];
+    metric(valid, par, G);
     if (valid) {
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        const T gx = par[d], gy = par[3 + d], gz = par[6 + d];
-        w[d] = gx + T(0.5) * (gy + gz);
-        w[3 + d] = gy + gz;
-        w[6 + d] = gz;
-      }
       irho = T(1) / par[9];
       lam = par[10];
       mu = par[11];
@@ -55,14 +99,62 @@ struct RowStar {
     src[0] = on ? base + q0 : lane;
     src[1] = on ? base + q1 : lane;
     src[2] = on ? base + q2 : lane;
-    c[0] = c0; c[1] = c1; c[2] = c2;
-    if constexpr (sizeof(T) == 8) {
+    const T cc[3] = {c0, c1, c2};
+    set(G, cc);
+  }
+  // the acoustic rows of lane 4 j + p (p = 0: sigma_xx, p = 1..3: v_x, v_y, v_z): the
+  // normal stress reads the velocities with lambda, a velocity the normal stress with 1 / rho
+  __device__ __forceinline__ void setup_acoustic(int lane, bool valid, const T* par) {
+    const int p = lane & 3, base = lane & ~3;
+    T lam = 0, irho = 0, G[9], cc[3];
+    metric(valid, par, G);
+    if (valid) {
+      irho = T(1) / par[9];
+      lam = par[10];
+    }
 #pragma unroll
-      for (int k = 0; k < 9; ++k) w[k] *= c[k % 3];
+    for (int d = 0; d < 3; ++d) {
+      cc[d] = p == 0 ? lam : (p == d + 1 ? irho : T(0));
+      src[d] = p == 0 ? base + 1 + d : (p == d + 1 ? base : lane);
+    }
+    set(G, cc);
+  }
+  // y[b][k]: the directions' values of the functions k = 0, 1
+  __device__ __forceinline__ void apply(const T (&y)[3][2], T& o0, T& o1) const {
+    if constexpr (f32) {
+      const F2 y0 = f2(y[0][0], y[0][1]), y1 = f2(y[1][0], y[1][1]), y2 = f2(y[2][0], y[2][1]);
+      F2 s;
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        float a, b;
+        f2_get(f2_fma(w[6 + d], y2, f2_fma(w[3 + d], y1, f2_mul(w[d], y0))), a, b);
+        const F2 x = f2(__shfl_sync(0xffffffffu, a, src[d]), __shfl_sync(0xffffffffu, b, src[d]));
+        s = d == 0 ? f2_mul(c[0], x) : f2_fma(c[d], x, s);
+      }
+      f2_get(s, o0, o1);
+    } else {
+      T s[2] = {T(0), T(0)};
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          s[k] = fma(w[d], __shfl_sync(0xffffffffu, y[0][k], src[d]), s[k]);
+          s[k] = fma(w[3 + d], __shfl_sync(0xffffffffu, y[1][k], src[d]), s[k]);
+          s[k] = fma(w[6 + d], __shfl_sync(0xffffffffu, y[2][k], src[d]), s[k]);
+        }
+      }
+      o0 = s[0];
+      o1 = s[1];
     }
   }
-  __device__ __forceinline__ T apply(T y0, T y1, T y2) const {
-    if constexpr (sizeof(T) == 8) {
+  // one function
+  __device__ __forceinline__ T apply1(T y0, T y1, T y2) const {
+    if constexpr (f32) {
+      const T y[3][2] = {{y0, T(0)}, {y1, T(0)}, {y2, T(0)}};
+      T a, b;
+      apply(y, a, b);
+      return a;
+    } else {
       T s = T(0);
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
@@ -71,17 +163,27 @@ struct RowStar {
         s = fma(w[6 + d], __shfl_sync(0xffffffffu, y2, src[d]), s);
       }
       return s;
-    } else {
-      T s = T(0);
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        const T X = fma(w[6 + d], y2, fma(w[3 + d], y1, w[d] * y0));
-        s = fma(c[d], __shfl_sync(0xffffffffu, X, src[d]), s);
-      }
-      return s;
     }
   }
 };
+// out[m] for m < M from the directions' values y(b, integral_constant<m>), two functions at a time
+template <int M, class T, class Y>
+__device__ __forceinline__ void star_rows(const RowStar<T>& st, T* out, Y&& yf) {
+  sp::each<M / 2>([&](auto hc) {
+    constexpr int m = 2 * decltype(hc)::value;
+    using A = std::integral_constant<int, m>;
+    using C = std::integral_constant<int, m + 1>;
+    const T y[3][2] = {{yf(std::integral_constant<int, 0>{}, A{}), yf(std::integral_constant<int, 0>{}, C{})},
+                       {yf(std::integral_constant<int, 1>{}, A{}), yf(std::integral_constant<int, 1>{}, C{})},
+                       {yf(std::integral_constant<int, 2>{}, A{}), yf(std::integral_constant<int, 2>{}, C{})}};
+    st.apply(y, out[m], out[m + 1]);
+  });
+  if constexpr (M % 2) {
+    using A = std::integral_constant<int, M - 1>;
+    out[M - 1] = st.apply1(yf(std::integral_constant<int, 0>{}, A{}), yf(std::integral_constant<int, 1>{}, A{}),
+                           yf(std::integral_constant<int, 2>{}, A{}));
+  }
+}
 
 // shared memory of one warp (values of T): dofs rows, the nine-quantity modes
 // of two faces, and with kSpec the rows' derivative stacks
@@ -90,7 +192,8 @@ struct LocalSmem {
   using S = Shape<T, N>;
   static constexpr int nQ = (9 * EW * S::SB + 3) / 4 * 4, nT = (2 * 9 * EW * S::Bf + 3) / 4 * 4;
   static constexpr int nD = kSpec ? 9 * EW * S::ND + (S::ND + 3) / 4 * 4 + 2 * S::Bf + 2 : 0;
-  static constexpr int warp = (nQ + nT + nD + 3) / 4 * 4;
+  static constexpr int nN = 16 * EW;  // the faces' normals
+  static constexpr int warp = (nQ + nN + nT + nD + 3) / 4 * 4;
   static constexpr int bytes(int threads) { return warp * (int)sizeof(T) * (threads / 32); }
 };
 
@@ -104,19 +207,21 @@ static __constant__ double kRowRcpFact[6] = {1.0, 1.0, 1.0 / 2, 1.0 / 6, 1.0 / 2
 
 // D^{K+1} rows from D^K, then the next levels; I accumulates the time integral
 template <class T, int N, int K, bool kSpec>
-__device__ __forceinline__ void predict(const T* D, T* I, const RowStar<T>& st, const double* tc, T* stack) {
+__device__ __forceinline__ void predict(const T* D, T* I, const RowStar<T>& st, const Seg& sg, T* stack) {
   constexpr int L = nb3(N - K), M = nb3(N - K - 1);
   T Dn[M];
-  sp::each<M>([&](auto mc) {
-    constexpr int m = decltype(mc)::value;
-    Dn[m] = st.apply(sp::dot<sp::KX, m, L>(T(0), D), sp::dot<sp::KY, m, L>(T(0), D), sp::dot<sp::KZ, m, L>(T(0), D));
+  star_rows<M>(st, Dn, [&](auto bc, auto mc) {
+    constexpr int b = decltype(bc)::value, m = decltype(mc)::value;
+    if constexpr (b == 0) return sp::dot<sp::KX, m, L>(T(0), D);
+    else if constexpr (b == 1) return sp::dot<sp::KY, m, L>(T(0), D);
+    else return sp::dot<sp::KZ, m, L>(T(0), D);
   });
   if constexpr (K == 0) {  // D^0 is not needed any more: its registers become I
-    const T c0 = (T)tc[0];
+    const T c0 = seg_tcoef<T>(sg, 0);
 #pragma unroll
     for (int l = 0; l < L; ++l) I[l] = c0 * D[l];
   }
-  const T ck = (T)tc[K + 1];
+  const T ck = seg_tcoef<T>(sg, K + 1);
 #pragma unroll
   for (int m = 0; m < M; ++m) I[m] = fma(ck, Dn[m], I[m]);
   if constexpr (kSpec) {
@@ -125,26 +230,37 @@ __device__ __forceinline__ void predict(const T* D, T* I, const RowStar<T>& st, 
       for (int m = 0; m < M; ++m) stack[stack_off(K + 1, N) + m] = Dn[m];
     }
   }
-  if constexpr (K + 1 < N) predict<T, N, K + 1, kSpec>(Dn, I, st, tc, stack);
+  if constexpr (K + 1 < N) predict<T, N, K + 1, kSpec>(Dn, I, st, sg, stack);
 }
 
+// the outward normals of the warp's faces into sN[4 j + f][4] (asynchronously)
+template <class T>
+__device__ __forceinline__ void normals_request(const StepArgs& a, T* sN, int64_t v0, int nE, int lane) {
+  constexpr int V = 16 / (int)sizeof(T), C = 4 / V;
+  for (int i = lane; i < nE * 4 * C; i += 32) {
+    const int jf = i / C, c = (i % C) * V;
+    tc::cp_async16(sN + jf * 4 + c, reinterpret_cast<const T*>(a.crec) +
+                                        (elem_of(v0 + (jf >> 2), a.S) * 4 + (jf & 3)) * CREC + c);
+  }
+}
 // the faces F0, F0 + 1 of the warp's elements: staged modes -> traction and
 // velocity blocks of the trace array (and the LTS buffers, in FP64)
 template <class T, int N, bool kSpec>
 __device__ __forceinline__ void faces_out(const StepArgs& a, const Seg& sg, int64_t v0, int nE, int f0, const T* sT,
-                                          int lane) {
+                                          const T* sN, int lane) {
   using S = Shape<T, N>;
   constexpr int Bf = S::Bf;
   T* const trace = reinterpret_cast<T*>(a.trace);
-  const T* const crec = reinterpret_cast<const T*>(a.crec);
-  for (int i = lane; i < nE * 2 * Bf; i += 32) {
-    const int jf = i / Bf, n = i - jf * Bf, j = jf >> 1, f = f0 + (jf & 1);
-    const int64_t v = v0 + j, e = v / a.S;
+#pragma unroll(sizeof(T) == 4 ? 8 : 1)
+  for (int it = 0; it < (2 * EW * Bf + 31) / 32; ++it) {
+    const int i = lane + 32 * it, jf = i / Bf, n = i - jf * Bf, j = jf >> 1, f = f0 + (jf & 1);
+    if (i >= nE * 2 * Bf) continue;
+    const int64_t v = v0 + j;
     const T* const s = sT + ((jf & 1) * 9 * EW + 9 * j) * Bf + n;
     T q[9];
 #pragma unroll
     for (int p = 0; p < 9; ++p) q[p] = s[p * Bf];
-    const T* const c = crec + (e * 4 + f) * CREC;
+    const T* const c = sN + (4 * j + f) * 4;
     const T nx = c[0], ny = c[1], nz = c[2];
     const T o[6] = {fma(q[5], nz, fma(q[3], ny, q[0] * nx)), fma(q[4], nz, fma(q[1], ny, q[3] * nx)),
                     fma(q[2], nz, fma(q[4], ny, q[5] * nx)), q[6], q[7], q[8]};
@@ -153,6 +269,7 @@ __device__ __forceinline__ void faces_out(const StepArgs& a, const Seg& sg, int6
     for (int k = 0; k < 6; ++k) out[k * Bf] = o[k];
     if constexpr (kSpec) {
       if (sg.btrace_mode && a.bslot) {
+        const int64_t e = elem_of(v, a.S);
         const int bs = a.bslot[e];
         if (bs >= 0) {
           double* const b = a.btrace + (((int64_t)bs * a.S + (v - e * a.S)) * 4 + f) * S::FS + n;
@@ -171,7 +288,7 @@ template <class T, int N>
 __device__ void special_faces(const StepArgs& a, const Seg& sg, int64_t v, const T* sD, T* sW, int lane) {
   using S = Shape<T, N>;
   constexpr int B = S::B, Bf = S::Bf, ND = S::ND;
-  const int64_t e = v / a.S;
+  const int64_t e = elem_of(v, a.S);
   const int s = (int)(v - e * a.S);
 #pragma unroll 1
   for (int f = 0; f < 4; ++f) {
@@ -275,16 +392,19 @@ __global__ void __launch_bounds__(kMaxThreads, sizeof(T) == 4 ? 2 : 1) local_row
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31;
   T* const sQ = reinterpret_cast<T*>(smem_raw) + (threadIdx.x >> 5) * M::warp;
-  T* const sT = sQ + M::nQ;
+  T* const sN = sQ + M::nQ;
+  T* const sT = sN + M::nN;
   const Unit u = unit_of(g);
   if (u.nE == 0) return;
   const Seg& sg = g.s[u.seg];
   T* const Q = reinterpret_cast<T*>(a.Q) + u.v0 * 9 * B;
+  normals_request(a, sN, u.v0, u.nE, lane);
+  tc::cp_async_commit();
   rows_in<T, N>(sQ, Q, u.nE, lane);
   const int j = lane / 9;
   const bool valid = lane < 9 * u.nE;
   RowStar<T> st;
-  st.setup(lane, valid, reinterpret_cast<const T*>(a.par) + (u.v0 + (valid ? j : 0)) / a.S * PAR);
+  st.setup(lane, valid, reinterpret_cast<const T*>(a.par) + elem_of(u.v0 + (valid ? j : 0), a.S) * PAR);
   T* const row = sQ + (valid ? lane : 0) * S::SB;
   T* const stack = kSpec && valid ? sT + M::nT + lane * S::ND : nullptr;
   __syncwarp();
@@ -303,7 +423,7 @@ __global__ void __launch_bounds__(kMaxThreads, sizeof(T) == 4 ? 2 : 1) local_row
       for (int l = 0; l < B; ++l) stack[l] = I[l];
     }
   }
-  predict<T, N, 0, kSpec>(I, I, st, sg.tcoef, stack);
+  predict<T, N, 0, kSpec>(I, I, st, sg, stack);
 
   // ---- modal face traces, two faces at a time through shared memory
   {
@@ -316,8 +436,9 @@ __global__ void __launch_bounds__(kMaxThreads, sizeof(T) == 4 ? 2 : 1) local_row
         s0[9 * EW * Bf + r] = ev - od;
       });
     }
+    tc::cp_async_wait<0>();
     __syncwarp();
-    faces_out<T, N, kSpec>(a, sg, u.v0, u.nE, 0, sT, lane);
+    faces_out<T, N, kSpec>(a, sg, u.v0, u.nE, 0, sT, sN, lane);
     __syncwarp();
     if (valid) {
       sp::each<Bf>([&](auto rc) {
@@ -327,17 +448,18 @@ __global__ void __launch_bounds__(kMaxThreads, sizeof(T) == 4 ? 2 : 1) local_row
       });
     }
     __syncwarp();
-    faces_out<T, N, kSpec>(a, sg, u.v0, u.nE, 2, sT, lane);
+    faces_out<T, N, kSpec>(a, sg, u.v0, u.nE, 2, sT, sN, lane);
   }
 
   // ---- volume: Q += sum_a A*_a K_a I (face terms follow in the neighbour kernel)
   sp::each<B / VW>([&](auto cc) {
     constexpr int m0 = decltype(cc)::value * VW;
     T x[VW];
-    sp::each<VW>([&](auto kc) {
-      constexpr int m = m0 + decltype(kc)::value;
-      x[decltype(kc)::value] = st.apply(sp::dot<sp::KXt, m, S::B1>(T(0), I), sp::dot<sp::KYt, m, S::B1>(T(0), I),
-                                        sp::dot<sp::KZt, m, S::B1>(T(0), I));
+    star_rows<VW>(st, x, [&](auto bc, auto kc) {
+      constexpr int b = decltype(bc)::value, m = m0 + decltype(kc)::value;
+      if constexpr (b == 0) return sp::dot<sp::KXt, m, S::B1>(T(0), I);
+      else if constexpr (b == 1) return sp::dot<sp::KYt, m, S::B1>(T(0), I);
+      else return sp::dot<sp::KZt, m, S::B1>(T(0), I);
     });
     if (valid) {
       Vec<T, VW> q = *reinterpret_cast<const Vec<T, VW>*>(row + m0);

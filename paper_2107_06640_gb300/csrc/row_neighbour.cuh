@@ -40,7 +40,7 @@ __global__ void __launch_bounds__(kMaxThreads, sizeof(T) == 4 ? 2 : 1) neighbour
   // lane 4 j + f (< 12): face f of element j, its neighbour and what it is
   int info = 0, nbr = -1;
   if (lane < 4 * u.nE) {
-    const int64_t ef = (u.v0 + (lane >> 2)) / a.S * 4 + (lane & 3);
+    const int64_t ef = elem_of(u.v0 + (lane >> 2), a.S) * 4 + (lane & 3);
     info = a.ninfo[ef];
     nbr = a.nbr[ef];
   }
@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(kMaxThreads, sizeof(T) == 4 ? 2 : 1) neighbour
   // flux row of face f (of this lane's element and quantity) -> gr
   auto face = [&](const int f, T(&gr)[Bf]) {
     T* const st = sSt + (f & 1) * F::stage;
-    cp_wait_all();
+    tc::cp_async_wait<0>();
     __syncwarp();
     if (f < 3) stage(f + 1);
     if constexpr (kSpec) {
@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(kMaxThreads, sizeof(T) == 4 ? 2 : 1) neighbour
       // a fault's flux comes from the friction solve, at the face nodes
       const int in = __shfl_sync(0xffffffffu, info, 4 * j + f);
       if (valid && ((in >> 5) & 7) == NK_FAULT) {
-        const int64_t v = u.v0 + j, e = v / a.S;
+        const int64_t v = u.v0 + j, e = elem_of(v, a.S);
         const int fsl = a.fslot[e * 4 + f];
         const T* const src = reinterpret_cast<const T*>(a.drout) +
                              ((((int64_t)(fsl >> 1) * a.S + (v - e * a.S)) * 2 + (fsl & 1)) * 9 + (lane - 9 * j)) * Bf;

@@ -58,6 +58,32 @@ __host__ __device__ constexpr int parity(int l) {
   return 0;
 }
 
+// ... and of i in psi_ij for mode r of a face (order: degree, then i)
+__host__ __device__ constexpr int fparity(int r) {
+  int n = 0;
+  while ((n + 1) * (n + 2) / 2 <= r) ++n;
+  return (r - n * (n + 1) / 2) & 1;
+}
+// how many of the first n modes have parity p, and the place of a mode among those of its parity
+__host__ __device__ constexpr int count_par(int n, int p) {
+  int c = 0;
+  for (int l = 0; l < n; ++l) c += parity(l) == p;
+  return c;
+}
+__host__ __device__ constexpr int count_fpar(int n, int p) {
+  int c = 0;
+  for (int r = 0; r < n; ++r) c += fparity(r) == p;
+  return c;
+}
+__host__ __device__ constexpr int par_index(int l) { return count_par(l, parity(l)); }
+__host__ __device__ constexpr int fpar_index(int r) { return count_fpar(r, fparity(r)); }
+// the i-th mode of parity p
+__host__ __device__ constexpr int par_mode(int p, int i) {
+  int l = 0;
+  while (parity(l) != p || par_index(l) != i) ++l;
+  return l;
+}
+
 #define ADG_SPARSE_OP(name, NR, kT, table)                                                     \
   struct name {                                                                                \
     static constexpr auto m = csr<NR, kT>(table);                                              \

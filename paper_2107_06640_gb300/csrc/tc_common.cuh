@@ -13,6 +13,7 @@
 // 16w..16w+15 in lanes 32w..32w+15 (w = 0..3); column j of D is TMEM column j.
 #pragma once
 #include <cstdint>
+#include <utility>
 
 namespace adg {
 namespace tc {
@@ -137,6 +138,10 @@ __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
 __device__ __forceinline__ void cp_async4(void* dst, const void* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
+// ... and of 16 bytes (both 16-byte aligned)
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int NPEND>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(NPEND) : "memory"); }
@@ -241,6 +246,62 @@ __device__ __forceinline__ void st_split8(uint32_t th, uint32_t tl, const float 
   asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(tl), "r"(l[0]),
                "r"(l[1]), "r"(l[2]), "r"(l[3]), "r"(l[4]), "r"(l[5]), "r"(l[6]), "r"(l[7]));
 }
+
+__host__ __device__ constexpr int up8(int x) { return (x + 7) / 8 * 8; }
+__host__ __device__ constexpr int up16(int x) { return (x + 15) / 16 * 16; }
+
+// C chunks of 8 columns of this lane's A row, value k from f(integral_constant<k>)
+template <int C, class F, int... I>
+__device__ __forceinline__ void put_chunk(uint32_t th, uint32_t tl, F&& f, std::integer_sequence<int, I...>) {
+  const float x[8] = {f(std::integral_constant<int, 8 * C + I>{})...};
+  st_split8(th + 8 * C, tl + 8 * C, x);
+}
+template <class F, int... C>
+__device__ __forceinline__ void put_chunks(uint32_t th, uint32_t tl, F&& f, std::integer_sequence<int, C...>) {
+  (put_chunk<C>(th, tl, f, std::make_integer_sequence<int, 8>{}), ...);
+}
+template <int C, class F>
+__device__ __forceinline__ void put_row(uint32_t th, uint32_t tl, F&& f) {
+  put_chunks(th, tl, f, std::make_integer_sequence<int, C>{});
+}
+
+constexpr int kWaitIters = 1 << 22;
+// the 128 threads of a slot (one tile in flight): named barrier slot + 1
+__device__ __forceinline__ void slot_bar(int slot) { asm volatile("bar.sync %0, 128;" ::"r"(slot + 1) : "memory"); }
+
+// The tensor-core products of one slot.  issue(f): the A columns that the
+// slot's threads wrote made visible, then f's MMAs by one thread.  done(): the
+// products complete; one lane per warp waits (more waiting lanes take issue
+// slots from the other slots' warps).  A wait that runs out is reported and the
+// slot goes on to the end of its tile, where it leaves together.
+struct SlotMma {
+  uint64_t* mbar;
+  int* abort;
+  unsigned int* err;
+  int slot, t, lane;
+  uint32_t phase;
+  template <class F>
+  __device__ __forceinline__ void issue(F&& f) {
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    fence_before();
+    slot_bar(slot);
+    fence_after();
+    if (t == 0) {
+      f();
+      commit(mbar);
+    }
+  }
+  __device__ __forceinline__ void done() {
+    if (lane == 0 && !mbar_wait(mbar, phase, *(volatile int*)abort ? 1 : kWaitIters)) {
+      atomicOr(err, 2u /* ERR_TIMEOUT */);
+      *(volatile int*)abort = 1;
+    }
+    __syncwarp();
+    mbar_wait(mbar, phase, 1);  // every thread observes the completed phase
+    phase ^= 1u;
+    fence_after();
+  }
+};
 
 
 }  // namespace tc

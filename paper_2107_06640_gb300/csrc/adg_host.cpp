@@ -955,7 +955,12 @@ void Ctx::launch_rupture_cluster(int c, double dt) {
   d.dt = dt;
   std::vector<double> x, w;
   gauss01(N + 1, x, w);
-  for (int j = 0; j <= N; ++j) { d.tp[j] = dt * x[j]; d.tw[j] = dt * w[j]; }
+  for (int j = 0; j <= N; ++j) {
+    d.tp[j] = dt * x[j];
+    d.tw[j] = dt * w[j];
+    d.tk[j][0] = 1.0;
+    for (int k = 1; k <= N; ++k) d.tk[j][k] = d.tk[j][k - 1] * d.tp[j] / k;
+  }
   d.newton = dNewton; d.err = dErr;
   d.mlp = mlp_on ? dMlp : nullptr;
   d.capture = cap_on ? dCapture : nullptr;

@@ -23,7 +23,7 @@ namespace adg {
 __host__ __device__ constexpr int nb3(int n) { return n < 0 ? 0 : (n + 1) * (n + 2) * (n + 3) / 6; }
 __host__ __device__ constexpr int nb2(int n) { return (n + 1) * (n + 2) / 2; }
 // values of one face in the trace array: traction and velocity in the face's
-// modes, [6][Bf], padded to a multiple of 4 so that a block starts on 16 bytes
+// modes, [Bf][6], padded to a multiple of 4 so that a block starts on 16 bytes
 __host__ __device__ constexpr int face_block(int n) { return (6 * nb2(n) + 3) / 4 * 4; }
 // values that the trace array (also the scratch of the FP32 dofs transfers) holds per face
 __host__ __device__ constexpr int face_stride(int n) { return (9 * nb2(n) + 3) / 4 * 4; }
@@ -185,6 +185,7 @@ struct DRArgs {
   int S;
   double dt;
   double tp[8], tw[8];  // Gauss-Legendre time points / weights on [0, dt]
+  double tk[6][6];      // Taylor weights of the time points, tp[j]^k / k!
   unsigned long long* newton;  // [0] solves, [1] iterations
   unsigned int* err;
   const float* mlp;     // network parameters (or null: plain start)

@@ -161,13 +161,11 @@ __device__ __forceinline__ void face_out_acoustic(const StepArgs& a, int64_t v0,
     const int64_t v = v0 + j;
     const float* const s = sT + 4 * j * Bf + n;
     const float* const c = reinterpret_cast<const float*>(a.crec) + (elem_of(v, a.S) * 4 + f) * CREC;
-    float* const out = reinterpret_cast<float*>(a.trace) + (v * 4 + f) * FS + n;
+    float2* const out = reinterpret_cast<float2*>(reinterpret_cast<float*>(a.trace) + (v * 4 + f) * FS + 6 * n);
     const float x = s[0];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      out[k * Bf] = x * c[k];
-      out[(3 + k) * Bf] = s[(1 + k) * Bf];
-    }
+    out[0] = make_float2(x * c[0], x * c[1]);
+    out[1] = make_float2(x * c[2], s[Bf]);
+    out[2] = make_float2(s[2 * Bf], s[3 * Bf]);
   }
 }
 
@@ -290,7 +288,16 @@ __global__ void __launch_bounds__(LSmem<N, M, kSpec>::threads, 1)
     if constexpr (!M::fluid) row::normals_request(a, sW + SM::oN, p.v0, p.nE, lane);
     tc::cp_async_commit();
     float* const rowp = sQ + (valid ? lane : 0) * S::SB;
-    float* const stack = kSpec && valid ? sW + SM::oD + lane * S::ND : nullptr;
+    std::conditional_t<kSpec, row::SpecLevels<float, N>, row::NoLevels> lev = [&] {
+      if constexpr (kSpec) {
+        tc::cp_async_wait<0>();
+        __syncwarp();  // the normals
+        return row::SpecLevels<float, N>(a, valid ? sW + SM::oD + lane * S::ND : nullptr, sT, sW + SM::oN, p.v0, p.nE,
+                                         lane);
+      } else {
+        return row::NoLevels{};
+      }
+    }();
 
     // ---- level 0 on the tensor cores: D^1 from D^0 = the dofs row
     float I[B];
@@ -303,20 +310,15 @@ __global__ void __launch_bounds__(LSmem<N, M, kSpec>::threads, 1)
       }
     };
     load_row();
-    if constexpr (kSpec) {
-      if (valid) {
-#pragma unroll
-        for (int l = 0; l < B; ++l) stack[l] = I[l];
-      }
-    }
     put(I, std::integral_constant<int, I_::KE>{}, std::integral_constant<int, I_::KO>{},
         std::integral_constant<int, B>{}, I_::cL);
-    mma.issue([&] {
+    mma.issue(0, [&] {
       tc::mma3_ts<I_::nPE, I_::KE>(tbase + I_::cD, tbase, tbase + I_::cL, sB + 4 * I_::oPE,
                                    sB + 4 * (I_::oPE + I_::sPE), false);
       tc::mma3_ts<I_::nPO, I_::KO>(tbase + I_::cD + I_::nPE, tbase + I_::KE, tbase + I_::cL + I_::KE,
                                    sB + 4 * I_::oPO, sB + 4 * (I_::oPO + I_::sPO), false);
     });
+    if constexpr (kSpec) lev(std::integral_constant<int, 0>{}, I);  // (while the product runs)
     mma.done();
     {
       float D1[B1];
@@ -345,17 +347,16 @@ __global__ void __launch_bounds__(LSmem<N, M, kSpec>::threads, 1)
 #pragma unroll
       for (int m = 0; m < B1; ++m) I[m] = fmaf(c1, D1[m], I[m]);
       if constexpr (kSpec) {
-        if (valid) {
-#pragma unroll
-          for (int m = 0; m < B1; ++m) stack[B + m] = D1[m];
-        }
+        lev(std::integral_constant<int, 1>{}, D1);
+        row::predict<float, N, 1>(D1, I, st, sg, lev);
+      } else {
+        row::predict<float, N, 1>(D1, I, st, sg, row::NoLevels{});
       }
-      row::predict<float, N, 1, kSpec>(D1, I, st, sg, stack);
     }
     // ---- modal face traces
     put(I, std::integral_constant<int, I_::KE>{}, std::integral_constant<int, I_::KO>{},
         std::integral_constant<int, B>{}, I_::cL);
-    mma.issue([&] {
+    mma.issue(1, [&] {
       tc::mma3_ts<I_::nTE, I_::KE>(tbase + I_::cD, tbase, tbase + I_::cL, sB + 4 * I_::oTE,
                                    sB + 4 * (I_::oTE + I_::sTE), false);
       tc::mma3_ts<I_::nTO, I_::KO>(tbase + I_::cD + I_::nTE, tbase + I_::KE, tbase + I_::cL + I_::KE,
@@ -369,7 +370,7 @@ __global__ void __launch_bounds__(LSmem<N, M, kSpec>::threads, 1)
       // ---- the volume product runs while the traces leave
       put(I, std::integral_constant<int, I_::VE>{}, std::integral_constant<int, I_::VO>{},
           std::integral_constant<int, B1>{}, I_::cVL);
-      mma.issue([&] {
+      mma.issue(2, [&] {
         tc::mma3_ts<I_::nVE, I_::VE>(tbase + I_::cV, tbase, tbase + I_::cVL, sB + 4 * I_::oVE,
                                      sB + 4 * (I_::oVE + I_::sVE), false);
         tc::mma3_ts<I_::nVO, I_::VO>(tbase + I_::cV + I_::nVE, tbase + I_::VE, tbase + I_::cVL + I_::VE,

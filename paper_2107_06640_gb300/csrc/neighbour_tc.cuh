@@ -8,17 +8,17 @@
 // of 128 threads and 128 TMEM columns; the warps of a slot meet only where an
 // operand of the lift is complete.  A warp forms, face by face,
 // the flux rows of row_flux.cuh; lane (element, quantity) then takes its row.
-// The lift Q[l] -= sum_f sum_r R_f[r][l] G_f[r] splits by the parity of i
-// (sparse_ops.inc): face 1 is face 0 with the odd modes negated and faces 2, 3
-// couple equal parities only, so four products (A in TMEM, one after another
-// in the same 48 columns, hi and lo)
-//   G_0 + G_1 -> even l,  G_0 - G_1 -> odd l,
-//   even modes of G_2, G_3 -> even l,  odd modes of G_2, G_3 -> odd l
-// replace the dense K = 84, N = 56 one with 62 % of its multiplications, and
-// each runs while the next face is worked on.
+// The lift Q[l] -= sum_f sum_r R_f[r][l] G_f[r] is one product per face (A in
+// TMEM, one face after another in the same 48 columns), which runs while the
+// next face is worked on, so that a thread holds one flux row at a time and 128
+// registers suffice for four tiles.  (Faces 0 and 1 through their sum and
+// difference and the parities of faces 2 and 3 apart take half the tensor
+// work, but hold two more rows: three tiles of 168 registers, 483 us on the
+// 183,456-tet degree-5 box where this form takes 398; the nodal kernel before,
+// nine quantities staged and two tiles in flight, took 652.)
 //
-// What bounds it: HBM (8.5 KB per element at degree 5) and instruction issue
-// alike.
+// What bounds it: shared-memory traffic (76 % of the L1 data pipe busy) and
+// instruction issue (49 %); 0.40 of the HBM bandwidth.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -35,13 +35,10 @@ namespace adg {
 namespace {
 
 constexpr int TE = kTileElems;
-constexpr int kSlotsN = 3, kThreadsN = 128 * kSlotsN;
+constexpr int kSlotsN = 4, kThreadsN = 128 * kSlotsN;
 using tc::kWaitIters;
 
-using sp::count_fpar;
 using sp::count_par;
-using sp::fpar_index;
-using sp::fparity;
 using sp::par_index;
 using tc::up16;
 using tc::up8;
@@ -50,11 +47,9 @@ template <int N>
 struct NImg {
   static constexpr int B = nb3(N), BF = nb2(N), FS = face_block(N);
   static constexpr int NE = up16(count_par(B, 0)), NO = up16(count_par(B, 1));    // outputs: even, odd l
-  static constexpr int FE = count_fpar(BF, 0), FO = count_fpar(BF, 1);            // a face's even and odd modes
-  static constexpr int KS = up8(BF), KE = up8(2 * FE), KO = up8(2 * FO);
-  // lift operands (floats), hi block then lo block each
-  static constexpr int sA = NE * KS, sB = NO * KS, sC = NE * KE, sD = NO * KO;
-  static constexpr int oA = 0, oB = oA + 2 * sA, oC = oB + 2 * sB, oD = oC + 2 * sC, image = oD + 2 * sD;
+  static constexpr int KS = up8(BF), NL = NE + NO;
+  // lift operands (floats): per face, hi block then lo block; rows: even l, then odd l from NE
+  static constexpr int sF = NL * KS, image = 4 * 2 * sF;
   using F = FaceSmem<float, N>;
   static constexpr int oPV = image;
   static constexpr int oW = oPV + (F::table + 3) / 4 * 4;   // per warp: two stage buffers, the flux rows
@@ -62,8 +57,8 @@ struct NImg {
   static_assert(F::stage + F::rows >= 27 * B, "the lifted rows take the second stage buffer and the flux rows");
   static_assert(oW % 4 == 0 && F::stage % 4 == 0 && sW % 4 == 0, "16-byte aligned buffers");
   static constexpr int bytes = (oW + 4 * kSlotsN * sW) * 4;
-  static constexpr int cAl = 24, cE = 48, cO = cE + NE;     // TMEM columns: A hi 0, A lo, even and odd accumulators
-  static_assert(KS <= 24 && KE <= 24 && KO <= 24 && cO + NO <= 128, "TMEM columns of a slot");
+  static constexpr int cAl = 24, cAcc = 48;  // TMEM columns: A hi 0, A lo, accumulator
+  static_assert(KS <= 24 && cAcc + NL <= 128, "TMEM columns of a slot");
   static_assert(bytes + 256 <= 232448, "neighbour tensor-core kernel exceeds the shared memory of one CTA");
 };
 
@@ -193,9 +188,6 @@ __global__ void __launch_bounds__(kThreadsN, 1) neighbour_tc_kernel(StepArgs a, 
     };
     float* const Q = reinterpret_cast<float*>(a.Q) + p.v0 * 9 * B;
     const int cnt = p.nE * 9 * B / VW;
-    float g0[BF], g1[BF];
-#pragma unroll
-    for (int r = 0; r < BF; ++r) g0[r] = g1[r] = 0.f;
 #pragma unroll 1
     for (int f = 0; f < 4; ++f) {
       tc::cp_async_wait<0>();
@@ -214,78 +206,25 @@ __global__ void __launch_bounds__(kThreadsN, 1) neighbour_tc_kernel(StepArgs a, 
       float x[BF];
       face_row<float, N>(sG, lane < 27 ? lane : 0, x);
       // (rows past the part's elements hold anything: no other row reads them)
-      if (f == 0) {
-#pragma unroll
-        for (int r = 0; r < BF; ++r) g0[r] = x[r];
-      } else if (f == 1) {
-#pragma unroll
-        for (int r = 0; r < BF; ++r) {
-          g1[r] = g0[r] - x[r];
-          g0[r] += x[r];
-        }
-        put(g0, std::integral_constant<int, BF>{});
-        mma.issue([&] {
-          tc::mma3_ts<NI::NE, NI::KS>(tbase + NI::cE, tbase, tbase + NI::cAl, sL + 4 * NI::oA,
-                                      sL + 4 * (NI::oA + NI::sA), false);
-        });
-      } else if (f == 2) {
-        mma.done();
-        put(g1, std::integral_constant<int, BF>{});
-        mma.issue([&] {
-          tc::mma3_ts<NI::NO, NI::KS>(tbase + NI::cO, tbase, tbase + NI::cAl, sL + 4 * NI::oB,
-                                      sL + 4 * (NI::oB + NI::sB), false);
-        });
-#pragma unroll
-        for (int r = 0; r < BF; ++r) g0[r] = x[r];
-      } else {
-#pragma unroll
-        for (int r = 0; r < BF; ++r) g1[r] = x[r];
-      }
-    }
-    mma.done();
-    {
-      float x[2 * NI::FE];
-      sp::each<BF>([&](auto rc) {
-        constexpr int r = decltype(rc)::value;
-        if constexpr (fparity(r) == 0) {
-          x[fpar_index(r)] = g0[r];
-          x[NI::FE + fpar_index(r)] = g1[r];
-        }
+      if (f > 0) mma.done();  // the face before has been lifted: its columns are free
+      put(x, std::integral_constant<int, BF>{});
+      mma.issue(f, [&] {
+        const uint32_t b = sL + 4 * f * 2 * NI::sF;
+        tc::mma3_ts<NI::NL, NI::KS>(tbase + NI::cAcc, tbase, tbase + NI::cAl, b, b + 4 * NI::sF, f > 0);
       });
-      put(x, std::integral_constant<int, 2 * NI::FE>{});
     }
-    mma.issue([&] {
-      tc::mma3_ts<NI::NE, NI::KE>(tbase + NI::cE, tbase, tbase + NI::cAl, sL + 4 * NI::oC, sL + 4 * (NI::oC + NI::sC),
-                                  true);
-    });
-    // the dofs of this warp's part, as they lie in memory, requested before the last products are waited for
+    // the dofs of this warp's part, as they lie in memory, requested before the last product is waited for
     V q[(nV + 31) / 32];
 #pragma unroll
     for (int k = 0; k < (nV + 31) / 32; ++k)
       if (lane + 32 * k < cnt) q[k] = reinterpret_cast<const V*>(Q)[lane + 32 * k];
     mma.done();
-    {
-      float x[2 * NI::FO];
-      sp::each<BF>([&](auto rc) {
-        constexpr int r = decltype(rc)::value;
-        if constexpr (fparity(r) == 1) {
-          x[fpar_index(r)] = g0[r];
-          x[NI::FO + fpar_index(r)] = g1[r];
-        }
-      });
-      put(x, std::integral_constant<int, 2 * NI::FO>{});
-    }
-    mma.issue([&] {
-      tc::mma3_ts<NI::NO, NI::KO>(tbase + NI::cO, tbase, tbase + NI::cAl, sL + 4 * NI::oD, sL + 4 * (NI::oD + NI::sD),
-                                  true);
-    });
-    mma.done();
     // ---- Q -= lift: the rows through shared memory, laid out as in memory
     {
       constexpr int CE = (count_par(B, 0) + 7) / 8, CO = (count_par(B, 1) + 7) / 8;
       float x[8 * (CE + CO)];
-      tc::ld8s<CE>(trow + NI::cE, x);
-      tc::ld8s<CO>(trow + NI::cO, x + 8 * CE);
+      tc::ld8s<CE>(trow + NI::cAcc, x);
+      tc::ld8s<CO>(trow + NI::cAcc + NI::NE, x + 8 * CE);
       if (valid) {
         float* const r = sRows + lane * B;
         sp::each<B / VW>([&](auto cc) {
@@ -364,24 +303,14 @@ void pack_lift_tc_deg(const double* rfc, float* out) {
   using NI = NImg<N>;
   constexpr int B = NI::B, BF = NI::BF;
   for (int i = 0; i < NI::image; ++i) out[i] = 0.f;
-  auto put = [&](int off, int size, int R, int n, int k, double x) {
-    const float xf = (float)x, hi = tc::tf32_trunc(xf);
-    const int o = tc::canon(n, k, R);
-    out[off + o] = hi;
-    out[off + size + o] = xf - hi;
-  };
-  auto at = [&](int f, int l, int r) { return rfc[((size_t)f * B + l) * BF + r]; };
-  for (int l = 0; l < B; ++l) {
-    const bool odd = sp::parity(l) == 1;
-    const int n = par_index(l), R = odd ? NI::NO : NI::NE;
-    for (int r = 0; r < BF; ++r) {
-      put(odd ? NI::oB : NI::oA, odd ? NI::sB : NI::sA, R, n, r, at(0, l, r));
-      if (fparity(r) == (odd ? 1 : 0))
-        for (int f = 2; f < 4; ++f)
-          put(odd ? NI::oD : NI::oC, odd ? NI::sD : NI::sC, R, n, (f - 2) * (odd ? NI::FO : NI::FE) + fpar_index(r),
-              at(f, l, r));
-    }
-  }
+  for (int f = 0; f < 4; ++f)
+    for (int l = 0; l < B; ++l)
+      for (int r = 0; r < BF; ++r) {
+        const float xf = (float)rfc[((size_t)f * B + l) * BF + r], hi = tc::tf32_trunc(xf);
+        const int o = f * 2 * NI::sF + tc::canon((sp::parity(l) ? NI::NE : 0) + par_index(l), r, NI::NL);
+        out[o] = hi;
+        out[o + NI::sF] = xf - hi;
+      }
 }
 
 }  // namespace adg

@@ -8,7 +8,7 @@
 //
 // Face data are modal: a face block holds traction sigma n (n the owner's
 // outward normal) and velocity, the six quantities that the Godunov flux
-// reads, in the face's orthonormal Dubiner modes: [6][Bf], padded to
+// reads, in the face's orthonormal Dubiner modes: [Bf][6], padded to
 // face_block(N) values.  An element's four blocks follow one another in the
 // trace array.  LTS buffers ([slot*S][4] blocks, FP64) and the derivative
 // traces of faces with a finer neighbour ([slot*S][N+1] blocks in the space of

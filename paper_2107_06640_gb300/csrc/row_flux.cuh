@@ -117,24 +117,32 @@ __device__ __forceinline__ void face_items(const StepArgs& a, const T* st, const
     const int in = __shfl_sync(0xffffffffu, info, 4 * je + f);
     if (i >= nE * BF) continue;
     const int kind = (in >> 5) & 7;
+    struct alignas(2 * sizeof(T)) V2 {
+      T x, y;
+    };
     T q[6], w[6];
 #pragma unroll
-    for (int d = 0; d < 6; ++d) {
-      q[d] = st[je * FS + d * BF + n];
-      w[d] = T(0);
+    for (int d = 0; d < 6; d += 2) {
+      const V2 x = *reinterpret_cast<const V2*>(st + je * FS + 6 * n + d);
+      q[d] = x.x; q[d + 1] = x.y;
+      w[d] = w[d + 1] = T(0);
     }
     T srt = T(0), srv = T(0);
     if (kind != NK_NONE) {
       int first = 0;  // of the modes of n's degree
 #pragma unroll
       for (int d = 1; d <= N; ++d) first = n >= d * (d + 1) / 2 ? d * (d + 1) / 2 : first;
-      const T* const u = st + (3 + je) * FS + first;
+      const T* const u = st + (3 + je) * FS + 6 * first;
       const T* const p = sP + ((in >> 2) & 7) * ((N + 1) * F::BP) + n;
 #pragma unroll
       for (int s = 0; s <= N; ++s) {
         const T x = p[s * F::BP];  // (zero past the degree's modes)
 #pragma unroll
-        for (int d = 0; d < 6; ++d) w[d] = fma(x, u[d * BF + s], w[d]);
+        for (int d = 0; d < 6; d += 2) {
+          const V2 y = *reinterpret_cast<const V2*>(u + 6 * s + d);
+          w[d] = fma(x, y.x, w[d]);
+          w[d + 1] = fma(x, y.y, w[d + 1]);
+        }
       }
     } else if (kLts && a.gslot) {
       // a gravitational surface's normal traction and velocity

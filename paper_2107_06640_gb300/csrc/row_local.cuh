@@ -205,9 +205,10 @@ static __constant__ double kRowRcp[48] = {
     1.0 / 45, 1.0 / 46, 1.0 / 47};
 static __constant__ double kRowRcpFact[6] = {1.0, 1.0, 1.0 / 2, 1.0 / 6, 1.0 / 24, 1.0 / 120};
 
-// D^{K+1} rows from D^K, then the next levels; I accumulates the time integral
-template <class T, int N, int K, bool kSpec>
-__device__ __forceinline__ void predict(const T* D, T* I, const RowStar<T>& st, const Seg& sg, T* stack) {
+// D^{K+1} rows from D^K, then the next levels; I accumulates the time
+// integral; lev(integral_constant<k>, D^k) sees every new level
+template <class T, int N, int K, class Lev>
+__device__ __forceinline__ void predict(const T* D, T* I, const RowStar<T>& st, const Seg& sg, Lev&& lev) {
   constexpr int L = nb3(N - K), M = nb3(N - K - 1);
   T Dn[M];
   star_rows<M>(st, Dn, [&](auto bc, auto mc) {
@@ -224,13 +225,8 @@ __device__ __forceinline__ void predict(const T* D, T* I, const RowStar<T>& st, 
   const T ck = seg_tcoef<T>(sg, K + 1);
 #pragma unroll
   for (int m = 0; m < M; ++m) I[m] = fma(ck, Dn[m], I[m]);
-  if constexpr (kSpec) {
-    if (stack) {
-#pragma unroll
-      for (int m = 0; m < M; ++m) stack[stack_off(K + 1, N) + m] = Dn[m];
-    }
-  }
-  if constexpr (K + 1 < N) predict<T, N, K + 1, kSpec>(Dn, I, st, sg, stack);
+  lev(std::integral_constant<int, K + 1>{}, Dn);
+  if constexpr (K + 1 < N) predict<T, N, K + 1>(Dn, I, st, sg, lev);
 }
 
 // the outward normals of the warp's faces into sN[4 j + f][4] (asynchronously)
@@ -264,26 +260,112 @@ __device__ __forceinline__ void faces_out(const StepArgs& a, const Seg& sg, int6
     const T nx = c[0], ny = c[1], nz = c[2];
     const T o[6] = {fma(q[5], nz, fma(q[3], ny, q[0] * nx)), fma(q[4], nz, fma(q[1], ny, q[3] * nx)),
                     fma(q[2], nz, fma(q[4], ny, q[5] * nx)), q[6], q[7], q[8]};
-    T* const out = trace + (v * 4 + f) * S::FS + n;
+    Vec<T, 2>* const out = reinterpret_cast<Vec<T, 2>*>(trace + (v * 4 + f) * S::FS + 6 * n);
 #pragma unroll
-    for (int k = 0; k < 6; ++k) out[k * Bf] = o[k];
+    for (int k = 0; k < 3; ++k) out[k] = {o[2 * k], o[2 * k + 1]};
     if constexpr (kSpec) {
       if (sg.btrace_mode && a.bslot) {
         const int64_t e = elem_of(v, a.S);
         const int bs = a.bslot[e];
         if (bs >= 0) {
-          double* const b = a.btrace + (((int64_t)bs * a.S + (v - e * a.S)) * 4 + f) * S::FS + n;
+          double* const b = a.btrace + (((int64_t)bs * a.S + (v - e * a.S)) * 4 + f) * S::FS + 6 * n;
 #pragma unroll
-          for (int k = 0; k < 6; ++k) b[k * Bf] = (sg.btrace_mode == 1 ? 0.0 : b[k * Bf]) + (double)o[k];
+          for (int k = 0; k < 6; ++k) b[k] = (sg.btrace_mode == 1 ? 0.0 : b[k]) + (double)o[k];
         }
       }
     }
   }
 }
 
-// faces of one element that need more than its trace (kSpec): derivative
-// traces for fault faces and finer neighbours, and the gravitational surface's
-// ODE.  sD: the element's nine stacks (stride ND), sW: scratch of ND + 2 Bf values.
+// What kSpec does with the rows of D^k: keeps them in the rows' stacks and, on
+// faces with a finer neighbour (which integrates this element's Taylor expansion
+// over its sub-steps), writes their modal traces.  The sparse projections of a
+// level are applied to the rows in registers, faces 0, 1 and 2, 3 together and
+// only where some element of the warp has such a face: 1,766 FMAs for all six
+// levels of four faces at degree 5, where dense sums over the stacks took 2,200
+// instructions per element and face.
+template <class T, int N>
+struct SpecLevels {
+  using S = Shape<T, N>;
+  const StepArgs& a;
+  T *stack, *sT;      // this row's stack (null: no row); staging as in faces_out
+  const T* sN;
+  int64_t v0;
+  int nE, lane;
+  int ds;             // lane 4 j + f: the slot of a face with a finer neighbour, else -1
+  unsigned mask;      // faces f with such an element in the warp
+  __device__ __forceinline__ SpecLevels(const StepArgs& args, T* st, T* t, const T* n, int64_t v, int e, int l)
+      : a(args), stack(st), sT(t), sN(n), v0(v), nE(e), lane(l), ds(-1), mask(0) {
+    if (lane < 4 * nE && a.dslot) {
+      const int64_t ef = elem_of(v0 + (lane >> 2), a.S) * 4 + (lane & 3);
+      if (((a.ninfo[ef] >> 5) & 7) == NK_FINE) ds = a.dslot[ef];
+    }
+    const unsigned b = __ballot_sync(0xffffffffu, ds >= 0);
+    mask = (b | b >> 4 | b >> 8) & 15u;
+  }
+  template <int K, int F0>
+  __device__ __forceinline__ void pair(const T* D) const {
+    constexpr int L = nb3(N - K), Bk = nb2(N - K), Bf = S::Bf;
+    if (stack) {
+      T* const s0 = sT + lane * Bf;
+      sp::each<Bk>([&](auto rc) {
+        constexpr int r = decltype(rc)::value;
+        if constexpr (F0 == 0) {
+          const T ev = sp::dot<sp::R0, r, L, 0>(T(0), D), od = sp::dot<sp::R0, r, L, 1>(T(0), D);
+          s0[r] = ev + od;
+          s0[9 * EW * Bf + r] = ev - od;
+        } else {
+          s0[r] = sp::dot<sp::R2, r, L>(T(0), D);
+          s0[9 * EW * Bf + r] = sp::dot<sp::R3, r, L>(T(0), D);
+        }
+      });
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int i = lane; i < (2 * EW * Bf + 31) / 32 * 32; i += 32) {
+      const int jf = i / Bf, n = i - jf * Bf, j = jf >> 1, f = F0 + (jf & 1);
+      const int slot = __shfl_sync(0xffffffffu, ds, (4 * j + f) & 31);
+      if (j >= nE || slot < 0) continue;
+      T o[6];
+#pragma unroll
+      for (int k = 0; k < 6; ++k) o[k] = T(0);
+      if (n < Bk) {  // (a polynomial of degree N - K: no higher modes)
+        const T* const s = sT + ((jf & 1) * 9 * EW + 9 * j) * Bf + n;
+        const T* const c = sN + (4 * j + f) * 4;
+        T q[9];
+#pragma unroll
+        for (int p = 0; p < 9; ++p) q[p] = s[p * Bf];
+        o[0] = fma(q[5], c[2], fma(q[3], c[1], q[0] * c[0]));
+        o[1] = fma(q[4], c[2], fma(q[1], c[1], q[3] * c[0]));
+        o[2] = fma(q[2], c[2], fma(q[4], c[1], q[5] * c[0]));
+        o[3] = q[6]; o[4] = q[7]; o[5] = q[8];
+      }
+      const int64_t v = v0 + j;
+      T* const d = reinterpret_cast<T*>(a.dtrace) +
+                   ((int64_t)slot * a.S + (v - elem_of(v, a.S) * a.S)) * (N + 1) * 9 * Bf + K * S::FS + 6 * n;
+#pragma unroll
+      for (int k = 0; k < 6; ++k) d[k] = o[k];
+    }
+    __syncwarp();
+  }
+  template <int K>
+  __device__ __forceinline__ void operator()(std::integral_constant<int, K>, const T* D) const {
+    if (stack) {
+#pragma unroll
+      for (int l = 0; l < nb3(N - K); ++l) stack[stack_off(K, N) + l] = D[l];
+    }
+    if (mask & 3u) pair<K, 0>(D);
+    if (mask & 12u) pair<K, 2>(D);
+  }
+};
+struct NoLevels {
+  template <int K, class T>
+  __device__ __forceinline__ void operator()(std::integral_constant<int, K>, const T*) const {}
+};
+
+// faces of one element that need more than its trace (kSpec): the nodal
+// derivative traces of fault faces, and the gravitational surface's ODE.  sD:
+// the element's nine stacks (stride ND), sW: scratch of ND + 2 Bf values.
 template <class T, int N>
 __device__ void special_faces(const StepArgs& a, const Seg& sg, int64_t v, const T* sD, T* sW, int lane) {
   using S = Shape<T, N>;
@@ -292,12 +374,9 @@ __device__ void special_faces(const StepArgs& a, const Seg& sg, int64_t v, const
   const int s = (int)(v - e * a.S);
 #pragma unroll 1
   for (int f = 0; f < 4; ++f) {
-    const T* const c = reinterpret_cast<const T*>(a.crec) + (e * 4 + f) * CREC;
-    const int ds = a.dslot ? a.dslot[e * 4 + f] : -1;
-    if (ds >= 0) {
-      const bool fault = ((a.ninfo[e * 4 + f] >> 5) & 7) == NK_FAULT;
-      const T* const tab = reinterpret_cast<const T*>(fault ? a.efcT : a.rfcT) + (size_t)f * B * Bf;
-      T* const out = reinterpret_cast<T*>(a.dtrace) + ((int64_t)ds * a.S + s) * (N + 1) * 9 * Bf;
+    if (a.dslot && ((a.ninfo[e * 4 + f] >> 5) & 7) == NK_FAULT) {
+      const T* const tab = reinterpret_cast<const T*>(a.efcT) + (size_t)f * B * Bf;
+      T* const out = reinterpret_cast<T*>(a.dtrace) + ((int64_t)a.dslot[e * 4 + f] * a.S + s) * (N + 1) * 9 * Bf;
       for (int i = lane; i < (N + 1) * Bf; i += 32) {
         const int k = i / Bf, n = i - k * Bf, Bk = nb3(N - k), o = stack_off(k, N);
         T q[9];
@@ -308,18 +387,8 @@ __device__ void special_faces(const StepArgs& a, const Seg& sg, int64_t v, const
 #pragma unroll
           for (int p = 0; p < 9; ++p) q[p] = fma(w, sD[p * ND + o + l], q[p]);
         }
-        if (fault) {
 #pragma unroll
-          for (int p = 0; p < 9; ++p) out[(k * 9 + p) * Bf + n] = q[p];
-        } else {
-          T* const d = out + k * S::FS + n;
-          d[0] = q[0] * c[0] + q[3] * c[1] + q[5] * c[2];
-          d[Bf] = q[3] * c[0] + q[1] * c[1] + q[4] * c[2];
-          d[2 * Bf] = q[5] * c[0] + q[4] * c[1] + q[2] * c[2];
-          d[3 * Bf] = q[6];
-          d[4 * Bf] = q[7];
-          d[5 * Bf] = q[8];
-        }
+        for (int p = 0; p < 9; ++p) out[(k * 9 + p) * Bf + n] = q[p];
       }
     }
     const int gs = a.gslot ? a.gslot[e * 4 + f] : -1;
@@ -418,12 +487,14 @@ __global__ void __launch_bounds__(kMaxThreads, sizeof(T) == 4 ? 2 : 1) local_row
     for (int k = 0; k < VW; ++k) I[c * VW + k] = valid ? x.x[k] : T(0);
   }
   if constexpr (kSpec) {
-    if (valid) {
-#pragma unroll
-      for (int l = 0; l < B; ++l) stack[l] = I[l];
-    }
+    tc::cp_async_wait<0>();
+    __syncwarp();  // the normals
+    const SpecLevels<T, N> lev(a, stack, sT, sN, u.v0, u.nE, lane);
+    lev(std::integral_constant<int, 0>{}, I);
+    predict<T, N, 0>(I, I, st, sg, lev);
+  } else {
+    predict<T, N, 0>(I, I, st, sg, NoLevels{});
   }
-  predict<T, N, 0, kSpec>(I, I, st, sg, stack);
 
   // ---- modal face traces, two faces at a time through shared memory
   {

@@ -280,13 +280,15 @@ struct SlotMma {
   unsigned int* err;
   int slot, t, lane;
   uint32_t phase;
+  // (by the first thread of warp `who`: the rounds of a tile take turns, a thread's
+  // MMA instructions would make one warp of the slot late)
   template <class F>
-  __device__ __forceinline__ void issue(F&& f) {
+  __device__ __forceinline__ void issue(int who, F&& f) {
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
     fence_before();
     slot_bar(slot);
     fence_after();
-    if (t == 0) {
+    if (t == 32 * who) {
       f();
       commit(mbar);
     }

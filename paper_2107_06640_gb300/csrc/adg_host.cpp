@@ -730,12 +730,9 @@ void Ctx::setup() {
     std::vector<float> tf(lift_tc_floats(N));
     pack_lift_tc(N, rt.rfcT.data(), tf.data());
     dTcLift = upload_raw<float>(tf, owned, dev_bytes);
-    int64_t ngrav = 0;
-    for (int c = 0; c < ncl; ++c) ngrav += cl_grav[c];
-    if (ngrav > 0 && n_gslots > 0)
-      dGscr = (float*)dalloc((size_t)n_gslots * S * gscr_floats(N) * sizeof(float), owned, dev_bytes);
   }
   dErr = (unsigned int*)dalloc(sizeof(unsigned int), owned, dev_bytes);
+  dTiles = (int*)dalloc(2 * kTileKinds * sizeof(int), owned, dev_bytes);
   if (acoustic) {
     std::vector<int64_t> fl;
     for (int64_t i = 0; i < E; ++i)
@@ -754,8 +751,10 @@ void Ctx::setup() {
     dMlp = (float*)dalloc(MLP_NPARAM * sizeof(float), owned, dev_bytes);
     dCapCount = (unsigned long long*)dalloc(sizeof(unsigned long long), owned, dev_bytes);
   }
+  int prio_low = 0, prio_high = 0;
+  CK(cudaDeviceGetStreamPriorityRange(&prio_low, &prio_high));
   for (int i = 0; i < kSide; ++i) {
-    CK(cudaStreamCreateWithFlags(&side[i], cudaStreamNonBlocking));
+    CK(cudaStreamCreateWithPriority(&side[i], cudaStreamNonBlocking, prio_high));
     CK(cudaEventCreateWithFlags(&side_done[i], cudaEventDisableTiming));
   }
   CK(cudaEventCreateWithFlags(&side_fork, cudaEventDisableTiming));
@@ -780,7 +779,7 @@ StepArgs Ctx::base_args() const {
   a.efcT = dEfc; a.perm = dPerm; a.gpar = dGpar;
   a.S = S; a.err = dErr;
   a.fslot = dFslot; a.drout = dDrout; a.gflux = dGflux; a.tc_local = dTcLocal; a.tc_lift = dTcLift;
-  a.gscr = dGscr;
+  a.tiles = dTiles;
   a.crec = dCrec; a.rfcT = dRfc; a.modalT = dModal; a.reorient = dReorient;
   return a;
 }
@@ -864,72 +863,67 @@ void Ctx::launch_tick(int s, double dtm) {
       CK(cudaEventRecord(ev.a, stream));
     }
     // The launches of a phase, the tensor-core kinds first.  They work on
-    // different elements and may run side by side.  A tensor-core kernel takes
-    // whole SMs for all of its tiles, so those are forked only where every CTA
-    // of all of them has an SM of its own from the start (small meshes and LTS
-    // ticks: 1,512 tets at degree 5, local phase, 107 us one after the other
-    // and 50 us side by side); with more tiles than that, kernels on shares of
-    // the SMs were no faster than one after the other on all (183,456 tets
-    // 1.29 against 1.31 ms per step, six-cluster box 6.86 against 6.57 ms).
-    // The row kernels' small blocks mix freely.  adg_profile measures the kinds
-    // one after the other.
+    // different elements and run side by side, the special kernel (the longest
+    // tiles) first: a tensor-core kernel keeps a CTA on every SM that it gets, but
+    // its tiles go to whoever is free (tc::TileFeed), so the kernels' last tiles
+    // overlap.  adg_profile measures the kinds one after the other.
     struct Launch {
       const std::vector<Seg>* v;
-      int unit, per_cta;  // elements of a work unit; of a tensor-core kernel: units in flight per CTA (0: row kernel)
-      std::function<int(const Segs&, int, void*)> fn;  // (segments, SMs to use, stream)
+      int unit;  // virtual elements of a work unit
+      bool tc;
+      std::function<int(const Segs&, void*)> fn;
     };
     const Launch all[] = {
-        {&grs, kTileElems, 1,
-         [&](const Segs& g, int sms, void* st) { return launch_local_tc(N, a, g, sms, st, true, false, true); }},
-        {&fls, kTileElemsFluid, 2,
-         [&](const Segs& g, int sms, void* st) { return launch_local_tc(N, a, g, sms, st, false, true); }},
-        {&tcb, kTileElems, 2,
-         [&](const Segs& g, int sms, void* st) { return launch_local_tc(N, a, g, sms, st, true); }},
-        {&tcs, kTileElems, phase == 0 ? 2 : 3,
-         [&](const Segs& g, int sms, void* st) {
-           return phase == 0 ? launch_local_tc(N, a, g, sms, st, false) : launch_neighbour_tc(N, a, g, sms, st, ltsf);
+        {&grs, kTileElems, true,
+         [&](const Segs& g, void* st) { return launch_local_tc(N, a, g, n_sms, st, true, false, true); }},
+        {&fls, kTileElemsFluid, true,
+         [&](const Segs& g, void* st) { return launch_local_tc(N, a, g, n_sms, st, false, true); }},
+        {&tcb, kTileElems, true,
+         [&](const Segs& g, void* st) { return launch_local_tc(N, a, g, n_sms, st, true); }},
+        {&tcs, kTileElems, true,
+         [&](const Segs& g, void* st) {
+           return phase == 0 ? launch_local_tc(N, a, g, n_sms, st, false) : launch_neighbour_tc(N, a, g, n_sms, st, ltsf);
          }},
-        {&rss, kRowElems, 0,
-         [&](const Segs& g, int sms, void* st) {
+        {&rss, kRowElems, false,
+         [&](const Segs& g, void* st) {
            return phase == 0 ? launch_local_row(fp64, N, a, g, st, cc_threads[0], true)
                              : launch_neighbour_row(fp64, N, a, g, st, cc_threads[1], true);
          }},
-        {&rws, kRowElems, 0,
-         [&](const Segs& g, int sms, void* st) {
+        {&rws, kRowElems, false,
+         [&](const Segs& g, void* st) {
            return phase == 0 ? launch_local_row(fp64, N, a, g, st, cc_threads[0], false)
                              : launch_neighbour_row(fp64, N, a, g, st, cc_threads[1], false);
          }}};
     constexpr int kKinds = (int)(sizeof(all) / sizeof(all[0]));
-    int64_t units[kKinds] = {}, ctas = 0, tiles = 0;
     int kinds = 0, last = -1;
+    bool any_tc = false;
     for (int k = 0; k < kKinds; ++k) {
-      for (const Seg& x : *all[k].v) units[k] += (x.n + all[k].unit - 1) / all[k].unit;
-      if (all[k].per_cta) ctas += (units[k] + all[k].per_cta - 1) / all[k].per_cta, tiles += units[k];
-      if (units[k]) ++kinds, last = k;
+      if (all[k].v->empty()) continue;
+      ++kinds;
+      last = k;
+      any_tc = any_tc || all[k].tc;
     }
-    const bool fork = kinds > 1 && !prof && ctas <= n_sms;
+    const bool fork = kinds > 1 && !prof;
     int rc = 0, side_used = 0;
     bool tc_open = prof != nullptr;
     if (fork) CK(cudaEventRecord(side_fork, stream));
     for (int k = 0; k < kKinds && !rc; ++k) {
-      if (tc_open && !all[k].per_cta && ctas) {  // (adg_profile: the tensor-core launches alone)
+      if (tc_open && !all[k].tc && any_tc) {  // (adg_profile: the tensor-core launches alone)
         CK(cudaEventCreate(&ev.m));
         CK(cudaEventRecord(ev.m, stream));
         tc_open = false;
       }
-      if (!units[k]) continue;
+      if (all[k].v->empty()) continue;
       cudaStream_t st = stream;
       if (fork && k != last) {
         st = side[side_used];
         CK(cudaStreamWaitEvent(st, side_fork, 0));
       }
       // one launch per kind and at most kMaxSeg segments
-      // (side by side: a CTA per tile where that fits, else full CTAs)
-      const int sms = fork && all[k].per_cta && tiles > n_sms ? (int)((units[k] + all[k].per_cta - 1) / all[k].per_cta) : n_sms;
       const std::vector<Seg>& v = *all[k].v;
       for (size_t i = 0; i < v.size() && !rc; i += kMaxSeg) {
         const int n = (int)std::min<size_t>(kMaxSeg, v.size() - i);
-        rc = all[k].fn(make_segs(v.data() + i, n, all[k].unit, all[k].per_cta ? tc_chunk[phase] : 1), sms, st);
+        rc = all[k].fn(make_segs(v.data() + i, n, all[k].unit, all[k].tc ? tc_chunk[phase] : 1), st);
         ev.launches++;
       }
       if (st != stream) CK(cudaEventRecord(side_done[side_used++], st));

@@ -98,10 +98,8 @@ struct Ctx {
   bool acoustic = false;
   std::vector<int64_t> cl_elastic, cl_fluid;
   // the last cl_grav[c] elements of cluster c's tensor-core range have one
-  // gravitational face or a finer neighbour (their own local launch; dGscr:
-  // the gravitational faces' scratch)
+  // gravitational face or a finer neighbour (their own local launch)
   std::vector<int64_t> cl_grav;
-  float* dGscr = nullptr;
   int64_t* dFluid = nullptr;  // library indices of all fluid elements (projection at upload)
   int64_t n_fluid = 0;
   void project_fluid(bool sync = true);  // fluid stress -> its isotropic part, on the device
@@ -123,6 +121,7 @@ struct Ctx {
   int *dNbr = nullptr, *dNinfo = nullptr, *dGslot = nullptr, *dBslot = nullptr, *dDslot = nullptr,
       *dPerm = nullptr;
   unsigned int* dErr = nullptr;
+  int* dTiles = nullptr;  // tile counters of the tensor-core kernels
   // the launches of one phase are independent of each other and run side by
   // side: forked onto these streams from the library stream and joined with it
   static constexpr int kSide = 4;

@@ -37,6 +37,9 @@ constexpr int PAR = 16;
 //   n[3], Z, kappa = rho g / Z, rho*g
 constexpr int GPAR = 6;
 
+// the tensor-core kernels that have a tile counter of their own
+enum { TILES_ELASTIC = 0, TILES_BUFFER, TILES_FLUID, TILES_SPECIAL, TILES_NEIGHBOUR, kTileKinds };
+
 struct StepArgs {
   void* Q;              // T [V][9][B]
   void* trace;          // T [V][4][face_block(N)]
@@ -58,9 +61,9 @@ struct StepArgs {
   const void* drout;    // T [nff*S][2][9][Bf] time-integrated fault flux per side
   void* gflux;          // T [ngslot*S][9][Bf], the first two rows: the modes of the time-integrated normal
                         // traction -rho g H and normal velocity of gravitational faces
+  int* tiles;            // [kTileKinds][2] tile counters of the tensor-core kernels (tc::TileFeed)
   const float* tc_local; // tensor-core operands of the local kernel (hi/lo, canonical layout), degree 5 or 4
   const float* tc_lift;  // tensor-core lift operand of the neighbour kernel (hi/lo, canonical layout), degree 5 or 4
-  float* gscr;           // [ngslot*S][gscr_floats(N)] scratch of the tensor-core local kernel's gravity faces
   const void* crec;      // T [E][4][CREC] face coefficients
   const void* rfcT;      // T [4][B(l)][Bf(r)]  face modes of phi_l, l-major
   const void* modalT;    // T [Bf(n)][Bf(r)]    face nodes to face modes, n-major
@@ -81,13 +84,6 @@ constexpr int kRowElems = 3;
 // (the same four), the neighbour's traction taken with its own normal; then
 // -s_f lambda, -s_f mu, -s_f / rho of the element (s_f = 2|S_f|/|J|); padding.
 constexpr int CREC = 24;
-// Per gravity slot and scenario, the tensor-core local kernel's scratch: the
-// normal-projected derivative rows g_m[l] = sum_p w_p D^m[p][l] (m = 0..N,
-// l < B(N - m); w: v_n - sigma_nn / Z), then the face nodes' time-integrated
-// normal traction and velocity.
-__host__ __device__ constexpr int gscr_off(int n, int m) { return m <= 0 ? 0 : gscr_off(n, m - 1) + nb3(n - m + 1); }
-__host__ __device__ constexpr int gscr_floats(int n) { return gscr_off(n, n + 1) + 2 * nb2(n); }
-
 // The clusters of one LTS phase (Sec. 4.4) in a single launch: segment i
 // covers the virtual elements [v_begin, v_begin + n) of one cluster with that
 // cluster's time coefficients, and the launch's work units (tiles of the
@@ -118,17 +114,10 @@ __host__ __device__ inline T seg_ccoef(const Seg& s, int k) {
 }
 struct Segs {
   int n;                        // segments
-  int chunk;                    // tensor-core kernels: consecutive tiles a CTA slot takes per sweep
+  int chunk;                    // tensor-core kernels: consecutive tiles a CTA slot takes at a time
   int64_t first[kMaxSeg + 1];   // first work unit of each segment; first[n] = all units
   Seg s[kMaxSeg];
 };
-// Tensor-core kernels: the i-th tile of slot `slot` (of `slots`, over all CTAs)
-// when every slot takes `chunk` consecutive tiles per sweep; increasing in i.
-// (Tile counts stay below 2^31.)
-__host__ __device__ inline int slot_tile(int i, int slot, int slots, int chunk) {
-  const int q = i / chunk;
-  return (q * slots + slot) * chunk + (i - q * chunk);
-}
 // segment of work unit u (segments are few: a linear scan)
 __host__ __device__ inline int seg_find(const Segs& g, int64_t u) {
   int i = 0;

@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(LSmem<N, M, kSpec>::threads, 1)
   float* const sm = reinterpret_cast<float*>(smem_raw);
   __shared__ uint32_t tmem_base;
   __shared__ __align__(8) uint64_t mbar[kSlots], s_img;
-  __shared__ int s_abort[kSlots];
+  __shared__ int s_abort[kSlots], s_next[kSlots][2];
 
   const int tid = threadIdx.x, slot = tid >> 7, t = tid & 127, w = t >> 5, lane = tid & 31;
   // the operand image into shared memory by the TMA engine, while the threads set up the rest
@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(LSmem<N, M, kSpec>::threads, 1)
 
   // this warp's part of tile tl: first virtual element, elements (may be 0), segment
   const int64_t ntiles = g.first[g.n];
-  const int slots = (int)gridDim.x * kSlots, me = (int)blockIdx.x * kSlots + slot;
+  const int slots = (int)gridDim.x * kSlots, me = slot * (int)gridDim.x + (int)blockIdx.x;
   struct Part {
     int64_t v0;
     int nE, seg;
@@ -209,8 +209,10 @@ __global__ void __launch_bounds__(LSmem<N, M, kSpec>::threads, 1)
   };
   float* const sW = sm + I_::floats + (slot * 4 + w) * SM::warp;
   float* const Qg = reinterpret_cast<float*>(a.Q);
+  const tc::TileFeed feed{a.tiles, s_next[slot], slots, g.chunk, ntiles};
   int it = 0;
-  int64_t tile = slot_tile(0, me, slots, g.chunk);
+  int64_t tile = feed.first(me);
+  if (t == 32) s_next[slot][1] = (int)feed.after(tile);
   Part p{0, 0, 0};
   // a part's dofs rows (buffer b) and element parameters
   auto request = [&](const Part& q, int b) {
@@ -243,6 +245,7 @@ __global__ void __launch_bounds__(LSmem<N, M, kSpec>::threads, 1)
     __syncthreads();
     tc::fence_after();
     if (tid < 32) tc::tmem_dealloc<256 * kSlots>(tmem_base);
+    if (tid == 0) feed.leave();
     return;
   }
 
@@ -264,8 +267,9 @@ __global__ void __launch_bounds__(LSmem<N, M, kSpec>::threads, 1)
     });
   };
 
-  for (; tile < ntiles;) {
-    const int64_t next = slot_tile(it + 1, me, slots, g.chunk);
+  for (int64_t next = s_next[slot][1]; tile < ntiles;) {
+    // the tile after the next, asked for now and handed to the slot at the end
+    const int64_t after = t == 32 ? feed.after(next) : 0;
     const Seg& sg = g.s[p.seg];
     float* const sQ = sW + (it & 1) * SM::nQ;
     tc::cp_async_wait<0>();  // this tile's rows and parameters
@@ -439,13 +443,14 @@ __global__ void __launch_bounds__(LSmem<N, M, kSpec>::threads, 1)
     __syncwarp();
     rows_back<N, M>(sQ, Qg + p.v0 * 9 * B, p.nE, lane);
     if constexpr (kSpec) {
-      for (int k = 0; k < p.nE; ++k)
-        row::special_faces<float, N>(a, sg, p.v0 + k, sW + SM::oD + 9 * k * S::ND, sW + SM::oD + 27 * S::ND, lane);
+      row::special_faces<float, N>(a, sg, p.v0, p.nE, sW + SM::oD, sT, lane);
     }
+    if (t == 32) s_next[slot][it & 1] = (int)after;
     tc::slot_bar(slot);
     if (*(volatile int*)&s_abort[slot]) break;
-    ++it;
     tile = next;
+    next = s_next[slot][it & 1];
+    ++it;
     p = pn;
   }
   tc::cp_async_wait<0>();  // no copy into shared memory outlives the loop
@@ -455,6 +460,7 @@ __global__ void __launch_bounds__(LSmem<N, M, kSpec>::threads, 1)
   __syncthreads();
   tc::fence_after();
   if (tid < 32) tc::tmem_dealloc<256 * kSlots>(tmem_base);
+  if (tid == 0) feed.leave();
 }
 
 }  // namespace
@@ -483,13 +489,16 @@ int launch_local_tc_deg(const StepArgs& a, const Segs& g, int n_sms, void* strea
   if (ntiles <= 0) return 0;
   if (acoustic && (buffers || grav)) return (int)cudaErrorInvalidValue;
   // one CTA per SM at most; fewer tiles than slots: a CTA each, so that no SM holds two
-  const unsigned grid = (unsigned)(ntiles < n_sms ? ntiles : n_sms);
+  const int64_t units = (ntiles + g.chunk - 1) / g.chunk;
+  const unsigned grid = (unsigned)(units < n_sms ? units : n_sms);
+  StepArgs b = a;
+  b.tiles = a.tiles + 2 * (grav ? TILES_SPECIAL : acoustic ? TILES_FLUID : buffers ? TILES_BUFFER : TILES_ELASTIC);
   if (grav)
-    spec<<<grid, LSmem<N, Elastic, true>::threads, bytes_sp, (cudaStream_t)stream>>>(a, g);
+    spec<<<grid, LSmem<N, Elastic, true>::threads, bytes_sp, (cudaStream_t)stream>>>(b, g);
   else if (acoustic)
-    fluid<<<grid, LSmem<N, Acoustic, false>::threads, bytes_fl, (cudaStream_t)stream>>>(a, g);
+    fluid<<<grid, LSmem<N, Acoustic, false>::threads, bytes_fl, (cudaStream_t)stream>>>(b, g);
   else
-    (buffers ? buf : plain)<<<grid, LSmem<N, Elastic, false>::threads, bytes_el, (cudaStream_t)stream>>>(a, g);
+    (buffers ? buf : plain)<<<grid, LSmem<N, Elastic, false>::threads, bytes_el, (cudaStream_t)stream>>>(b, g);
   return (int)cudaGetLastError();
 }
 

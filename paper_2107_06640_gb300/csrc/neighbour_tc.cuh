@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(kThreadsN, 1) neighbour_tc_kernel(StepArgs a, 
   float* const sm = reinterpret_cast<float*>(smem_raw);
   __shared__ uint32_t tmem_base;
   __shared__ __align__(8) uint64_t mbar[kSlotsN], s_img;
-  __shared__ int s_abort[kSlotsN];
+  __shared__ int s_abort[kSlotsN], s_next[kSlotsN][2];
 
   const int tid = threadIdx.x, slot = tid >> 7, t = tid & 127, w = t >> 5, lane = tid & 31;
   if (tid == 0) {
@@ -87,6 +87,11 @@ __global__ void __launch_bounds__(kThreadsN, 1) neighbour_tc_kernel(StepArgs a, 
     tc::mbar_init(&mbar[tid], 1);
     s_abort[tid] = 0;
   }
+  const int64_t ntiles = g.first[g.n];
+  const int slots = (int)gridDim.x * kSlotsN, me = slot * (int)gridDim.x + (int)blockIdx.x;
+  const tc::TileFeed feed{a.tiles, s_next[slot], slots, g.chunk, ntiles};
+  int64_t tile = feed.first(me);
+  if (t == 32) s_next[slot][1] = (int)feed.after(tile);
   if (tid < 32) tc::tmem_alloc<512>(&tmem_base);
   __syncthreads();  // (the image barrier is initialised)
   const bool img_ok = tc::mbar_wait(&s_img, 0, kWaitIters);
@@ -105,6 +110,7 @@ __global__ void __launch_bounds__(kThreadsN, 1) neighbour_tc_kernel(StepArgs a, 
     __syncthreads();
     tc::fence_after();
     if (tid < 32) tc::tmem_dealloc<512>(tmem_base);
+    if (tid == 0) feed.leave();
     return;
   }
 
@@ -115,9 +121,6 @@ __global__ void __launch_bounds__(kThreadsN, 1) neighbour_tc_kernel(StepArgs a, 
   float* const sRows = sStage + F::stage;  // the lifted rows at a tile's end
   const float* const trace = reinterpret_cast<const float*>(a.trace);
   auto elem = [&](int64_t vv) -> int64_t { return kOne ? vv : elem_of(vv, a.S); };
-  const int64_t ntiles = g.first[g.n];
-  const int slots = (int)gridDim.x * kSlotsN, me = (int)blockIdx.x * kSlotsN + slot;
-
   // this warp's part of tile tl: first virtual element, elements (<= 3, may be 0), segment
   struct Part {
     int64_t v0;
@@ -154,7 +157,6 @@ __global__ void __launch_bounds__(kThreadsN, 1) neighbour_tc_kernel(StepArgs a, 
   };
 
   int it = 0;
-  int64_t tile = slot_tile(0, me, slots, g.chunk);
   Part p{0, 0, 0};
   int info = 0, nbr = 0;
   if (tile < ntiles) {
@@ -162,8 +164,9 @@ __global__ void __launch_bounds__(kThreadsN, 1) neighbour_tc_kernel(StepArgs a, 
     faces_of(p, info, nbr);
     stage(p, info, nbr, 0, 0);
   }
-  for (; tile < ntiles;) {
-    const int64_t next = slot_tile(it + 1, me, slots, g.chunk);
+  for (int64_t next = s_next[slot][1]; tile < ntiles;) {
+    // the tile after the next, asked for now and handed to the slot at the end
+    const int64_t after = t == 32 ? feed.after(next) : 0;
     Part pn{0, 0, 0};
     int info_n = 0, nbr_n = 0;
     if (next < ntiles) {
@@ -253,10 +256,12 @@ __global__ void __launch_bounds__(kThreadsN, 1) neighbour_tc_kernel(StepArgs a, 
       }
       __syncwarp();  // the rows are read before the next tile's fluxes overwrite them
     }
+    if (t == 32) s_next[slot][it & 1] = (int)after;
     tc::slot_bar(slot);
     if (*(volatile int*)&s_abort[slot]) break;
-    ++it;
     tile = next;
+    next = s_next[slot][it & 1];
+    ++it;
     p = pn;
     info = info_n;
     nbr = nbr_n;
@@ -269,6 +274,7 @@ __global__ void __launch_bounds__(kThreadsN, 1) neighbour_tc_kernel(StepArgs a, 
   __syncthreads();
   tc::fence_after();
   if (tid < 32) tc::tmem_dealloc<512>(tmem_base);
+  if (tid == 0) feed.leave();
 }
 
 }  // namespace
@@ -291,8 +297,11 @@ int launch_neighbour_tc_deg(const StepArgs& a, const Segs& g, int n_sms, void* s
   if (rc) return rc;
   const int64_t ntiles = g.n ? g.first[g.n] : 0;
   if (ntiles <= 0) return 0;
-  const unsigned grid = (unsigned)(ntiles < n_sms ? ntiles : n_sms);
-  kern[a.S == 1 ? 1 : 0][lts ? 1 : 0]<<<grid, kThreadsN, NImg<N>::bytes, (cudaStream_t)stream>>>(a, g);
+  const int64_t units = (ntiles + g.chunk - 1) / g.chunk;
+  const unsigned grid = (unsigned)(units < n_sms ? units : n_sms);
+  StepArgs b = a;
+  b.tiles = a.tiles + 2 * TILES_NEIGHBOUR;
+  kern[a.S == 1 ? 1 : 0][lts ? 1 : 0]<<<grid, kThreadsN, NImg<N>::bytes, (cudaStream_t)stream>>>(b, g);
   return (int)cudaGetLastError();
 }
 

@@ -191,7 +191,7 @@ template <class T, int N, bool kSpec>
 struct LocalSmem {
   using S = Shape<T, N>;
   static constexpr int nQ = (9 * EW * S::SB + 3) / 4 * 4, nT = (2 * 9 * EW * S::Bf + 3) / 4 * 4;
-  static constexpr int nD = kSpec ? 9 * EW * S::ND + (S::ND + 3) / 4 * 4 + 2 * S::Bf + 2 : 0;
+  static constexpr int nD = kSpec ? 9 * EW * S::ND : 0;
   static constexpr int nN = 16 * EW;  // the faces' normals
   static constexpr int warp = (nQ + nN + nT + nD + 3) / 4 * 4;
   static constexpr int bytes(int threads) { return warp * (int)sizeof(T) * (threads / 32); }
@@ -363,88 +363,122 @@ struct NoLevels {
   __device__ __forceinline__ void operator()(std::integral_constant<int, K>, const T*) const {}
 };
 
-// faces of one element that need more than its trace (kSpec): the nodal
-// derivative traces of fault faces, and the gravitational surface's ODE.  sD:
-// the element's nine stacks (stride ND), sW: scratch of ND + 2 Bf values.
+// Faces of the warp's elements that need more than their traces (kSpec): the
+// nodal derivative traces of fault faces, and the gravitational surface's ODE.
+// sD: the elements' stacks (row stride ND); sW: scratch (the trace staging).
+// The elements with such a face f go side by side, one (element, node) per
+// lane, and the operator's columns are loaded several at a time: the latency
+// of one warp is what a small mesh waits for.
 template <class T, int N>
-__device__ void special_faces(const StepArgs& a, const Seg& sg, int64_t v, const T* sD, T* sW, int lane) {
+__device__ void special_faces(const StepArgs& a, const Seg& sg, int64_t v0, int nE, const T* sD, T* sW, int lane) {
   using S = Shape<T, N>;
   constexpr int B = S::B, Bf = S::Bf, ND = S::ND;
-  const int64_t e = elem_of(v, a.S);
-  const int s = (int)(v - e * a.S);
+  static_assert(EW * (ND + 2 * Bf) <= 2 * 9 * EW * Bf, "scratch");
+  T* const sS = sW + EW * ND;
+  // lane 4 j + f: the gravity slot and the fault's derivative-trace slot of face f of element j
+  int grav = -1, fault = -1;
+  if (lane < 4 * nE) {
+    const int64_t ef = elem_of(v0 + (lane >> 2), a.S) * 4 + (lane & 3);
+    if (a.gslot) grav = a.gslot[ef];
+    if (a.dslot && ((a.ninfo[ef] >> 5) & 7) == NK_FAULT) fault = a.dslot[ef];
+  }
+  const unsigned gmask = __ballot_sync(0xffffffffu, grav >= 0), fmask = __ballot_sync(0xffffffffu, fault >= 0);
+  auto scenario = [&](int j) { return (int)(v0 + j - elem_of(v0 + j, a.S) * a.S); };
 #pragma unroll 1
   for (int f = 0; f < 4; ++f) {
-    if (a.dslot && ((a.ninfo[e * 4 + f] >> 5) & 7) == NK_FAULT) {
-      const T* const tab = reinterpret_cast<const T*>(a.efcT) + (size_t)f * B * Bf;
-      T* const out = reinterpret_cast<T*>(a.dtrace) + ((int64_t)a.dslot[e * 4 + f] * a.S + s) * (N + 1) * 9 * Bf;
-      for (int i = lane; i < (N + 1) * Bf; i += 32) {
-        const int k = i / Bf, n = i - k * Bf, Bk = nb3(N - k), o = stack_off(k, N);
-        T q[9];
+    const T* const E = reinterpret_cast<const T*>(a.efcT) + (size_t)f * B * Bf;
+    if (fmask & (0x111u << f)) {
+#pragma unroll 1
+      for (int k = 0; k <= N; ++k) {
+        const int Bk = nb3(N - k), o = stack_off(k, N);
 #pragma unroll
-        for (int p = 0; p < 9; ++p) q[p] = T(0);
-        for (int l = 0; l < Bk; ++l) {
-          const T w = tab[(size_t)l * Bf + n];
+        for (int it = 0; it < (EW * Bf + 31) / 32; ++it) {
+          const int i = lane + 32 * it, j = i < EW * Bf ? i / Bf : 0, n = i - j * Bf;
+          const int slot = __shfl_sync(0xffffffffu, fault, 4 * j + f);
+          if (i >= nE * Bf || slot < 0) continue;
+          T q[9];
 #pragma unroll
-          for (int p = 0; p < 9; ++p) q[p] = fma(w, sD[p * ND + o + l], q[p]);
+          for (int p = 0; p < 9; ++p) q[p] = T(0);
+#pragma unroll 5
+          for (int l = 0; l < Bk; ++l) {
+            const T w = E[(size_t)l * Bf + n];
+#pragma unroll
+            for (int p = 0; p < 9; ++p) q[p] = fma(w, sD[(9 * j + p) * ND + o + l], q[p]);
+          }
+          T* const out = reinterpret_cast<T*>(a.dtrace) + (((int64_t)slot * a.S + scenario(j)) * (N + 1) + k) * 9 * Bf + n;
+#pragma unroll
+          for (int p = 0; p < 9; ++p) out[p * Bf] = q[p];
         }
-#pragma unroll
-        for (int p = 0; p < 9; ++p) out[(k * 9 + p) * Bf + n] = q[p];
       }
     }
-    const int gs = a.gslot ? a.gslot[e * 4 + f] : -1;
-    if (gs >= 0) {
+    if (gmask & (0x111u << f)) {
       // g_m[l]: v_n - sigma_nn / Z of the derivative rows, then per face node
       // f_m = E g_m / m!, the (eta, H) series in FP64, and the modes of
       // -rho g H and eta^{n+1} - eta^n
-      const double* const gp = a.gpar + (size_t)gs * GPAR;
-      const T nx = (T)gp[0], ny = (T)gp[1], nz = (T)gp[2], iz = (T)(1.0 / gp[3]);
-      T* const sS = sW + (ND + 3) / 4 * 4;
-      for (int l = lane; l < ND; l += 32) {
-        const T snn = nx * nx * sD[l] + ny * ny * sD[ND + l] + nz * nz * sD[2 * ND + l] +
-                      T(2) * (nx * ny * sD[3 * ND + l] + ny * nz * sD[4 * ND + l] + nx * nz * sD[5 * ND + l]);
-        const T vn = nx * sD[6 * ND + l] + ny * sD[7 * ND + l] + nz * sD[8 * ND + l];
-        sW[l] = vn - snn * iz;
+      for (int j = 0; j < nE; ++j) {
+        const int gs = __shfl_sync(0xffffffffu, grav, 4 * j + f);
+        if (gs < 0) continue;
+        const double* const gp = a.gpar + (size_t)gs * GPAR;
+        const T nx = (T)gp[0], ny = (T)gp[1], nz = (T)gp[2], iz = (T)(1.0 / gp[3]);
+        const T* const D = sD + 9 * j * ND;
+        for (int l = lane; l < ND; l += 32) {
+          const T snn = nx * nx * D[l] + ny * ny * D[ND + l] + nz * nz * D[2 * ND + l] +
+                        T(2) * (nx * ny * D[3 * ND + l] + ny * nz * D[4 * ND + l] + nx * nz * D[5 * ND + l]);
+          const T vn = nx * D[6 * ND + l] + ny * D[7 * ND + l] + nz * D[8 * ND + l];
+          sW[j * ND + l] = vn - snn * iz;
+        }
       }
       __syncwarp();
-      if (lane < Bf) {
-        const T* const tab = reinterpret_cast<const T*>(a.efcT) + (size_t)f * B * Bf + lane;
+#pragma unroll 1
+      for (int it = 0; it < (EW * Bf + 31) / 32; ++it) {
+        const int i = lane + 32 * it, j = i < EW * Bf ? i / Bf : 0, n = i - j * Bf;
+        const int gs = __shfl_sync(0xffffffffu, grav, 4 * j + f);
+        if (i >= nE * Bf || gs < 0) continue;
+        const T* const gj = sW + j * ND;
         double fm[N + 1];
 #pragma unroll
         for (int m = 0; m <= N; ++m) {
           T acc = T(0);
-          for (int l = 0; l < nb3(N - m); ++l) acc = fma(tab[(size_t)l * Bf], sW[stack_off(m, N) + l], acc);
+#pragma unroll 14
+          for (int l = 0; l < nb3(N - m); ++l) acc = fma(E[(size_t)l * Bf + n], gj[stack_off(m, N) + l], acc);
           fm[m] = (double)acc * kRowRcpFact[m];
         }
-        double* const eta = a.eta + ((int64_t)gs * a.S + s) * Bf + lane;
+        const double* const gp = a.gpar + (size_t)gs * GPAR;
+        double* const eta = a.eta + ((int64_t)gs * a.S + scenario(j)) * Bf + n;
         const double kappa = gp[4], rg = gp[5], dt = sg.dt, eta0 = *eta;
         double cm = eta0, e1 = eta0, H = eta0 * dt, pw = 1.0;
-#pragma unroll 1
-        for (int m = 0; m < N + 40; ++m) {
-          double fv = 0.0;
-#pragma unroll
-          for (int k = 0; k <= N; ++k)
-            if (k == m) fv = fm[k];
+        auto term = [&](int m, double fv) {
           cm = (fv - kappa * cm) * kRowRcp[m + 1];
           pw *= dt;
           const double t = cm * pw;
           e1 += t;
           H += t * dt * kRowRcp[m + 2];
-          if (m > N && fabs(t) <= 1e-17 * fabs(e1)) break;
-        }
+          return t;
+        };
+#pragma unroll
+        for (int m = 0; m <= N; ++m) term(m, fm[m]);
+#pragma unroll 1
+        for (int m = N + 1; m < N + 40; ++m)
+          if (fabs(term(m, 0.0)) <= 1e-17 * fabs(e1)) break;
         *eta = e1;
-        sS[lane] = (T)(-rg * H);
-        sS[Bf + lane] = (T)(e1 - eta0);
+        sS[j * 2 * Bf + n] = (T)(-rg * H);
+        sS[(j * 2 + 1) * Bf + n] = (T)(e1 - eta0);
       }
       __syncwarp();
-      if (lane < Bf) {
-        const T* const mn = reinterpret_cast<const T*>(a.modalT) + lane;
+#pragma unroll 1
+      for (int it = 0; it < (EW * Bf + 31) / 32; ++it) {
+        const int i = lane + 32 * it, j = i < EW * Bf ? i / Bf : 0, r = i - j * Bf;
+        const int gs = __shfl_sync(0xffffffffu, grav, 4 * j + f);
+        if (i >= nE * Bf || gs < 0) continue;
+        const T* const mn = reinterpret_cast<const T*>(a.modalT) + r;
         T h = T(0), d = T(0);
+#pragma unroll
         for (int n = 0; n < Bf; ++n) {
           const T w = mn[n * Bf];
-          h = fma(w, sS[n], h);
-          d = fma(w, sS[Bf + n], d);
+          h = fma(w, sS[j * 2 * Bf + n], h);
+          d = fma(w, sS[(j * 2 + 1) * Bf + n], d);
         }
-        T* const out = reinterpret_cast<T*>(a.gflux) + ((int64_t)gs * a.S + s) * 9 * Bf + lane;
+        T* const out = reinterpret_cast<T*>(a.gflux) + ((int64_t)gs * a.S + scenario(j)) * 9 * Bf + r;
         out[0] = h;
         out[Bf] = d;
       }
@@ -542,8 +576,8 @@ __global__ void __launch_bounds__(kMaxThreads, sizeof(T) == 4 ? 2 : 1) local_row
   __syncwarp();
   rows_out<T, N>(sQ, Q, u.nE, lane);
   if constexpr (kSpec) {
-    for (int k = 0; k < u.nE; ++k)
-      special_faces<T, N>(a, sg, u.v0 + k, sT + M::nT + 9 * k * S::ND, sT + M::nT + 9 * EW * S::ND, lane);
+    __syncwarp();
+    special_faces<T, N>(a, sg, u.v0, u.nE, sT + M::nT, sT, lane);
   }
 }
 

@@ -306,5 +306,33 @@ struct SlotMma {
 };
 
 
+// The tiles of a slot.  Its first one is fixed (slot `me` of `slots` over all
+// CTAs), later ones come from a counter in global memory, `chunk` consecutive
+// tiles at a time, so that CTAs that start late (the kernels of a phase run side
+// by side and share the SMs) or meet slow tiles take fewer.  One thread of the slot asks for the tile
+// after the next at the start of a tile; the slot reads the answer after the
+// barrier at its end.  The last CTA to leave resets the counter for the next
+// launch.
+struct TileFeed {
+  int* counter;  // [0] units handed out, [1] CTAs that have left
+  int* box;      // shared, [2] of this slot
+  int slots, chunk;
+  int64_t n;
+  __device__ __forceinline__ int64_t after(int64_t tile) const {  // (by one thread)
+    if (chunk > 1 && ((int)tile + 1) % chunk) return tile + 1;
+    return tile < n ? ((int64_t)slots + atomicAdd(counter, 1)) * chunk : n;
+  }
+  __device__ __forceinline__ int64_t first(int me) const { return (int64_t)me * chunk; }
+  // one thread of the CTA, when its slots are done
+  __device__ __forceinline__ void leave() const {
+    __threadfence();
+    if (atomicAdd(counter + 1, 1) == (int)gridDim.x - 1) {
+      counter[0] = 0;
+      counter[1] = 0;
+    }
+  }
+};
+
+
 }  // namespace tc
 }  // namespace adg

@@ -676,11 +676,6 @@ void Ctx::setup() {
   fault_set = false;
 
   // ---- reference operators in device layouts (l-major / n-major)
-  std::vector<double> efcT((size_t)4 * B * Bf);
-  for (int f = 0; f < 4; ++f)
-    for (int n = 0; n < Bf; ++n)
-      for (int l = 0; l < B; ++l) efcT[((size_t)f * B + l) * Bf + n] = ops.efc[((size_t)f * Bf + n) * B + l];
-
   const RowTables rt = make_row_tables(ops);
   if (rt.max_err > 1e-10) throw Err(ADG_E_STATE, "internal: the sparse operators do not match the basis");
 
@@ -703,17 +698,15 @@ void Ctx::setup() {
   if (fp64) {
     dPar = upload_vec<double>(par, owned, dev_bytes);
     dCrec = upload_vec<double>(crec, owned, dev_bytes);
-    dRfc = upload_vec<double>(rt.rfcT, owned, dev_bytes);
+    dNodal = upload_vec<double>(rt.nodalT, owned, dev_bytes);
     dModal = upload_vec<double>(rt.modalT, owned, dev_bytes);
     dReorient = upload_vec<double>(rt.reorient, owned, dev_bytes);
-    dEfc = upload_vec<double>(efcT, owned, dev_bytes);
   } else {
     dPar = upload_vec<float>(par, owned, dev_bytes);
     dCrec = upload_vec<float>(crec, owned, dev_bytes);
-    dRfc = upload_vec<float>(rt.rfcT, owned, dev_bytes);
+    dNodal = upload_vec<float>(rt.nodalT, owned, dev_bytes);
     dModal = upload_vec<float>(rt.modalT, owned, dev_bytes);
     dReorient = upload_vec<float>(rt.reorient, owned, dev_bytes);
-    dEfc = upload_vec<float>(efcT, owned, dev_bytes);
   }
   dNbr = upload_raw<int>(nbr, owned, dev_bytes);
   dNinfo = upload_raw<int>(ninfo, owned, dev_bytes);
@@ -776,11 +769,11 @@ StepArgs Ctx::base_args() const {
   a.Q = dQ; a.trace = dTrace; a.btrace = dBtrace; a.dtrace = dDtrace; a.eta = dEta;
   a.par = dPar; a.nbr = dNbr; a.ninfo = dNinfo;
   a.gslot = dGslot; a.bslot = dBslot; a.dslot = dDslot;
-  a.efcT = dEfc; a.perm = dPerm; a.gpar = dGpar;
+  a.perm = dPerm; a.gpar = dGpar;
   a.S = S; a.err = dErr;
   a.fslot = dFslot; a.drout = dDrout; a.gflux = dGflux; a.tc_local = dTcLocal; a.tc_lift = dTcLift;
   a.tiles = dTiles;
-  a.crec = dCrec; a.rfcT = dRfc; a.modalT = dModal; a.reorient = dReorient;
+  a.crec = dCrec; a.nodalT = dNodal; a.modalT = dModal; a.reorient = dReorient;
   return a;
 }
 

@@ -40,10 +40,11 @@ int launch_isotropic_fluid(int fp64, void* Q, const int64_t* elems, int64_t n, i
 int launch_receivers(int fp64, int B, const void* Q, int S, int64_t n, const int64_t* elem,
                      const double* phi, double* out, void* stream);
 
-// Modal face tables (StepArgs rfcT, modalT, reorient); max_err: the
+// Modal face tables: rfcT [4][B(l)][Bf(r)], the face modes of phi_l, and
+// StepArgs' modalT, nodalT, reorient; max_err: the
 // largest difference between the operators' compiled-in entries and `o`'s
 struct RowTables {
-  std::vector<double> rfcT, modalT, reorient;
+  std::vector<double> rfcT, modalT, nodalT, reorient;
   double max_err = 0;
 };
 RowTables make_row_tables(const RefOps& o);
@@ -117,7 +118,7 @@ struct Ctx {
   int64_t* dOrder = nullptr;  // order on the device: the caller's element of library element i
   double *dBtrace = nullptr, *dEta = nullptr, *dGpar = nullptr;
   void* dPar = nullptr;
-  void *dCrec = nullptr, *dRfc = nullptr, *dModal = nullptr, *dReorient = nullptr, *dEfc = nullptr;
+  void *dCrec = nullptr, *dNodal = nullptr, *dModal = nullptr, *dReorient = nullptr;
   int *dNbr = nullptr, *dNinfo = nullptr, *dGslot = nullptr, *dBslot = nullptr, *dDslot = nullptr,
       *dPerm = nullptr;
   unsigned int* dErr = nullptr;

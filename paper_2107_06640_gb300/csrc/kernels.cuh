@@ -52,7 +52,6 @@ struct StepArgs {
   const int* gslot;     // [E][4] gravity slot or -1
   const int* bslot;     // [E]    LTS buffer slot or -1
   const int* dslot;     // [E][4] LTS derivative-trace slot or -1
-  const void* efcT;     // T [4][B(l)][Bf(n)]  phi_l at node n stored l-major
   const int* perm;      // [6][Bf]
   const double* gpar;   // [ngslot][GPAR]
   int S;                // ensemble size
@@ -65,7 +64,7 @@ struct StepArgs {
   const float* tc_local; // tensor-core operands of the local kernel (hi/lo, canonical layout), degree 5 or 4
   const float* tc_lift;  // tensor-core lift operand of the neighbour kernel (hi/lo, canonical layout), degree 5 or 4
   const void* crec;      // T [E][4][CREC] face coefficients
-  const void* rfcT;      // T [4][B(l)][Bf(r)]  face modes of phi_l, l-major
+  const void* nodalT;    // T [Bf(r)][Bf(n)]    face modes at the face nodes, r-major
   const void* modalT;    // T [Bf(n)][Bf(r)]    face nodes to face modes, n-major
   const void* reorient;  // T [6][sum (n+1)^2]  a neighbour's face modes in this side's, blocks by degree
 };

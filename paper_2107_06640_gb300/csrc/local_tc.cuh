@@ -29,9 +29,9 @@
 // velocity rows; a tile is 32 elements x 4 quantities (warp w: elements
 // 8w..8w+7, lane 4j+p).  Face blocks are those of every other element.
 //
-// kSpec: elements with one gravitational face or a finer LTS neighbour; the
-// rows' derivative stacks stay in shared memory for special_faces
-// (row_local.cuh), one slot per CTA.
+// kSpec: elements with one gravitational face or a finer LTS neighbour, with
+// row_local.cuh's SpecLevels between the levels (one buffer of dofs rows: the
+// room goes to the surfaces' modes).
 //
 // What bounds it: the latency of a warp's own instruction stream (eight warps
 // per SM, 0.39 instructions per clock and scheduler), not a roof: 0.23 of the
@@ -103,16 +103,18 @@ struct LImg {
 
 // Shared memory of one warp (floats): two buffers of dofs rows, the element
 // parameters, the faces' normals, the modes of
-// two faces' rows (acoustic: of one, there are more rows), with kSpec the derivative stacks and their scratch.
+// two faces' rows (acoustic: of one, there are more rows), with kSpec the modes
+// of the gravitational faces.
 template <int N, class M, bool kSpec>
 struct LSmem {
   using S = row::Shape<float, N>;
   static constexpr int rowsN = M::Q * M::EW;
   static constexpr int nQ = (rowsN * S::SB + 3) / 4 * 4, nT = ((M::fluid ? 1 : 2) * rowsN * S::Bf + 3) / 4 * 4;
-  static constexpr int nD = kSpec ? row::LocalSmem<float, N, true>::nD : 0;
+  static constexpr int nD = kSpec ? row::SpecLevels<float, N, true>::values : 0;
   static constexpr int nP = M::EW * PAR, nN = M::fluid ? 0 : row::LocalSmem<float, N, kSpec>::nN;
-  static constexpr int oP = 2 * nQ, oN = oP + nP, oT = oN + nN, oD = oT + nT, warp = (oD + nD + 3) / 4 * 4;
-  static constexpr int slots = kSpec ? 1 : 2, threads = 128 * slots;
+  static constexpr int bufs = kSpec ? 1 : 2;
+  static constexpr int oP = bufs * nQ, oN = oP + nP, oT = oN + nN, oD = oT + nT, warp = (oD + nD + 3) / 4 * 4;
+  static constexpr int slots = 2, threads = 128 * slots;
   static constexpr int bytes = (LImg<N>::floats + 4 * slots * warp) * 4;
   static_assert(bytes + 256 <= 232448, "local tensor-core kernel exceeds the shared memory of one CTA");
 };
@@ -271,7 +273,7 @@ __global__ void __launch_bounds__(LSmem<N, M, kSpec>::threads, 1)
     // the tile after the next, asked for now and handed to the slot at the end
     const int64_t after = t == 32 ? feed.after(next) : 0;
     const Seg& sg = g.s[p.seg];
-    float* const sQ = sW + (it & 1) * SM::nQ;
+    float* const sQ = sW + (SM::bufs > 1 ? it & 1 : 0) * SM::nQ;
     tc::cp_async_wait<0>();  // this tile's rows and parameters
     __syncwarp();
     const bool valid = lane < M::Q * p.nE;
@@ -287,17 +289,16 @@ __global__ void __launch_bounds__(LSmem<N, M, kSpec>::threads, 1)
     Part pn{0, 0, 0};
     if (next < ntiles) {
       pn = part_of(next);
-      request(pn, (it + 1) & 1);
+      if constexpr (SM::bufs > 1) request(pn, (it + 1) & 1);
     }
     if constexpr (!M::fluid) row::normals_request(a, sW + SM::oN, p.v0, p.nE, lane);
     tc::cp_async_commit();
     float* const rowp = sQ + (valid ? lane : 0) * S::SB;
-    std::conditional_t<kSpec, row::SpecLevels<float, N>, row::NoLevels> lev = [&] {
+    std::conditional_t<kSpec, row::SpecLevels<float, N, true>, row::NoLevels> lev = [&] {
       if constexpr (kSpec) {
         tc::cp_async_wait<0>();
         __syncwarp();  // the normals
-        return row::SpecLevels<float, N>(a, valid ? sW + SM::oD + lane * S::ND : nullptr, sT, sW + SM::oN, p.v0, p.nE,
-                                         lane);
+        return row::SpecLevels<float, N, true>(a, valid, sT, sW + SM::oD, sW + SM::oN, p.v0, p.nE, lane);
       } else {
         return row::NoLevels{};
       }
@@ -322,7 +323,7 @@ __global__ void __launch_bounds__(LSmem<N, M, kSpec>::threads, 1)
       tc::mma3_ts<I_::nPO, I_::KO>(tbase + I_::cD + I_::nPE, tbase + I_::KE, tbase + I_::cL + I_::KE,
                                    sB + 4 * I_::oPO, sB + 4 * (I_::oPO + I_::sPO), false);
     });
-    if constexpr (kSpec) lev(std::integral_constant<int, 0>{}, I);  // (while the product runs)
+    lev(std::integral_constant<int, 0>{}, I);  // (while the product runs)
     mma.done();
     {
       float D1[B1];
@@ -350,12 +351,8 @@ __global__ void __launch_bounds__(LSmem<N, M, kSpec>::threads, 1)
       for (int l = 0; l < B; ++l) I[l] *= c0;
 #pragma unroll
       for (int m = 0; m < B1; ++m) I[m] = fmaf(c1, D1[m], I[m]);
-      if constexpr (kSpec) {
-        lev(std::integral_constant<int, 1>{}, D1);
-        row::predict<float, N, 1>(D1, I, st, sg, lev);
-      } else {
-        row::predict<float, N, 1>(D1, I, st, sg, row::NoLevels{});
-      }
+      lev(std::integral_constant<int, 1>{}, D1);
+      row::predict<float, N, 1>(D1, I, st, sg, lev);
     }
     // ---- modal face traces
     put(I, std::integral_constant<int, I_::KE>{}, std::integral_constant<int, I_::KO>{},
@@ -443,7 +440,10 @@ __global__ void __launch_bounds__(LSmem<N, M, kSpec>::threads, 1)
     __syncwarp();
     rows_back<N, M>(sQ, Qg + p.v0 * 9 * B, p.nE, lane);
     if constexpr (kSpec) {
-      row::special_faces<float, N>(a, sg, p.v0, p.nE, sW + SM::oD, sT, lane);
+      lev.surface(sg);
+      __syncwarp();  // the rows have left: the next tile's take their place
+      if (next < ntiles) request(pn, 0);
+      tc::cp_async_commit();
     }
     if (t == 32) s_next[slot][it & 1] = (int)after;
     tc::slot_bar(slot);

@@ -48,15 +48,7 @@ struct Shape {
   // 16-byte accesses: the stride in 16-byte units must be odd
   static constexpr int SB = VW == 1 ? (sizeof(T) == 4 ? (B | 1) : B) : (B / VW % 2 ? B : B + VW);
   static constexpr int FS = face_block(N);     // values of a face block
-  static constexpr int ND = nb3(N) + nb3(N - 1) + nb3(N - 2) + nb3(N - 3) + nb3(N - 4) + nb3(N - 5);
 };
-// row offset of D^k in a row's derivative stack
-__host__ __device__ constexpr int stack_off(int k, int N) {
-  int s = 0;
-  for (int j = 0; j < k; ++j) s += nb3(N - j);
-  return s;
-}
-
 template <class T, int VW>
 struct alignas(VW * sizeof(T)) Vec {
   T x[VW];

@@ -2,7 +2,7 @@
 // Cauchy-Kovalewski predictor, time integral, modal face traces and volume
 // term of three elements per warp.  kSpec: the launch's elements may have
 // gravitational faces (Sec. 4.3), fault faces or neighbours in another LTS
-// cluster (Sec. 4.4); their derivative stack is kept in shared memory for it.
+// cluster (Sec. 4.4).
 #pragma once
 #include "row_common.cuh"
 #include "tc_common.cuh"
@@ -186,12 +186,12 @@ __device__ __forceinline__ void star_rows(const RowStar<T>& st, T* out, Y&& yf) 
 }
 
 // shared memory of one warp (values of T): dofs rows, the nine-quantity modes
-// of two faces, and with kSpec the rows' derivative stacks
+// of two faces, and with kSpec the modes of the gravitational faces
 template <class T, int N, bool kSpec>
 struct LocalSmem {
   using S = Shape<T, N>;
   static constexpr int nQ = (9 * EW * S::SB + 3) / 4 * 4, nT = (2 * 9 * EW * S::Bf + 3) / 4 * 4;
-  static constexpr int nD = kSpec ? 9 * EW * S::ND : 0;
+  static constexpr int nD = kSpec ? 4 * EW * (N + 1) * S::Bf : 0;
   static constexpr int nN = 16 * EW;  // the faces' normals
   static constexpr int warp = (nQ + nN + nT + nD + 3) / 4 * 4;
   static constexpr int bytes(int threads) { return warp * (int)sizeof(T) * (threads / 32); }
@@ -277,36 +277,63 @@ __device__ __forceinline__ void faces_out(const StepArgs& a, const Seg& sg, int6
   }
 }
 
-// What kSpec does with the rows of D^k: keeps them in the rows' stacks and, on
-// faces with a finer neighbour (which integrates this element's Taylor expansion
-// over its sub-steps), writes their modal traces.  The sparse projections of a
-// level are applied to the rows in registers, faces 0, 1 and 2, 3 together and
-// only where some element of the warp has such a face: 1,766 FMAs for all six
-// levels of four faces at degree 5, where dense sums over the stacks took 2,200
-// instructions per element and face.
-template <class T, int N>
+// Faces that need more than their traces (kSpec): a finer neighbour integrates
+// this element's Taylor expansion over its sub-steps, a fault's friction solve
+// evaluates it at its time points, and a gravitational surface's ODE (Sec. 4.3)
+// is driven by it.  All three read the derivatives' traces, formed level by
+// level from the rows in registers with the sparse face projections (faces 0, 1
+// and 2, 3 together, only where some element of the warp has such a face):
+//   finer neighbour  the modal blocks of every level, to the derivative traces
+//   fault            nine quantities at the face nodes (as the solve reads them)
+//   gravity          the modes of v_n - sigma_nn / Z, kept in shared memory for
+//                    surface() at the end
+// No level outlives its registers.  kOneGrav: at most one gravitational face
+// per element (the tensor-core kernels).
+template <class T, int N, bool kOneGrav>
 struct SpecLevels {
   using S = Shape<T, N>;
+  enum { NONE = 0, FINE = 1, GRAVITY = 2, FAULT = 3 };
+  static constexpr int values = (kOneGrav ? 1 : 4) * EW * (N + 1) * S::Bf;  // of sF
   const StepArgs& a;
-  T *stack, *sT;      // this row's stack (null: no row); staging as in faces_out
+  bool on;            // this lane holds a row
+  T *sT, *sF;         // staging as in faces_out; the surfaces' modes [face][level][Bf]
   const T* sN;
   int64_t v0;
   int nE, lane;
-  int ds;             // lane 4 j + f: the slot of a face with a finer neighbour, else -1
-  unsigned mask;      // faces f with such an element in the warp
-  __device__ __forceinline__ SpecLevels(const StepArgs& args, T* st, T* t, const T* n, int64_t v, int e, int l)
-      : a(args), stack(st), sT(t), sN(n), v0(v), nE(e), lane(l), ds(-1), mask(0) {
-    if (lane < 4 * nE && a.dslot) {
+  int what, slot;     // lane 4 j + f: of face f of element j
+  T iz;               // 1 / Z (gravity)
+  unsigned mask, surf;  // faces f to project; bit 4 j + f: a gravitational face
+  __device__ __forceinline__ SpecLevels(const StepArgs& args, bool row, T* t, T* sf, const T* n, int64_t v, int e, int l)
+      : a(args), on(row), sT(t), sF(sf), sN(n), v0(v), nE(e), lane(l), what(NONE), slot(-1), iz(T(0)) {
+    if (lane < 4 * nE) {
       const int64_t ef = elem_of(v0 + (lane >> 2), a.S) * 4 + (lane & 3);
-      if (((a.ninfo[ef] >> 5) & 7) == NK_FINE) ds = a.dslot[ef];
+      const int kind = (a.ninfo[ef] >> 5) & 7;
+      if (kind == NK_FINE || kind == NK_FAULT) {
+        what = kind == NK_FINE ? FINE : FAULT;
+        slot = a.dslot[ef];
+      } else if (a.gslot) {
+        slot = a.gslot[ef];
+        if (slot >= 0) {
+          what = GRAVITY;
+          iz = (T)(1.0 / a.gpar[(size_t)slot * GPAR + 3]);
+        }
+      }
     }
-    const unsigned b = __ballot_sync(0xffffffffu, ds >= 0);
+    const unsigned b = __ballot_sync(0xffffffffu, what != NONE);
     mask = (b | b >> 4 | b >> 8) & 15u;
+    surf = __ballot_sync(0xffffffffu, what == GRAVITY);
+  }
+  __device__ __forceinline__ int scenario(int j) const {
+    return a.S == 1 ? 0 : (int)(v0 + j - elem_of(v0 + j, a.S) * a.S);
+  }
+  // the surface modes of face f of element j
+  __device__ __forceinline__ T* face_modes(int j, int f) const {
+    return sF + (kOneGrav ? j : 4 * j + f) * (N + 1) * S::Bf;
   }
   template <int K, int F0>
   __device__ __forceinline__ void pair(const T* D) const {
-    constexpr int L = nb3(N - K), Bk = nb2(N - K), Bf = S::Bf;
-    if (stack) {
+    constexpr int L = nb3(N - K), Bk = nb2(N - K), Bf = S::Bf;  // (degree N - K: no higher modes)
+    if (on) {
       T* const s0 = sT + lane * Bf;
       sp::each<Bk>([&](auto rc) {
         constexpr int r = decltype(rc)::value;
@@ -324,128 +351,80 @@ struct SpecLevels {
 #pragma unroll 1
     for (int i = lane; i < (2 * EW * Bf + 31) / 32 * 32; i += 32) {
       const int jf = i / Bf, n = i - jf * Bf, j = jf >> 1, f = F0 + (jf & 1);
-      const int slot = __shfl_sync(0xffffffffu, ds, (4 * j + f) & 31);
-      if (j >= nE || slot < 0) continue;
-      T o[6];
+      const int w = __shfl_sync(0xffffffffu, what, (4 * j + f) & 31), sl = __shfl_sync(0xffffffffu, slot, (4 * j + f) & 31);
+      const T z = __shfl_sync(0xffffffffu, iz, (4 * j + f) & 31);
+      if (j >= nE || w == NONE) continue;
+      const T* const s = sT + ((jf & 1) * 9 * EW + 9 * j) * Bf;
+      T* const d = reinterpret_cast<T*>(a.dtrace) + ((int64_t)sl * a.S + scenario(j)) * (N + 1) * 9 * Bf;
+      T q[9];
+      if (w == FAULT) {
 #pragma unroll
-      for (int k = 0; k < 6; ++k) o[k] = T(0);
-      if (n < Bk) {  // (a polynomial of degree N - K: no higher modes)
-        const T* const s = sT + ((jf & 1) * 9 * EW + 9 * j) * Bf + n;
-        const T* const c = sN + (4 * j + f) * 4;
-        T q[9];
+        for (int p = 0; p < 9; ++p) q[p] = T(0);
+        const T* const nd = reinterpret_cast<const T*>(a.nodalT) + n;
+#pragma unroll 3
+        for (int r = 0; r < Bk; ++r) {
+          const T x = nd[r * Bf];
 #pragma unroll
-        for (int p = 0; p < 9; ++p) q[p] = s[p * Bf];
-        o[0] = fma(q[5], c[2], fma(q[3], c[1], q[0] * c[0]));
-        o[1] = fma(q[4], c[2], fma(q[1], c[1], q[3] * c[0]));
-        o[2] = fma(q[2], c[2], fma(q[4], c[1], q[5] * c[0]));
-        o[3] = q[6]; o[4] = q[7]; o[5] = q[8];
+          for (int p = 0; p < 9; ++p) q[p] = fma(x, s[p * Bf + r], q[p]);
+        }
+#pragma unroll
+        for (int p = 0; p < 9; ++p) d[(K * 9 + p) * Bf + n] = q[p];
+        continue;
       }
-      const int64_t v = v0 + j;
-      T* const d = reinterpret_cast<T*>(a.dtrace) +
-                   ((int64_t)slot * a.S + (v - elem_of(v, a.S) * a.S)) * (N + 1) * 9 * Bf + K * S::FS + 6 * n;
+      const T* const c = sN + (4 * j + f) * 4;
 #pragma unroll
-      for (int k = 0; k < 6; ++k) d[k] = o[k];
+      for (int p = 0; p < 9; ++p) q[p] = n < Bk ? s[p * Bf + n] : T(0);
+      const T o[6] = {fma(q[5], c[2], fma(q[3], c[1], q[0] * c[0])), fma(q[4], c[2], fma(q[1], c[1], q[3] * c[0])),
+                      fma(q[2], c[2], fma(q[4], c[1], q[5] * c[0])), q[6], q[7], q[8]};
+      if (w == FINE) {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) d[K * S::FS + 6 * n + k] = o[k];
+      } else {
+        face_modes(j, f)[K * Bf + n] = fma(o[5], c[2], fma(o[4], c[1], o[3] * c[0])) -
+                                       fma(o[2], c[2], fma(o[1], c[1], o[0] * c[0])) * z;
+      }
     }
     __syncwarp();
   }
   template <int K>
   __device__ __forceinline__ void operator()(std::integral_constant<int, K>, const T* D) const {
-    if (stack) {
-#pragma unroll
-      for (int l = 0; l < nb3(N - K); ++l) stack[stack_off(K, N) + l] = D[l];
-    }
     if (mask & 3u) pair<K, 0>(D);
     if (mask & 12u) pair<K, 2>(D);
   }
-};
-struct NoLevels {
-  template <int K, class T>
-  __device__ __forceinline__ void operator()(std::integral_constant<int, K>, const T*) const {}
-};
-
-// Faces of the warp's elements that need more than their traces (kSpec): the
-// nodal derivative traces of fault faces, and the gravitational surface's ODE.
-// sD: the elements' stacks (row stride ND); sW: scratch (the trace staging).
-// The elements with such a face f go side by side, one (element, node) per
-// lane, and the operator's columns are loaded several at a time: the latency
-// of one warp is what a small mesh waits for.
-template <class T, int N>
-__device__ void special_faces(const StepArgs& a, const Seg& sg, int64_t v0, int nE, const T* sD, T* sW, int lane) {
-  using S = Shape<T, N>;
-  constexpr int B = S::B, Bf = S::Bf, ND = S::ND;
-  static_assert(EW * (ND + 2 * Bf) <= 2 * 9 * EW * Bf, "scratch");
-  T* const sS = sW + EW * ND;
-  // lane 4 j + f: the gravity slot and the fault's derivative-trace slot of face f of element j
-  int grav = -1, fault = -1;
-  if (lane < 4 * nE) {
-    const int64_t ef = elem_of(v0 + (lane >> 2), a.S) * 4 + (lane & 3);
-    if (a.gslot) grav = a.gslot[ef];
-    if (a.dslot && ((a.ninfo[ef] >> 5) & 7) == NK_FAULT) fault = a.dslot[ef];
-  }
-  const unsigned gmask = __ballot_sync(0xffffffffu, grav >= 0), fmask = __ballot_sync(0xffffffffu, fault >= 0);
-  auto scenario = [&](int j) { return (int)(v0 + j - elem_of(v0 + j, a.S) * a.S); };
-#pragma unroll 1
-  for (int f = 0; f < 4; ++f) {
-    const T* const E = reinterpret_cast<const T*>(a.efcT) + (size_t)f * B * Bf;
-    if (fmask & (0x111u << f)) {
-#pragma unroll 1
-      for (int k = 0; k <= N; ++k) {
-        const int Bk = nb3(N - k), o = stack_off(k, N);
+  // The gravitational surfaces over the step, up to three faces at a time, one
+  // (face, node) per lane: f_m = modes of level m at the node / m!, the (eta, H)
+  // series in FP64, then the modes of -rho g H and eta^{n+1} - eta^n.
+  __device__ void surface(const Seg& sg) const {
+    constexpr int Bf = S::Bf;
+    unsigned left = surf;
+    while (left) {
+      int face[EW];  // 4 j + f, or -1
 #pragma unroll
-        for (int it = 0; it < (EW * Bf + 31) / 32; ++it) {
-          const int i = lane + 32 * it, j = i < EW * Bf ? i / Bf : 0, n = i - j * Bf;
-          const int slot = __shfl_sync(0xffffffffu, fault, 4 * j + f);
-          if (i >= nE * Bf || slot < 0) continue;
-          T q[9];
-#pragma unroll
-          for (int p = 0; p < 9; ++p) q[p] = T(0);
-#pragma unroll 5
-          for (int l = 0; l < Bk; ++l) {
-            const T w = E[(size_t)l * Bf + n];
-#pragma unroll
-            for (int p = 0; p < 9; ++p) q[p] = fma(w, sD[(9 * j + p) * ND + o + l], q[p]);
-          }
-          T* const out = reinterpret_cast<T*>(a.dtrace) + (((int64_t)slot * a.S + scenario(j)) * (N + 1) + k) * 9 * Bf + n;
-#pragma unroll
-          for (int p = 0; p < 9; ++p) out[p * Bf] = q[p];
-        }
+      for (int c = 0; c < EW; ++c) {
+        face[c] = __ffs(left) - 1;
+        left &= left - 1;
       }
-    }
-    if (gmask & (0x111u << f)) {
-      // g_m[l]: v_n - sigma_nn / Z of the derivative rows, then per face node
-      // f_m = E g_m / m!, the (eta, H) series in FP64, and the modes of
-      // -rho g H and eta^{n+1} - eta^n
-      for (int j = 0; j < nE; ++j) {
-        const int gs = __shfl_sync(0xffffffffu, grav, 4 * j + f);
-        if (gs < 0) continue;
-        const double* const gp = a.gpar + (size_t)gs * GPAR;
-        const T nx = (T)gp[0], ny = (T)gp[1], nz = (T)gp[2], iz = (T)(1.0 / gp[3]);
-        const T* const D = sD + 9 * j * ND;
-        for (int l = lane; l < ND; l += 32) {
-          const T snn = nx * nx * D[l] + ny * ny * D[ND + l] + nz * nz * D[2 * ND + l] +
-                        T(2) * (nx * ny * D[3 * ND + l] + ny * nz * D[4 * ND + l] + nx * nz * D[5 * ND + l]);
-          const T vn = nx * D[6 * ND + l] + ny * D[7 * ND + l] + nz * D[8 * ND + l];
-          sW[j * ND + l] = vn - snn * iz;
-        }
-      }
-      __syncwarp();
+      auto which = [&](int c) { return c == 0 ? face[0] : c == 1 ? face[1] : face[2]; };
 #pragma unroll 1
       for (int it = 0; it < (EW * Bf + 31) / 32; ++it) {
-        const int i = lane + 32 * it, j = i < EW * Bf ? i / Bf : 0, n = i - j * Bf;
-        const int gs = __shfl_sync(0xffffffffu, grav, 4 * j + f);
-        if (i >= nE * Bf || gs < 0) continue;
-        const T* const gj = sW + j * ND;
-        double fm[N + 1];
-#pragma unroll
-        for (int m = 0; m <= N; ++m) {
-          T acc = T(0);
-#pragma unroll 14
-          for (int l = 0; l < nb3(N - m); ++l) acc = fma(E[(size_t)l * Bf + n], gj[stack_off(m, N) + l], acc);
-          fm[m] = (double)acc * kRowRcpFact[m];
-        }
+        const int i = lane + 32 * it, c = i < EW * Bf ? i / Bf : 0, n = i - c * Bf, jf = which(c);
+        const int gs = __shfl_sync(0xffffffffu, slot, jf & 31);
+        if (i >= EW * Bf || jf < 0) continue;
+        const T* const F = face_modes(jf >> 2, jf & 3);
         const double* const gp = a.gpar + (size_t)gs * GPAR;
-        double* const eta = a.eta + ((int64_t)gs * a.S + scenario(j)) * Bf + n;
+        double* const eta = a.eta + ((int64_t)gs * a.S + scenario(jf >> 2)) * Bf + n;
         const double kappa = gp[4], rg = gp[5], dt = sg.dt, eta0 = *eta;
+        const T* const nd = reinterpret_cast<const T*>(a.nodalT) + n;
+        T acc[N + 1];
+#pragma unroll
+        for (int m = 0; m <= N; ++m) acc[m] = T(0);
+#pragma unroll
+        for (int r = 0; r < Bf; ++r) {
+          const T w = nd[r * Bf];
+#pragma unroll
+          for (int m = 0; m <= N; ++m)
+            if (r < nb2(N - m)) acc[m] = fma(w, F[m * Bf + r], acc[m]);
+        }
         double cm = eta0, e1 = eta0, H = eta0 * dt, pw = 1.0;
         auto term = [&](int m, double fv) {
           cm = (fv - kappa * cm) * kRowRcp[m + 1];
@@ -456,36 +435,40 @@ __device__ void special_faces(const StepArgs& a, const Seg& sg, int64_t v0, int 
           return t;
         };
 #pragma unroll
-        for (int m = 0; m <= N; ++m) term(m, fm[m]);
+        for (int m = 0; m <= N; ++m) term(m, (double)acc[m] * kRowRcpFact[m]);
 #pragma unroll 1
         for (int m = N + 1; m < N + 40; ++m)
           if (fabs(term(m, 0.0)) <= 1e-17 * fabs(e1)) break;
         *eta = e1;
-        sS[j * 2 * Bf + n] = (T)(-rg * H);
-        sS[(j * 2 + 1) * Bf + n] = (T)(e1 - eta0);
+        sT[c * 2 * Bf + n] = (T)(-rg * H);
+        sT[(c * 2 + 1) * Bf + n] = (T)(e1 - eta0);
       }
       __syncwarp();
 #pragma unroll 1
       for (int it = 0; it < (EW * Bf + 31) / 32; ++it) {
-        const int i = lane + 32 * it, j = i < EW * Bf ? i / Bf : 0, r = i - j * Bf;
-        const int gs = __shfl_sync(0xffffffffu, grav, 4 * j + f);
-        if (i >= nE * Bf || gs < 0) continue;
+        const int i = lane + 32 * it, c = i < EW * Bf ? i / Bf : 0, r = i - c * Bf, jf = which(c);
+        const int gs = __shfl_sync(0xffffffffu, slot, jf & 31);
+        if (i >= EW * Bf || jf < 0) continue;
         const T* const mn = reinterpret_cast<const T*>(a.modalT) + r;
         T h = T(0), d = T(0);
 #pragma unroll
         for (int n = 0; n < Bf; ++n) {
           const T w = mn[n * Bf];
-          h = fma(w, sS[j * 2 * Bf + n], h);
-          d = fma(w, sS[(j * 2 + 1) * Bf + n], d);
+          h = fma(w, sT[c * 2 * Bf + n], h);
+          d = fma(w, sT[(c * 2 + 1) * Bf + n], d);
         }
-        T* const out = reinterpret_cast<T*>(a.gflux) + ((int64_t)gs * a.S + scenario(j)) * 9 * Bf + r;
+        T* const out = reinterpret_cast<T*>(a.gflux) + ((int64_t)gs * a.S + scenario(jf >> 2)) * 9 * Bf + r;
         out[0] = h;
         out[Bf] = d;
       }
       __syncwarp();
     }
   }
-}
+};
+struct NoLevels {
+  template <int K, class T>
+  __device__ __forceinline__ void operator()(std::integral_constant<int, K>, const T*) const {}
+};
 
 template <class T, int N, bool kSpec>
 __global__ void __launch_bounds__(kMaxThreads, sizeof(T) == 4 ? 2 : 1) local_row_kernel(StepArgs a, const __grid_constant__ Segs g) {
@@ -509,7 +492,6 @@ __global__ void __launch_bounds__(kMaxThreads, sizeof(T) == 4 ? 2 : 1) local_row
   RowStar<T> st;
   st.setup(lane, valid, reinterpret_cast<const T*>(a.par) + elem_of(u.v0 + (valid ? j : 0), a.S) * PAR);
   T* const row = sQ + (valid ? lane : 0) * S::SB;
-  T* const stack = kSpec && valid ? sT + M::nT + lane * S::ND : nullptr;
   __syncwarp();
 
   // ---- D^0, the predictor levels and the time integral
@@ -523,12 +505,13 @@ __global__ void __launch_bounds__(kMaxThreads, sizeof(T) == 4 ? 2 : 1) local_row
   if constexpr (kSpec) {
     tc::cp_async_wait<0>();
     __syncwarp();  // the normals
-    const SpecLevels<T, N> lev(a, stack, sT, sN, u.v0, u.nE, lane);
-    lev(std::integral_constant<int, 0>{}, I);
-    predict<T, N, 0>(I, I, st, sg, lev);
-  } else {
-    predict<T, N, 0>(I, I, st, sg, NoLevels{});
   }
+  std::conditional_t<kSpec, SpecLevels<T, N, false>, NoLevels> lev = [&] {
+    if constexpr (kSpec) return SpecLevels<T, N, false>(a, valid, sT, sT + M::nT, sN, u.v0, u.nE, lane);
+    else return NoLevels{};
+  }();
+  lev(std::integral_constant<int, 0>{}, I);
+  predict<T, N, 0>(I, I, st, sg, lev);
 
   // ---- modal face traces, two faces at a time through shared memory
   {
@@ -575,10 +558,7 @@ __global__ void __launch_bounds__(kMaxThreads, sizeof(T) == 4 ? 2 : 1) local_row
   });
   __syncwarp();
   rows_out<T, N>(sQ, Q, u.nE, lane);
-  if constexpr (kSpec) {
-    __syncwarp();
-    special_faces<T, N>(a, sg, u.v0, u.nE, sT + M::nT, sT, lane);
-  }
+  if constexpr (kSpec) lev.surface(sg);
 }
 
 template <class T, int N>
@@ -588,14 +568,14 @@ int launch_local_row_t(const StepArgs& a, const Segs& g, int threads, bool spec,
                                           LocalSmem<T, N, false>::bytes(kMaxThreads));
     if (ce == cudaSuccess)
       ce = cudaFuncSetAttribute(local_row_kernel<T, N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                LocalSmem<T, N, true>::bytes(64));
+                                LocalSmem<T, N, true>::bytes(128));
     return ce;
   });
   if (rc) return rc;
   const int64_t units = g.n ? g.first[g.n] : 0;
   if (units <= 0) return 0;
   if (threads < 32 || threads > kMaxThreads || threads % 32) return (int)cudaErrorInvalidValue;
-  if (spec && threads > 64) threads = 64;  // (the derivative stacks in shared memory)
+  if (spec && threads > 128) threads = 128;  // (shared memory)
   const int w = threads / 32;
   const unsigned blocks = (unsigned)((units + w - 1) / w);
   if (spec)

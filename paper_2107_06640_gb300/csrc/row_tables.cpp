@@ -55,6 +55,11 @@ RowTables make_row_tables(const RefOps& o) {
   for (const Entry& x : kR3)
     if (x.r < Bf && x.c < B)
       for (int n = 0; n < Bf; ++n) t.modalT[(size_t)n * Bf + x.r] = o.lift[((size_t)3 * B + x.c) * Bf + n] / x.v;
+  // modes at the nodes, from the same multiples: efc[3][n][l] = v psi_r(n)
+  t.nodalT.assign((size_t)Bf * Bf, 0.0);
+  for (const Entry& x : kR3)
+    if (x.r < Bf && x.c < B)
+      for (int n = 0; n < Bf; ++n) t.nodalT[(size_t)x.r * Bf + n] = o.efc[((size_t)3 * Bf + n) * B + x.c] / x.v;
   // both ways of lifting a node: over the modes, and the nodal lift
   for (int f = 0; f < 4; ++f)
     for (int m = 0; m < B; ++m)

@@ -977,7 +977,11 @@ int adg_save_state(adg_ctx* ctx, void* buf, size_t* len) {
     std::memcpy(p, hdr, sizeof(hdr));
     char* body = p + kStateHeader;
     check_cuda(cudaStreamSynchronize(c.stream), "save");
-    check_cuda(cudaMemcpy(body, c.dQ, qb, cudaMemcpyDeviceToHost), "save dofs");
+    const std::vector<int64_t> place = c.state_places();
+    const size_t per = c.nt ? qb / c.nt : 0;
+    std::vector<char> tmp(place.empty() ? 0 : qb);
+    check_cuda(cudaMemcpy(place.empty() ? body : tmp.data(), c.dQ, qb, cudaMemcpyDeviceToHost), "save dofs");
+    for (size_t i = 0; i < place.size(); ++i) std::memcpy(body + place[i] * per, tmp.data() + i * per, per);
     if (eb) check_cuda(cudaMemcpy(body + qb, c.dEta, eb, cudaMemcpyDeviceToHost), "save eta");
     if (fb) check_cuda(cudaMemcpy(body + qb + eb, c.dFstate, fb, cudaMemcpyDeviceToHost), "save fault state");
     *len = need;
@@ -1002,7 +1006,11 @@ int adg_load_state(adg_ctx* ctx, const void* buf, size_t len) {
       adg::throw_err(ADG_E_INVALID, "state does not match this context");
     const char* body = p + kStateHeader;
     check_cuda(cudaStreamSynchronize(c.stream), "load");
-    check_cuda(cudaMemcpy(c.dQ, body, qb, cudaMemcpyHostToDevice), "load dofs");
+    const std::vector<int64_t> place = c.state_places();
+    const size_t per = c.nt ? qb / c.nt : 0;
+    std::vector<char> tmp(place.empty() ? 0 : qb);
+    for (size_t i = 0; i < place.size(); ++i) std::memcpy(tmp.data() + i * per, body + place[i] * per, per);
+    check_cuda(cudaMemcpy(c.dQ, place.empty() ? body : tmp.data(), qb, cudaMemcpyHostToDevice), "load dofs");
     c.project_fluid();
     if (eb) check_cuda(cudaMemcpy(c.dEta, body + qb, eb, cudaMemcpyHostToDevice), "load eta");
     if (fb) {

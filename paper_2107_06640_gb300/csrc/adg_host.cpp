@@ -993,6 +993,24 @@ int64_t Ctx::launches_per_macro() const {
   return L;
 }
 
+// Place of every element in a saved state: the tensor-core contexts' own order,
+// else by cluster and the caller's numbering alone (empty: nothing to move).
+std::vector<int64_t> Ctx::state_places() const {
+  std::vector<int64_t> p;
+  if (tc) return p;
+  bool moved = false;
+  for (int c = 0; c < ncl; ++c) {
+    std::vector<int64_t> user(order.begin() + cl_begin[c], order.begin() + cl_begin[c + 1]);
+    std::sort(user.begin(), user.end());
+    for (int64_t i = cl_begin[c]; i < cl_begin[c + 1]; ++i) {
+      p.push_back(cl_begin[c] + (std::lower_bound(user.begin(), user.end(), order[i]) - user.begin()));
+      moved = moved || p.back() != i;
+    }
+  }
+  if (!moved) p.clear();
+  return p;
+}
+
 void Ctx::project_fluid(bool sync) {
   if (!acoustic || !n_fluid) return;
   const int rc = launch_isotropic_fluid(fp64, dQ, dFluid, n_fluid, S * B, B, stream);

@@ -206,6 +206,7 @@ struct Ctx {
   void launch_tick(int s, double dtm);
   void run_macro(double scale);
   int64_t launches_per_macro() const;
+  std::vector<int64_t> state_places() const;
   void autotune(int reps, bool force, int* choice, double* ms);
   void check_err();
   ~Ctx();

@@ -525,14 +525,14 @@ void Ctx::setup() {
     else  // the row kernels: their special instantiation takes all of these
       special[e] = cc || ng_e || coarser || finer ? 2 : 0;
   }
-  // order key within a cluster: 0 plain elastic, 1 plain fluid on the
+  // order key within a cluster: 0 plain elastic, 1 plain fluid on an
   // acoustic local kernel, 2 with a coarser neighbour, 3 with a gravitational
-  // face or a finer neighbour (all four on the tensor-core kernels), 4 the
-  // CUDA-core rest
+  // face or a finer neighbour (with the tensor-core kernels all four on them),
+  // 4 the rest
   std::vector<char> key(E, 0);
   for (int64_t e = 0; e < E; ++e)
     key[e] = special[e] == 1 ? 2 : special[e] == 3 ? 3 : special[e] == 2 ? 4
-                                 : (char)(tc && acoustic && mu[e] == 0.0 ? 1 : 0);
+                                 : (char)(acoustic && mu[e] == 0.0 ? 1 : 0);
   order.resize(E);
   for (int64_t e = 0; e < E; ++e) order[e] = e;
   std::stable_sort(order.begin(), order.end(), [&](int64_t a, int64_t b) {
@@ -543,6 +543,7 @@ void Ctx::setup() {
   cl_begin.assign(ncl + 1, 0);
   cl_plain.assign(ncl, 0);
   cl_row.assign(ncl, 0);
+  cl_row_fluid.assign(ncl, 0);
   cl_elastic.assign(ncl, 0);
   cl_fluid.assign(ncl, 0);
   cl_grav.assign(ncl, 0);
@@ -551,7 +552,8 @@ void Ctx::setup() {
     const int k = key[order[i]], c = cl[order[i]];
     cl_begin[c + 1]++;
     if (tc && k < 4) cl_plain[c]++;
-    if (!tc && k == 0) cl_row[c]++;
+    if (!tc && k <= 1) cl_row[c]++;
+    if (!tc && k == 1) cl_row_fluid[c]++;
     if (tc && k == 0) cl_elastic[c]++;
     if (tc && k == 1) cl_fluid[c]++;
     if (tc && k == 3) cl_grav[c]++;
@@ -798,11 +800,11 @@ void Ctx::launch_tick(int s, double dtm) {
   StepArgs a = base_args();
   for (int phase = 0; phase < 2; ++phase) {
     // per kernel kind the clusters' segments: tensor-core elastic, tensor-core
-    // acoustic and gravitational-face (local phase only), the row kernels' plain
-    // and special elements
+    // acoustic and gravitational-face (local phase only), the row kernels' plain,
+    // acoustic (local phase) and special elements
     // (tcb: the local phase's elements with a coarser neighbour outside the
     // special range, on the instantiation with the LTS-buffer code)
-    std::vector<Seg> tcs, tcb, fls, grs, rws, rss;
+    std::vector<Seg> tcs, tcb, fls, grs, rws, rfs, rss;
     bool ltsf = false;
     for (int c = 0; c < ncl; ++c) {
       const bool active = phase == 0 ? s % (1 << c) == 0 : (s + 1) % (1 << c) == 0;
@@ -844,11 +846,13 @@ void Ctx::launch_tick(int s, double dtm) {
       if (tc) {
         if (n > np) rss.push_back(seg(cl_begin[c] + np, n - np));
       } else {
-        if (cl_row[c] > 0) rws.push_back(seg(cl_begin[c], cl_row[c]));
+        const int64_t nf = phase == 0 ? cl_row_fluid[c] : 0, nr = cl_row[c] - nf;
+        if (nr > 0) rws.push_back(seg(cl_begin[c], nr));
+        if (nf > 0) rfs.push_back(seg(cl_begin[c] + nr, nf));
         if (n > cl_row[c]) rss.push_back(seg(cl_begin[c] + cl_row[c], n - cl_row[c]));
       }
     }
-    if (tcs.empty() && tcb.empty() && fls.empty() && grs.empty() && rws.empty() && rss.empty()) continue;
+    if (tcs.empty() && tcb.empty() && fls.empty() && grs.empty() && rws.empty() && rfs.empty() && rss.empty()) continue;
     ProfEv ev{phase, nullptr, nullptr, 0};
     if (prof) {
       CK(cudaEventCreate(&ev.a));
@@ -882,6 +886,8 @@ void Ctx::launch_tick(int s, double dtm) {
            return phase == 0 ? launch_local_row(fp64, N, a, g, st, cc_threads[0], true)
                              : launch_neighbour_row(fp64, N, a, g, st, cc_threads[1], true);
          }},
+        {&rfs, kRowElemsFluid, false,
+         [&](const Segs& g, void* st) { return launch_local_fluid(fp64, N, a, g, st, cc_threads[0]); }},
         {&rws, kRowElems, false,
          [&](const Segs& g, void* st) {
            return phase == 0 ? launch_local_row(fp64, N, a, g, st, cc_threads[0], false)
@@ -970,7 +976,7 @@ int64_t Ctx::launches_per_macro() const {
   const int ticks = 1 << (ncl - 1);
   for (int s = 0; s < ticks; ++s)
     for (int phase = 0; phase < 2; ++phase) {
-      bool tcl = false, tbl = false, fll = false, grl = false, ccl = false, rwl = false;
+      bool tcl = false, tbl = false, fll = false, grl = false, ccl = false, rwl = false, rfl = false;
       for (int c = 0; c < ncl; ++c) {
         const int64_t n = cl_begin[c + 1] - cl_begin[c];
         if (!n || (phase == 0 ? s % (1 << c) : (s + 1) % (1 << c))) continue;
@@ -986,9 +992,11 @@ int64_t Ctx::launches_per_macro() const {
           tcl = tcl || np > 0;
         }
         ccl = ccl || (tc ? n > np : n > cl_row[c]);
-        rwl = rwl || (!tc && cl_row[c] > 0);
+        const int64_t rf = tc || phase ? 0 : cl_row_fluid[c];
+        rfl = rfl || rf > 0;
+        rwl = rwl || (!tc && cl_row[c] > rf);
       }
-      L += tcl + tbl + fll + grl + ccl + rwl;
+      L += tcl + tbl + fll + grl + ccl + rwl + rfl;
     }
   return L;
 }

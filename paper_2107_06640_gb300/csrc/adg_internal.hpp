@@ -90,6 +90,9 @@ struct Ctx {
   // have no gravitational or fault face and no neighbour in another cluster
   // (the row kernels' plain instantiation)
   std::vector<int64_t> cl_row;
+  // of them the last cl_row_fluid[c] are acoustic (the row kernel of eight
+  // elements per warp, local phase)
+  std::vector<int64_t> cl_row_fluid;
   // cluster c's tensor-core range includes elements with a coarser or finer
   // neighbour or a gravitational face (the neighbour kernel's code for them)
   std::vector<char> cl_tc_lts;
@@ -131,9 +134,9 @@ struct Ctx {
   cudaGraphExec_t graph_exec = nullptr;
   bool use_graph = true;
   // launch shapes (adg_autotune; phase 0 local, 1 neighbour): threads per
-  // element block of the CUDA-core kernels, consecutive tiles per CTA-slot
-  // sweep of the tensor-core kernels
-  int cc_threads[2] = {128, 128};
+  // block of the row kernels (0: by their own rule), consecutive tiles that a
+  // CTA slot of the tensor-core kernels takes at a time
+  int cc_threads[2] = {0, 0};
   int tc_chunk[2] = {1, 1};
   // dynamic rupture: fault faces in internal (cluster) order
   int64_t nff = 0;

@@ -77,6 +77,7 @@ __host__ __device__ inline int64_t elem_of(int64_t v, int S) {
 }
 // Virtual elements per warp of the row kernels
 constexpr int kRowElems = 3;
+constexpr int kRowElemsFluid = 8;  // of its acoustic form
 // Face coefficients: outward normal n[3]; the middle
 // state's tangential coefficients of the own and of the neighbour's side (t^b
 // from t and v, v^b from t and v) and what the normal components add to them
@@ -190,11 +191,13 @@ int launch_rupture(int fp64, int N, const DRArgs& a, void* stream);
 enum { ERR_NAN = 1u, ERR_TIMEOUT = 2u, ERR_NEWTON = 4u };
 
 // host-side launchers; return cudaError_t as int
-// (threads: per block, a multiple of 32 up to 256)
+// (threads: per block, a multiple of 32 up to 256; 0: by row::block_threads)
 // row kernels (row_local.cuh, row_neighbour.cuh): both precisions, every degree;
 // spec: the launch's elements may have gravitational or fault faces or
 // neighbours in another cluster
 int launch_local_row(int fp64, int N, const StepArgs& a, const Segs& g, void* stream, int threads, bool spec);
 int launch_neighbour_row(int fp64, int N, const StepArgs& a, const Segs& g, void* stream, int threads, bool spec);
+// the local row kernel of plain acoustic elements (adg_set_acoustic_ocean)
+int launch_local_fluid(int fp64, int N, const StepArgs& a, const Segs& g, void* stream, int threads);
 
 }  // namespace adg

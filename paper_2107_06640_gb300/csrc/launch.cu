@@ -7,6 +7,8 @@ int launch_local_row_f32(int N, const StepArgs& a, const Segs& g, int threads, b
 int launch_local_row_f64(int N, const StepArgs& a, const Segs& g, int threads, bool spec, void* stream);
 int launch_neighbour_row_f32(int N, const StepArgs& a, const Segs& g, int threads, bool spec, void* stream);
 int launch_neighbour_row_f64(int N, const StepArgs& a, const Segs& g, int threads, bool spec, void* stream);
+int launch_local_fluid_f32(int N, const StepArgs& a, const Segs& g, int threads, void* stream);
+int launch_local_fluid_f64(int N, const StepArgs& a, const Segs& g, int threads, void* stream);
 
 int launch_local_row(int fp64, int N, const StepArgs& a, const Segs& g, void* stream, int threads, bool spec) {
   return fp64 ? launch_local_row_f64(N, a, g, threads, spec, stream)
@@ -15,6 +17,9 @@ int launch_local_row(int fp64, int N, const StepArgs& a, const Segs& g, void* st
 int launch_neighbour_row(int fp64, int N, const StepArgs& a, const Segs& g, void* stream, int threads, bool spec) {
   return fp64 ? launch_neighbour_row_f64(N, a, g, threads, spec, stream)
               : launch_neighbour_row_f32(N, a, g, threads, spec, stream);
+}
+int launch_local_fluid(int fp64, int N, const StepArgs& a, const Segs& g, void* stream, int threads) {
+  return fp64 ? launch_local_fluid_f64(N, a, g, threads, stream) : launch_local_fluid_f32(N, a, g, threads, stream);
 }
 
 Segs make_segs(const Seg* s, int n, int unit, int chunk) {

@@ -72,7 +72,7 @@ struct Elastic {
 };
 struct Acoustic {
   static constexpr bool fluid = true;
-  static constexpr int Q = 4, EW = 8, TE = kTileElemsFluid;
+  static constexpr int Q = 4, EW = row::EWF, TE = kTileElemsFluid;
 };
 static_assert(Elastic::TE == 4 * Elastic::EW && Acoustic::TE == 4 * Acoustic::EW, "tile of 4 warps");
 
@@ -129,7 +129,7 @@ __device__ __forceinline__ void rows_request(float* sQ, const float* Q, int nE, 
   for (int k = 0; k < (M::Q * M::EW * C + 31) / 32; ++k) {
     const int i = lane + 32 * k, r = i / C, c = (i - r * C) * S::VW;
     if (r >= M::Q * nE) continue;
-    const int gr = M::fluid ? 9 * (r >> 2) + ((r & 3) ? 5 + (r & 3) : 0) : r;
+    const int gr = M::fluid ? row::fluid_row(r) : r;
     if constexpr (S::VW == 4)
       tc::cp_async16(sQ + r * S::SB + c, Q + gr * S::B + c);
     else
@@ -140,35 +140,10 @@ __device__ __forceinline__ void rows_request(float* sQ, const float* Q, int nE, 
 template <int N, class M>
 __device__ __forceinline__ void rows_back(const float* sQ, float* Q, int nE, int lane) {
   using S = row::Shape<float, N>;
-  using V = row::Vec<float, S::VW>;
-  constexpr int C = S::B / S::VW, R = M::fluid ? 6 : 9;
-#pragma unroll 4
-  for (int i = lane; i < nE * R * C; i += 32) {
-    const int r = i / C, c = (i - r * C) * S::VW;
-    const int e = r / R, q = r - e * R;  // acoustic: q = 0..2 the stresses, 3..5 the velocities
-    const int sr = M::fluid ? 4 * e + (q < 3 ? 0 : q - 2) : r, gr = M::fluid ? 9 * e + (q < 3 ? q : q + 3) : r;
-    *reinterpret_cast<V*>(Q + gr * S::B + c) = *reinterpret_cast<const V*>(sQ + sr * S::SB + c);
-  }
-}
-
-// acoustic: face f of the warp's elements, staged (sigma, v) modes -> face blocks
-template <int N>
-__device__ __forceinline__ void face_out_acoustic(const StepArgs& a, int64_t v0, int nE, int f, const float* sT,
-                                                  int lane) {
-  constexpr int Bf = nb2(N), FS = face_block(N), EW = Acoustic::EW;
-#pragma unroll
-  for (int it = 0; it < (EW * Bf + 31) / 32; ++it) {
-    const int i = lane + 32 * it, j = i / Bf, n = i - j * Bf;
-    if (i >= nE * Bf) continue;
-    const int64_t v = v0 + j;
-    const float* const s = sT + 4 * j * Bf + n;
-    const float* const c = reinterpret_cast<const float*>(a.crec) + (elem_of(v, a.S) * 4 + f) * CREC;
-    float2* const out = reinterpret_cast<float2*>(reinterpret_cast<float*>(a.trace) + (v * 4 + f) * FS + 6 * n);
-    const float x = s[0];
-    out[0] = make_float2(x * c[0], x * c[1]);
-    out[1] = make_float2(x * c[2], s[Bf]);
-    out[2] = make_float2(s[2 * Bf], s[3 * Bf]);
-  }
+  if constexpr (M::fluid)
+    row::fluid_rows_out<float, N>(sQ, Q, nE, lane);
+  else
+    row::rows_out_v<float, N, S::VW>(sQ, Q, nE, lane);
 }
 
 // kBuf: some elements of the launch have an LTS buffer (a coarser neighbour)
@@ -402,7 +377,7 @@ __global__ void __launch_bounds__(LSmem<N, M, kSpec>::threads, 1)
         }
         __syncwarp();
         if constexpr (M::fluid)
-          face_out_acoustic<N>(a, p.v0, p.nE, f0, sT, lane);
+          row::fluid_face_out<float, N>(a, p.v0, p.nE, f0, sT, lane);
         else
           row::faces_out<float, N, kBuf>(a, sg, p.v0, p.nE, f0, sT, sW + SM::oN, lane);
         __syncwarp();

@@ -92,8 +92,8 @@ extern "C" int adg_step_noalloc(adg_ctx* ctx, void* d_Q, int n_steps, void* stre
   }
   const adg::Segs g = adg::make_segs(&sg, 1, adg::kRowElems);
   for (int i = 0; i < n_steps; ++i) {
-    int rc = adg::launch_local_row(c.fp64, c.N, a, g, st, 128, false);
-    if (!rc) rc = adg::launch_neighbour_row(c.fp64, c.N, a, g, st, 128, false);
+    int rc = adg::launch_local_row(c.fp64, c.N, a, g, st, 0, false);
+    if (!rc) rc = adg::launch_neighbour_row(c.fp64, c.N, a, g, st, 0, false);
     if (rc) {
       c.last_error = std::string("adg_step_noalloc: launch failed: ") + cudaGetErrorString((cudaError_t)rc);
       return ADG_E_CUDA;

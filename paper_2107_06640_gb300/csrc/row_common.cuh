@@ -95,11 +95,27 @@ __device__ __forceinline__ void rows_out(const T* sQ, T* Q, int nE, int lane) {
     rows_out_v<T, N, 1>(sQ, Q, nE, lane);
 }
 
+// Threads per block where the caller leaves the choice (threads = 0).  The warps
+// of a block share nothing but, in the neighbour kernel, the re-orientation
+// table, so blocks are as small as that allows: with at most eight warps per SM
+// single warps spread best (degree 3 FP64, 3,072 tets: 110 us per step with 32
+// threads, 120 with 128), above that 128 (13,182 tets, FP32: 29.7 with 128,
+// 32.6 with 32).  FP32 at degrees 4 and 5 holds one block of 256 per SM either
+// way, and its table is filled once instead of twice (183,456 tets: degree 5
+// 1106 -> 1028 us, degree 4 782 -> 759 us); at degree 3 256 is slower (225 -> 231).
+template <class T, int N>
+inline int block_threads(int threads, int64_t units) {
+  if (threads) return threads;
+  if (units <= 8 * 152) return 32;
+  return sizeof(T) == 4 && N >= 4 ? 256 : 128;
+}
+
 // this warp's work unit: its segment, first virtual element and element count (0: none)
 struct Unit {
   int seg, nE;
   int64_t v0;
 };
+template <int EW = kRowElems>
 __device__ __forceinline__ Unit unit_of(const Segs& g) {
   const int64_t u = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (u >= g.first[g.n]) return {0, 0, 0};

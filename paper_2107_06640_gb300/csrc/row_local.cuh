@@ -277,6 +277,45 @@ __device__ __forceinline__ void faces_out(const StepArgs& a, const Seg& sg, int6
   }
 }
 
+// Acoustic elements (mu = 0, stress -p I; kept so by the solver when it runs with
+// acoustic media): lane 4 j + p holds sigma_xx (p = 0) or a velocity of element j
+// of eight; sigma_yy = sigma_zz = sigma_xx, no shear.
+constexpr int EWF = kRowElemsFluid;
+__device__ __forceinline__ int fluid_row(int r) { return 9 * (r >> 2) + ((r & 3) ? 5 + (r & 3) : 0); }  // of the dofs
+
+// the warp's rows from shared memory to the dofs: the normal stress three times, the velocities
+template <class T, int N>
+__device__ __forceinline__ void fluid_rows_out(const T* sQ, T* Q, int nE, int lane) {
+  using S = Shape<T, N>;
+  using V = Vec<T, S::VW>;
+  constexpr int C = S::B / S::VW;
+#pragma unroll 4
+  for (int i = lane; i < nE * 6 * C; i += 32) {
+    const int r = i / C, c = (i - r * C) * S::VW, e = r / 6, q = r - e * 6;  // q = 0..2 the stresses, 3..5 the velocities
+    const int sr = 4 * e + (q < 3 ? 0 : q - 2), gr = 9 * e + (q < 3 ? q : q + 3);
+    *reinterpret_cast<V*>(Q + gr * S::B + c) = *reinterpret_cast<const V*>(sQ + sr * S::SB + c);
+  }
+}
+// face f of the warp's elements, staged (sigma, v) modes -> face blocks
+template <class T, int N>
+__device__ __forceinline__ void fluid_face_out(const StepArgs& a, int64_t v0, int nE, int f, const T* sT, int lane) {
+  constexpr int Bf = Shape<T, N>::Bf;
+#pragma unroll(sizeof(T) == 4 ? 8 : 1)
+  for (int it = 0; it < (EWF * Bf + 31) / 32; ++it) {
+    const int i = lane + 32 * it, j = i / Bf, n = i - j * Bf;
+    if (i >= nE * Bf) continue;
+    const int64_t v = v0 + j;
+    const T* const s = sT + 4 * j * Bf + n;
+    const T* const c = reinterpret_cast<const T*>(a.crec) + (elem_of(v, a.S) * 4 + f) * CREC;
+    Vec<T, 2>* const out =
+        reinterpret_cast<Vec<T, 2>*>(reinterpret_cast<T*>(a.trace) + (v * 4 + f) * Shape<T, N>::FS + 6 * n);
+    const T x = s[0];
+    out[0] = {x * c[0], x * c[1]};
+    out[1] = {x * c[2], s[Bf]};
+    out[2] = {s[2 * Bf], s[3 * Bf]};
+  }
+}
+
 // Faces that need more than their traces (kSpec): a finer neighbour integrates
 // this element's Taylor expansion over its sub-steps, a fault's friction solve
 // evaluates it at its time points, and a gravitational surface's ODE (Sec. 4.3)
@@ -470,6 +509,29 @@ struct NoLevels {
   __device__ __forceinline__ void operator()(std::integral_constant<int, K>, const T*) const {}
 };
 
+// row -= this lane's row of the volume term sum_a A*_a K_a I
+template <class T, int N>
+__device__ __forceinline__ void volume_row(const RowStar<T>& st, const T* I, bool valid, T* row) {
+  using S = Shape<T, N>;
+  constexpr int VW = S::VW;
+  sp::each<S::B / VW>([&](auto cc) {
+    constexpr int m0 = decltype(cc)::value * VW;
+    T x[VW];
+    star_rows<VW>(st, x, [&](auto bc, auto kc) {
+      constexpr int b = decltype(bc)::value, m = m0 + decltype(kc)::value;
+      if constexpr (b == 0) return sp::dot<sp::KXt, m, S::B1>(T(0), I);
+      else if constexpr (b == 1) return sp::dot<sp::KYt, m, S::B1>(T(0), I);
+      else return sp::dot<sp::KZt, m, S::B1>(T(0), I);
+    });
+    if (valid) {
+      Vec<T, VW> q = *reinterpret_cast<const Vec<T, VW>*>(row + m0);
+#pragma unroll
+      for (int k = 0; k < VW; ++k) q.x[k] -= x[k];
+      *reinterpret_cast<Vec<T, VW>*>(row + m0) = q;
+    }
+  });
+}
+
 template <class T, int N, bool kSpec>
 __global__ void __launch_bounds__(kMaxThreads, sizeof(T) == 4 ? 2 : 1) local_row_kernel(StepArgs a, const __grid_constant__ Segs g) {
   using S = Shape<T, N>;
@@ -539,26 +601,96 @@ __global__ void __launch_bounds__(kMaxThreads, sizeof(T) == 4 ? 2 : 1) local_row
     faces_out<T, N, kSpec>(a, sg, u.v0, u.nE, 2, sT, sN, lane);
   }
 
-  // ---- volume: Q += sum_a A*_a K_a I (face terms follow in the neighbour kernel)
-  sp::each<B / VW>([&](auto cc) {
-    constexpr int m0 = decltype(cc)::value * VW;
-    T x[VW];
-    star_rows<VW>(st, x, [&](auto bc, auto kc) {
-      constexpr int b = decltype(bc)::value, m = m0 + decltype(kc)::value;
-      if constexpr (b == 0) return sp::dot<sp::KXt, m, S::B1>(T(0), I);
-      else if constexpr (b == 1) return sp::dot<sp::KYt, m, S::B1>(T(0), I);
-      else return sp::dot<sp::KZt, m, S::B1>(T(0), I);
-    });
-    if (valid) {
-      Vec<T, VW> q = *reinterpret_cast<const Vec<T, VW>*>(row + m0);
-#pragma unroll
-      for (int k = 0; k < VW; ++k) q.x[k] -= x[k];
-      *reinterpret_cast<Vec<T, VW>*>(row + m0) = q;
-    }
-  });
+  // ---- volume term (face terms follow in the neighbour kernel)
+  volume_row<T, N>(st, I, valid, row);
   __syncwarp();
   rows_out<T, N>(sQ, Q, u.nE, lane);
   if constexpr (kSpec) lev.surface(sg);
+}
+
+// Acoustic elements without any special face: four rows instead of nine, eight
+// elements per warp, otherwise as local_row_kernel.  What bounds it and where
+// the rows wait is the same; the work is 4 / 9.
+template <class T, int N>
+struct FluidSmem {
+  using S = Shape<T, N>;
+  static constexpr int nQ = (32 * S::SB + 3) / 4 * 4, warp = (nQ + 2 * 32 * S::Bf + 3) / 4 * 4;
+  static constexpr int bytes(int threads) { return warp * (int)sizeof(T) * (threads / 32); }
+  static_assert(bytes(kMaxThreads) <= 232448, "acoustic row kernel exceeds the shared memory of one block");
+};
+template <class T, int N>
+__global__ void __launch_bounds__(kMaxThreads, sizeof(T) == 4 ? 2 : 1) local_fluid_kernel(StepArgs a, const __grid_constant__ Segs g) {
+  using S = Shape<T, N>;
+  using M = FluidSmem<T, N>;
+  constexpr int B = S::B, Bf = S::Bf, VW = S::VW, C = B / VW;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int lane = threadIdx.x & 31;
+  T* const sQ = reinterpret_cast<T*>(smem_raw) + (threadIdx.x >> 5) * M::warp;
+  T* const sT = sQ + M::nQ;
+  const Unit u = unit_of<EWF>(g);
+  if (u.nE == 0) return;
+  T* const Q = reinterpret_cast<T*>(a.Q) + u.v0 * 9 * B;
+  for (int i = lane; i < 4 * u.nE * C; i += 32) {
+    const int r = i / C, c = (i - r * C) * VW;
+    *reinterpret_cast<Vec<T, VW>*>(sQ + r * S::SB + c) =
+        *reinterpret_cast<const Vec<T, VW>*>(Q + fluid_row(r) * B + c);
+  }
+  const bool valid = lane < 4 * u.nE;
+  RowStar<T> st;
+  st.setup_acoustic(lane, valid, reinterpret_cast<const T*>(a.par) + elem_of(u.v0 + (valid ? lane >> 2 : 0), a.S) * PAR);
+  T* const row = sQ + (valid ? lane : 0) * S::SB;
+  __syncwarp();
+  T I[B];
+#pragma unroll
+  for (int c = 0; c < C; ++c) {
+    const Vec<T, VW> x = *reinterpret_cast<const Vec<T, VW>*>(row + c * VW);
+#pragma unroll
+    for (int k = 0; k < VW; ++k) I[c * VW + k] = valid ? x.x[k] : T(0);
+  }
+  predict<T, N, 0>(I, I, st, g.s[u.seg], NoLevels{});
+  T* const s0 = sT + lane * Bf;
+  if (valid) {
+    sp::each<Bf>([&](auto rc) {
+      constexpr int r = decltype(rc)::value;
+      const T ev = sp::dot<sp::R0, r, B, 0>(T(0), I), od = sp::dot<sp::R0, r, B, 1>(T(0), I);
+      s0[r] = ev + od;
+      s0[32 * Bf + r] = ev - od;
+    });
+  }
+  __syncwarp();
+  fluid_face_out<T, N>(a, u.v0, u.nE, 0, sT, lane);
+  fluid_face_out<T, N>(a, u.v0, u.nE, 1, sT + 32 * Bf, lane);
+  __syncwarp();
+  if (valid) {
+    sp::each<Bf>([&](auto rc) {
+      constexpr int r = decltype(rc)::value;
+      s0[r] = sp::dot<sp::R2, r, B>(T(0), I);
+      s0[32 * Bf + r] = sp::dot<sp::R3, r, B>(T(0), I);
+    });
+  }
+  __syncwarp();
+  fluid_face_out<T, N>(a, u.v0, u.nE, 2, sT, lane);
+  fluid_face_out<T, N>(a, u.v0, u.nE, 3, sT + 32 * Bf, lane);
+  volume_row<T, N>(st, I, valid, row);
+  __syncwarp();
+  fluid_rows_out<T, N>(sQ, Q, u.nE, lane);
+}
+
+template <class T, int N>
+int launch_local_fluid_t(const StepArgs& a, const Segs& g, int threads, cudaStream_t st) {
+  using M = FluidSmem<T, N>;
+  const int rc = configure_on_device((const void*)local_fluid_kernel<T, N>, [] {
+    return cudaFuncSetAttribute(local_fluid_kernel<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                M::bytes(kMaxThreads));
+  });
+  if (rc) return rc;
+  const int64_t units = g.n ? g.first[g.n] : 0;
+  if (units <= 0) return 0;
+  threads = block_threads<T, N>(threads, units);
+  if (threads < 32 || threads > kMaxThreads || threads % 32) return (int)cudaErrorInvalidValue;
+  const int w = threads / 32;
+  local_fluid_kernel<T, N><<<(unsigned)((units + w - 1) / w), threads, M::bytes(threads), st>>>(a, g);
+  return (int)cudaGetLastError();
 }
 
 template <class T, int N>
@@ -574,6 +706,7 @@ int launch_local_row_t(const StepArgs& a, const Segs& g, int threads, bool spec,
   if (rc) return rc;
   const int64_t units = g.n ? g.first[g.n] : 0;
   if (units <= 0) return 0;
+  threads = block_threads<T, N>(threads, units);
   if (threads < 32 || threads > kMaxThreads || threads % 32) return (int)cudaErrorInvalidValue;
   if (spec && threads > 128) threads = 128;  // (shared memory)
   const int w = threads / 32;
@@ -583,6 +716,18 @@ int launch_local_row_t(const StepArgs& a, const Segs& g, int threads, bool spec,
   else
     local_row_kernel<T, N, false><<<blocks, threads, LocalSmem<T, N, false>::bytes(threads), st>>>(a, g);
   return (int)cudaGetLastError();
+}
+
+template <class T>
+int launch_local_fluid_n(int N, const StepArgs& a, const Segs& g, int th, cudaStream_t st) {
+  switch (N) {
+    case 1: return launch_local_fluid_t<T, 1>(a, g, th, st);
+    case 2: return launch_local_fluid_t<T, 2>(a, g, th, st);
+    case 3: return launch_local_fluid_t<T, 3>(a, g, th, st);
+    case 4: return launch_local_fluid_t<T, 4>(a, g, th, st);
+    case 5: return launch_local_fluid_t<T, 5>(a, g, th, st);
+  }
+  return (int)cudaErrorInvalidValue;
 }
 
 template <class T>

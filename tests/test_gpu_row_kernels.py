@@ -53,3 +53,27 @@ def test_noalloc_dofs_at_any_element_alignment(precision, N):
         assert float(buf[:off].abs().sum()) == 0 and float(buf[off + Q0.numel():].abs().sum()) == 0
     s.sync()
     assert np.array_equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("N,S,nxy", [(1, 1, 3), (2, 3, 3), (3, 1, 4), (4, 1, 2), (5, 2, 3)])
+def test_acoustic_rows(N, S, nxy, precision):
+    """The acoustic local kernel (eight elements per warp) on element counts that are no multiple of eight."""
+    from synthetic.workloads import coupled_box, random_dofs
+    m, mat = coupled_box(nxy=nxy, n_water=3, n_crust=1, L=6e3, depth=4e3, water=2e3, rigid_bottom=True)
+    o, s = make_pair(m, mat, N, precision=precision, ensemble=S, acoustic_ocean=True)
+    Q0 = random_dofs((S, m.nt, s.B, 9), 7, N=N)
+    fluid = mat[2] == 0
+    Q0[:, fluid, :, 0:3] = Q0[:, fluid, :, 0:3].mean(axis=-1, keepdims=True)
+    Q0[:, fluid, :, 3:6] = 0
+    s.set_dofs(np.ascontiguousarray(np.stack([to_gpu_layout(q) for q in Q0], axis=1)))
+    s.set_eta(np.zeros((int(s.info.n_gravity_faces), S, s.Bf)))
+    s.advance(2)
+    got = s.get_dofs().reshape(m.nt, S, 9, s.B)
+    assert np.array_equal(got[fluid][:, :, 0], got[fluid][:, :, 2]) and not got[fluid][:, :, 3:6].any()
+    for k in range(S):
+        o.Q, o._D, o.t = Q0[k].copy(), None, 0.0
+        o.eta[:] = 0
+        for _ in range(2):
+            o.advance_macro()
+        assert rel_l2(to_oracle_layout(got[:, k]), o.Q) <= TOL[precision]

@@ -338,6 +338,8 @@ __global__ void __launch_bounds__(LSmem<N, M, kSpec>::threads, 1)
       tc::mma3_ts<I_::nTO, I_::KO>(tbase + I_::cD + I_::nTE, tbase + I_::KE, tbase + I_::cL + I_::KE,
                                    sB + 4 * I_::oTO, sB + 4 * (I_::oTO + I_::sTO), false);
     });
+    [[maybe_unused]] float nrm[3];  // (acoustic; requested while the product runs)
+    if constexpr (M::fluid) row::fluid_normal(a, p.v0, p.nE, lane, nrm);
     mma.done();
     {
       float te[I_::nTE], to[I_::nTO];
@@ -377,7 +379,7 @@ __global__ void __launch_bounds__(LSmem<N, M, kSpec>::threads, 1)
         }
         __syncwarp();
         if constexpr (M::fluid)
-          row::fluid_face_out<float, N>(a, p.v0, p.nE, f0, sT, lane);
+          row::fluid_face_out<float, N>(a, p.v0, p.nE, f0, sT, nrm, lane);
         else
           row::faces_out<float, N, kBuf>(a, sg, p.v0, p.nE, f0, sT, sW + SM::oN, lane);
         __syncwarp();

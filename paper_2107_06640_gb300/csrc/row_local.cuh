@@ -296,17 +296,30 @@ __device__ __forceinline__ void fluid_rows_out(const T* sQ, T* Q, int nE, int la
     *reinterpret_cast<V*>(Q + gr * S::B + c) = *reinterpret_cast<const V*>(sQ + sr * S::SB + c);
   }
 }
-// face f of the warp's elements, staged (sigma, v) modes -> face blocks
+// the normal of face f of element j, in lane 4 j + f
+template <class T>
+__device__ __forceinline__ void fluid_normal(const StepArgs& a, int64_t v0, int nE, int lane, T (&n)[3]) {
+  const T* const c = reinterpret_cast<const T*>(a.crec) +
+                     (elem_of(v0 + (lane < 4 * nE ? lane >> 2 : 0), a.S) * 4 + (lane & 3)) * CREC;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) n[d] = c[d];
+}
+// Face f of the warp's elements, staged (sigma, v) modes -> face blocks; nrm: of
+// fluid_normal.  (Read from global memory here, each of the four faces waits for
+// its normals with every 32 modes: 40 % of the tensor-core kernel's time.)
 template <class T, int N>
-__device__ __forceinline__ void fluid_face_out(const StepArgs& a, int64_t v0, int nE, int f, const T* sT, int lane) {
+__device__ __forceinline__ void fluid_face_out(const StepArgs& a, int64_t v0, int nE, int f, const T* sT,
+                                               const T (&nrm)[3], int lane) {
   constexpr int Bf = Shape<T, N>::Bf;
 #pragma unroll(sizeof(T) == 4 ? 8 : 1)
   for (int it = 0; it < (EWF * Bf + 31) / 32; ++it) {
     const int i = lane + 32 * it, j = i / Bf, n = i - j * Bf;
+    T c[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) c[d] = __shfl_sync(0xffffffffu, nrm[d], (4 * j + f) & 31);
     if (i >= nE * Bf) continue;
     const int64_t v = v0 + j;
     const T* const s = sT + 4 * j * Bf + n;
-    const T* const c = reinterpret_cast<const T*>(a.crec) + (elem_of(v, a.S) * 4 + f) * CREC;
     Vec<T, 2>* const out =
         reinterpret_cast<Vec<T, 2>*>(reinterpret_cast<T*>(a.trace) + (v * 4 + f) * Shape<T, N>::FS + 6 * n);
     const T x = s[0];
@@ -648,6 +661,8 @@ __global__ void __launch_bounds__(kMaxThreads, sizeof(T) == 4 ? 2 : 1) local_flu
     for (int k = 0; k < VW; ++k) I[c * VW + k] = valid ? x.x[k] : T(0);
   }
   predict<T, N, 0>(I, I, st, g.s[u.seg], NoLevels{});
+  T nrm[3];
+  fluid_normal(a, u.v0, u.nE, lane, nrm);
   T* const s0 = sT + lane * Bf;
   if (valid) {
     sp::each<Bf>([&](auto rc) {
@@ -658,8 +673,8 @@ __global__ void __launch_bounds__(kMaxThreads, sizeof(T) == 4 ? 2 : 1) local_flu
     });
   }
   __syncwarp();
-  fluid_face_out<T, N>(a, u.v0, u.nE, 0, sT, lane);
-  fluid_face_out<T, N>(a, u.v0, u.nE, 1, sT + 32 * Bf, lane);
+  fluid_face_out<T, N>(a, u.v0, u.nE, 0, sT, nrm, lane);
+  fluid_face_out<T, N>(a, u.v0, u.nE, 1, sT + 32 * Bf, nrm, lane);
   __syncwarp();
   if (valid) {
     sp::each<Bf>([&](auto rc) {
@@ -669,8 +684,8 @@ __global__ void __launch_bounds__(kMaxThreads, sizeof(T) == 4 ? 2 : 1) local_flu
     });
   }
   __syncwarp();
-  fluid_face_out<T, N>(a, u.v0, u.nE, 2, sT, lane);
-  fluid_face_out<T, N>(a, u.v0, u.nE, 3, sT + 32 * Bf, lane);
+  fluid_face_out<T, N>(a, u.v0, u.nE, 2, sT, nrm, lane);
+  fluid_face_out<T, N>(a, u.v0, u.nE, 3, sT + 32 * Bf, nrm, lane);
   volume_row<T, N>(st, I, valid, row);
   __syncwarp();
   fluid_rows_out<T, N>(sQ, Q, u.nE, lane);

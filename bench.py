@@ -21,6 +21,7 @@ the host cores, one bounded sample of the workload per step.
 import argparse
 import json
 import os
+import re
 import subprocess
 import tempfile
 import sys
@@ -49,20 +50,18 @@ def flops_per_update(N):
     # kernel split: the local kernel projects the time integral onto the 4
     # faces; the neighbour kernel does both flux products and the lift
     local = pred + vol + 4 * 18 * Bf * B
-    # reference-matrix products the tensor-core local kernel runs as MMAs:
-    # predictor levels 0..N-3, the volume term and the face traces
+    # the dense reference-matrix products of predictor levels 0..N-3, the volume term and the face traces
     tensor = sum(54 * nb(N - k - 1) * nb(N - k) for k in range(N - 2)) + 54 * B * nb(N - 1) + 72 * Bf * B
     return {"pred": pred, "vol": vol, "loc": loc, "nb": nbf, "local_kernel": local,
             "neighbour_kernel": total - local, "total": total, "local_tensor": tensor}
 
 
 def bytes_per_update(N, w):
-    """Algorithmic HBM bytes per element update and kernel: the local kernel
-    reads and writes the dofs and writes 4 face traces; the neighbour kernel
-    reads the own and the neighbours' traces and reads and writes the dofs.
-    The tensor-core forms count what they move: face blocks padded to a
-    multiple of 4 floats, the element parameters, and (neighbour) the four
-    32-byte face records (normal, neighbour impedances, face code)."""
+    """HBM bytes per element update and kernel of the scheme with nodal faces
+    of all nine quantities (fixed counting convention): the local kernel reads
+    and writes the dofs and writes 4 face traces; the neighbour kernel reads
+    the own and the neighbours' traces and reads and writes the dofs.  What
+    the kernels move: modal_bytes_per_update."""
     B, Bf = (N + 1) * (N + 2) * (N + 3) // 6, (N + 1) * (N + 2) // 2
     FS = (9 * Bf + 3) // 4 * 4
     return {"local_kernel": (2 * 9 * B + 4 * 9 * Bf) * w, "neighbour_kernel": (2 * 9 * B + 8 * 9 * Bf) * w,
@@ -70,6 +69,45 @@ def bytes_per_update(N, w):
             # acoustic element: reads its 4 (p, v) rows, writes the three normal-stress rows and v
             "local_tc_kernel_acoustic": ((4 + 6) * B + 4 * FS + 16) * w,
             "neighbour_tc_kernel": (2 * 9 * B + 8 * FS + 16) * w + 4 * 32}
+
+
+def modal_bytes_per_update(N, w):
+    """Bytes per element update that the kernels cannot do without: dofs read
+    and written (an acoustic element: 4 rows read, 6 written), face blocks of
+    six quantities' modes padded to 4 values, element parameters, normals
+    (local) or flux coefficients and face codes (neighbour)."""
+    B, FS = (N + 1) * (N + 2) * (N + 3) // 6, (6 * (N + 1) * (N + 2) // 2 + 3) // 4 * 4
+    return {"local": (18 * B + 4 * FS + 32) * w, "local_acoustic": (10 * B + 4 * FS + 32) * w,
+            "neighbour": (18 * B + 8 * FS + 96) * w + 32}
+
+
+def sparse_ops():
+    """(row, column) of the nonzero operator entries that the kernels are compiled with."""
+    text = open(os.path.join(ROOT, "paper_2107_06640_gb300", "csrc", "sparse_ops.inc")).read()
+    return {name: [tuple(int(x) for x in t.split(",")[:2]) for t in re.findall(r"\{(.*?)\}", body)]
+            for name, body in re.findall(r"constexpr Entry k(\w+)\[\] = \{(.*?)\};", text, re.S)}
+
+
+def sparse_local_flops(N, rows=9):
+    """FP operations (an FMA is two) of the local row kernel per element of `rows` quantities: the sparse
+    operators, 9 FMAs of the star product per basis function and level, the time integral."""
+    nb = lambda n: (n + 1) * (n + 2) * (n + 3) // 6 if n >= 0 else 0
+    ops, Bf = sparse_ops(), (N + 1) * (N + 2) // 2
+    nnz = lambda name, r, c: sum(1 for x, y in ops[name] if x < r and y < c)
+    k = lambda n: sum(nnz(a, nb(n - 1), nb(n)) for a in ("KX", "KY", "KZ"))
+    fma = sum(k(N - l) + 10 * nb(N - l - 1) for l in range(N)) + nb(N)
+    fma += sum(nnz(a, Bf, nb(N)) for a in ("R0", "R2", "R3")) + Bf
+    return 2 * rows * (fma + k(N) + 9 * nb(N))
+
+
+def tc_local_flops(N):
+    """Useful flops of the tensor-core products per element of nine quantities: level 0, traces and
+    volume, each split by the parity of the basis functions' first index."""
+    par = lambda n, p: sum((n - i + 1) * (n - i + 2) // 2 for i in range(p, n + 1, 2))
+    fpar = lambda n, p: sum(n - i + 1 for i in range(p, n + 1, 2))
+    be, bo, me, mo, bf = par(N, 0), par(N, 1), par(N - 1, 0), par(N - 1, 1), (N + 1) * (N + 2) // 2
+    return 18 * (be * (2 * me + mo) + bo * (2 * mo + me) + be * (bf + 2 * fpar(N, 0)) + bo * (bf + 2 * fpar(N, 1)) +
+                 me * (2 * be + bo) + mo * (2 * bo + be))
 
 
 # DRAM bytes (read + write) per element of the tensor-core kernels (elastic and
@@ -651,7 +689,7 @@ def main():
 
     peaks, src = load_peaks()
     fl = flops_per_update(N_DEG)
-    by = bytes_per_update(N_DEG, 4)
+    by = modal_bytes_per_update(N_DEG, 4)
     kms = r32["kms"]
     # elements of one launch of the dominant kernel and that launch's own duration:
     # with the tensor-core form the tensor-core launches are timed alone (kms[3], kms[4])
@@ -669,27 +707,20 @@ def main():
     alu_peak, alu_src = alu_peak_tflops(False, peaks.get("sm_max_mhz", 2070.0), units, n_sm)
     achieved_flops = fl[kname.replace("_tc", "")] * n_k / (t_k[dom] * 1e-3) / 1e12
     # an acoustic element's reference-matrix products act on 4 of the 9 quantity rows
-    local_bytes = by["local_tc_kernel"] * (n_k - n_ac) + by["local_tc_kernel_acoustic"] * n_ac
-    launch_bytes = local_bytes if kname == "local_tc_kernel" else by[kname] * n_k
+    local_bytes = by["local"] * (n_k - n_ac) + by["local_acoustic"] * n_ac
+    launch_bytes = local_bytes if kname.startswith("local") else by["neighbour"] * n_k
     achieved_bytes = launch_bytes / (t_k[dom] * 1e-3) / 1e9
     frac_alu = achieved_flops / alu_peak
     frac_hbm = achieved_bytes / peaks["hbm_gbs"]
     tc_peak, tc_src = tf32x3_peak_tflops(peaks, units)
-    tensor_flops = fl["local_tensor"] * ((n_k - n_ac) + n_ac * 4.0 / 9.0)
+    tensor_flops = tc_local_flops(N_DEG) * ((n_k - n_ac) + n_ac * 4.0 / 9.0)
     achieved_tc = tensor_flops / (t_k[0] * 1e-3) / 1e12 if tc_form else None
-    if kname == "local_tc_kernel":
-        roof = {"bound": "tensor", "achieved": achieved_tc, "peak": tc_peak, "unit": "TFLOP/s",
-                "frac": achieved_tc / tc_peak, "traffic": None, "kernel": kname,
-                "peak_source": tc_src,
-                "flops_counted": "reference-matrix products only (predictor levels 0-2, volume, traces); "
-                                 "an acoustic element's count 4/9 of an elastic one's",
-                "elements": {"elastic": n_k - n_ac, "acoustic": n_ac}}
-    elif kname == "neighbour_tc_kernel":
-        # the lift runs on the tensor cores and the fluxes are ~27 kflop per update:
-        # HBM (traces, flux matrices, dofs) is the roof
+    if kname.endswith("_tc_kernel"):
+        # the products on the tensor cores take half as long at their peak as the bytes at theirs
         roof = {"bound": "hbm", "achieved": achieved_bytes, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                 "frac": frac_hbm, "traffic": None, "kernel": kname, "peak_source": src,
-                "bytes_counted": f"{by[kname]} B per update: own and neighbour face blocks, face records, dofs read+write"}
+                "bytes_counted": {"elastic": by["local"], "acoustic": by["local_acoustic"]} if dom == 0 else by["neighbour"],
+                "elements": {"elastic": n_k - n_ac, "acoustic": n_ac}}
     elif frac_alu >= frac_hbm:
         roof = {"bound": "alu", "achieved": achieved_flops, "peak": alu_peak, "unit": "TFLOP/s",
                 "frac": frac_alu, "traffic": None, "kernel": kname,
@@ -708,12 +739,15 @@ def main():
                  "kernel_ms": {"local": kms[0], "neighbour": kms[1]}})
     if tc_form:
         roof.update({"tc_kernel_ms": {"local_tc": kms[3], "neighbour_tc": kms[4]},
-                     "local_tc_tensor_frac": achieved_tc / tc_peak,
+                     "local_tc_tensor_frac": achieved_tc / tc_peak, "local_tc_tensor_peak": tc_peak,
+                     "local_tc_tensor_peak_source": tc_src,
                      "local_tc_hbm_frac": local_bytes / (kms[3] * 1e-3) / 1e9 / peaks["hbm_gbs"],
-                     "neighbour_tc_hbm_frac": by["neighbour_tc_kernel"] * n_k / (kms[4] * 1e-3) / 1e9
+                     "neighbour_tc_hbm_frac": by["neighbour"] * n_k / (kms[4] * 1e-3) / 1e9
                      / peaks["hbm_gbs"]})
     r64k = r64["kms"]
-    fp64_alu = fl["local_kernel"] * s.nt / (r64k[0] * 1e-3) / 1e12
+    # (the fluid's elements without a sea-surface face: four rows)
+    fp64_flops = sparse_local_flops(N_DEG) * (s.nt - n_ac) + sparse_local_flops(N_DEG, 4) * n_ac
+    fp64_alu = fp64_flops / (r64k[0] * 1e-3) / 1e12
     fp64_peak, fp64_src = alu_peak_tflops(True, r64["clocks"].get("sm_mhz") or 2070.0, units, n_sm)
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": r32["steps"],

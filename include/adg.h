@@ -50,8 +50,8 @@ extern "C" {
 
 #define ADG_FP64 0
 #define ADG_FP32 1
-/* FP32 dofs; at degrees 5 and 4 the reference-matrix products (predictor,
- * face traces, volume term, lift) of every element without a fault face or
+/* FP32 dofs; at degrees 5 and 4 the large reference-matrix products (first
+ * predictor level, face traces, volume term, lift) of every element without a fault face or
  * two or more gravitational faces run on the tensor cores (tcgen05) as 3xTF32
  * split products with FP32 accumulation (elements at LTS cluster borders and
  * with one gravitational face included), everything else as in ADG_FP32;
@@ -130,12 +130,13 @@ int adg_upload_material(adg_ctx* ctx, const double* rho, const double* lambda, c
  *    with no shear stress; the scheme keeps that form (the acoustic subspace
  *    is invariant), so the results equal those of the 9-quantity system on
  *    such data;
- *  - with the tensor-core kernels (ADG_3XTF32, degree 5 or 4), the fluid elements
- *    without gravitational face, fault face or LTS neighbour in another
- *    cluster take a 4-quantity (p, v) local kernel (the others the 9-quantity
- *    ones): 32 elements per 128-row
- *    tile, the acoustic star product, 4 of the 9 dofs rows read; their face
- *    traces are written in the usual 9-quantity layout.
+ *  - the fluid elements without gravitational face, fault face or LTS
+ *    neighbour in another cluster take a 4-quantity (p, v) local kernel (the
+ *    others the 9-quantity ones): 32 elements per 128-row tile on the tensor
+ *    cores, eight per warp otherwise, the acoustic star product, 4 of the 9
+ *    dofs rows read; face traces as of every element.  (Contexts that
+ *    adg_step_noalloc accepts, without tensor-core kernels, keep the
+ *    9-quantity kernel.)
  * Without it the fluid carries whatever stress the caller uploads (a
  * deviatoric part stays constant in a fluid but drives velocities). */
 int adg_set_acoustic_ocean(adg_ctx* ctx, int enable);
@@ -278,7 +279,7 @@ int adg_sync(adg_ctx* ctx);
  * kernel kind of a cluster on the library stream.  ms[k] = mean duration of
  * one such phase of kind k, launches[k] = number of kernel launches (arrays
  * of 5), k = 0 local (predictor, volume, traces; with ADG_3XTF32 at degree 5
- * or 4 tensor-core and CUDA-core launches), 1 neighbour flux,
+ * or 4 tensor-core and other launches, one after the other), 1 neighbour flux,
  * 2 fault friction solve, 3 and 4 the tensor-core launch of the local and
  * of the neighbour phase alone (0 without one).  Advances the simulation
  * like adg_advance. */
@@ -301,7 +302,7 @@ int adg_profile(adg_ctx* ctx, int n_macro, double* ms, int64_t* launches);
  *    stream, as in any CUDA call, so work the caller enqueued on it (torch's
  *    default stream, handle 0) is ordered before these kernels.  The call
  *    only enqueues work (no synchronisation).
- *  - Arithmetic: the CUDA-core kernels in the context's precision.  In an
+ *  - Arithmetic: the row kernels (CUDA cores) in the context's precision.  In an
  *    ADG_3XTF32 context those are the FP32 kernels of ADG_FP32 (the
  *    tensor-core kernels stage through shared memory the library allocates
  *    with the context), so the result is the ADG_FP32 one: within 2e-5
@@ -326,9 +327,8 @@ int adg_step_noalloc(adg_ctx* ctx, void* d_Q, int n_steps, void* stream);
  * events as in adg_profile, after one untimed macro step):
  *   choice[0] / [1]: threads per block of the CUDA-core local /
  *                    neighbour kernels, of {64, 128, 256};
- *   choice[2] / [3]: consecutive 12-element tiles one CTA slot of the
- *                    tensor-core local / neighbour kernel takes per sweep
- *                    (elements per CTA before it strides on), of {1, 2, 4};
+ *   choice[2] / [3]: consecutive tiles that one CTA slot of the tensor-core
+ *                    local / neighbour kernel takes at a time, of {1, 2, 4};
  *   0 for a kernel kind this context does not launch.
  * ms (optional, [4][3]): mean milliseconds per macro step of that kernel kind
  * for each candidate (-1 where not timed).  reps >= 1 timed macro steps per

@@ -499,15 +499,13 @@ void Ctx::setup() {
   const std::vector<int>&nface_u = pl.nface, &nperm_u = pl.nperm, &cl = pl.cl;
   dtmin = pl.dtmin;
   ncl = pl.ncl;
-  // ---- internal order: by cluster, stable; with the tensor-core kernels,
-  // the elements of a cluster without gravitational face, fault face or
-  // finer neighbour come first (those with a coarser neighbour, which the
-  // tensor-core kernels handle at some extra cost, at the end of that range,
-  // so that they fill few tiles)
+  // ---- internal order: by cluster, then by kernel kind, stable: plain elements
+  // first (acoustic ones apart), those that a kernel handles at some extra cost
+  // at the end, so that they fill few tiles and warps
   // (special: 1 a coarser neighbour, 3 one gravitational face or a finer
   // neighbour (both on the tensor-core kernels, 3 on their special local
-  // instantiation), 2 the CUDA-core kernels: a fault face or more than one
-  // gravitational face)
+  // instantiation), 2 the row kernels: a fault face or more than one
+  // gravitational face; without the tensor-core kernels any of these)
   std::vector<char> special(E, 0);
   for (int64_t e = 0; e < E; ++e) {
     int ng_e = 0;
@@ -529,10 +527,17 @@ void Ctx::setup() {
   // acoustic local kernel, 2 with a coarser neighbour, 3 with a gravitational
   // face or a finer neighbour (with the tensor-core kernels all four on them),
   // 4 the rest
+  // (contexts that adg_step_noalloc takes keep the caller's order, which its dofs are in)
+  bool sort_fluid = acoustic;
+  if (!tc && ncl == 1 && S == 1) {
+    sort_fluid = false;
+    for (int64_t i = 0; i < 4 * E; ++i)
+      sort_fluid = sort_fluid || (acoustic && (tag[i] == ADG_TAG_GRAVITY || tag[i] == ADG_TAG_FAULT));
+  }
   std::vector<char> key(E, 0);
   for (int64_t e = 0; e < E; ++e)
     key[e] = special[e] == 1 ? 2 : special[e] == 3 ? 3 : special[e] == 2 ? 4
-                                 : (char)(acoustic && mu[e] == 0.0 ? 1 : 0);
+                                 : (char)(sort_fluid && mu[e] == 0.0 ? 1 : 0);
   order.resize(E);
   for (int64_t e = 0; e < E; ++e) order[e] = e;
   std::stable_sort(order.begin(), order.end(), [&](int64_t a, int64_t b) {
@@ -794,8 +799,8 @@ static void taylor_int(int N, double ta, double tb, double* out) {
 // tick, then the friction solves and the neighbour phase of every cluster
 // that ends one.  Each phase is one launch per kernel kind covering all its
 // clusters (a segment per cluster with that cluster's step and coefficients):
-// the tensor-core kernels take the plain elements, the CUDA-core kernels the
-// rest (all elements without the tensor-core form).
+// the tensor-core kernels take what they can, the row kernels the rest (all
+// elements without the tensor-core form).
 void Ctx::launch_tick(int s, double dtm) {
   StepArgs a = base_args();
   for (int phase = 0; phase < 2; ++phase) {

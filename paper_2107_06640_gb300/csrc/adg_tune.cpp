@@ -1,10 +1,10 @@
 // Autotuner of the launch shapes (adg_autotune).  The work of a step is fixed
 // by the scheme; how it is cut into launches is a choice per kernel kind:
-//   knob 0 / 1: threads per block of the CUDA-core local / neighbour
-//               kernels (64, 128, 256);
-//   knob 2 / 3: consecutive 12-element tiles a CTA slot of the tensor-core
-//               local / neighbour kernel takes per sweep (1, 2, 4), i.e. the
-//               elements one CTA works through before striding on.
+//   knob 0 / 1: threads per block of the local / neighbour row kernels (64,
+//               128, 256; untuned: row::block_threads);
+//   knob 2 / 3: consecutive tiles a CTA slot of the tensor-core local /
+//               neighbour kernel takes from the launch's tile counter at a
+//               time (1, 2, 4).
 // Each candidate is timed with CUDA events on this context's own clusters
 // (whole macro steps of adg_profile's per-phase events, after one untimed
 // macro step), one knob after the other; the fastest is kept.  The solver
@@ -125,7 +125,7 @@ void Ctx::autotune(int reps, bool force, int* choice, double* ms) {
         for (auto& e : evs) {
           float x = 0.f;
           if (e.kind == phase) {
-            // the tensor-core launch is timed alone (a -> m); the CUDA-core one after it (m -> b)
+            // the tensor-core launch is timed alone (a -> m); the row kernels' after it (m -> b)
             if (tc_knob && e.m) ck(cudaEventElapsedTime(&x, e.a, e.m), "autotune: events");
             if (!tc_knob && e.launches > (e.m ? 1 : 0)) ck(cudaEventElapsedTime(&x, e.m ? e.m : e.a, e.b), "autotune: events");
           }

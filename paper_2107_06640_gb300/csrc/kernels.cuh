@@ -87,7 +87,7 @@ constexpr int CREC = 24;
 // The clusters of one LTS phase (Sec. 4.4) in a single launch: segment i
 // covers the virtual elements [v_begin, v_begin + n) of one cluster with that
 // cluster's time coefficients, and the launch's work units (tiles of the
-// tensor-core kernels, blocks of the CUDA-core kernels) [first[i], first[i+1]).
+// tensor-core kernels, warps of the row kernels) [first[i], first[i+1]).
 // The launch takes the table by value (kernel parameter space), so a CUDA
 // graph keeps it and no device buffer is involved.
 constexpr int kMaxSeg = 16;
@@ -128,8 +128,8 @@ __host__ __device__ inline int seg_find(const Segs& g, int64_t u) {
 Segs make_segs(const Seg* s, int n, int unit, int chunk = 1);
 
 // tensor-core (tcgen05, 3xTF32) local kernel, degree 5 or 4, FP32 dofs
-// (local_tc.cuh; one translation unit per degree), for elements without
-// gravitational faces, fault faces or finer LTS neighbours
+// (local_tc.cuh; one translation unit per degree), for elements without fault
+// faces or two or more gravitational faces
 // buffers: the launch's elements include some with an LTS buffer (a coarser neighbour)
 // acoustic: the launch's elements are fluid (mu = 0) without LTS buffer, on the
 // 4-quantity (p, v) instantiation; their stress must be isotropic (-p I)

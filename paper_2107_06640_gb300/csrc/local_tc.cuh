@@ -37,8 +37,10 @@
 // per SM, 0.39 instructions per clock and scheduler), not a roof: 0.23 of the
 // HBM bandwidth, tensor pipe active 18 % of the time.  Local phase of the
 // 183,456-tet degree-5 coupled box (all kinds): 788 us with 256 threads per
-// tile, five dense MMA rounds and nodal nine-quantity faces, 618 us now; plain
-// elastic launch of its 93,600-tet version 392 -> 274 us.  Degree 4: 593 -> 468 us.
+// tile, five dense MMA rounds and nodal nine-quantity faces, 594 us now; plain
+// elastic launch of its 93,600-tet version 392 -> 266 us.  Degree 4: 593 -> 435 us;
+// 81,600 acoustic tets at degree 4: 101 us (161 with the faces' normals read from
+// global memory where they are used), 0.29 of the HBM bandwidth.
 #pragma once
 #include <cuda_runtime.h>
 

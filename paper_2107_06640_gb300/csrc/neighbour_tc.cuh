@@ -14,7 +14,7 @@
 // registers suffice for four tiles.  (Faces 0 and 1 through their sum and
 // difference and the parities of faces 2 and 3 apart take half the tensor
 // work, but hold two more rows: three tiles of 168 registers, 483 us on the
-// 183,456-tet degree-5 box where this form takes 398; the nodal kernel before,
+// 183,456-tet degree-5 box where this form takes 378; the nodal kernel before,
 // nine quantities staged and two tiles in flight, took 652.)
 //
 // What bounds it: shared-memory traffic (76 % of the L1 data pipe busy) and

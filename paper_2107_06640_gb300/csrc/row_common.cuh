@@ -1,9 +1,11 @@
 // What the two row kernels (row_local.cuh, row_neighbour.cuh) share.
 //
 // They are the CUDA-core form of the element update, in both precisions and at
-// every degree (in a tensor-core context for its fault elements): one warp works on three (virtual) elements, lane 9 j + p holds
-// the row of quantity p of element j in registers (lanes 27..31 idle), the
-// operators are straight-line sparse code (sparse_ops.cuh), the quantities of
+// every degree (in a tensor-core context for its fault elements): one warp works
+// on three (virtual) elements, lane 9 j + p holds
+// the row of quantity p of element j in registers (lanes 27..31 idle; plain
+// acoustic elements in the local phase: eight elements, lane 4 j + p, all lanes
+// busy), the operators are straight-line sparse code (sparse_ops.cuh), the quantities of
 // an element meet in warp shuffles, and no block barrier is needed.
 //
 // Face data are modal: a face block holds traction sigma n (n the owner's
@@ -17,11 +19,12 @@
 //
 // What bounds them: FP64, the 2 FMA per clock and SM (the sparse form has 3.4
 // to 4 times fewer of them than dense nodal products, and no lane waits on an
-// operand); FP32, instruction issue.  Against one block per element with dense
+// operand; 87 % of the FP64 pipe busy at degree 5); FP32, instruction issue and
+// the latency of the copies (50 % of issue slots at degree 3).  Against one block per element with dense
 // operands in global memory and block barriers between the levels: degree 3
-// FP64, 3,072 tets, 366 -> 130 us per step; degree 5 FP64, 33,696 tets, 17.2 ->
-// 5.9 ms; degree 3 FP32, 13,182 tets, 130 -> 35 us; 102,258 tets, 1.13 -> 0.33
-// ms (steps as a caller sees them, transfers included).
+// FP64, 3,072 tets, 366 -> 110 us per step; degree 5 FP64, 33,696 tets, 17.0 ->
+// 4.4 ms; degree 3 FP32, 13,182 tets, 130 -> 30 us; 102,258 tets, 1.13 -> 0.22
+// ms.
 #pragma once
 #include <cuda_runtime.h>
 

@@ -77,3 +77,30 @@ def test_acoustic_rows(N, S, nxy, precision):
         for _ in range(2):
             o.advance_macro()
         assert rel_l2(to_oracle_layout(got[:, k]), o.Q) <= TOL[precision]
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_noalloc_on_an_acoustic_context_without_gravity(precision):
+    """Its dofs are in the caller's order, also where fluid and solid elements alternate."""
+    import torch
+    from paper_2107_06640_gb300 import _lib
+    from synthetic.workloads import coupled_box, random_dofs
+    m, mat = coupled_box(nxy=2, n_water=1, n_crust=2, L=6e3, depth=4e3, water=2e3)
+    m.face_tag[m.face_tag == 2] = 1  # no gravitational surface
+    mat = [x.copy() for x in mat]
+    for x, solid in zip(mat, (2700.0, 3e10, 3e10)):  # a solid tet between fluid ones
+        x[-2] = solid
+    N = 3
+    o, s = make_pair(m, mat, N, precision=precision, acoustic_ocean=True)
+    assert s.info.n_gravity_faces == 0
+    Q0 = random_dofs((m.nt, s.B, 9), 17, N=N)
+    fluid = mat[2] == 0
+    Q0[fluid, :, 0:3] = Q0[fluid, :, 0:3].mean(axis=-1, keepdims=True)
+    Q0[fluid, :, 3:6] = 0
+    o.Q, o._D, o.t = Q0.copy(), None, 0.0
+    d = torch.from_numpy(to_gpu_layout(Q0).copy()).to("cuda", torch.float64 if precision == 0 else torch.float32)
+    _lib.adg_step_noalloc(s.ctx, d.data_ptr(), 2, torch.cuda.current_stream().cuda_stream)
+    s.sync()
+    for _ in range(2):
+        o.advance_macro()
+    assert rel_l2(to_oracle_layout(d.cpu().numpy().reshape(m.nt, 9, s.B)), o.Q) <= TOL[precision]

@@ -210,6 +210,7 @@ struct Ctx {
   void run_macro(double scale);
   int64_t launches_per_macro() const;
   std::vector<int64_t> state_places() const;
+  int64_t row_plain(int c) const;
   void autotune(int reps, bool force, int* choice, double* ms);
   void check_err();
   ~Ctx();

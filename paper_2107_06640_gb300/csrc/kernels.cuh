@@ -78,6 +78,7 @@ __host__ __device__ inline int64_t elem_of(int64_t v, int S) {
 // Virtual elements per warp of the row kernels
 constexpr int kRowElems = 3;
 constexpr int kRowElemsFluid = 8;  // of its acoustic form
+constexpr int64_t kSmallLaunch = 8 * 152;  // warps of a row launch, eight per SM
 // Face coefficients: outward normal n[3]; the middle
 // state's tangential coefficients of the own and of the neighbour's side (t^b
 // from t and v, v^b from t and v) and what the normal components add to them

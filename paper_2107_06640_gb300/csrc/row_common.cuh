@@ -109,7 +109,7 @@ __device__ __forceinline__ void rows_out(const T* sQ, T* Q, int nE, int lane) {
 template <class T, int N>
 inline int block_threads(int threads, int64_t units) {
   if (threads) return threads;
-  if (units <= 8 * 152) return 32;
+  if (units <= kSmallLaunch) return 32;
   return sizeof(T) == 4 && N >= 4 ? 256 : 128;
 }
 

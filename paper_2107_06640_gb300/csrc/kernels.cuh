@@ -125,6 +125,23 @@ __host__ __device__ inline int seg_find(const Segs& g, int64_t u) {
   while (i + 1 < g.n && u >= g.first[i + 1]) ++i;
   return i;
 }
+// The part of tile `tl` (TE virtual elements) that warp `w` of a slot works on, EW
+// elements each: first virtual element, elements, segment.  Warps past a segment's
+// end have nE = 0 and a v0 that is no element of the launch: nothing may be read there.
+struct TilePart {
+  int64_t v0;
+  int nE, seg;
+};
+template <int TE, int EW>
+__host__ __device__ inline TilePart tile_part(const Segs& g, int64_t tl, int w) {
+  const int i = seg_find(g, tl);
+  const int64_t o = (tl - g.first[i]) * TE + EW * w, left = g.s[i].n - o;
+  return {g.s[i].v_begin + o, (int)(left < 0 ? 0 : left < EW ? left : EW), i};
+}
+// Face 4 element + f that lane 4 j + f of a warp with elements v0 .. v0 + nE - 1 stands for; -1: none
+__host__ __device__ inline int64_t lane_face(int64_t v0, int nE, int lane, int S) {
+  return lane < 4 * nE ? elem_of(v0 + (lane >> 2), S) * 4 + (lane & 3) : -1;
+}
 // Segs of the given segments with `unit` virtual elements per work unit
 Segs make_segs(const Seg* s, int n, int unit, int chunk = 1);
 

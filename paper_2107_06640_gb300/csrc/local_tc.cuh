@@ -177,15 +177,8 @@ __global__ void __launch_bounds__(LSmem<N, M, kSpec>::threads, 1)
   // this warp's part of tile tl: first virtual element, elements (may be 0), segment
   const int64_t ntiles = g.first[g.n];
   const int slots = (int)gridDim.x * kSlots, me = slot * (int)gridDim.x + (int)blockIdx.x;
-  struct Part {
-    int64_t v0;
-    int nE, seg;
-  };
-  auto part_of = [&](int64_t tl) {
-    const int i = seg_find(g, tl);
-    const int64_t o = (tl - g.first[i]) * M::TE + M::EW * w, left = g.s[i].n - o;
-    return Part{g.s[i].v_begin + o, (int)(left < 0 ? 0 : left < M::EW ? left : M::EW), i};
-  };
+  using Part = TilePart;
+  auto part_of = [&](int64_t tl) { return tile_part<M::TE, M::EW>(g, tl, w); };
   float* const sW = sm + I_::floats + (slot * 4 + w) * SM::warp;
   float* const Qg = reinterpret_cast<float*>(a.Q);
   const tc::TileFeed feed{a.tiles, s_next[slot], slots, g.chunk, ntiles};

@@ -122,15 +122,8 @@ __global__ void __launch_bounds__(kThreadsN, 1) neighbour_tc_kernel(StepArgs a, 
   const float* const trace = reinterpret_cast<const float*>(a.trace);
   auto elem = [&](int64_t vv) -> int64_t { return kOne ? vv : elem_of(vv, a.S); };
   // this warp's part of tile tl: first virtual element, elements (<= 3, may be 0), segment
-  struct Part {
-    int64_t v0;
-    int nE, seg;
-  };
-  auto part_of = [&](int64_t tl) {
-    const int i = seg_find(g, tl);
-    const int64_t o = (tl - g.first[i]) * TE + 3 * w, left = g.s[i].n - o;
-    return Part{g.s[i].v_begin + o, (int)(left < 0 ? 0 : left < 3 ? left : 3), i};
-  };
+  using Part = TilePart;
+  auto part_of = [&](int64_t tl) { return tile_part<TE, 3>(g, tl, w); };
   // lane 4 j + f (< 12): face f of the part's element j
   auto faces_of = [&](const Part& p, int& info, int& nbr) {
     info = 0;

@@ -296,13 +296,16 @@ __device__ __forceinline__ void fluid_rows_out(const T* sQ, T* Q, int nE, int la
     *reinterpret_cast<V*>(Q + gr * S::B + c) = *reinterpret_cast<const V*>(sQ + sr * S::SB + c);
   }
 }
-// the normal of face f of element j, in lane 4 j + f
+// the normal of face f of element j, in lane 4 j + f (nE may be 0: nothing is read)
 template <class T>
 __device__ __forceinline__ void fluid_normal(const StepArgs& a, int64_t v0, int nE, int lane, T (&n)[3]) {
-  const T* const c = reinterpret_cast<const T*>(a.crec) +
-                     (elem_of(v0 + (lane < 4 * nE ? lane >> 2 : 0), a.S) * 4 + (lane & 3)) * CREC;
+  const int64_t face = lane_face(v0, nE, lane, a.S);
+  n[0] = n[1] = n[2] = T(0);
+  if (face >= 0) {
+    const T* const c = reinterpret_cast<const T*>(a.crec) + face * CREC;
 #pragma unroll
-  for (int d = 0; d < 3; ++d) n[d] = c[d];
+    for (int d = 0; d < 3; ++d) n[d] = c[d];
+  }
 }
 // Face f of the warp's elements, staged (sigma, v) modes -> face blocks; nrm: of
 // fluid_normal.  (Read from global memory here, each of the four faces waits for

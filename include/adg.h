@@ -296,8 +296,9 @@ int adg_profile(adg_ctx* ctx, int n_macro, double* ms, int64_t* launches);
  *    gravitational or fault faces (else ADG_E_INVALID); its tables are read,
  *    its own dofs are not touched.
  *  - d_Q: DEVICE pointer to the caller's dofs in the context's precision,
- *    layout [tet][9][B] in user tet order (for such contexts the internal
- *    order is the user order), updated in place.  Owned by the caller.
+ *    layout [tet][9][B] in user tet order, updated in place.  Owned by the
+ *    caller.  (Where the library works in another order, in acoustic
+ *    ADG_3XTF32 contexts, the call has element tables in the user order.)
  *  - stream: cudaStream_t to launch on; NULL is CUDA's default (legacy)
  *    stream, as in any CUDA call, so work the caller enqueued on it (torch's
  *    default stream, handle 0) is ordered before these kernels.  The call

@@ -527,7 +527,8 @@ void Ctx::setup() {
   // acoustic local kernel, 2 with a coarser neighbour, 3 with a gravitational
   // face or a finer neighbour (with the tensor-core kernels all four on them),
   // 4 the rest
-  // (contexts that adg_step_noalloc takes keep the caller's order, which its dofs are in)
+  // (contexts without the tensor-core kernels that adg_step_noalloc takes keep the
+  // caller's order, which its dofs are in; those with them get tables in that order)
   bool sort_fluid = acoustic;
   if (!tc && ncl == 1 && S == 1) {
     sort_fluid = false;
@@ -715,6 +716,23 @@ void Ctx::setup() {
     dModal = upload_vec<float>(rt.modalT, owned, dev_bytes);
     dReorient = upload_vec<float>(rt.reorient, owned, dev_bytes);
   }
+  if (takes_noalloc() && noalloc_scratch() <= kNoallocScratch && !std::is_sorted(order.begin(), order.end())) {
+    std::vector<double> par_u(par.size()), crec_u(crec.size());
+    std::vector<int> nbr_u2(nbr.size()), ninfo_u(ninfo.size());
+    for (int64_t i = 0; i < E; ++i) {
+      const int64_t eu = order[i];
+      std::copy_n(&par[i * PAR], PAR, &par_u[eu * PAR]);
+      std::copy_n(&crec[i * 4 * CREC], 4 * CREC, &crec_u[eu * 4 * CREC]);
+      for (int f = 0; f < 4; ++f) {
+        nbr_u2[eu * 4 + f] = nbr[i * 4 + f] < 0 ? -1 : (int)order[nbr[i * 4 + f]];
+        ninfo_u[eu * 4 + f] = ninfo[i * 4 + f];
+      }
+    }
+    dParUser = fp64 ? upload_vec<double>(par_u, owned, dev_bytes) : upload_vec<float>(par_u, owned, dev_bytes);
+    dCrecUser = fp64 ? upload_vec<double>(crec_u, owned, dev_bytes) : upload_vec<float>(crec_u, owned, dev_bytes);
+    dNbrUser = upload_raw<int>(nbr_u2, owned, dev_bytes);
+    dNinfoUser = upload_raw<int>(ninfo_u, owned, dev_bytes);
+  }
   dNbr = upload_raw<int>(nbr, owned, dev_bytes);
   dNinfo = upload_raw<int>(ninfo, owned, dev_bytes);
   dGslot = ng ? upload_raw<int>(gslot, owned, dev_bytes) : nullptr;
@@ -770,6 +788,9 @@ void Ctx::setup() {
   time = 0.0;
   inited = true;
 }
+
+bool Ctx::takes_noalloc() const { return ncl == 1 && S == 1 && gfaces.empty() && n_fault_faces == 0; }
+size_t Ctx::noalloc_scratch() const { return (size_t)nt * 4 * face_stride(N) * (fp64 ? 8 : 4); }
 
 StepArgs Ctx::base_args() const {
   StepArgs a{};

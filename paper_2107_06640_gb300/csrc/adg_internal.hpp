@@ -49,6 +49,9 @@ struct RowTables {
 };
 RowTables make_row_tables(const RefOps& o);
 
+// adg_step_noalloc: 32 MiB of face traces in static device memory
+constexpr size_t kNoallocScratch = (size_t)32 << 20;
+
 // Host-side plan of a mesh (caller's element order): geometry, face
 // connectivity, CFL time steps and rate-2 clusters (Sec. 4.4)
 struct MeshPlan {
@@ -121,6 +124,10 @@ struct Ctx {
   int64_t* dOrder = nullptr;  // order on the device: the caller's element of library element i
   double *dBtrace = nullptr, *dEta = nullptr, *dGpar = nullptr;
   void* dPar = nullptr;
+  // adg_step_noalloc, whose dofs are in the caller's order: the element tables
+  // in that order, where the library's differs (else null)
+  void *dParUser = nullptr, *dCrecUser = nullptr;
+  int *dNbrUser = nullptr, *dNinfoUser = nullptr;
   void *dCrec = nullptr, *dNodal = nullptr, *dModal = nullptr, *dReorient = nullptr;
   int *dNbr = nullptr, *dNinfo = nullptr, *dGslot = nullptr, *dBslot = nullptr, *dDslot = nullptr,
       *dPerm = nullptr;
@@ -205,6 +212,8 @@ struct Ctx {
   void face_neighbour(const MeshPlan& pl, const RefOps& o, int64_t eu, int f, int64_t* nb, int* nf,
                       int32_t* node_map) const;
   void setup();
+  bool takes_noalloc() const;  // contexts that adg_step_noalloc accepts
+  size_t noalloc_scratch() const;  // bytes of face traces it needs
   StepArgs base_args() const;
   void launch_tick(int s, double dtm);
   void run_macro(double scale);

@@ -26,7 +26,7 @@
 
 namespace {
 
-constexpr size_t kScratchBytes = (size_t)32 << 20;  // 32 MiB of face traces
+constexpr size_t kScratchBytes = adg::kNoallocScratch;
 static __device__ __align__(256) unsigned char g_trace_scratch[kScratchBytes];
 
 constexpr int kMaxDevices = 64;
@@ -42,12 +42,12 @@ extern "C" int adg_step_noalloc(adg_ctx* ctx, void* d_Q, int n_steps, void* stre
     c.last_error = "call adg_init first";
     return ADG_E_STATE;
   }
-  if (c.ncl != 1 || c.S != 1 || !c.gfaces.empty() || c.n_fault_faces) {
+  if (!c.takes_noalloc()) {
     c.last_error = "adg_step_noalloc needs a global-time-stepping context (one cluster), ensemble 1, "
                    "and no gravitational or fault faces";
     return ADG_E_INVALID;
   }
-  const size_t need = (size_t)c.nt * 4 * adg::face_stride(c.N) * (c.fp64 ? 8 : 4);
+  const size_t need = c.noalloc_scratch();
   if (need > kScratchBytes) {
     c.last_error = "adg_step_noalloc: the face traces of this mesh need " + std::to_string(need) +
                    " bytes of scratch; the fixed maximum is " + std::to_string(kScratchBytes) + " bytes";
@@ -80,6 +80,12 @@ extern "C" int adg_step_noalloc(adg_ctx* ctx, void* d_Q, int n_steps, void* stre
   adg::StepArgs a = c.base_args();
   a.Q = d_Q;
   a.trace = scratch;
+  if (c.dNbrUser) {  // the library's order is not the caller's
+    a.par = c.dParUser;
+    a.crec = c.dCrecUser;
+    a.nbr = c.dNbrUser;
+    a.ninfo = c.dNinfoUser;
+  }
   adg::Seg sg{};  // the whole mesh, one global step of dt_min
   sg.v_begin = 0;
   sg.n = c.nt;

@@ -104,3 +104,32 @@ def test_noalloc_on_an_acoustic_context_without_gravity(precision):
     for _ in range(2):
         o.advance_macro()
     assert rel_l2(to_oracle_layout(d.cpu().numpy().reshape(m.nt, 9, s.B)), o.Q) <= TOL[precision]
+
+
+@pytest.mark.parametrize("N", [4, 5])
+def test_noalloc_on_an_acoustic_tensor_core_context(N):
+    """There the library sorts the fluid elements behind the solid ones; the caller's dofs keep the caller's order."""
+    import torch
+    from paper_2107_06640_gb300 import _lib
+    from synthetic.workloads import coupled_box, random_dofs
+    m, mat = coupled_box(nxy=2, n_water=1, n_crust=2, L=6e3, depth=4e3, water=2e3)
+    m.face_tag[m.face_tag == 2] = 1  # no gravitational surface
+    mat = [x.copy() for x in mat]
+    for x, water, rock in zip(mat, (1000.0, 2.25e9, 0.0), (2700.0, 3e10, 3e10)):
+        x[:] = np.where(np.arange(m.nt) % 3 == 1, rock, water)  # fluid and solid tets alternate
+    o, s = make_pair(m, mat, N, precision=2, acoustic_ocean=True)
+    fluid = mat[2] == 0
+    assert s.info.n_gravity_faces == 0 and s.info.acoustic_updates_per_macro == fluid.sum()
+    Q0 = random_dofs((m.nt, s.B, 9), 17, N=N)
+    Q0[fluid, :, 0:3] = Q0[fluid, :, 0:3].mean(axis=-1, keepdims=True)
+    Q0[fluid, :, 3:6] = 0
+    o.Q, o._D, o.t = Q0.copy(), None, 0.0
+    s.set_dofs(to_gpu_layout(Q0))
+    d = torch.from_numpy(to_gpu_layout(Q0).copy()).to("cuda", torch.float32)
+    _lib.adg_step_noalloc(s.ctx, d.data_ptr(), 2, torch.cuda.current_stream().cuda_stream)
+    s.sync()
+    s.advance(2)
+    for _ in range(2):
+        o.advance_macro()
+    for got in (d.cpu().numpy().reshape(m.nt, 9, s.B), s.get_dofs()):
+        assert rel_l2(to_oracle_layout(got), o.Q) <= TOL[1]

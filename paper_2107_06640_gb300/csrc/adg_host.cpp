@@ -205,8 +205,10 @@ void face_coefficients(const double n[3], int tag, double Zp, double Zs, double 
     const double s = nb ? (k % 2 ? 1.0 : -1.0) : 0.0;  // the neighbour's traction has the opposite normal
     c[3 + k] = at[k];
     c[7 + k] = s * bt[k];
-    c[11 + k] = an[k] - at[k];
-    c[15 + k] = s * (bn[k] - bt[k]);
+    // (traction: what the normal part adds to the tangential coefficients' product;
+    // velocity: the normal state itself, see row_flux.cuh)
+    c[11 + k] = k < 2 ? an[k] - at[k] : an[k];
+    c[15 + k] = s * (k < 2 ? bn[k] - bt[k] : bn[k]);
   }
   c[19] = -sf * lam;
   c[20] = -sf * mu;

@@ -81,8 +81,9 @@ constexpr int kRowElemsFluid = 8;  // of its acoustic form
 constexpr int64_t kSmallLaunch = 8 * 152;  // warps of a row launch, eight per SM
 // Face coefficients: outward normal n[3]; the middle
 // state's tangential coefficients of the own and of the neighbour's side (t^b
-// from t and v, v^b from t and v) and what the normal components add to them
-// (the same four), the neighbour's traction taken with its own normal; then
+// from t and v, v^b from t and v) and of both sides' normal components (t^b: what
+// they add to the tangential product, v^b: the normal velocity itself), the
+// neighbour's traction taken with its own normal; then
 // -s_f lambda, -s_f mu, -s_f / rho of the element (s_f = 2|S_f|/|J|); padding.
 constexpr int CREC = 24;
 // The clusters of one LTS phase (Sec. 4.4) in a single launch: segment i

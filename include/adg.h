@@ -327,7 +327,9 @@ int adg_step_noalloc(adg_ctx* ctx, void* d_Q, int n_steps, void* stream);
  * context's own clusters with CUDA events (whole macro steps, per-phase
  * events as in adg_profile, after one untimed macro step):
  *   choice[0] / [1]: threads per block of the CUDA-core local /
- *                    neighbour kernels, of {64, 128, 256};
+ *                    neighbour kernels in launches of more than eight
+ *                    warps per SM (smaller ones take blocks of one
+ *                    warp), of {64, 128, 256};
  *   choice[2] / [3]: consecutive tiles that one CTA slot of the tensor-core
  *                    local / neighbour kernel takes at a time, of {1, 2, 4};
  *   0 for a kernel kind this context does not launch.

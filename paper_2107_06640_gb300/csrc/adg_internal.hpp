@@ -142,7 +142,8 @@ struct Ctx {
   cudaGraphExec_t graph_exec = nullptr;
   bool use_graph = true;
   // launch shapes (adg_autotune; phase 0 local, 1 neighbour): threads per
-  // block of the row kernels (0: by their own rule), consecutive tiles that a
+  // block of the row kernels (0: by their own rule; launches too small to fill
+  // the GPU keep to the rule), consecutive tiles that a
   // CTA slot of the tensor-core kernels takes at a time
   int cc_threads[2] = {0, 0};
   int tc_chunk[2] = {1, 1};

@@ -1,7 +1,9 @@
 // Autotuner of the launch shapes (adg_autotune).  The work of a step is fixed
 // by the scheme; how it is cut into launches is a choice per kernel kind:
 //   knob 0 / 1: threads per block of the local / neighbour row kernels (64,
-//               128, 256; untuned: row::block_threads);
+//               128, 256) in launches above row::block_threads' small ones,
+//               which take single warps whatever the choice: what the rule
+//               does untuned is among the candidates for every launch;
 //   knob 2 / 3: consecutive tiles a CTA slot of the tensor-core local /
 //               neighbour kernel takes from the launch's tile counter at a
 //               time (1, 2, 4).

@@ -98,8 +98,8 @@ __device__ __forceinline__ void rows_out(const T* sQ, T* Q, int nE, int lane) {
     rows_out_v<T, N, 1>(sQ, Q, nE, lane);
 }
 
-// Threads per block where the caller leaves the choice (threads = 0).  The warps
-// of a block share nothing but, in the neighbour kernel, the re-orientation
+// Threads per block; `threads` (0: none) is the choice of adg_autotune for launches
+// above eight warps per SM.  The warps of a block share nothing but, in the neighbour kernel, the re-orientation
 // table, so blocks are as small as that allows: with at most eight warps per SM
 // single warps spread best (degree 3 FP64, 3,072 tets: 110 us per step with 32
 // threads, 120 with 128), above that 128 (13,182 tets, FP32: 29.7 with 128,
@@ -108,8 +108,8 @@ __device__ __forceinline__ void rows_out(const T* sQ, T* Q, int nE, int lane) {
 // 1106 -> 1028 us, degree 4 782 -> 759 us); at degree 3 256 is slower (225 -> 231).
 template <class T, int N>
 inline int block_threads(int threads, int64_t units) {
-  if (threads) return threads;
   if (units <= kSmallLaunch) return 32;
+  if (threads) return threads;
   return sizeof(T) == 4 && N >= 4 ? 256 : 128;
 }
 

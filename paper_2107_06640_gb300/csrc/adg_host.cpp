@@ -802,7 +802,7 @@ StepArgs Ctx::base_args() const {
   a.par = dPar; a.nbr = dNbr; a.ninfo = dNinfo;
   a.gslot = dGslot; a.bslot = dBslot; a.dslot = dDslot;
   a.perm = dPerm; a.gpar = dGpar;
-  a.S = S; a.err = dErr;
+  a.S = S; a.err = dErr; a.n_sms = n_sms;
   a.fslot = dFslot; a.drout = dDrout; a.gflux = dGflux; a.tc_local = dTcLocal; a.tc_lift = dTcLift;
   a.tiles = dTiles;
   a.crec = dCrec; a.nodalT = dNodal; a.modalT = dModal; a.nodal64 = dNodal64; a.modal64 = dModal64; a.reorient = dReorient;
@@ -1009,7 +1009,7 @@ void Ctx::launch_rupture_cluster(int c, double dt) {
 // that costs more than it saves (degree 2 FP64 2.36 -> 2.57 ms).
 int64_t Ctx::row_plain(int c) const {
   const int64_t n = cl_begin[c + 1] - cl_begin[c];
-  return n > cl_row[c] && n * S <= kSmallLaunch * kRowElems ? 0 : cl_row[c];
+  return n > cl_row[c] && n * S <= (int64_t)kSmallLaunchWarps * n_sms * kRowElems ? 0 : cl_row[c];
 }
 
 int64_t Ctx::launches_per_macro() const {

@@ -66,6 +66,7 @@ struct StepArgs {
   const void* crec;      // T [E][4][CREC] face coefficients
   const void* nodalT;    // T [Bf(r)][Bf(n)]    face modes at the face nodes, r-major
   const void* modalT;    // T [Bf(n)][Bf(r)]    face nodes to face modes, n-major
+  int n_sms;             // of the context's GPU (read by the launchers)
   const double *nodal64, *modal64;  // the same in FP64 (gravitational surfaces of the row kernels)
   const void* reorient;  // T [6][sum (n+1)^2]  a neighbour's face modes in this side's, blocks by degree
 };
@@ -79,7 +80,7 @@ __host__ __device__ inline int64_t elem_of(int64_t v, int S) {
 // Virtual elements per warp of the row kernels
 constexpr int kRowElems = 3;
 constexpr int kRowElemsFluid = 8;  // of its acoustic form
-constexpr int64_t kSmallLaunch = 8 * 152;  // warps of a row launch, eight per SM
+constexpr int kSmallLaunchWarps = 8;  // warps per SM of a row launch that counts as small
 // Face coefficients: outward normal n[3]; the middle
 // state's tangential coefficients of the own and of the neighbour's side (t^b
 // from t and v, v^b from t and v) and of both sides' normal components (t^b: what

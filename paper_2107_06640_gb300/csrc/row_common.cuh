@@ -107,8 +107,8 @@ __device__ __forceinline__ void rows_out(const T* sQ, T* Q, int nE, int lane) {
 // way, and its table is filled once instead of twice (183,456 tets: degree 5
 // 1106 -> 1028 us, degree 4 782 -> 759 us); at degree 3 256 is slower (225 -> 231).
 template <class T, int N>
-inline int block_threads(int threads, int64_t units) {
-  if (units <= kSmallLaunch) return 32;
+inline int block_threads(int threads, int64_t units, int n_sms) {
+  if (units <= (int64_t)kSmallLaunchWarps * n_sms) return 32;
   if (threads) return threads;
   return sizeof(T) == 4 && N >= 4 ? 256 : 128;
 }

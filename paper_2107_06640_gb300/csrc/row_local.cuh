@@ -717,7 +717,7 @@ int launch_local_fluid_t(const StepArgs& a, const Segs& g, int threads, cudaStre
   if (rc) return rc;
   const int64_t units = g.n ? g.first[g.n] : 0;
   if (units <= 0) return 0;
-  threads = block_threads<T, N>(threads, units);
+  threads = block_threads<T, N>(threads, units, a.n_sms);
   if (threads < 32 || threads > kMaxThreads || threads % 32) return (int)cudaErrorInvalidValue;
   const int w = threads / 32;
   local_fluid_kernel<T, N><<<(unsigned)((units + w - 1) / w), threads, M::bytes(threads), st>>>(a, g);
@@ -737,7 +737,7 @@ int launch_local_row_t(const StepArgs& a, const Segs& g, int threads, bool spec,
   if (rc) return rc;
   const int64_t units = g.n ? g.first[g.n] : 0;
   if (units <= 0) return 0;
-  threads = block_threads<T, N>(threads, units);
+  threads = block_threads<T, N>(threads, units, a.n_sms);
   if (threads < 32 || threads > kMaxThreads || threads % 32) return (int)cudaErrorInvalidValue;
   if (spec && threads > 128) threads = 128;  // (shared memory)
   const int w = threads / 32;

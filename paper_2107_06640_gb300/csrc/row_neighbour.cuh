@@ -176,7 +176,7 @@ int launch_neighbour_row_t(const StepArgs& a, const Segs& g, int threads, bool s
   if (rc) return rc;
   const int64_t units = g.n ? g.first[g.n] : 0;
   if (units <= 0) return 0;
-  threads = block_threads<T, N>(threads, units);
+  threads = block_threads<T, N>(threads, units, a.n_sms);
   if (threads < 32 || threads > kMaxThreads || threads % 32) return (int)cudaErrorInvalidValue;
   const int w = threads / 32;
   const unsigned blocks = (unsigned)((units + w - 1) / w);

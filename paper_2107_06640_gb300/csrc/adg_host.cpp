@@ -780,11 +780,13 @@ void Ctx::setup() {
     CK(cudaEventCreateWithFlags(&side_done[i], cudaEventDisableTiming));
   }
   CK(cudaEventCreateWithFlags(&side_fork, cudaEventDisableTiming));
-  // configure kernels once (outside any stream capture)
+  // configure every kernel that a step of this context may launch (outside any stream capture)
   StepArgs a0 = base_args();
   const Segs none = make_segs(nullptr, 0, 1);
   int rc = launch_local_row(fp64, N, a0, none, stream, 128, false);
   if (!rc) rc = launch_neighbour_row(fp64, N, a0, none, stream, 128, false);
+  if (!rc && acoustic && !tc) rc = launch_local_fluid(fp64, N, a0, none, stream, 128);
+  if (!rc && nff) rc = launch_rupture(fp64, N, DRArgs{}, stream);
   if (!rc && tc) rc = launch_local_tc(N, a0, none, n_sms, stream, false);
   if (!rc && tc) rc = launch_neighbour_tc(N, a0, none, n_sms, stream, false);
   if (rc) throw Err(ADG_E_CUDA, std::string("kernel configuration: ") + cudaGetErrorString((cudaError_t)rc));

@@ -207,6 +207,7 @@ struct DRArgs {
 
 enum { FRIC_RS = 0, FRIC_LSW = 1 };  // the ADG_FRICTION_* values of adg.h
 
+// (no faces: the kernels are configured on the current device, nothing is launched)
 int launch_rupture(int fp64, int N, const DRArgs& a, void* stream);
 
 enum { ERR_NAN = 1u, ERR_TIMEOUT = 2u, ERR_NEWTON = 4u };

@@ -424,33 +424,34 @@ __global__ void __launch_bounds__(128) rupture_kernel(DRArgs a) {
   atomicAdd(&a.newton[1], n_iters);
 }
 
-template <typename T>
-int dispatch(int N, const DRArgs& a, cudaStream_t st) {
+template <typename T, int N>
+int dispatch_deg(const DRArgs& a, cudaStream_t st) {
+  // (12 (N + 1) doubles per thread: at most 72 KB, above the default limit from N = 4 on)
+  constexpr int bytes = 12 * (N + 1) * 128 * (int)sizeof(double);
+  const auto net = rupture_kernel<T, N, true>, plain = rupture_kernel<T, N, false>;
+  const int rc = configure_on_device((const void*)plain, [&] {
+    cudaError_t ce = cudaFuncSetAttribute((const void*)plain, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (ce == cudaSuccess)
+      ce = cudaFuncSetAttribute((const void*)net, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    return ce;
+  });
+  if (rc) return rc;
   const int64_t total = a.n_faces * a.S * nb2(N);
   if (total <= 0) return 0;
-  const unsigned grid = (unsigned)((total + 127) / 128);
-  const bool net = a.mlp || a.capture;
-  // (12 (N + 1) doubles per thread: at most 72 KB, above the default limit from N = 4 on)
-  const int bytes = 12 * (N + 1) * 128 * (int)sizeof(double);
-#define ADG_RK(n)                                                                                          \
-  {                                                                                                        \
-    const auto k = net ? rupture_kernel<T, n, true> : rupture_kernel<T, n, false>;                         \
-    const int rc = configure_on_device((const void*)k, [&] {                                               \
-      return cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);     \
-    });                                                                                                    \
-    if (rc) return rc;                                                                                     \
-    k<<<grid, 128, bytes, st>>>(a);                                                                        \
-  }
-  switch (N) {
-    case 1: ADG_RK(1); break;
-    case 2: ADG_RK(2); break;
-    case 3: ADG_RK(3); break;
-    case 4: ADG_RK(4); break;
-    case 5: ADG_RK(5); break;
-    default: return (int)cudaErrorInvalidValue;
-  }
-#undef ADG_RK
+  (a.mlp || a.capture ? net : plain)<<<(unsigned)((total + 127) / 128), 128, bytes, st>>>(a);
   return (int)cudaGetLastError();
+}
+
+template <typename T>
+int dispatch(int N, const DRArgs& a, cudaStream_t st) {
+  switch (N) {
+    case 1: return dispatch_deg<T, 1>(a, st);
+    case 2: return dispatch_deg<T, 2>(a, st);
+    case 3: return dispatch_deg<T, 3>(a, st);
+    case 4: return dispatch_deg<T, 4>(a, st);
+    case 5: return dispatch_deg<T, 5>(a, st);
+  }
+  return (int)cudaErrorInvalidValue;
 }
 
 }  // namespace

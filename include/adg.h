@@ -162,9 +162,10 @@ int adg_init(adg_ctx* ctx);
  * upload. */
 int adg_plan(adg_ctx* ctx, double* dt_elem, int32_t* cluster, double* dt_min, int* n_clusters);
 
-/* Host-only: the Godunov flux matrices adg_init builds for local face `face`
- * of user tet `tet` (Sec. 4.2, Eq. numerical-flux), global frame, row-major
- * 9x9, caller-owned Fm[81], Fp[81] (either may be NULL).  The flux T A^- w^b
+/* Host-only: the Godunov flux through local face `face` of user tet `tet`
+ * (Sec. 4.2, Eq. numerical-flux) as matrices: what the kernels compute from
+ * adg_init's coefficients of the face, in double on unit states; global frame,
+ * row-major 9x9, caller-owned Fm[81], Fp[81] (either may be NULL).  The flux T A^- w^b
  * through the face is Fm q^- + Fp q^+ for interior and periodic faces (q^+ the
  * neighbour's state at the same point) and Fm q^- for free-surface, rigid-wall
  * and absorbing faces (Fp zero); both are zero for gravitational and fault

@@ -61,56 +61,6 @@ M9 jac_x(double rho, double lam, double mu) {
   return A;
 }
 
-// Orthonormal frame (n, s, t) and the maps T (rotated -> global) and T^-1.
-void frame(const double n[3], double R[3][3]) {
-  int k = 0;
-  for (int d = 1; d < 3; ++d)
-    if (std::fabs(n[d]) < std::fabs(n[k])) k = d;
-  double a[3] = {0, 0, 0};
-  a[k] = 1;
-  double dot = a[0] * n[0] + a[1] * n[1] + a[2] * n[2];
-  double s[3] = {a[0] - dot * n[0], a[1] - dot * n[1], a[2] - dot * n[2]};
-  double ns = std::sqrt(s[0] * s[0] + s[1] * s[1] + s[2] * s[2]);
-  for (double& v : s) v /= ns;
-  double t[3] = {n[1] * s[2] - n[2] * s[1], n[2] * s[0] - n[0] * s[2], n[0] * s[1] - n[1] * s[0]};
-  for (int d = 0; d < 3; ++d) { R[d][0] = n[d]; R[d][1] = s[d]; R[d][2] = t[d]; }
-}
-const int kVo[6][2] = {{0, 0}, {1, 1}, {2, 2}, {0, 1}, {1, 2}, {0, 2}};
-// out = rotate(vec): fwd => stress R S R^T, vel R v ; inverse => R^T S R, R^T v
-void rot9(const double R[3][3], const double* in, double* out, bool to_global) {
-  double S[3][3];
-  for (int c = 0; c < 6; ++c) { S[kVo[c][0]][kVo[c][1]] = in[c]; S[kVo[c][1]][kVo[c][0]] = in[c]; }
-  double Rm[3][3];
-  for (int i = 0; i < 3; ++i)
-    for (int j = 0; j < 3; ++j) Rm[i][j] = to_global ? R[i][j] : R[j][i];
-  double Y[3][3];
-  for (int i = 0; i < 3; ++i)
-    for (int l = 0; l < 3; ++l) {
-      double acc = 0;
-      for (int j = 0; j < 3; ++j)
-        for (int k = 0; k < 3; ++k) acc += Rm[i][j] * S[j][k] * Rm[l][k];
-      Y[i][l] = acc;
-    }
-  for (int c = 0; c < 6; ++c) out[c] = Y[kVo[c][0]][kVo[c][1]];
-  for (int i = 0; i < 3; ++i) {
-    double acc = 0;
-    for (int j = 0; j < 3; ++j) acc += Rm[i][j] * in[6 + j];
-    out[6 + i] = acc;
-  }
-}
-void rot_mats(const double n[3], M9& T, M9& Ti) {
-  double R[3][3];
-  frame(n, R);
-  for (int c = 0; c < 9; ++c) {
-    double e[9] = {0}, o[9];
-    e[c] = 1;
-    rot9(R, e, o, true);
-    for (int r = 0; r < 9; ++r) T[r * 9 + c] = o[r];
-    rot9(R, e, o, false);
-    for (int r = 0; r < 9; ++r) Ti[r * 9 + c] = o[r];
-  }
-}
-
 // Middle state w^b = Mm w^- + Mp w^+ (Sec. 4.2, Eq. boundary-state; solid-solid
 // shear with the same welded form using Z_s).
 void middle_state(double Zpm, double Zpp, double Zsm, double Zsp, M9& Mm, M9& Mp) {
@@ -145,76 +95,57 @@ M9 diag9(std::initializer_list<double> d) {
   return r;
 }
 
-// Godunov flux matrices of a face in the global frame (Sec. 4.2, Eq.
-// numerical-flux): with TA = T A^- and Ti = T^-1 for the face's normal, the
-// flux T A^- w^b, w^b = Mm T^-1 q^- + Mp T^-1 q^+, is Fm q^- + Fp q^+.
-void godunov_pair(const M9& TA, const M9& Ti, double Zpm, double Zpp, double Zsm, double Zsp, M9& Fm, M9& Fp) {
-  M9 Mm, Mp;
-  middle_state(Zpm, Zpp, Zsm, Zsp, Mm, Mp);
-  Fm = mm(mm(TA, Mm), Ti);
-  Fp = mm(mm(TA, Mp), Ti);
-}
-
-// Linear boundaries (Sec. 4.3): the ghost state w^+ = G w^- (free surface:
-// traction w1, w4, w6 mirrored; rigid wall: w7, w4, w6 mirrored; absorbing:
-// G = 0) with the minus material folds into Fm = T A^- (Mm + Mp G) T^-1.
-M9 boundary_matrix(const M9& TA, const M9& Ti, double Zp, double Zs, int tag) {
-  M9 Mm, Mp;
-  middle_state(Zp, Zp, Zs, Zs, Mm, Mp);
+// Ghost state w^+ = G w^- of a linear boundary (Sec. 4.3), with the minus
+// material: free surface, traction w1, w4, w6 mirrored; rigid wall, w7, w4, w6
+// mirrored; absorbing, zero.
+M9 ghost(int tag) {
   M9 G{};
   if (tag == ADG_TAG_FREE) G = diag9({-1, 1, 1, -1, 1, -1, 1, 1, 1});
   else if (tag == ADG_TAG_RIGID) G = diag9({1, 1, 1, -1, 1, -1, -1, 1, 1});
-  return mm(mm(TA, madd(Mm, mm(Mp, G))), Ti);
+  return G;
 }
 
-// ---------------- Gauss-Legendre on [0,1] (Newton on P_n) ----------------
-// Coefficients of one face for the row kernels (kernels.cuh, CREC) from the
-// middle state of Sec. 4.2 (Eq. boundary-state), a linear boundary's ghost
-// folded into the own side (free surface: traction mirrored; rigid wall: normal
-// velocity and shear traction mirrored; absorbing: zero).  A gravitational
-// face keeps the own tangential velocity and takes its normal state from the
-// (eta, H) ODE; a fault face's flux is the friction solve's.
+// Coefficients of one face for the kernels (kernels.cuh, CREC) from the middle
+// state of Sec. 4.2 (Eq. boundary-state), a linear boundary's ghost folded into
+// the own side.  A gravitational face keeps the own tangential velocity and takes
+// its normal state from the (eta, H) ODE; a fault face's flux is the friction
+// solve's.
 void face_coefficients(const double n[3], int tag, double Zp, double Zs, double Zpp, double Zsp, double rho, double lam,
                        double mu, double sf, double* c) {
   for (int d = 0; d < 3; ++d) c[d] = n[d];
   if (tag == ADG_TAG_FAULT) return;
-  // normal pair: (t^b, v^b) from own (t, v) and the neighbour's; tangential the same
-  const double z = Zp * Zpp / (Zp + Zpp);
-  double an[4] = {1 - z / Zpp, -z, -z / (Zpp * Zp), 1 - z / Zp}, bn[4] = {z / Zpp, z, z / (Zpp * Zp), z / Zp};
-  double at[4] = {0, 0, Zs > 0 ? -1 / Zs : 0.0, 1}, bt[4] = {0, 0, 0, 0};
-  if (Zs > 0 && Zsp > 0) {
-    const double zs = Zs * Zsp / (Zs + Zsp);
-    at[0] = 1 - zs / Zsp; at[1] = -zs; at[2] = -zs / (Zsp * Zs); at[3] = 1 - zs / Zs;
-    bt[0] = zs / Zsp; bt[1] = zs; bt[2] = zs / (Zsp * Zs); bt[3] = zs / Zs;
-  }
-  if (tag == ADG_TAG_GRAVITY) {
-    an[0] = an[1] = an[2] = an[3] = at[0] = at[1] = 0;
-    at[2] = Zs > 0 ? -1 / Zs : 0.0;
-    at[3] = 1;
-  } else if (tag != ADG_TAG_INTERIOR && tag != ADG_TAG_PERIODIC) {
-    const double gtn = tag == ADG_TAG_FREE ? -1 : tag == ADG_TAG_RIGID ? 1 : 0;
-    const double gvn = tag == ADG_TAG_FREE ? 1 : tag == ADG_TAG_RIGID ? -1 : 0;
-    const double gts = tag == ADG_TAG_ABSORB ? 0 : -1, gvs = tag == ADG_TAG_ABSORB ? 0 : 1;
-    for (int k = 0; k < 4; ++k) {
-      an[k] += bn[k] * (k % 2 ? gvn : gtn);
-      at[k] += bt[k] * (k % 2 ? gvs : gts);
-    }
-  }
   const bool nb = tag == ADG_TAG_INTERIOR || tag == ADG_TAG_PERIODIC;
-  for (int k = 0; k < 4; ++k) {
-    const double s = nb ? (k % 2 ? 1.0 : -1.0) : 0.0;  // the neighbour's traction has the opposite normal
-    c[3 + k] = at[k];
-    c[7 + k] = s * bt[k];
-    // (traction: what the normal part adds to the tangential coefficients' product;
-    // velocity: the normal state itself, see row_flux.cuh)
-    c[11 + k] = k < 2 ? an[k] - at[k] : an[k];
-    c[15 + k] = s * (k < 2 ? bn[k] - bt[k] : bn[k]);
+  M9 Mm, Mp;
+  middle_state(Zp, nb ? Zpp : Zp, Zs, nb ? Zsp : Zs, Mm, Mp);
+  if (tag == ADG_TAG_GRAVITY) {
+    for (int r : {0, 6}) Mm[r * 9 + 0] = Mm[r * 9 + 6] = 0;
+    Mm[3 * 9 + 3] = Mm[3 * 9 + 7] = 0;
+    Mm[7 * 9 + 3] = Zs > 0 ? -1 / Zs : 0.0;
+    Mm[7 * 9 + 7] = 1;
+  } else if (!nb) {
+    Mm = madd(Mm, mm(Mp, ghost(tag)));
   }
-  c[19] = -sf * lam;
-  c[20] = -sf * mu;
-  c[21] = -sf / rho;
+  // normal pair (w1, w7) and tangential pair (w4, w8; w6, w9 alike): the rows of
+  // traction and velocity, each from traction and velocity
+  for (int k = 0; k < 4; ++k) {
+    const int rn = k < 2 ? 0 : 6, cn = k % 2 ? 6 : 0, rt = k < 2 ? 3 : 7, ct = k % 2 ? 7 : 3;
+    const double an = Mm[rn * 9 + cn], at = Mm[rt * 9 + ct];
+    const double s = nb ? (k % 2 ? 1.0 : -1.0) : 0.0;  // the neighbour's traction has the opposite normal
+    const double bn = s * Mp[rn * 9 + cn], bt = s * Mp[rt * 9 + ct];
+    c[3 + k] = at;
+    c[7 + k] = bt;
+    // (traction: what the normal part adds to the tangential coefficients' product;
+    // velocity: the normal state itself, see face_flux_state)
+    c[11 + k] = k < 2 ? an - at : an;
+    c[15 + k] = k < 2 ? bn - bt : bn;
+  }
+  const M9 A = jac_x(rho, lam, mu);
+  c[19] = sf * (A[0 * 9 + 6] - 2 * A[3 * 9 + 7]);  // (A holds -(lam + 2 mu), -mu, -1 / rho)
+  c[20] = sf * A[3 * 9 + 7];
+  c[21] = sf * A[6 * 9 + 0];
 }
 
+// ---------------- Gauss-Legendre on [0,1] (Newton on P_n) ----------------
 void gauss01(int n, std::vector<double>& x, std::vector<double>& w) {
   x.resize(n);
   w.resize(n);
@@ -446,26 +377,37 @@ void Ctx::plan_mesh(const RefOps& o, int degree, MeshPlan& plan) const {
   for (int64_t e = 0; e < E; ++e) plan.ncl = std::max(plan.ncl, cl[e] + 1);
 }
 
-// The flux matrices setup() builds for face f of user tet eu (global frame,
-// row-major): interior and periodic faces Fm, Fp; free, rigid and absorbing
+// The flux through face f of user tet eu as matrices (global frame, row-major):
+// the kernels' face_flux_state with the coefficients that setup() gives them, on
+// unit states.  Interior and periodic faces Fm, Fp; free, rigid and absorbing
 // faces Fm (Fp zero); gravitational and fault faces zero (their fluxes come
 // from the (eta, H) ODE and the friction solve).
 void Ctx::face_flux(const MeshPlan& pl, int64_t eu, int f, double* Fm, double* Fp) const {
-  M9 FmM{}, FpM{};
   const int tg = tag[4 * eu + f];
-  const double Zpm = std::sqrt(rho[eu] * (lam[eu] + 2 * mu[eu])), Zsm = std::sqrt(rho[eu] * mu[eu]);
-  M9 T, Ti;
-  rot_mats(&pl.nrm[12 * eu + 3 * f], T, Ti);
-  const M9 TA = mm(T, jac_x(rho[eu], lam[eu], mu[eu]));
-  if (tg == ADG_TAG_INTERIOR || tg == ADG_TAG_PERIODIC) {
-    const int64_t e2u = pl.nbr[4 * eu + f];
-    const double Zpp = std::sqrt(rho[e2u] * (lam[e2u] + 2 * mu[e2u])), Zsp = std::sqrt(rho[e2u] * mu[e2u]);
-    godunov_pair(TA, Ti, Zpm, Zpp, Zsm, Zsp, FmM, FpM);
-  } else if (tg == ADG_TAG_FREE || tg == ADG_TAG_RIGID || tg == ADG_TAG_ABSORB) {
-    FmM = boundary_matrix(TA, Ti, Zpm, Zsm, tg);
+  for (double* F : {Fm, Fp})
+    if (F) std::fill(F, F + 81, 0.0);
+  if (tg == ADG_TAG_GRAVITY || tg == ADG_TAG_FAULT) return;
+  const double* n = &pl.nrm[12 * eu + 3 * f];
+  const int64_t e2 = pl.nbr[4 * eu + f] < 0 ? eu : pl.nbr[4 * eu + f];
+  double c[CREC] = {0};
+  face_coefficients(n, tg, std::sqrt(rho[eu] * (lam[eu] + 2 * mu[eu])), std::sqrt(rho[eu] * mu[eu]),
+                    std::sqrt(rho[e2] * (lam[e2] + 2 * mu[e2])), std::sqrt(rho[e2] * mu[e2]), rho[eu], lam[eu], mu[eu],
+                    1.0, c);
+  const int vo[3][3] = {{0, 3, 5}, {3, 1, 4}, {5, 4, 2}};  // the stress tensor's entries
+  const double zero[6] = {0};
+  for (int side = 0; side < 2; ++side) {
+    double* const F = side ? Fp : Fm;
+    if (!F) continue;
+    for (int k = 0; k < 9; ++k) {
+      double q[6] = {0}, g[9];  // a trace: traction with the owner's outward normal, velocity
+      for (int d = 0; d < 3; ++d)
+        for (int x = 0; x < 3; ++x)
+          if (vo[d][x] == k) q[d] += side ? -n[x] : n[x];
+      if (k >= 6) q[k - 3] = 1;
+      face_flux_state(c, side ? zero : q, side ? q : zero, 0.0, 0.0, g);
+      for (int r = 0; r < 9; ++r) F[r * 9 + k] = g[r];
+    }
   }
-  if (Fm) std::copy(FmM.begin(), FmM.end(), Fm);
-  if (Fp) std::copy(FpM.begin(), FpM.end(), Fp);
 }
 
 // Face f of user tet eu seen from its neighbour (interior, periodic and fault

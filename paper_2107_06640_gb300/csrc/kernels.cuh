@@ -16,6 +16,7 @@
 //                     stored fluxes of gravitational and fault faces; one lift.
 // Dofs layout: Q[v][9][B] (basis fastest).  Face data: modal, see row_common.cuh.
 #pragma once
+#include <cmath>
 #include <cstdint>
 
 namespace adg {
@@ -88,6 +89,40 @@ constexpr int kSmallLaunchWarps = 8;  // warps per SM of a row launch that count
 // neighbour's traction taken with its own normal; then
 // -s_f lambda, -s_f mu, -s_f / rho of the element (s_f = 2|S_f|/|J|); padding.
 constexpr int CREC = 24;
+// The scaled flux s_f T A^- w^b of one mode (or point) of a face: c the face's
+// coefficients, q and w the own and the neighbour's traction and velocity (each
+// traction with its owner's outward normal), srt and srv a gravitational surface's
+// normal traction and velocity.
+// The normal velocity state vs is formed by itself and goes into the lambda
+// rows directly.  The tangential velocity coefficients hold 1 / Z_s: in a soft
+// solid (Z_s << Z_p) the normal part of their product is large, and what is left
+// of it in vb.n after the subtraction is rounding of that size, which the mu rows
+// bear (mu / Z_s is small) and the lambda rows do not (FP32, v_s 50 m/s beside
+// water: 3e-6 of the row where this form has 8e-8).
+template <class T>
+__host__ __device__ __forceinline__ void face_flux_state(const T* c, const T* q, const T* w, T srt, T srv, T* g) {
+  const T tn = fma(q[2], c[2], fma(q[1], c[1], q[0] * c[0])), vn = fma(q[5], c[2], fma(q[4], c[1], q[3] * c[0]));
+  const T tm = fma(w[2], c[2], fma(w[1], c[1], w[0] * c[0])), vm = fma(w[5], c[2], fma(w[4], c[1], w[3] * c[0]));
+  const T an = fma(c[11], tn, fma(c[12], vn, fma(c[15], tm, fma(c[16], vm, srt))));
+  const T vs = fma(c[13], tn, fma(c[14], vn, fma(c[17], tm, fma(c[18], vm, srv))));
+  const T bn = vs - fma(c[5], tn, fma(c[6], vn, fma(c[9], tm, c[10] * vm)));
+  T tb[3], vb[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    tb[d] = fma(an, c[d], fma(c[3], q[d], fma(c[4], q[3 + d], fma(c[7], w[d], c[8] * w[3 + d]))));
+    vb[d] = fma(bn, c[d], fma(c[5], q[d], fma(c[6], q[3 + d], fma(c[9], w[d], c[10] * w[3 + d]))));
+  }
+  const T l = c[19] * vs;
+  const T m[3] = {c[20] * vb[0], c[20] * vb[1], c[20] * vb[2]};
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    g[d] = fma(T(2) * c[d], m[d], l);
+    g[6 + d] = c[21] * tb[d];
+  }
+  g[3] = fma(c[0], m[1], c[1] * m[0]);
+  g[4] = fma(c[1], m[2], c[2] * m[1]);
+  g[5] = fma(c[0], m[2], c[2] * m[0]);
+}
 // The clusters of one LTS phase (Sec. 4.4) in a single launch: segment i
 // covers the virtual elements [v_begin, v_begin + n) of one cluster with that
 // cluster's time coefficients, and the launch's work units (tiles of the

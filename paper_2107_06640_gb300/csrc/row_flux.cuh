@@ -154,7 +154,6 @@ __device__ __forceinline__ void face_items(const StepArgs& a, const T* st, const
         srv = src[BF];
       }
     }
-    // coefficients: n[3], own and the neighbour's tangential, own and the neighbour's normal, material
     T c[CREC];
 #pragma unroll
     for (int d = 0; d < CREC / F::V; ++d) {
@@ -165,34 +164,11 @@ __device__ __forceinline__ void face_items(const StepArgs& a, const T* st, const
 #pragma unroll
       for (int t = 0; t < F::V; ++t) c[d * F::V + t] = x.x[t];
     }
-    const T tn = fma(q[2], c[2], fma(q[1], c[1], q[0] * c[0])), vn = fma(q[5], c[2], fma(q[4], c[1], q[3] * c[0]));
-    const T tm = fma(w[2], c[2], fma(w[1], c[1], w[0] * c[0])), vm = fma(w[5], c[2], fma(w[4], c[1], w[3] * c[0]));
-    const T an = fma(c[11], tn, fma(c[12], vn, fma(c[15], tm, fma(c[16], vm, srt))));
-    // The normal velocity state vs is formed by itself and goes into the lambda
-    // rows directly.  The tangential velocity coefficients hold 1 / Z_s: in a soft
-    // solid (Z_s << Z_p) the normal part of their product is large, and what is left
-    // of it in vb.n after the subtraction is rounding of that size, which the mu rows
-    // bear (mu / Z_s is small) and the lambda rows do not (FP32, v_s 50 m/s beside
-    // water: 3e-6 of the row where this form has 8e-8).
-    const T vs = fma(c[13], tn, fma(c[14], vn, fma(c[17], tm, fma(c[18], vm, srv))));
-    const T bn = vs - fma(c[5], tn, fma(c[6], vn, fma(c[9], tm, c[10] * vm)));
-    T tb[3], vb[3];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      tb[d] = fma(an, c[d], fma(c[3], q[d], fma(c[4], q[3 + d], fma(c[7], w[d], c[8] * w[3 + d]))));
-      vb[d] = fma(bn, c[d], fma(c[5], q[d], fma(c[6], q[3 + d], fma(c[9], w[d], c[10] * w[3 + d]))));
-    }
-    const T l = c[19] * vs;
-    const T m[3] = {c[20] * vb[0], c[20] * vb[1], c[20] * vb[2]};
+    T r[9];
+    face_flux_state(c, q, w, srt, srv, r);
     T* const g = sG + 9 * je * F::GS + n;
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      g[d * F::GS] = fma(T(2) * c[d], m[d], l);
-      g[(6 + d) * F::GS] = c[21] * tb[d];
-    }
-    g[3 * F::GS] = fma(c[0], m[1], c[1] * m[0]);
-    g[4 * F::GS] = fma(c[1], m[2], c[2] * m[1]);
-    g[5 * F::GS] = fma(c[0], m[2], c[2] * m[0]);
+    for (int p = 0; p < 9; ++p) g[p * F::GS] = r[p];
   }
 }
 

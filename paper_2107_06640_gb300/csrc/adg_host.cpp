@@ -745,7 +745,7 @@ StepArgs Ctx::base_args() const {
   a.Q = dQ; a.trace = dTrace; a.btrace = dBtrace; a.dtrace = dDtrace; a.eta = dEta;
   a.par = dPar; a.nbr = dNbr; a.ninfo = dNinfo;
   a.gslot = dGslot; a.bslot = dBslot; a.dslot = dDslot;
-  a.perm = dPerm; a.gpar = dGpar;
+  a.gpar = dGpar;
   a.S = S; a.err = dErr; a.n_sms = n_sms;
   a.fslot = dFslot; a.drout = dDrout; a.gflux = dGflux; a.tc_local = dTcLocal; a.tc_lift = dTcLift;
   a.tiles = dTiles;

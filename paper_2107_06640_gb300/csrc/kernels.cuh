@@ -53,7 +53,6 @@ struct StepArgs {
   const int* gslot;     // [E][4] gravity slot or -1
   const int* bslot;     // [E]    LTS buffer slot or -1
   const int* dslot;     // [E][4] LTS derivative-trace slot or -1
-  const int* perm;      // [6][Bf]
   const double* gpar;   // [ngslot][GPAR]
   int S;                // ensemble size
   unsigned int* err;    // device error word

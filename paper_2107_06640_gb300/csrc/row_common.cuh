@@ -47,7 +47,6 @@ struct Shape {
   static constexpr int B = nb3(N), Bf = nb2(N), B1 = nb3(N - 1);
   static constexpr int V16 = 16 / (int)sizeof(T);
   static constexpr int VW = B % V16 == 0 ? V16 : 1;
-  static constexpr int words(int s) { return s * (int)sizeof(T) / 4; }
   // 16-byte accesses: the stride in 16-byte units must be odd
   static constexpr int SB = VW == 1 ? (sizeof(T) == 4 ? (B | 1) : B) : (B / VW % 2 ? B : B + VW);
   static constexpr int FS = face_block(N);     // values of a face block

@@ -140,7 +140,6 @@ __device__ __forceinline__ void each(F&& f) {
 
 // the re-orientation of a face's modes: entries of one permutation, block n at blk(n)
 __host__ __device__ constexpr int blk(int n) { return n * (n + 1) * (2 * n + 1) / 6; }
-constexpr int kPVn = blk(6);
 
 }  // namespace sp
 }  // namespace adg

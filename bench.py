@@ -704,13 +704,10 @@ def main():
     sm_mhz = clk.get("sm_mhz") or peaks.get("sm_max_mhz", 2070.0)
     units = unit_peaks()
     n_sm = torch.cuda.get_device_properties(local).multi_processor_count
-    alu_peak, alu_src = alu_peak_tflops(False, peaks.get("sm_max_mhz", 2070.0), units, n_sm)
-    achieved_flops = fl[kname.replace("_tc", "")] * n_k / (t_k[dom] * 1e-3) / 1e12
     # an acoustic element's reference-matrix products act on 4 of the 9 quantity rows
     local_bytes = by["local"] * (n_k - n_ac) + by["local_acoustic"] * n_ac
     launch_bytes = local_bytes if kname.startswith("local") else by["neighbour"] * n_k
     achieved_bytes = launch_bytes / (t_k[dom] * 1e-3) / 1e9
-    frac_alu = achieved_flops / alu_peak
     frac_hbm = achieved_bytes / peaks["hbm_gbs"]
     tc_peak, tc_src = tf32x3_peak_tflops(peaks, units)
     tensor_flops = tc_local_flops(N_DEG) * ((n_k - n_ac) + n_ac * 4.0 / 9.0)
@@ -721,11 +718,7 @@ def main():
                 "frac": frac_hbm, "traffic": None, "kernel": kname, "peak_source": src,
                 "bytes_counted": {"elastic": by["local"], "acoustic": by["local_acoustic"]} if dom == 0 else by["neighbour"],
                 "elements": {"elastic": n_k - n_ac, "acoustic": n_ac}}
-    elif frac_alu >= frac_hbm:
-        roof = {"bound": "alu", "achieved": achieved_flops, "peak": alu_peak, "unit": "TFLOP/s",
-                "frac": frac_alu, "traffic": None, "kernel": kname,
-                "peak_source": alu_src}
-    else:
+    else:  # (row kernels; flops_per_update is a count of dense nodal products, not of what they execute)
         roof = {"bound": "hbm", "achieved": achieved_bytes, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                 "frac": frac_hbm, "traffic": None, "kernel": kname, "peak_source": src}
     if kname in TC_DRAM_BYTES_PER_ELEMENT:
@@ -734,8 +727,7 @@ def main():
                            if kname == "local_tc_kernel" else TC_DRAM_BYTES_PER_ELEMENT[kname] * n_k)
         roof["traffic_note"] = "DRAM bytes per launch, ncu on the 374,400-tet box scaled by elements"
     roof.update({"ms_per_launch": t_k[dom], "elements_per_launch": n_k, "hbm_frac": frac_hbm,
-                 # the CUDA-core ALU fraction of a tensor-core kernel's whole flop count means nothing
-                 "alu_frac": None if kname.endswith("_tc_kernel") else frac_alu,
+                 "alu_frac": None,
                  "kernel_ms": {"local": kms[0], "neighbour": kms[1]}})
     if tc_form:
         roof.update({"tc_kernel_ms": {"local_tc": kms[3], "neighbour_tc": kms[4]},
@@ -756,6 +748,8 @@ def main():
         "config": {"workload": WORKLOAD if args.nxy == 80 else f"{args.nxy}x{args.nxy}-column box", "n_tets": s.nt, "degree": N_DEG, "time_stepping": "global (1 cluster)",
                    "parallelism": f"replicas x{world}", "l2": "inputs larger than L2 (3 GB FP32 dofs)"},
         "gflops": value * fl["total"] / 1e9,
+        "gflops_note": "dense nodal products as counted by flops_per_update; the kernels' sparse and modal form "
+                       "executes fewer",
         "precision": "FP32 dofs; reference-matrix products of the local kernel as tcgen05 3xTF32 MMAs with "
                      "FP32 accumulation, star and flux products on FP32 CUDA cores (eta, LTS buffers, friction FP64)",
         "fp32_cuda_cores": {"value": value_cc, "unit": UNIT, "ms_per_step": rcc["ms"] / rcc["steps"],

@@ -119,8 +119,9 @@ int adg_upload_mesh(adg_ctx* ctx, int64_t nv, const double* xyz, int64_t nt,
 /* Element-wise constant material (Sec. 4.1): density, Lame lambda, mu (mu = 0: fluid). */
 int adg_upload_material(adg_ctx* ctx, const double* rho, const double* lambda, const double* mu);
 
-/* Geometry, CFL time steps, rate-2 clustering, Godunov flux matrices F-/F+
- * per face (Sec. 4.2, Eq. numerical-flux), device allocation.  Dofs start at 0. */
+/* (adg_init, declared below:) geometry, CFL time steps, rate-2 clustering, the
+ * coefficients of every face's Godunov flux (Sec. 4.2, Eq. numerical-flux),
+ * device allocation.  Dofs start at 0. */
 /* The ocean as the acoustic system (Sec. 4.1: the fluid is the elastic
  * system with mu = 0, its stress -p I).  Call before adg_init (else
  * ADG_E_STATE); enable = 0 restores the default.  With it:
@@ -180,8 +181,9 @@ int adg_face_flux(adg_ctx* ctx, int64_t tet, int face, double* Fm, double* Fp);
  * and its local face (-1, -1 for a face without neighbour), and
  * node_map[Bf] = for each face node n (equispaced, see above) the
  * neighbour's face node at the same physical point (for periodic faces:
- * after the translation between the two faces).  This is the re-orientation
- * the neighbour flux applies to the neighbour's trace (Sec. 4.2).  Outputs
+ * after the translation between the two faces).  The vertex permutation behind
+ * it is the one by which the neighbour flux re-orients the neighbour's trace
+ * (Sec. 4.2; the kernels do so mode by mode).  Outputs
  * caller-owned, each may be NULL; node_map is left untouched without a
  * neighbour.  No device needed.  Errors as adg_face_flux. */
 int adg_face_neighbour(adg_ctx* ctx, int64_t tet, int face, int64_t* nb_tet, int* nb_face,

@@ -1,5 +1,5 @@
 // Host side of the C ABI (include/adg.h): mesh set-up, geometry, clustering,
-// Godunov flux matrices, device memory, the rate-2 LTS tick schedule and the
+// coefficients of the face fluxes, device memory, the rate-2 LTS tick schedule and the
 // per-macro-step CUDA graph.
 #include <cuda_runtime.h>
 
@@ -33,19 +33,8 @@ using Err = adg::AdgError;
     if (_e != cudaSuccess) throw Err(ADG_E_CUDA, std::string(#call) + ": " + cudaGetErrorString(_e)); \
   } while (0)
 
-// ---------------- small dense 9x9 helpers (row-major) ----------------
+// ---------------- 9x9 matrices (row-major) ----------------
 typedef std::array<double, 81> M9;
-M9 mm(const M9& a, const M9& b) {
-  M9 r{};
-  for (int i = 0; i < 9; ++i)
-    for (int k = 0; k < 9; ++k) {
-      double v = a[i * 9 + k];
-      if (v == 0) continue;
-      for (int j = 0; j < 9; ++j) r[i * 9 + j] += v * b[k * 9 + j];
-    }
-  return r;
-}
-M9 madd(const M9& a, const M9& b) { M9 r; for (int i = 0; i < 81; ++i) r[i] = a[i] + b[i]; return r; }
 
 // x-Jacobian of Eq. (elasticity-pde) (the rotated 1-D problem uses A only)
 M9 jac_x(double rho, double lam, double mu) {
@@ -123,7 +112,9 @@ void face_coefficients(const double n[3], int tag, double Zp, double Zs, double 
     Mm[7 * 9 + 3] = Zs > 0 ? -1 / Zs : 0.0;
     Mm[7 * 9 + 7] = 1;
   } else if (!nb) {
-    Mm = madd(Mm, mm(Mp, ghost(tag)));
+    const M9 G = ghost(tag);  // diagonal
+    for (int r : {0, 3, 6, 7})
+      for (int k : {0, 3, 6, 7}) Mm[r * 9 + k] += Mp[r * 9 + k] * G[k * 9 + k];
   }
   // normal pair (w1, w7) and tangential pair (w4, w8; w6, w9 alike): the rows of
   // traction and velocity, each from traction and velocity
@@ -412,8 +403,9 @@ void Ctx::face_flux(const MeshPlan& pl, int64_t eu, int f, double* Fm, double* F
 
 // Face f of user tet eu seen from its neighbour (interior, periodic and fault
 // faces): the neighbour tet and local face, and node_map[n] = the neighbour's
-// face node at the place of my face node n (the permutation the neighbour
-// kernel applies to the neighbour's trace); nb = -1 for faces without one.
+// face node at the place of my face node n (the friction solve's; the neighbour
+// kernels re-orient modes by the same vertex permutation); nb = -1 for faces
+// without one.
 void Ctx::face_neighbour(const MeshPlan& pl, const RefOps& o, int64_t eu, int f, int64_t* nb, int* nf,
                          int32_t* node_map) const {
   const int64_t e2 = pl.nbr[4 * eu + f];
@@ -532,7 +524,7 @@ void Ctx::setup() {
   gpar.assign((size_t)ng * GPAR, 0.0);
   // per element in parallel; LTS/fault slots are flagged here and numbered in
   // element order afterwards
-#pragma omp parallel for schedule(dynamic, 4096)
+#pragma omp parallel for schedule(dynamic, 256)
   for (int64_t i = 0; i < E; ++i) {
     const int64_t eu = order[i];
     for (int k = 0; k < 9; ++k) par[i * PAR + k] = Jinv[9 * eu + k];

@@ -5,15 +5,17 @@
 //   local kernel      Sec. 4.1: Cauchy-Kovalewski predictor
 //                       D^{k+1} = -sum_a KT_a D^k A*_a^T,  KT_a[m][l] = int phi_m dphi_l/dxi_a,
 //                     time integral I = sum_k dt^{k+1}/(k+1)! D^k (Eq. taylor),
-//                     volume sum_a K_a I A*_a^T, its own nodal face traces
-//                     (and LTS buffers / derivative traces); gravitational
-//                     faces (Sec. 4.3): exact (eta, H) Taylor recursion in
-//                     FP64 at the face nodes and that face's time-integrated
-//                     flux from int w1^b = -rho g H and int w7^b = eta^{n+1} - eta^n.
+//                     volume sum_a K_a I A*_a^T, traction and velocity of its
+//                     faces in the faces' modes (and LTS buffers / derivative
+//                     traces); gravitational faces (Sec. 4.3): exact (eta, H)
+//                     Taylor recursion in FP64 at the face nodes, driven by the
+//                     derivatives' traces, and the modes of the integrated
+//                     normal state int w1^b = -rho g H, int w7^b = eta^{n+1} - eta^n.
 //   neighbour kernel  Godunov fluxes of all four faces (Sec. 4.2, Eq.
-//                     numerical-flux): F^- on the own traces, F^+ on the
-//                     neighbours' (re-oriented by a node permutation), the
-//                     stored fluxes of gravitational and fault faces; one lift.
+//                     numerical-flux) mode by mode: the neighbour's modes
+//                     re-oriented to this side's, one middle state from the
+//                     face's coefficients (face_flux_state), gravitational
+//                     surfaces' normal states and fault fluxes added; one lift.
 // Dofs layout: Q[v][9][B] (basis fastest).  Face data: modal, see row_common.cuh.
 #pragma once
 #include <cmath>

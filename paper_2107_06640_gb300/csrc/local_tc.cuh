@@ -34,8 +34,9 @@
 // room goes to the surfaces' modes).
 //
 // What bounds it: the latency of a warp's own instruction stream (eight warps
-// per SM, 0.39 instructions per clock and scheduler), not a roof: 0.23 of the
-// HBM bandwidth, tensor pipe active 18 % of the time.  Local phase of the
+// per SM, 0.40 instructions per clock and scheduler), not a roof: DRAM 28 % busy
+// (0.32 of the copy bandwidth in needed bytes at 1,497,600 tets), tensor pipe
+// active 19 % of the time (374,400 tets, elastic launch).  Local phase of the
 // 183,456-tet degree-5 coupled box (all kinds): 788 us with 256 threads per
 // tile, five dense MMA rounds and nodal nine-quantity faces, 594 us now; plain
 // elastic launch of its 93,600-tet version 392 -> 266 us.  Degree 4: 593 -> 435 us;

@@ -17,8 +17,10 @@
 // 183,456-tet degree-5 box where this form takes 378; the nodal kernel before,
 // nine quantities staged and two tiles in flight, took 652.)
 //
-// What bounds it: shared-memory traffic (76 % of the L1 data pipe busy) and
-// instruction issue (49 %); 0.40 of the HBM bandwidth.
+// What bounds it: shared-memory traffic (L1 / shared-memory pipe 81 % busy) and
+// instruction issue (52 %); DRAM 50 % busy (374,400 tets; 0.66 of the copy
+// bandwidth in needed bytes at 1,497,600).  The 128 registers spill 36 bytes at
+// degree 5, up to 148 with LTS faces, none at degree 4.
 #pragma once
 #include <cuda_runtime.h>
 

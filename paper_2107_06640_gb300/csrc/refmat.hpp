@@ -12,9 +12,11 @@
 //
 // Face f of the tet is the face opposite vertex f; its vertices in increasing
 // local order (a,b,c) define x(chi) = Va + chi1 (Vb - Va) + chi2 (Vc - Va).
-// Face data are nodal on the (N+1)(N+2)/2 equispaced points of the reference
-// triangle, chi = (i1/N, i2/N); the point set is invariant under the six vertex
-// permutations, so re-orienting a neighbour's trace is a permutation of nodes.
+// Face nodes (of eta, the friction solve and adg_face_neighbour) are the
+// (N+1)(N+2)/2 equispaced points of the reference triangle, chi = (i1/N, i2/N);
+// the point set is invariant under the six vertex permutations, so that a
+// neighbour's node values are re-oriented by a permutation.  The element kernels'
+// face traces are modal (row_common.cuh, row_tables.cpp).
 #pragma once
 #include <vector>
 

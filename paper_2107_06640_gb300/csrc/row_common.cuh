@@ -20,7 +20,7 @@
 // What bounds them: FP64, the 2 FMA per clock and SM (the sparse form has 3.4
 // to 4 times fewer of them than dense nodal products, and no lane waits on an
 // operand; 87 % of the FP64 pipe busy at degree 5); FP32, instruction issue and
-// the latency of the copies (50 % of issue slots at degree 3).  Against one block per element with dense
+// the latency of the copies (50 to 58 % of issue slots at degree 3).  Against one block per element with dense
 // operands in global memory and block barriers between the levels: degree 3
 // FP64, 3,072 tets, 366 -> 110 us per step; degree 5 FP64, 33,696 tets, 17.0 ->
 // 4.4 ms; degree 3 FP32, 13,182 tets, 130 -> 30 us; 102,258 tets, 1.13 -> 0.22
@@ -102,9 +102,12 @@ __device__ __forceinline__ void rows_out(const T* sQ, T* Q, int nE, int lane) {
 // table, so blocks are as small as that allows: with at most eight warps per SM
 // single warps spread best (degree 3 FP64, 3,072 tets: 110 us per step with 32
 // threads, 120 with 128), above that 128 (13,182 tets, FP32: 29.7 with 128,
-// 32.6 with 32).  FP32 at degrees 4 and 5 holds one block of 256 per SM either
-// way, and its table is filled once instead of twice (183,456 tets: degree 5
-// 1106 -> 1028 us, degree 4 782 -> 759 us); at degree 3 256 is slower (225 -> 231).
+// 32.6 with 32).  FP32 at degrees 4 and 5 gains more from filling the table once
+// for eight warps instead of four (183,456 tets: degree 5 1106 -> 1028 us, degree 4
+// 782 -> 759 us) than degree 3 does (102,258 tets: 225 -> 231).  FP32 kernels are
+// held to 128 registers (two blocks of 256 per SM): at degree 4 the local ones
+// spill 288 to 400 bytes for it, at degree 5 20 to 320, below that nothing; FP64 at
+// degree 5 (255 registers) spills 250 to 500 bytes.
 template <class T, int N>
 inline int block_threads(int threads, int64_t units, int n_sms) {
   if (units <= (int64_t)kSmallLaunchWarps * n_sms) return 32;

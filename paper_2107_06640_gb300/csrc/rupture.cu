@@ -27,7 +27,11 @@
 // f = mu_s - (mu_s - mu_d) min(psi/D_c, 1), strength tau_S = C + f S and
 // |V| = max(0, Theta - tau_S)/eta_s in closed form, with the same time points
 // and two passes (psi advanced exactly for a frozen slip rate: psi + |V| h).
-// What bounds it: FP64 operations, 2 FMA per clock and SM.  So the nodes'
+// What bounds it: FP64 operations, 2 FMA per clock and SM: 19,200 nodes at degree
+// 4 are 150 blocks, one warp per scheduler (255 registers, 260 bytes of spill), and
+// while an SM has its block the FP64 pipe is busy 77 % of the time; the blocks
+// differ in what their nodes need (Newton iterations, the power of f_ss), an SM is
+// active 62 % of the launch.  So the nodes'
 // derivatives are projected to traction and velocity once for all time points,
 // reciprocals replace divisions, ln V is carried along, and asinh and its slope
 // take their asymptotes where those are exact: 19,200 nodes at degree 4, 374 ->

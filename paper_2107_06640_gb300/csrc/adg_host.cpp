@@ -652,8 +652,6 @@ void Ctx::setup() {
     dModal = upload_vec<float>(rt.modalT, owned, dev_bytes);
     dReorient = upload_vec<float>(rt.reorient, owned, dev_bytes);
   }
-  dNodal64 = fp64 ? (double*)dNodal : upload_raw(rt.nodalT, owned, dev_bytes);
-  dModal64 = fp64 ? (double*)dModal : upload_raw(rt.modalT, owned, dev_bytes);
   if (takes_noalloc() && noalloc_scratch() <= kNoallocScratch && !std::is_sorted(order.begin(), order.end())) {
     std::vector<double> par_u(par.size()), crec_u(crec.size());
     std::vector<int> nbr_u2(nbr.size()), ninfo_u(ninfo.size());
@@ -741,7 +739,7 @@ StepArgs Ctx::base_args() const {
   a.S = S; a.err = dErr; a.n_sms = n_sms;
   a.fslot = dFslot; a.drout = dDrout; a.gflux = dGflux; a.tc_local = dTcLocal; a.tc_lift = dTcLift;
   a.tiles = dTiles;
-  a.crec = dCrec; a.nodalT = dNodal; a.modalT = dModal; a.nodal64 = dNodal64; a.modal64 = dModal64; a.reorient = dReorient;
+  a.crec = dCrec; a.nodalT = dNodal; a.modalT = dModal; a.reorient = dReorient;
   return a;
 }
 

@@ -129,7 +129,6 @@ struct Ctx {
   void *dParUser = nullptr, *dCrecUser = nullptr;
   int *dNbrUser = nullptr, *dNinfoUser = nullptr;
   void *dCrec = nullptr, *dNodal = nullptr, *dModal = nullptr, *dReorient = nullptr;
-  double *dNodal64 = nullptr, *dModal64 = nullptr;
   int *dNbr = nullptr, *dNinfo = nullptr, *dGslot = nullptr, *dBslot = nullptr, *dDslot = nullptr,
       *dPerm = nullptr;
   unsigned int* dErr = nullptr;

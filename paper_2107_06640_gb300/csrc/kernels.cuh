@@ -69,7 +69,6 @@ struct StepArgs {
   const void* nodalT;    // T [Bf(r)][Bf(n)]    face modes at the face nodes, r-major
   const void* modalT;    // T [Bf(n)][Bf(r)]    face nodes to face modes, n-major
   int n_sms;             // of the context's GPU (read by the launchers)
-  const double *nodal64, *modal64;  // the same in FP64 (gravitational surfaces of the row kernels)
   const void* reorient;  // T [6][sum (n+1)^2]  a neighbour's face modes in this side's, blocks by degree
 };
 // Element of a virtual element, S scenarios per element: the 64-bit division

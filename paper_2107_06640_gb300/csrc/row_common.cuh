@@ -106,7 +106,7 @@ __device__ __forceinline__ void rows_out(const T* sQ, T* Q, int nE, int lane) {
 // for eight warps instead of four (183,456 tets: degree 5 1106 -> 1028 us, degree 4
 // 782 -> 759 us) than degree 3 does (102,258 tets: 225 -> 231).  FP32 kernels are
 // held to 128 registers (two blocks of 256 per SM): at degree 4 the local ones
-// spill 288 to 400 bytes for it, at degree 5 20 to 320, below that nothing; FP64 at
+// spill 288 to 400 bytes for it, at degree 5 20 to 304, below that nothing; FP64 at
 // degree 5 (255 registers) spills 250 to 500 bytes.
 template <class T, int N>
 inline int block_threads(int threads, int64_t units, int n_sms) {

@@ -191,7 +191,7 @@ template <class T, int N, bool kSpec>
 struct LocalSmem {
   using S = Shape<T, N>;
   static constexpr int nQ = (9 * EW * S::SB + 3) / 4 * 4, nT = (2 * 9 * EW * S::Bf + 3) / 4 * 4;
-  static constexpr int nD = kSpec ? 4 * EW * (N + 1) * S::Bf * (int)(sizeof(double) / sizeof(T)) : 0;
+  static constexpr int nD = kSpec ? 4 * EW * (N + 1) * S::Bf : 0;
   static constexpr int nN = 16 * EW;  // the faces' normals
   static constexpr int warp = (nQ + nN + nT + nD + 3) / 4 * 4;
   static constexpr int bytes(int threads) { return warp * (int)sizeof(T) * (threads / 32); }
@@ -343,31 +343,32 @@ __device__ __forceinline__ void fluid_face_out(const StepArgs& a, int64_t v0, in
 //   gravity          the modes of v_n - sigma_nn / Z, kept in shared memory for
 //                    surface() at the end
 // No level outlives its registers.  kOneGrav: at most one gravitational face
-// per element (the tensor-core kernels), whose surface works on forcing in the
-// dofs' precision; else the difference, the sums over its modes and the fluxes'
-// modes are FP64, also for FP32 dofs (their traces are in the dofs' precision).
-// Only the surface's own series is FP64 in both.  (Small coupled box, 1,500 steps,
-// error of eta against FP64 dofs: 1.0e-5 in FP32 and in 3xTF32, as with nodal
-// traces and fluxes.)
+// per element (the tensor-core kernels).
+// A surface's forcing is a difference that cancels for incoming waves: 1 / Z is
+// held in two values of T, so that the difference of the traces is exact to one
+// rounding of the result, as if formed in FP64 (with 1 / Z rounded to FP32 it was
+// 6e-3 off where the parts cancel to four millionths).  Its series is FP64.  (FP64
+// differences and sums for FP32 dofs made steps of small FP32 meshes with a sea
+// surface 2 to 9 % longer.  Error of eta against FP64 dofs, coupled boxes of 864
+// and 648 tets, degrees 3 to 5, FP32 and 3xTF32: 1.0e-5 to 1.4e-5 after 1,500 steps,
+// 0.7 to 1.03 times that of nodal traces with FP64 differences.)
 template <class T, int N, bool kOneGrav>
 struct SpecLevels {
   using S = Shape<T, N>;
   enum { NONE = 0, FINE = 1, GRAVITY = 2, FAULT = 3 };
-  using A = std::conditional_t<kOneGrav, T, double>;  // of a surface's modes
   static constexpr int values = (kOneGrav ? 1 : 4) * EW * (N + 1) * S::Bf;  // of sF
   const StepArgs& a;
   bool on;            // this lane holds a row
-  T* sT;              // staging as in faces_out
-  A* sF;              // the surfaces' modes [face][level][Bf]
+  T *sT, *sF;         // staging as in faces_out; the surfaces' modes [face][level][Bf]
   const T* sN;
   int64_t v0;
   int nE, lane;
   int what, slot;     // lane 4 j + f: of face f of element j
-  A iz;               // 1 / Z (gravity)
+  T iz, iz2;          // 1 / Z (gravity) rounded to T and what that leaves
   unsigned mask, surf;  // faces f to project; bit 4 j + f: a gravitational face
   __device__ __forceinline__ SpecLevels(const StepArgs& args, bool row, T* t, T* sf, const T* n, int64_t v, int e, int l)
-      : a(args), on(row), sT(t), sF(reinterpret_cast<A*>(sf)), sN(n), v0(v), nE(e), lane(l), what(NONE), slot(-1),
-        iz(A(0)) {
+      : a(args), on(row), sT(t), sF(sf), sN(n), v0(v), nE(e), lane(l), what(NONE), slot(-1), iz(T(0)),
+        iz2(T(0)) {
     if (lane < 4 * nE) {
       const int64_t ef = elem_of(v0 + (lane >> 2), a.S) * 4 + (lane & 3);
       const int kind = (a.ninfo[ef] >> 5) & 7;
@@ -378,7 +379,9 @@ struct SpecLevels {
         slot = a.gslot[ef];
         if (slot >= 0) {
           what = GRAVITY;
-          iz = (A)(1.0 / a.gpar[(size_t)slot * GPAR + 3]);
+          const double r = 1.0 / a.gpar[(size_t)slot * GPAR + 3];
+          iz = (T)r;
+          iz2 = (T)(r - (double)iz);
         }
       }
     }
@@ -389,12 +392,8 @@ struct SpecLevels {
   __device__ __forceinline__ int scenario(int j) const {
     return a.S == 1 ? 0 : (int)(v0 + j - elem_of(v0 + j, a.S) * a.S);
   }
-  static __device__ __forceinline__ const A* table(const void* t, const double* t64) {
-    if constexpr (kOneGrav) return reinterpret_cast<const A*>(t);
-    else return t64;
-  }
   // the surface modes of face f of element j
-  __device__ __forceinline__ A* face_modes(int j, int f) const {
+  __device__ __forceinline__ T* face_modes(int j, int f) const {
     return sF + (kOneGrav ? j : 4 * j + f) * (N + 1) * S::Bf;
   }
   template <int K, int F0>
@@ -419,7 +418,7 @@ struct SpecLevels {
     for (int i = lane; i < (2 * EW * Bf + 31) / 32 * 32; i += 32) {
       const int jf = i / Bf, n = i - jf * Bf, j = jf >> 1, f = F0 + (jf & 1);
       const int w = __shfl_sync(0xffffffffu, what, (4 * j + f) & 31), sl = __shfl_sync(0xffffffffu, slot, (4 * j + f) & 31);
-      const A z = __shfl_sync(0xffffffffu, iz, (4 * j + f) & 31);
+      const T z = __shfl_sync(0xffffffffu, iz, (4 * j + f) & 31), z2 = __shfl_sync(0xffffffffu, iz2, (4 * j + f) & 31);
       if (j >= nE || w == NONE) continue;
       const T* const s = sT + ((jf & 1) * 9 * EW + 9 * j) * Bf;
       T* const d = reinterpret_cast<T*>(a.dtrace) + ((int64_t)sl * a.S + scenario(j)) * (N + 1) * 9 * Bf;
@@ -447,8 +446,8 @@ struct SpecLevels {
 #pragma unroll
         for (int k = 0; k < 6; ++k) d[K * S::FS + 6 * n + k] = o[k];
       } else {
-        face_modes(j, f)[K * Bf + n] = (A)fma(o[5], c[2], fma(o[4], c[1], o[3] * c[0])) -
-                                       (A)fma(o[2], c[2], fma(o[1], c[1], o[0] * c[0])) * z;
+        const T vn = fma(o[5], c[2], fma(o[4], c[1], o[3] * c[0])), tn = fma(o[2], c[2], fma(o[1], c[1], o[0] * c[0]));
+        face_modes(j, f)[K * Bf + n] = fma(-tn, z2, fma(-tn, z, vn));
       }
     }
     __syncwarp();
@@ -463,7 +462,6 @@ struct SpecLevels {
   // series in FP64, then the modes of -rho g H and eta^{n+1} - eta^n.
   __device__ void surface(const Seg& sg) const {
     constexpr int Bf = S::Bf;
-    A* const sH = reinterpret_cast<A*>(sT);
     unsigned left = surf;
     while (left) {
       int face[EW];  // 4 j + f, or -1
@@ -478,17 +476,17 @@ struct SpecLevels {
         const int i = lane + 32 * it, c = i < EW * Bf ? i / Bf : 0, n = i - c * Bf, jf = which(c);
         const int gs = __shfl_sync(0xffffffffu, slot, jf & 31);
         if (i >= EW * Bf || jf < 0) continue;
-        const A* const F = face_modes(jf >> 2, jf & 3);
+        const T* const F = face_modes(jf >> 2, jf & 3);
         const double* const gp = a.gpar + (size_t)gs * GPAR;
         double* const eta = a.eta + ((int64_t)gs * a.S + scenario(jf >> 2)) * Bf + n;
         const double kappa = gp[4], rg = gp[5], dt = sg.dt, eta0 = *eta;
-        const A* const nd = table(a.nodalT, a.nodal64) + n;
-        A acc[N + 1];
+        const T* const nd = reinterpret_cast<const T*>(a.nodalT) + n;
+        T acc[N + 1];
 #pragma unroll
-        for (int m = 0; m <= N; ++m) acc[m] = A(0);
+        for (int m = 0; m <= N; ++m) acc[m] = T(0);
 #pragma unroll
         for (int r = 0; r < Bf; ++r) {
-          const A w = nd[r * Bf];
+          const T w = nd[r * Bf];
 #pragma unroll
           for (int m = 0; m <= N; ++m)
             if (r < nb2(N - m)) acc[m] = fma(w, F[m * Bf + r], acc[m]);
@@ -508,8 +506,8 @@ struct SpecLevels {
         for (int m = N + 1; m < N + 40; ++m)
           if (fabs(term(m, 0.0)) <= 1e-17 * fabs(e1)) break;
         *eta = e1;
-        sH[c * 2 * Bf + n] = (A)(-rg * H);
-        sH[(c * 2 + 1) * Bf + n] = (A)(e1 - eta0);
+        sT[c * 2 * Bf + n] = (T)(-rg * H);
+        sT[(c * 2 + 1) * Bf + n] = (T)(e1 - eta0);
       }
       __syncwarp();
 #pragma unroll 1
@@ -517,17 +515,17 @@ struct SpecLevels {
         const int i = lane + 32 * it, c = i < EW * Bf ? i / Bf : 0, r = i - c * Bf, jf = which(c);
         const int gs = __shfl_sync(0xffffffffu, slot, jf & 31);
         if (i >= EW * Bf || jf < 0) continue;
-        const A* const mn = table(a.modalT, a.modal64) + r;
-        A h = A(0), d = A(0);
+        const T* const mn = reinterpret_cast<const T*>(a.modalT) + r;
+        T h = T(0), d = T(0);
 #pragma unroll
         for (int n = 0; n < Bf; ++n) {
-          const A w = mn[n * Bf];
-          h = fma(w, sH[c * 2 * Bf + n], h);
-          d = fma(w, sH[(c * 2 + 1) * Bf + n], d);
+          const T w = mn[n * Bf];
+          h = fma(w, sT[c * 2 * Bf + n], h);
+          d = fma(w, sT[(c * 2 + 1) * Bf + n], d);
         }
         T* const out = reinterpret_cast<T*>(a.gflux) + ((int64_t)gs * a.S + scenario(jf >> 2)) * 9 * Bf + r;
-        out[0] = (T)h;
-        out[Bf] = (T)d;
+        out[0] = h;
+        out[Bf] = d;
       }
       __syncwarp();
     }

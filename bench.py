@@ -114,8 +114,8 @@ def tc_local_flops(N):
 # acoustic local, neighbour), from the one-kernel ncu captures of the
 # 374,400-tet box (profiles/tensor_core_kernels_box40.md); a launch's traffic
 # is scaled from them by its elements of each kind
-TC_DRAM_BYTES_PER_ELEMENT = {"local_tc_kernel": 6450.4, "local_tc_kernel_acoustic": 3753.6,
-                             "neighbour_tc_kernel": 7841.6}
+TC_DRAM_BYTES_PER_ELEMENT = {"local_tc_kernel": 6452.6, "local_tc_kernel_acoustic": 3755.2,
+                             "neighbour_tc_kernel": 7840.0}
 
 
 def load_peaks():
